@@ -23,6 +23,11 @@ int launch_gemv(const int8_t *a, const float *a_scale, const void *x_bf16, int8_
                 int count, const uint32_t *const *packed, const float *const *w_scale, float *const *y,
                 const int *N, const int *ldy, int M, int K, int group, cudaStream_t st);
 
+bool stat_takes(int M, int K, int group, int tiles, int count, bool h16);
+int launch_stat(const int8_t *a, const float *a_scale, int count, const uint32_t *const *packed,
+                const void *const *w_scale, void *const *y, const int *N, const int *ldy, int M, int K, int group,
+                cudaStream_t st, bool h16, bool y16);
+
 bool prefill_supported(int M, int N, int K, int group);
 bool prefill_preferred(int M, int N, int K, int group, bool can_split);
 size_t prefill_workspace_bytes(int M, int N, int K, int group);
@@ -496,6 +501,8 @@ int gemm_dispatch(const int8_t *a, const float *a_scale, const uint32_t *packed,
                              reinterpret_cast<char *>(y) + (size_t)n_tc * y_bytes, nullptr, M, N - n_tc, K,
                              group, rest, workspace, (cudaStream_t)stream, h16, y16, a16, N);
     }
+    if (!a16 && !partials && stat_takes(M, K, group, N / 16, 1, h16))
+        return launch_stat(a, a_scale, 1, &packed, &w_scale, &y, &N, &N, M, K, group, (cudaStream_t)stream, h16, y16);
     return launch_decode(a, a_scale, packed, w_scale, y, partials, M, N, K, group, si, workspace,
                          (cudaStream_t)stream, h16, y16, a16, N);
 }
@@ -568,7 +575,7 @@ static int grouped_plan(int count, const int *N, int M, int K, int group, int fu
     if (have_x && fuse != W2A8_FUSE_OFF && gemv_can_fuse(M, K, group) &&
         (fuse == W2A8_FUSE_ON || gemv_fuse_preferred(M, K, group)))
         plan = 3;
-    else if (gemv_preferred(M, K, group, tiles, count))
+    else if (stat_takes(M, K, group, tiles, count, false) || gemv_preferred(M, K, group, tiles, count))
         plan = 1;
     return plan;
 }
@@ -616,6 +623,11 @@ static int grouped_common(const void *x_bf16, const int8_t *a_in, const float *a
         a_in = a;
         a_scale_in = a_scale;
     }
+    int tiles = 0;
+    for (int i = 0; i < count; ++i) tiles += N[i] / 16;
+    if (plan == 1 && stat_takes(M, K, group, tiles, count, false))
+        return launch_stat(a_in, a_scale_in, count, packed, reinterpret_cast<const void *const *>(w_scale),
+                           reinterpret_cast<void *const *>(y), N, N, M, K, group, (cudaStream_t)stream, false, false);
     if (plan == 1)          // one launch over all matrices
         return launch_gemv(a_in, a_scale_in, nullptr, nullptr, nullptr, count, packed, w_scale, y, N, N, M, K, group,
                            (cudaStream_t)stream);

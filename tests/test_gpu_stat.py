@@ -1,0 +1,76 @@
+"""GPU parity of the streaming kernel with stationary activations (9 .. 32 tokens) against the CPU
+reference: edges of token slabs, half channel pairs, every scale group form, K shares with unequal
+block counts, cells cut between warps, several rounds of pairs, grouped matrices, both scale types."""
+import numpy as np
+import pytest
+
+from conftest import Guarded
+from paper_2508_06753_b200 import synth
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-4
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2508_06753_b200 import binding, build
+    build.build()
+    binding.lib()
+    return torch, binding
+
+
+def _dev(torch, arr):
+    return torch.from_numpy(np.ascontiguousarray(arr)).cuda()
+
+
+CASES = [
+    # M, K, [N], group (0 = K), forced K shares (0 = the plan's)
+    (9, 256, [16], 64, 0),                    # one cell, half a pair
+    (16, 512, [48, 16], 128, 0),              # half pairs at the end of both matrices
+    (17, 1280, [64], 64, 2),                  # shares of 2 and 3 blocks
+    (24, 1792, [160, 32], 256, 3),
+    (25, 2048, [4096], 0, 2),                 # one scale per channel
+    (32, 4096, [4096, 1024, 1024], 64, 4),
+    (32, 14336, [272], 64, 0),                # long rows: eight shares
+    (31, 512, [20480], 128, 1),               # no cluster, several rounds of pairs
+    (1, 1024, [96], 64, 0),                   # forced below its range: a single token
+    (8, 4352, [80], 64, 2),
+]
+
+
+@pytest.mark.parametrize("h16", [False, True])
+@pytest.mark.parametrize("M,K,Ns,group,shares", CASES)
+def test_stat_against_reference(gpu, oracle, monkeypatch, M, K, Ns, group, shares, h16):
+    torch, b = gpu
+    monkeypatch.setenv("W2A8_STAT", "2")
+    if shares:
+        monkeypatch.setenv("W2A8_STAT_C", str(shares))
+    g = K if group == 0 else group
+    mats = [synth.make_linear(5 * M + K + i, K, N, g) for i, N in enumerate(Ns)]
+    if h16:
+        mats = [(c, s.astype(np.float16)) for c, s in mats]
+    bits = synth.activations_bf16(M + K, M, K, 0.01)
+    a, s_a = b.a8_quantize(_dev(torch, bits.view(np.int16)).view(torch.bfloat16))
+    packed, scales = [b.w2_pack(_dev(torch, c)) for c, _ in mats], [_dev(torch, s) for _, s in mats]
+    ws = b.new_workspace(b.w2a8_grouped_workspace_bytes(Ns, M, K, g))
+    ys = []
+    for _ in range(2):
+        guards = [Guarded(torch, (M, N), torch.float32, float("nan")) for N in Ns]
+        if h16:
+            for pk, sc, gd in zip(packed, scales, guards):
+                b.w2a8_gemm_h16(a, s_a, pk, sc, g, ws, y=gd.view)
+        else:
+            b.w2a8_gemm_grouped(a, s_a, b.Group(packed, scales), g, ws, y=[gd.view for gd in guards])
+        torch.cuda.synchronize()
+        for gd in guards:
+            gd.check("y")
+        ys.append([gd.view.clone() for gd in guards])
+    a_ref, s_ref = oracle.quantize(bits)
+    for (codes, s_w), y, again in zip(mats, *ys):
+        assert torch.equal(y, again)
+        ref = oracle.gemm(a_ref, s_ref, codes, s_w.astype(np.float32), g)
+        err = np.abs(y.cpu().numpy().astype(np.float64) - ref).max(axis=1)
+        assert (err <= TOL * np.abs(ref).max(axis=1)).all(), float(err.max())
