@@ -133,9 +133,9 @@ int w2a8_workspace_status(const void *workspace, void *stream);
  * read once per slab of up to 32 tokens): the one-shot kernel when the problem
  * is about one wave of its CTAs, the persistent one (at most 32 tokens,
  * K % 256 == 0) for small matrices with K <= 4096 and for problems of more
- * than one wave; and the one with stationary activations (9 .. 32 tokens,
- * K % 256 == 0), which unpacks every weight once for all tokens, for the larger
- * problems.  w2a8_kernel_for reports tensor-core or streaming.
+ * than one wave; and the one with stationary activations (5 .. 256 tokens,
+ * K % 256 == 0), which unpacks every weight once per 64 tokens, where its estimate
+ * is ahead: larger problems of few tokens, smaller ones of many.  w2a8_kernel_for reports tensor-core or streaming.
  * A problem given to the tensor-core kernel may leave its last (at most
  * eight) 128-channel tiles to the streaming kernel, as a second launch on the
  * same stream (w2a8_tensor_core_channels); the result does not depend on it
@@ -282,7 +282,7 @@ int w2a8_gemm_partials(const int8_t *a, const uint32_t *packed, int32_t *partial
  *   workspace                      w2a8_grouped_workspace_bytes(count, N, M, K, group)
  * Each y[i] holds what w2a8_gemm computes for matrix i: bit for bit when both
  * calls take the same kernel, except that the kernel with stationary activations
- * (9 .. 32 tokens, larger problems) deals the work of a launch to its CTAs as a
+ * (more than four tokens, larger problems) deals the work of a launch to its CTAs as a
  * whole, so there the order of the fp32 additions may differ.  With any kernel
  * it is within the tolerance of w2a8_gemm's contract and repeated calls give
  * equal bits.

@@ -44,10 +44,54 @@ int launch_prefill_f16(const void *x_bf16, const float *a_scale, const uint32_t 
                        int ldy);
 int launch_a8_to_bf16(const int8_t *a, void *scratch, int M, int K, cudaStream_t st);
 
-int env_int(const char *name, int dflt) {
-    const char *v = getenv(name);
-    return (v && *v) ? atoi(v) : dflt;
+// ---- W2A8_* switches of the environment ---------------------------------------------
+// A call asks for some forty of them; reading each with getenv was 2 us of a call that launches a 2 us
+// kernel.  Values are kept per thread, together with a fingerprint of the environment block: the
+// addresses of its strings (the C library makes a new string whenever a variable is set to a new value,
+// so any change moves the fingerprint).  Inside an EnvScope, i.e. once per call, the fingerprint is taken
+// once.
+extern "C" char **environ;
+namespace {
+struct EnvCache {
+    uint64_t print = 0;
+    int depth = 0, n = 0;
+    struct { const char *name; bool set; int value; } entry[64];
+};
+thread_local EnvCache t_env;
+
+uint64_t take_fingerprint() {
+    uint64_t h = 1469598103934665603ull;
+    for (char **e = environ; e && *e; ++e) h = (h ^ (uint64_t)(uintptr_t)*e) * 1099511628211ull;
+    return h;
 }
+void refresh_env(EnvCache &c) {
+    const uint64_t h = take_fingerprint();
+    if (h != c.print) { c.print = h; c.n = 0; }
+}
+// the variable's entry; names are string literals, so equal addresses are equal names (the same name at
+// two addresses just gets two entries)
+bool env_lookup(const char *name, int *value) {
+    EnvCache &c = t_env;
+    if (c.depth == 0) refresh_env(c);
+    for (int i = 0; i < c.n; ++i)
+        if (c.entry[i].name == name) { *value = c.entry[i].value; return c.entry[i].set; }
+    const char *v = getenv(name);
+    const bool set = v && *v;
+    *value = set ? atoi(v) : 0;
+    if (c.n < 64) { c.entry[c.n] = {name, set, *value}; ++c.n; }
+    return set;
+}
+}  // namespace
+
+EnvScope::EnvScope() { if (t_env.depth++ == 0) refresh_env(t_env); }
+EnvScope::~EnvScope() { --t_env.depth; }
+
+uint64_t env_fingerprint() {
+    if (t_env.depth == 0) refresh_env(t_env);
+    return t_env.print;
+}
+bool env_set(const char *name) { int v; return env_lookup(name, &v); }
+int env_int(const char *name, int dflt) { int v; return env_lookup(name, &v) ? v : dflt; }
 
 bool pdl_enabled() {
     static const bool on = env_int("W2A8_PDL", 1) != 0;
@@ -336,6 +380,7 @@ static size_t kernel_workspace_bytes(int M, int N, int K, int group) {
 }
 
 size_t w2a8_workspace_bytes(int M, int N, int K, int group) {
+    EnvScope scope;
     size_t need = kernel_workspace_bytes(M, N, K, group);
     if (need == 0) return 0;
     // the 16-bit tensor-core kernel reads the int8 activations from a bf16 copy kept behind that
@@ -372,7 +417,8 @@ static bool takes_tensor_core_kernel_ex(int M, int N, int K, int group, bool can
 }
 // int8 activations: the int8 kernel can split K for problems with few output tiles, the 16-bit one cannot
 static bool takes_tensor_core_kernel(int M, int N, int K, int group) {
-    return takes_tensor_core_kernel_ex(M, N, K, group, !tensor_core_kind_is_16(M, N, K, group));
+    return takes_tensor_core_kernel_ex(M, N, K, group, !tensor_core_kind_is_16(M, N, K, group)) &&
+           !stat_takes(M, K, group, N / 16, 1, false);
 }
 
 // Channels the tensor-core kernel takes (the rest, if any, goes to the streaming kernel in a
@@ -413,6 +459,7 @@ int w2a8_tensor_core_kind(int M, int N, int K, int group) {
 }
 
 int w2a8_kernel_for(int M, int N, int K, int group) {
+    EnvScope scope;
     ShapeInfo si;
     if (!shape_ok(M, N, K, group, &si)) return W2A8_ERR_SHAPE;
     return takes_tensor_core_kernel(M, N, K, group) ? 1 : 0;
@@ -467,6 +514,8 @@ size_t gemm_header_bytes(int M, int N, int K, int group) {
 int gemm_dispatch(const int8_t *a, const float *a_scale, const uint32_t *packed, const void *w_scale,
                   void *y, int32_t *partials, int M, int N, int K, int group, const ShapeInfo &si,
                   void *workspace, void *stream, bool h16, bool y16, bool a16) {
+    if (!a16 && !partials && stat_takes(M, K, group, N / 16, 1, h16))
+        return launch_stat(a, a_scale, 1, &packed, &w_scale, &y, &N, &N, M, K, group, (cudaStream_t)stream, h16, y16);
     const bool takes = a16 ? takes_tensor_core_kernel_ex(M, N, K, group, false) : takes_tensor_core_kernel(M, N, K, group);
     const bool tc16 = !h16 && takes && prefill_f16_supported(M, N, K, group) &&
                       (a16 || tensor_core_kind_is_16(M, N, K, group));
@@ -501,8 +550,6 @@ int gemm_dispatch(const int8_t *a, const float *a_scale, const uint32_t *packed,
                              reinterpret_cast<char *>(y) + (size_t)n_tc * y_bytes, nullptr, M, N - n_tc, K,
                              group, rest, workspace, (cudaStream_t)stream, h16, y16, a16, N);
     }
-    if (!a16 && !partials && stat_takes(M, K, group, N / 16, 1, h16))
-        return launch_stat(a, a_scale, 1, &packed, &w_scale, &y, &N, &N, M, K, group, (cudaStream_t)stream, h16, y16);
     return launch_decode(a, a_scale, packed, w_scale, y, partials, M, N, K, group, si, workspace,
                          (cudaStream_t)stream, h16, y16, a16, N);
 }
@@ -514,6 +561,7 @@ static int gemm_common(const int8_t *a, const float *a_scale, const uint32_t *pa
                        const void *w_scale, void *y, int32_t *partials, int M, int N, int K,
                        int group, void *workspace, size_t workspace_bytes, void *stream,
                        bool h16 = false, bool y16 = false, bool a16 = false) {
+    EnvScope scope;
     ShapeInfo si;
     if (!shape_ok(M, N, K, group, &si)) return W2A8_ERR_SHAPE;
     if (!aligned16(a) || !aligned16(packed) || (y && !aligned16(y)) ||
@@ -581,6 +629,7 @@ static int grouped_plan(int count, const int *N, int M, int K, int group, int fu
 }
 
 size_t w2a8_grouped_workspace_bytes(int count, const int *N, int M, int K, int group) {
+    EnvScope scope;
     if (count < 1 || count > kMaxGroup || !N) return 0;
     size_t need = 0;
     for (int i = 0; i < count; ++i) {
@@ -599,6 +648,7 @@ static int grouped_common(const void *x_bf16, const int8_t *a_in, const float *a
                           int count, const uint32_t *const *packed, const float *const *w_scale, float *const *y,
                           const int *N, int M, int K, int group, int fuse, void *workspace, size_t workspace_bytes,
                           void *stream) {
+    EnvScope scope;
     if (!packed || !w_scale || !y || !N) return W2A8_ERR_NULL;
     const int plan = grouped_plan(count, N, M, K, group, fuse, x_bf16 != nullptr);
     if (plan < 0) return plan;
@@ -664,6 +714,7 @@ int w2a8_linear(const void *x_bf16, int8_t *a, float *a_scale, const uint32_t *p
 }
 
 size_t w2a8_linear_host_workspace_bytes(int M, int N, int K, int group) {
+    EnvScope scope;
     const size_t g = w2a8_workspace_bytes(M, N, K, group);
     if (g == 0) return 0;
     return up256(g) + up256((size_t)M * K * 2) + up256((size_t)M * K) + up256((size_t)M * 4) +
@@ -687,6 +738,7 @@ static void *mapped_device_pointer(const void *host) {
 int w2a8_linear_host(const void *x_host, int M, int K, const uint32_t *packed,
                      const float *w_scale, int N, int group, float *y_host, void *workspace,
                      size_t workspace_bytes, void *stream) {
+    EnvScope scope;
     if (!x_host || !packed || !w_scale || !y_host) return W2A8_ERR_NULL;
     const size_t need = w2a8_linear_host_workspace_bytes(M, N, K, group);
     if (need == 0) return W2A8_ERR_SHAPE;
@@ -722,6 +774,7 @@ int w2a8_linear_host(const void *x_host, int M, int K, const uint32_t *packed,
 }
 
 size_t w2a8_linear_grouped_host_workspace_bytes(int count, const int *N, int M, int K, int group) {
+    EnvScope scope;
     const size_t g = w2a8_grouped_workspace_bytes(count, N, M, K, group);
     if (g == 0) return 0;
     size_t need = up256(g) + up256((size_t)M * K * 2) + up256((size_t)M * K) + up256((size_t)M * 4);
@@ -732,6 +785,7 @@ size_t w2a8_linear_grouped_host_workspace_bytes(int count, const int *N, int M, 
 int w2a8_linear_grouped_host(const void *x_host, int M, int K, int count, const uint32_t *const *packed,
                              const float *const *w_scale, const int *N, int group, float *const *y_host,
                              void *workspace, size_t workspace_bytes, void *stream) {
+    EnvScope scope;
     if (!x_host || !packed || !w_scale || !N || !y_host) return W2A8_ERR_NULL;
     const size_t need = w2a8_linear_grouped_host_workspace_bytes(count, N, M, K, group);
     if (need == 0) return W2A8_ERR_SHAPE;

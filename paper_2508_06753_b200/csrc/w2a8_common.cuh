@@ -197,6 +197,12 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
     return launch_kernel_cluster(kernel, grid, block, smem, stream, pdl, 1u, static_cast<Args &&>(args)...);
 }
 
+// Switches of the environment (W2A8_*): the value of a variable that is set and not empty, else dflt.
+int env_int(const char *name, int dflt);
+bool env_set(const char *name);
+uint64_t env_fingerprint();      // changes whenever the environment does
+struct EnvScope { EnvScope(); ~EnvScope(); };      // one look at the environment for the calls inside
+
 bool pdl_enabled();
 int check_device();  // W2A8_OK or W2A8_ERR_ARCH / W2A8_ERR_CUDA
 

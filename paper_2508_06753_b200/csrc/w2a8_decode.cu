@@ -485,7 +485,6 @@ w2a8_decode_kernel(const DecodeParams p) {
 }
 
 // ---- host side -----------------------------------------------------------------
-int env_int(const char *name, int dflt);
 bool gemv_preferred(int M, int K, int group, int tiles, int count);
 int launch_gemv(const int8_t *a, const float *a_scale, const void *x_bf16, int8_t *a_out, float *a_scale_out,
                 int count, const uint32_t *const *packed, const float *const *w_scale, float *const *y,
@@ -566,17 +565,8 @@ static DecodePlan decode_plan_uncached(int M, int N, int K, const ShapeInfo &si,
 }
 
 // The plan depends on the shape and on the W2A8_* switches of the environment.  Every entry
-// point asks for it two to four times per call (workspace check, launch), and each evaluation
-// reads a dozen environment variables, so the last plan is kept per thread together with a
-// fingerprint of the environment block: the addresses of its strings (the C library makes a
-// new string whenever a variable is set to a new value, so any change moves the fingerprint).
-extern "C" char **environ;
-static uint64_t env_fingerprint() {
-    uint64_t h = 1469598103934665603ull;
-    for (char **e = environ; e && *e; ++e) h = (h ^ (uint64_t)(uintptr_t)*e) * 1099511628211ull;
-    return h;
-}
-
+// point asks for it two to four times per call (workspace check, launch), so the last plan is kept per
+// thread together with the fingerprint of the environment.
 static DecodePlan decode_plan(int M, int N, int K, const ShapeInfo &si, bool h16 = false) {
     struct Key { int M, N, K, G, h16, dev; uint64_t env; };
     thread_local Key key = {0, 0, 0, 0, 0, -2, 0};

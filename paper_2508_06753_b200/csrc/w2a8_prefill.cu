@@ -530,7 +530,6 @@ __global__ void pf_splitk_reduce_kernel(const float *__restrict__ split_out, voi
 }
 
 // ---- host side -----------------------------------------------------------------------
-int env_int(const char *name, int dflt);
 
 // Unpack warps (warp layout) by scale group; W2A8_PF_UNPACK_WARPS = 2 or 4 overrides.
 int prefill_unpack_warps(int group) {
@@ -622,6 +621,20 @@ bool prefill_preferred(int M, int N, int K, int group, bool can_split) {
     }
     const double t_stream = kStreamSecondsPerMac * (double)M * (double)N * (double)K;
     return t_tc * (950000.0 / 875000.0) < t_stream;
+}
+
+// Expected time of a problem on the faster of the tensor-core path and the one-shot streaming kernel.
+double many_token_seconds(int M, int N, int K, int group) {
+    double t = kStreamSecondsPerMac * (double)M * (double)N * (double)K;
+    if (!prefill_supported(M, N, K, group)) return t;
+    const double t_tc = prefill_seconds(M, N, K, group, prefill_ksplit(M, N, K, group));
+    if (t_tc < t) t = t_tc;
+    if (prefill_uses_wide(M, N, K, group)) {
+        int c;
+        const double t_wide = split_plan(M, N, K, 256, kWideRoundSecondsPerK, &c);
+        if (t_wide < t) t = t_wide;
+    }
+    return t;
 }
 
 bool prefill_wide_supported(int M, int N, int K, int group);

@@ -24,7 +24,6 @@
 
 namespace w2a8 {
 
-int env_int(const char *name, int dflt);
 
 // Four warpgroups, with the register file re-balanced between them at kernel entry (setmaxnreg):
 //   warps 0-3   two MMA issuers, the TMA producer, one spare       (56 registers per thread)

@@ -280,7 +280,6 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
 }
 
 // ---- host side -----------------------------------------------------------------------
-int env_int(const char *name, int dflt);
 
 bool prefill_wide_supported(int M, int N, int K, int group) {
     if (group != K) return false;

@@ -1,5 +1,5 @@
-// Streaming kernel with stationary activations (9 .. 32 tokens): the weights stream once past
-// activations that stay in shared memory, and every weight is unpacked once for all tokens.
+// Streaming kernel with stationary activations (a few to a few hundred tokens): the weights stream past
+// activations that stay in shared memory, and every weight is unpacked once per group of up to 64 tokens.
 //
 //  * Work.  A cluster of C CTAs owns a contiguous range of channel pairs (32 channels); rank r of it
 //    owns the r-th share of the 256-k blocks (K-splitting of Sec. II-D) and keeps the activations of
@@ -12,19 +12,20 @@
 //  * Inner step: mma.sync m16n8k32 int8, the weight tile as the 16-row operand (w2a8_cell.cuh).  Two
 //    tiles share each activation fragment, so a fragment is read from shared memory once per 32
 //    channels.
+//  * One CTA of 8 warps per SM with up to 255 registers: two warps per scheduler, but enough registers for
+//    the compiler to keep many MMAs in flight.  Against two CTAs (128 registers) or 16 and 12 warps:
+//    14336 x 4096 at 32 tokens 12.9 / 13.7 us, at 64 tokens 22.1 / 26.9; 8192 x (28672 + 28672) at 16 tokens
+//    35.3 / 44.
 //  * Bound.  32 tokens: issue slots (about 540 warp instructions per cell, of which 64 MMAs, 128 packed
-//    promotions and 112 of unpack) and, on small problems, the 4 to 5 us that a launch costs beside the
-//    stream: a cold prologue, the activations after the dependency wait, two cluster barriers.
-//    Measured (us per launch, group 64, back to back over distinct weights; before / this kernel):
-//    gate|up 4096 x (14336 + 14336) at 32 tokens 29.3 / 19.3, 8192 x (28672 + 28672) 133 / 71.
-#include <stdlib.h>
-
+//    promotions and 112 of unpack); 64 tokens: the MMA pipe at half its rate (425 of 1190 TOPS with 2 warps
+//    per scheduler); small problems: the 4 to 5 us that a launch costs beside the stream (a cold prologue, the
+//    activations after the dependency wait, two cluster barriers).
 #include "w2a8_cell.cuh"
 
 namespace w2a8 {
 
-int env_int(const char *name, int dflt);
 bool gemv_preferred(int M, int K, int group, int tiles, int count);
+double many_token_seconds(int M, int N, int K, int group);
 
 constexpr int kStMaxMats = 4;
 constexpr int kStWSlot = 4 * 32 * 16;         // weights of a cell: four channel rows per lane x 16 B
@@ -52,6 +53,7 @@ struct StParams {
     uint32_t nb_inv[2];           // ceil(65536 / n) for n = blk_per, blk_per + 1
     int pair_per, pair_extra;     // cluster c owns pair_per (+ 1 if c < pair_extra) pairs
     int round_pairs;              // pairs per round = sum slots
+    int tgroups;                  // token groups of 8 * MT tokens; neighbouring clusters take the same pairs of different groups
     int y16;
     int pairs;                    // (host)
 };
@@ -65,12 +67,14 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t local, uint32_t rank
     return v;
 }
 
-// MT: 8-token slabs; SPP: 64-k slices per scale group (capped at 4); H16: binary16 scales; W: warps
-// per CTA -- 8 (two CTAs per SM) or 16 (one); RING: landing slots (cells) per warp.
-template <int MT, int SPP, bool H16, int W, int RING>
-__global__ void __launch_bounds__(W * 32, 16 / W)
+constexpr int kStWarps = 8;
+
+// MT: 8-token slabs of a token group; SPP: 64-k slices per scale group (capped at 4); H16: binary16
+// scales; RING: landing slots (cells) per warp.
+template <int MT, int SPP, bool H16, int RING>
+__global__ void __launch_bounds__(kStWarps * 32, 1)
 w2a8_stat_kernel(const __grid_constant__ StParams p) {
-    constexpr int kThreads = W * 32;
+    constexpr int W = kStWarps, kThreads = W * 32;
     constexpr int SPB = 4 / SPP;                    // scales per block and channel
     constexpr int kActBlock = 8 * MT * 256;         // activations of one block in shared memory
     constexpr int kSlotFloats = MT * 2 * 32 * 4;    // sums of one pair
@@ -81,6 +85,9 @@ w2a8_stat_kernel(const __grid_constant__ StParams p) {
     const int C = p.C, rank = C > 1 ? (int)cluster_ctarank() : 0;
     int cl;
     asm("mov.u32 %0, %%clusterid.x;" : "=r"(cl));
+    int m_base = 0;                        // first token of this cluster's group
+    if (p.tgroups > 1) { const int all = cl; cl = all / p.tgroups; m_base = (all - cl * p.tgroups) * (8 * MT); }
+    const int mrows = min(8 * MT, p.M - m_base);
     // (shares computed on the host: a launch runs its prologue once, and divisions are long cold code)
     const int kb_lo = rank * p.blk_per + min(rank, p.blk_extra), nb = p.blk_per + (rank < p.blk_extra ? 1 : 0);
     const uint32_t nb_inv = rank < p.blk_extra ? p.nb_inv[1] : p.nb_inv[0];
@@ -193,15 +200,15 @@ w2a8_stat_kernel(const __grid_constant__ StParams p) {
         const int ch = (threadIdx.x & 15) * 16;
         int m = threadIdx.x >> 4, kb = 0;
         for (;;) {
-            while (m >= p.M) { m -= p.M; ++kb; }
+            while (m >= mrows) { m -= mrows; ++kb; }
             if (kb >= nb) break;
             cp_async16(act_u32 + kb * kActBlock + m * 256 + (ch ^ ((m & 1) << 6)),
-                       p.a + (size_t)m * p.K + (kb_lo + kb) * kBlockK + ch);
+                       p.a + (size_t)(m_base + m) * p.K + (kb_lo + kb) * kBlockK + ch);
             m += kThreads / 16;
         }
     }
     cp_async_commit();
-    if (threadIdx.x < 8 * MT) tok_scale[threadIdx.x] = p.a_scale[min((int)threadIdx.x, p.M - 1)] * (1.0f / kCodeGain);
+    if (threadIdx.x < 8 * MT) tok_scale[threadIdx.x] = p.a_scale[m_base + min((int)threadIdx.x, mrows - 1)] * (1.0f / kCodeGain);
     cp_async_wait_all();
     __syncthreads();
     const uint32_t b_even = act_u32 + gq * 256 + t * 16 + ((gq & 1) << 6), b_odd = b_even - ((gq & 1) << 7);
@@ -377,16 +384,16 @@ w2a8_stat_kernel(const __grid_constant__ StParams p) {
             if (n0 + i * 16 < p.mat[mi].N) {
                 const size_t ldy = p.mat[mi].ldy;
                 const int m = mt * 8 + 2 * t;
-                const size_t at = m * ldy + n0 + i * 16 + gq;
+                const size_t at = (size_t)(m_base + m) * ldy + n0 + i * 16 + gq;
                 const float s0 = tok_scale[m], s1 = tok_scale[m + 1];
                 if (H16 && p.y16) {
                     __nv_bfloat16 *y = reinterpret_cast<__nv_bfloat16 *>(p.mat[mi].y) + at;
-                    if (m < p.M) { y[0] = __float2bfloat16_rn(v.x * s0); y[8] = __float2bfloat16_rn(v.z * s0); }
-                    if (m + 1 < p.M) { y[ldy] = __float2bfloat16_rn(v.y * s1); y[ldy + 8] = __float2bfloat16_rn(v.w * s1); }
+                    if (m < mrows) { y[0] = __float2bfloat16_rn(v.x * s0); y[8] = __float2bfloat16_rn(v.z * s0); }
+                    if (m + 1 < mrows) { y[ldy] = __float2bfloat16_rn(v.y * s1); y[ldy + 8] = __float2bfloat16_rn(v.w * s1); }
                 } else {
                     float *y = reinterpret_cast<float *>(p.mat[mi].y) + at;
-                    if (m < p.M) { y[0] = v.x * s0; y[8] = v.z * s0; }
-                    if (m + 1 < p.M) { y[ldy] = v.y * s1; y[ldy + 8] = v.w * s1; }
+                    if (m < mrows) { y[0] = v.x * s0; y[8] = v.z * s0; }
+                    if (m + 1 < mrows) { y[ldy] = v.y * s1; y[ldy + 8] = v.w * s1; }
                 }
             }
         }
@@ -398,30 +405,37 @@ w2a8_stat_kernel(const __grid_constant__ StParams p) {
 }
 
 // ---- host side -----------------------------------------------------------------------
-constexpr size_t kStBudget8 = 112 * 1024, kStBudget16 = 225 * 1024;   // dynamic shared memory per CTA
-constexpr int st_warps(int mt) { return mt <= 2 ? 8 : 16; }
-constexpr int st_ring(int mt) { return mt <= 2 ? 3 : 2; }
+constexpr size_t kStBudget = 225 * 1024;      // dynamic shared memory per CTA
+constexpr int st_ring(int mt) { return mt <= 2 ? 4 : mt <= 4 ? 3 : 2; }
+// Token groups and slabs per group: groups of at most 64 tokens, all of the same width.
+static int st_tgroups(int M) { return (M + 63) / 64; }
+static int st_slabs(int M) { return ((M + 7) / 8 + st_tgroups(M) - 1) / st_tgroups(M); }
 
 static bool stat_supported(int M, int K, int group) {
-    if (K % kBlockK != 0 || M < 1 || M > 32) return false;
+    if (K % kBlockK != 0 || M < 1 || st_tgroups(M) > 16) return false;
     // the activations of an eighth of K have to fit beside the rings and one slot of sums
-    const int mt = (M + 7) / 8, nb = (K / kBlockK + kStMaxCluster - 1) / kStMaxCluster;
-    const size_t budget = st_warps(mt) == 8 ? kStBudget8 : kStBudget16;
-    if ((size_t)st_warps(mt) * st_ring(mt) * kStSlot + (size_t)nb * mt * 2048 + mt * 1024 > budget) return false;
+    const int mt = st_slabs(M), nb = (K / kBlockK + kStMaxCluster - 1) / kStMaxCluster;
+    const size_t budget = kStBudget;
+    if ((size_t)kStWarps * st_ring(mt) * kStSlot + (size_t)nb * mt * 2048 + mt * 1024 > budget) return false;
     return group == 64 || group == 128 || group % 256 == 0;
 }
 
 // Whether the kernel takes a launch over `count` matrices of `tiles` 16-channel tiles in all.  Measured on
-// B200 (us per GEMM call, back to back over rotating weight copies; before / this kernel):
-//   20 .. 32 tokens: 4096 x 14336 12.7 / 11.1, 14.7 / 12.6; gate|up 4096 x (14336 + 14336) 25.5 / 17,
-//     29.3 / 19.3; 14336 x 4096 16.5 / 14.6, 17.3 / 13.7; 8192 x 8192 18.6 / 11.7, 19.6 / 13.0;
-//     8192 x (28672 + 28672) 127 / 50, 133 / 71; q|k|v 4096 x 6144 12.0 / 8.7, 12.7 / 9.3; but 4096 x 4096
-//     4.8 / 6.8, 5.6 / 7.1 and 8192 x 1024 4.0 / 7.5: small problems stay where they were, unless the
-//     alternative is a launch per matrix.
-//   9 .. 16 tokens: the persistent kernel keeps what it serves with register-resident activations (K <= 4096:
-//     4096 x 14336 8.3 / 9.1) and 14336 x 4096 (9.6 / 10.4); longer problems come here: 8192 x 8192
-//     10.5 / 10.1, q|k|v of 8192 13.5 / 11.5, 8192 x (28672 + 28672) 65.6 / 44.0.  Where only the one-shot
+// B200 (us per GEMM call, group 64, back to back over rotating weight copies; before / this kernel):
+//   5 .. 8 tokens: 8192 x 8192 8.3 / 7.7, 8192 x (28672 + 28672) 36.0 / 30.9, 28672 x 8192 23.0 / 18.3; but
+//     14336 x 4096 7.8 / 8.6, gate|up 4096 x (14336 + 14336) 9.0 / 11.0;
+//   9 .. 16 tokens: gate|up 13.9 / 13.0, 8192 x 8192 10.6 / 9.7, 8192 x (28672 + 28672) 65.2 / 35.3,
+//     28672 x 8192 29.9 / 21.8; but 4096 x 14336 8.3 / 8.8, 14336 x 4096 9.5 / 9.7.  Where only the one-shot
 //     kernel is left (binary16 scales): 4096 x 14336 9.9 / 8.2, 14336 x 4096 11.1 / 9.6, 4096 x 4096 4.1 / 4.9.
+//   17 .. 32 tokens: 4096 x 14336 12.7 / 9.8, 14.7 / 11.9; gate|up 25.5 / 15.7, 29.3 / 18.9; 14336 x 4096
+//     16.5 / 10.7, 17.3 / 12.9; 8192 x (28672 + 28672) 127 / 49, 133 / 63; but 4096 x 4096 4.9 / 5.5, 5.6 / 6.9:
+//     a launch costs 4 to 5 us beside the stream, so small problems stay where they were, unless the
+//     alternative is a launch per matrix (q|k|v 4096 x 6144 12.0 / 8.7).
+//   33 .. 64 tokens: 4096 x 4096 8.8 / 7.2, 11.8 / 9.9; 4096 x 14336 20.6 / 13.5, 27.9 / 20.3; 14336 x 4096
+//     29.1 / 14.6, 34.4 / 22.1; 8192 x 8192 29.1 / 16.1, 37.2 / 23.5.
+//   65 .. 256 tokens: about 5 us + 0.27 ns per cell and slab (a little more for K > 8192, where clusters of six
+//     and eight leave SMs idle), against the model of the tensor-core kernels: 4096 x 4096 at 100 tokens
+//     15.1 / 12.6, at 200 20.9 / 19.8, but 4096 x 14336 at 100 29.6 / 31.3.
 // W2A8_STAT = 0 never, 2 whenever it supports the shape; any switch that forces a plan of another kernel
 // keeps it out.
 bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
@@ -429,26 +443,34 @@ bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
     const int mode = env_int("W2A8_STAT", 1);
     if (mode == 0) return false;
     if (mode == 2) return true;
-    if (M < 9) return false;
+    if (M < 5 || M > 256) return false;
     for (const char *name : {"W2A8_CHUNKS", "W2A8_TG", "W2A8_RING", "W2A8_MT", "W2A8_CLUSTER", "W2A8_MIN_WARPS",
                              "W2A8_RELAX"})
-        if (const char *v = getenv(name); v && *v) return false;
+        if (env_set(name)) return false;
     if (env_int("W2A8_GEMV", 1) == 2) return false;
     const long long blocks = K / kBlockK, cells = (long long)((tiles + 1) / 2) * blocks;
-    if (M <= 16 && !h16 && gemv_preferred(M, K, group, tiles, count)) return blocks > 16 && cells >= 8192;
-    return cells >= (count > 1 ? 1536 : 4096);
+    if (M <= 8) return gemv_preferred(M, K, group, tiles, count) && blocks > 16 && cells >= 8192;
+    if (M <= 16 && !h16 && gemv_preferred(M, K, group, tiles, count)) return cells >= (blocks > 16 ? 8192 : 12288);
+    if (M <= 32) return cells >= (count > 1 ? 1536 : 4096);
+    if (count > 1) return false;                  // (more than 32 tokens: a launch per matrix)
+    if (M <= 64) return cells >= 1024;
+    for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE",
+                             "W2A8_PF_UNPACK_WARPS"})
+        if (env_set(name)) return false;
+    const double mine = 5.0e-6 + 0.27e-9 * (blocks > 32 ? 1.15 : 1.0) * (double)cells * st_tgroups(M) * st_slabs(M);
+    return mine < 0.95 * many_token_seconds(M, tiles * 16, K, group);
 }
 
 // Clusters of C CTAs that are resident at once (clusters are placed inside one GPC, so the count is not
-// slots / C: with one CTA per SM 74, 45, 33 for C = 2, 3, 4; with two 148, 93, 71, 33 for C = 2, 3, 4, 8).
-// A larger grid would run a second wave of a few clusters.  Looked up once per device and form.
+// slots / C: 74, 45, 33, 26, 22, 15 for C = 2, 3, 4, 5, 6, 8).
+// A larger grid would run a second wave of a few clusters.  Looked up once per device and instance.
 struct StClusters { std::atomic<int> known; int n[kStMaxCluster + 1]; };
 
 template <typename K>
-static int stat_clusters(K kernel, int w, int C, size_t smem, int fallback) {
+static int stat_clusters(K kernel, int C, size_t smem, int fallback) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(w * 32);
+    cfg.blockDim = dim3(kStWarps * 32);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -469,8 +491,8 @@ struct StPlan { int C, round_pairs, nclusters; size_t smem; };
 // cells per warp: gate|up of the 8B layer 19.3 / 21.9 us at 32 tokens, 13.4 / 14.2 at 16.)
 static bool stat_plan(int M, int K, int pairs, const int *resident, StPlan *out) {
     StPlan pl = {};
-    const int mt = (M + 7) / 8, w = st_warps(mt), blocks = K / kBlockK;
-    const size_t budget = w == 8 ? kStBudget8 : kStBudget16;
+    const int mt = st_slabs(M), w = kStWarps, blocks = K / kBlockK, tg = st_tgroups(M);
+    const size_t budget = kStBudget;
     const size_t slot_bytes = (size_t)mt * 1024, act_block = (size_t)mt * 2048;
     const int forced = env_int("W2A8_STAT_C", 0);
     double best = 1e30;
@@ -479,7 +501,9 @@ static bool stat_plan(int M, int K, int pairs, const int *resident, StPlan *out)
         const int nb = (blocks + C - 1) / C;
         const size_t fixed = (size_t)w * st_ring(mt) * kStSlot + nb * act_block;
         if (fixed + slot_bytes > budget) continue;
-        const int ncl = resident[C] < pairs ? resident[C] : pairs;
+        int ncl = resident[C] / tg;                       // clusters per token group
+        if (ncl < 1) continue;
+        if (ncl > pairs) ncl = pairs;
         const int per = (pairs + ncl - 1) / ncl;
         int cap = (int)((budget - fixed) / slot_bytes);
         while (cap > 1 && (long long)cap * nb * nb >= 65536) --cap;      // (the kernel divides by nb with a 16-bit reciprocal)
@@ -499,15 +523,14 @@ static bool stat_plan(int M, int K, int pairs, const int *resident, StPlan *out)
 
 template <int MT, int SPP, bool H16>
 static cudaError_t launch_stat_inst(StParams &p, cudaStream_t st) {
-    constexpr int W = st_warps(MT);
-    auto kernel = w2a8_stat_kernel<MT, SPP, H16, W, st_ring(MT)>;
-    constexpr size_t budget = W == 8 ? kStBudget8 : kStBudget16;
+    auto kernel = w2a8_stat_kernel<MT, SPP, H16, st_ring(MT)>;
+    constexpr size_t budget = kStBudget;
     static PerDeviceFlags configured;   // per kernel instantiation
     if (cudaError_t e = allow_dynamic_smem(kernel, configured, (int)budget)) return e;
     static StClusters clusters[kMaxDevices];
     StClusters &cs = clusters[current_device()];
     if (!cs.known.load(std::memory_order_acquire)) {      // racing threads write the same values
-        for (int C = 1; C <= kStMaxCluster; ++C) cs.n[C] = stat_clusters(kernel, W, C, budget, sm_count() * (16 / W) / C);
+        for (int C = 1; C <= kStMaxCluster; ++C) cs.n[C] = stat_clusters(kernel, C, budget, sm_count() / C);
         cs.known.store(1, std::memory_order_release);
     }
     StPlan pl;
@@ -515,8 +538,9 @@ static cudaError_t launch_stat_inst(StParams &p, cudaStream_t st) {
     p.C = pl.C; p.round_pairs = pl.round_pairs;
     p.blk_per = p.blocks / pl.C; p.blk_extra = p.blocks % pl.C;
     for (int i = 0; i < 2; ++i) p.nb_inv[i] = (65536 + p.blk_per + i - 1) / (p.blk_per + i);
+    p.tgroups = st_tgroups(p.M);
     p.pair_per = p.pairs / pl.nclusters; p.pair_extra = p.pairs % pl.nclusters;
-    return launch_kernel_clusters(kernel, dim3(pl.nclusters * pl.C), dim3(W * 32), pl.smem, st, pdl_enabled(),
+    return launch_kernel_clusters(kernel, dim3(pl.nclusters * p.tgroups * pl.C), dim3(kStWarps * 32), pl.smem, st, pdl_enabled(),
                                   make_uint2((unsigned)pl.C, 1u), p);
 }
 template <int MT, bool H16>
@@ -526,11 +550,15 @@ static cudaError_t launch_stat_spp(StParams &p, int spp, cudaStream_t st) {
 }
 template <bool H16>
 static cudaError_t launch_stat_mt(StParams &p, int spp, cudaStream_t st) {
-    switch ((p.M + 7) / 8) {
+    switch (st_slabs(p.M)) {
         case 1: return launch_stat_spp<1, H16>(p, spp, st);
         case 2: return launch_stat_spp<2, H16>(p, spp, st);
         case 3: return launch_stat_spp<3, H16>(p, spp, st);
-        default: return launch_stat_spp<4, H16>(p, spp, st);
+        case 4: return launch_stat_spp<4, H16>(p, spp, st);
+        case 5: return launch_stat_spp<5, H16>(p, spp, st);
+        case 6: return launch_stat_spp<6, H16>(p, spp, st);
+        case 7: return launch_stat_spp<7, H16>(p, spp, st);
+        default: return launch_stat_spp<8, H16>(p, spp, st);
     }
 }
 

@@ -1,4 +1,4 @@
-"""GPU parity of the streaming kernel with stationary activations (9 .. 32 tokens) against the CPU
+"""GPU parity of the streaming kernel with stationary activations against the CPU
 reference: edges of token slabs, half channel pairs, every scale group form, K shares with unequal
 block counts, cells cut between warps, several rounds of pairs, grouped matrices, both scale types."""
 import numpy as np
@@ -38,6 +38,11 @@ CASES = [
     (31, 512, [20480], 128, 1),               # no cluster, several rounds of pairs
     (1, 1024, [96], 64, 0),                   # forced below its range: a single token
     (8, 4352, [80], 64, 2),
+    (40, 1024, [2048], 64, 0),                # five slabs
+    (47, 768, [96, 48], 256, 2),              # six
+    (64, 4096, [1024], 128, 0),               # eight: a full group
+    (100, 2048, [272], 64, 2),                # two groups of seven slabs, the second not full
+    (130, 512, [1024], 0, 0),                 # three groups
 ]
 
 
