@@ -36,8 +36,6 @@
 
 namespace w2a8 {
 
-int env_int(const char *name, int dflt);
-
 constexpr int kGvWarps = 16;                      // warps per CTA of the full-SM form (the other has 8, two CTAs per SM)
 constexpr int kGvRing = 4;                        // landing slots (cells) per warp (a power of two)
 constexpr int kGvMaxMats = 4;                     // weight matrices per launch
@@ -196,7 +194,49 @@ w2a8_gemv_kernel(const __grid_constant__ GemvParams p) {
 
     // ---- activations into shared memory (ASMEM) ---------------------------------------
     if constexpr (ASMEM) {
-        if (p.x) {
+        if (BCACHE && p.x) {
+            // Every warp quantises just the values that its K-lane multiplies (NB blocks, 16 values per lane),
+            // and the warps meet once, for the abs-max.  The stores need no second barrier: a warp reads
+            // back what its own lanes stored (warps of other tiles with the same K-lane store the same bytes).
+            const bool mine = lane < 16 * NB;
+            const int k0 = b0 * kBlockK + 16 * lane;
+            for (int m0 = 0; m0 < p.M; m0 += 4) {
+                uint4 v[4][2];
+#pragma unroll
+                for (int j = 0; j < (ONE ? 1 : 4); ++j)
+                    if (m0 + j < p.M && mine) {
+                        const int8_t *src = reinterpret_cast<const int8_t *>(p.x + (size_t)(m0 + j) * p.K + k0);
+                        v[j][0] = ld_act16(src);
+                        v[j][1] = ld_act16(src + 16);
+                    }
+#pragma unroll
+                for (int j = 0; j < (ONE ? 1 : 4); ++j)
+                    if (m0 + j < p.M) {
+                        const uint32_t am = mine ? amax8(amax8(0u, v[j][0]), v[j][1]) : 0u;
+                        const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, am);
+                        if (lane == 0) wmax[m0 + j][warp] = top;
+                    }
+            }
+            __syncthreads();
+#pragma unroll 1
+            for (int m = 0; m < p.M; ++m) {
+                float inv;
+                const float s = quant_scale(__reduce_max_sync(0xFFFFFFFFu, wmax[m][lane & (W - 1)]), &inv);
+                if (threadIdx.x == 0) {
+                    s_scale[m] = s;
+                    if (p.a_scale_out && blockIdx.x == 0) p.a_scale_out[m] = s;
+                }
+                if (mine) {
+                    const int8_t *src = reinterpret_cast<const int8_t *>(p.x + (size_t)m * p.K + k0);   // from L1
+                    const uint4 lo = ld_act16(src), hi = ld_act16(src + 16);
+                    const uint4 q = make_uint4(quant4(lo.x, lo.y, inv), quant4(lo.z, lo.w, inv),
+                                               quant4(hi.x, hi.y, inv), quant4(hi.z, hi.w, inv));
+                    *reinterpret_cast<uint4 *>(act + (size_t)m * p.act_stride + k0) = q;
+                    if (p.a_out && blockIdx.x == 0 && tl == 0) *reinterpret_cast<uint4 *>(p.a_out + (size_t)m * p.K + k0) = q;
+                }
+            }
+            __syncwarp();
+        } else if (p.x) {
             // Quantise the M <= 8 token rows here (same operations as a8_quantize, same bits).
             const int nvec = p.K >> 3;                    // 16-byte vectors (8 bf16) per row
             uint32_t am[kGvMaxFuseM];
@@ -248,7 +288,7 @@ w2a8_gemv_kernel(const __grid_constant__ GemvParams p) {
                     *reinterpret_cast<uint4 *>(act + (size_t)m * p.act_stride + 16 * i) =
                         ld_act16(p.a + (size_t)m * p.K + 16 * i);
         }
-        __syncthreads();
+        if (!(BCACHE && p.x)) __syncthreads();
     }
     const uint32_t act_u32 = smem_u32(act);
 
@@ -415,7 +455,7 @@ bool gemv_supported(int M, int K, int group) {
     if (env_int("W2A8_GEMV", 1) == 0) return false;
     for (const char *name : {"W2A8_CHUNKS", "W2A8_TG", "W2A8_RING", "W2A8_MT", "W2A8_CLUSTER", "W2A8_MIN_WARPS",
                              "W2A8_RELAX"})
-        if (getenv(name) && *getenv(name)) return false;
+        if (env_set(name)) return false;
     return true;
 }
 
