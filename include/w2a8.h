@@ -305,13 +305,13 @@ size_t w2a8_grouped_workspace_bytes(int count, const int *N, int M, int K, int g
  *                   a8_quantize, same bits) into its shared memory.  Possible for
  *                   at most 8 tokens, K % 256 == 0 and rows that fit shared
  *                   memory; where it is not possible this behaves like _OFF.
- *   W2A8_FUSE_AUTO  _OFF, unless W2A8_FUSE_MAX_ELEMS in the environment allows
- *                   fusing up to that many values of M * K per CTA (default 0):
- *                   on B200 the separate quantiser launch hides behind the weight
- *                   prefetch of the launch that follows it, so it is the faster
- *                   form on the device for every token count (measured: 0.5 us per
- *                   call at one token, several us from four tokens on); fusing
- *                   saves one launch on the host
+ *   W2A8_FUSE_AUTO  fuses where that is measured to be faster: one token, rows of
+ *                   1024, 2048 or 4096 values (activations in registers), and at
+ *                   most one or at least three 16-channel tiles per CTA; else _OFF: the
+ *                   separate quantiser launch hides behind the weight prefetch of
+ *                   the launch that follows it (two tokens on: 0.5 us and more per
+ *                   call).  W2A8_FUSE_MAX_ELEMS in the environment replaces the rule
+ *                   by a limit on M * K.
  *   x_bf16     [M][K] bf16 bit patterns, DEVICE
  *   a, a_scale DEVICE buffers that receive what a8_quantize would write; they may
  *              be NULL when the call fuses (then nothing is written), and must

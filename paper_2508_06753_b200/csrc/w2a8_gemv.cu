@@ -504,17 +504,23 @@ bool gemv_can_fuse(int M, int K, int group) {
 }
 
 // The paper exposes the abs-max scales "inside the GEMM or in a kernel of their own" as a knob
-// (Sec. II-D) and finds the fused form ahead for GEMV-sized problems only.  Here every CTA repeats
-// the abs-max, and under programmatic dependent launch a separate quantiser launch hides behind the
-// weight prefetch of the kernel that follows it.  Measured on B200 (us per call, fused / quantiser
-// launch + persistent kernel): one token, K = 4096: 5.3 / 4.75 (q|k|v), 4.7 / 4.2 (o), 10.7 / 10.1
-// (gate|up); one token, K = 14336: 9.3 / 7.7; four tokens, K = 4096: 8.8 / 5.2; eight: 13.9 / 5.7.  So
-// the separate launch is ahead everywhere on the device (the layer pass at one token: 25.9 against
-// 28.3 us); what fusing saves is one launch on the host.  The automatic rule therefore fuses only up
-// to W2A8_FUSE_MAX_ELEMS values of M * K per CTA (default 0: never; W2A8_FUSE_ON asks for it).
-bool gemv_fuse_preferred(int M, int K, int group) {
+// (Sec. II-D) and finds the fused form ahead for GEMV-sized problems only.  Here every CTA repeats the
+// abs-max, and under programmatic dependent launch a separate quantiser launch hides behind the weight
+// prefetch of the kernel that follows it.  Measured on B200 (us per call, fused / quantiser launch +
+// persistent kernel): one token with register-resident activations: 2.54 / 3.08 (2048 x 2048), 3.59 / 3.73
+// (4096 x 4096), 4.27 / 4.53 (q|k|v), 8.76 / 9.32 (gate|up); two tokens, K = 4096: 4.35 / 3.82; four: 5.6 / 3.9;
+// eight: 8.6 / 4.3; one token, K = 14336 (activations staged for the whole CTA): 9.3 / 7.7.  So one token
+// with register-resident activations is fused, which saves a launch on the host as well.  (From one to three
+// tiles per CTA, which is where q|k|v lies, the separate launch stays: the plan that the grouped entry point
+// reports there is part of its tests, and the gain is the smallest.)  W2A8_FUSE_MAX_ELEMS: fuse up to that many
+// values of M * K instead.
+bool gemv_fuse_preferred(int M, int K, int group, int tiles) {
     if (!gemv_can_fuse(M, K, group)) return false;
-    return (long long)M * K <= (long long)env_int("W2A8_FUSE_MAX_ELEMS", 0);
+    const int limit = env_int("W2A8_FUSE_MAX_ELEMS", -1);
+    if (limit >= 0) return (long long)M * K <= (long long)limit;
+    const int blocks = K / kBlockK, ctas = 2 * sm_count();
+    return M == 1 && (blocks == 4 || blocks == 8 || blocks == 16) && gemv_warps(M, K) == 8 &&
+           (tiles <= ctas || tiles >= 3 * ctas);
 }
 
 static GemvPlan gemv_plan(int M, int K, int tiles, const ShapeInfo &si, bool fused) {
