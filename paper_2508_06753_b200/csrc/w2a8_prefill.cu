@@ -134,6 +134,11 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
     __syncthreads();
     pf_tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    // Programmatic dependent launch: the set-up above and the first weights overlap the tail of the previous
+    // kernel of the stream; the roles that touch anything else (activations, token scales, outputs) wait for it.
+    // Measured (us per call, plain / dependent launch): 4096 x 14336 at 100 tokens 29.3 / 27.8, at 512 83.0 / 80.7;
+    // quantiser and one scale per channel, 2048 tokens, 119.5 / 110.7.
+    pdl_launch_dependents();
 
     constexpr int kFirstUnpack = pf_first_unpack(UW), kFirstDrain = pf_first_drain(UW);
     if (warp < kFirstUnpack) {
@@ -141,6 +146,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
             pf_setmaxnreg_dec<56>();
             if (warp == 2 && lane == 0) {
                 // ===== TMA producer: activations, 128 tokens x 256 k per stage ===============
+                pdl_wait();
                 int s = 0, round = 0;
                 for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
                     const int m0 = item_m0(tile), k0 = item_stage0(tile) * kPfBK;
@@ -317,6 +323,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
         int s = team, round = 0;                    // slot and use count of the slot for this team's stage
         uint4 w_nxt[kUnits];
         if (tile < ntiles) request(w_nxt, tile, it);
+        if (UW == 2 && warp == kFirstUnpack) pdl_wait();      // its first lane brings the activations
         while (tile < ntiles) {
             uint4 w[kUnits];
 #pragma unroll
@@ -360,6 +367,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
         // ===== drain warps: TMEM -> registers, fp32 accumulate with the group scale ======
         const int q4 = warp & 3;                    // TMEM lane quarter this warp may access
         if constexpr (UW == 4) pf_setmaxnreg_inc<176>();
+        pdl_wait();
         const int col0 = ((warp - kFirstDrain) >> 2) * kPfDrainCols;   // first token column of this warp
         const int ch = q4 * 32 + lane;              // channel inside the tile = TMEM lane
         const uint32_t tlane = tmem_base + ((uint32_t)(q4 * 32) << 16) + col0;
@@ -511,6 +519,8 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
 // which CTA finished first).  One thread per four consecutive channels.
 __global__ void pf_splitk_reduce_kernel(const float *__restrict__ split_out, void *__restrict__ y, int M, int N,
                                         int nsplit, int ldy, int y16) {
+    pdl_launch_dependents();
+    pdl_wait();
     const size_t quads = (size_t)M * (N / 4);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < quads; i += (size_t)gridDim.x * blockDim.x) {
         const int m = (int)(i / (N / 4)), n = (int)(i % (N / 4)) * 4;
@@ -722,8 +732,7 @@ int launch_prefill(const int8_t *a, const float *a_scale, const uint32_t *packed
     static PerDeviceFlags configured[21];
     auto launch = [&](auto kernel, int slot, int threads) -> bool {
         if (allow_dynamic_smem(kernel, configured[slot], (int)smem) != cudaSuccess) return false;
-        kernel<<<grid, threads, smem, st>>>(map, p);
-        return true;
+        return launch_kernel(kernel, grid, dim3(threads), smem, st, pdl_enabled(), map, p) == cudaSuccess;
     };
     // The MMA-issuing code is specialised on the 64-k slices per scale group: 1, 2, or whole stages
     // (0); the warp layout on the number of unpack warps (the parity export keeps the 12-warp one).
@@ -755,7 +764,9 @@ int launch_prefill(const int8_t *a, const float *a_scale, const uint32_t *packed
     if (nsplit > 1) {
         const size_t quads = (size_t)M * (N / 4);
         const unsigned blocks = (unsigned)((quads + 255) / 256 < (size_t)(8 * sms) ? (quads + 255) / 256 : (size_t)(8 * sms));
-        pf_splitk_reduce_kernel<<<blocks, 256, 0, st>>>(p.split_out, y, M, N, nsplit, ldy, p.y16);
+        if (launch_kernel(pf_splitk_reduce_kernel, dim3(blocks), dim3(256), 0, st, pdl_enabled(), p.split_out, y, M, N,
+                          nsplit, ldy, p.y16) != cudaSuccess)
+            return W2A8_ERR_CUDA;
     }
     return cudaGetLastError() == cudaSuccess ? W2A8_OK : W2A8_ERR_CUDA;
 }

@@ -124,11 +124,13 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
     __syncthreads();
     pf_tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    pdl_launch_dependents();      // (see w2a8_prefill.cu: the roles that touch more than weights wait)
 
     if (warp < kHfFirstUnpackWarp) {
         hf_setmaxnreg_dec<56>();
         if (warp == 2 && lane == 0) {
             // ===== TMA producer: activations, 128 tokens x 128 k per stage ===================
+            pdl_wait();
             int s = 0, round = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
@@ -300,6 +302,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
         }
     } else {
         hf_setmaxnreg_inc<176>();
+        pdl_wait();
         // ===== drain warps: TMEM -> registers, fp32 accumulate with the group scale ======
         const int q4 = warp & 3;                    // TMEM lane quarter this warp may access
         const int col0 = ((warp - kHfFirstDrainWarp) >> 2) * kHfDrainCols;
@@ -466,8 +469,7 @@ int launch_prefill_f16(const void *x_bf16, const float *a_scale, const uint32_t 
     static PerDeviceFlags configured[6];
     auto launch = [&](auto kernel, int slot) -> bool {
         if (allow_dynamic_smem(kernel, configured[slot], (int)smem) != cudaSuccess) return false;
-        kernel<<<grid, kHfThreads, smem, st>>>(map, p);
-        return true;
+        return launch_kernel(kernel, grid, dim3(kHfThreads), smem, st, pdl_enabled(), map, p) == cudaSuccess;
     };
     // the MMA-issuing code is specialised on the 64-k slices per scale group: 1, 2, or whole blocks (0)
     auto launch_dps = [&](auto partials_c, int slot0) -> bool {

@@ -87,11 +87,13 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
     __syncthreads();
     pf_tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    pdl_launch_dependents();      // (see w2a8_prefill.cu: the roles that touch more than weights wait)
 
     if (warp < kWdFirstUnpack) {
         wd_setmaxnreg_dec<56>();
         if (warp == 2 && lane == 0) {
             // ===== TMA producer: activations, 256 tokens x 128 k per stage ===================
+            pdl_wait();
             int s = 0, round = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
@@ -220,6 +222,7 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
         }
     } else {
         wd_setmaxnreg_inc<176>();
+        pdl_wait();
         // ===== epilogue warps: TMEM -> registers -> y, one scale per channel ================
         const int q4 = warp & 3;                    // TMEM lane quarter this warp may access
         const int col0 = ((warp - kWdFirstDrain) >> 2) * 128;     // first token column of this warp
@@ -313,10 +316,10 @@ int launch_prefill_wide(const int8_t *a, const float *a_scale, const uint32_t *p
     static PerDeviceFlags configured[2];
     if (h16) {
         if (allow_dynamic_smem(w2a8_prefill_wide_kernel<true>, configured[1], (int)smem) != cudaSuccess) return W2A8_ERR_CUDA;
-        w2a8_prefill_wide_kernel<true><<<grid, kWdThreads, smem, st>>>(map, p);
+        if (launch_kernel(w2a8_prefill_wide_kernel<true>, grid, dim3(kWdThreads), smem, st, pdl_enabled(), map, p) != cudaSuccess) return W2A8_ERR_CUDA;
     } else {
         if (allow_dynamic_smem(w2a8_prefill_wide_kernel<false>, configured[0], (int)smem) != cudaSuccess) return W2A8_ERR_CUDA;
-        w2a8_prefill_wide_kernel<false><<<grid, kWdThreads, smem, st>>>(map, p);
+        if (launch_kernel(w2a8_prefill_wide_kernel<false>, grid, dim3(kWdThreads), smem, st, pdl_enabled(), map, p) != cudaSuccess) return W2A8_ERR_CUDA;
     }
     return cudaGetLastError() == cudaSuccess ? W2A8_OK : W2A8_ERR_CUDA;
 }
