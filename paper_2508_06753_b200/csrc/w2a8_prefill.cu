@@ -96,7 +96,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
     __shared__ int abort_flag_s;
     volatile int *abort_flag = &abort_flag_s;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: known to be uniform
     const int ks_shift = SPLIT ? p.ks_shift : 0;
     const int nsplit = 1 << ks_shift;       // K splits: a work item is one tile over K / nsplit
     const int nstages = (p.K / kPfBK) >> ks_shift;        // stages per work item
@@ -178,7 +178,10 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
         // the kernel is specialised on the slices per group (DPS = 1, 2, or 0 for groups of
         // whole stages), K-step offsets are immediates added to the low descriptor word --
         // the same pair issues at the tensor pipe's rate (3.2-3.3 POPS in that test).
-        if (warp < 2 && lane == 0) {
+        // The whole warp walks the loop and one elected lane issues: the waits cost a third of a lone lane's and
+        // descriptors stay warp-uniform.
+        if (warp < 2) {
+            const bool lead = pf_elect();
             const int w = warp;             // this thread's unit slot: accumulator buffers 2 w and 2 w + 1
             const uint64_t a_desc0 = pf_smem_desc(smem_base);
             const uint64_t b_desc0 = pf_smem_desc(smem_base + 2 * kPfHalfBytes);
@@ -201,7 +204,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                 pf_mma_i8(t0 + b * kPfBN, ad, bd, pf_instr_desc(kPfBM, kPfBN), accumulate);
             };
             auto next_stage = [&]() {
-                pf_mma_commit(pf_smem_u32(&bar_empty[s]));   // stage can be refilled once these MMAs are done
+                if (lead) pf_mma_commit(pf_smem_u32(&bar_empty[s]));   // stage can be refilled once these MMAs are done
                 so += kPfStageBytes >> 4;
                 if (++s == kPfStages) { s = 0; so = 0; full_parity ^= 1u; }
             };
@@ -215,20 +218,24 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                 int c = 0;                  // units this thread has issued so far
                 for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                     for (int it = 0; it < nstages && ok; ++it, ++c) {
-                        ok = pf_wait(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
+                        ok = pf_wait_all(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
                         if (!ok) break;
                         // each buffer must have been read out by the drain warps since its last use
-                        if (c >= 1) ok = pf_wait(acc_empty_bar0, (uint32_t)(c - 1) & 1u, abort_flag);
+                        if (c >= 1) ok = pf_wait_all(acc_empty_bar0, (uint32_t)(c - 1) & 1u, abort_flag);
                         if (!ok) break;
                         pf_tc_fence_after();
-                        if (w == 0) { step(J0{}, 0, 0u); step(J1{}, 0, 1u); }
-                        else        { step(J4{}, 0, 0u); step(J5{}, 0, 1u); }
-                        if (c >= 1) ok = pf_wait(acc_empty_bar1, (uint32_t)(c - 1) & 1u, abort_flag);
+                        if (lead) {
+                            if (w == 0) { step(J0{}, 0, 0u); step(J1{}, 0, 1u); }
+                            else        { step(J4{}, 0, 0u); step(J5{}, 0, 1u); }
+                        }
+                        if (c >= 1) ok = pf_wait_all(acc_empty_bar1, (uint32_t)(c - 1) & 1u, abort_flag);
                         if (!ok) break;
                         pf_tc_fence_after();
-                        if (w == 0) { step(J2{}, 1, 0u); step(J3{}, 1, 1u); }
-                        else        { step(J6{}, 1, 0u); step(J7{}, 1, 1u); }
-                        pf_mma_commit(acc_full_bar);
+                        if (lead) {
+                            if (w == 0) { step(J2{}, 1, 0u); step(J3{}, 1, 1u); }
+                            else        { step(J6{}, 1, 0u); step(J7{}, 1, 1u); }
+                            pf_mma_commit(acc_full_bar);
+                        }
                         next_stage();
                     }
                 }
@@ -237,18 +244,20 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                 int u = 0;                  // unit (= stage) index across tiles
                 for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                     for (int it = 0; it < nstages && ok; ++it, ++u) {
-                        ok = pf_wait(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
+                        ok = pf_wait_all(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
                         if (!ok) break;
                         if ((u & 1) == w) {
-                            if (u >= kPfUnits) ok = pf_wait(acc_empty_bar0, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
+                            if (u >= kPfUnits) ok = pf_wait_all(acc_empty_bar0, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
                             if (!ok) break;
                             pf_tc_fence_after();
-                            step(J0{}, 0, 0u); step(J1{}, 0, 1u); step(J2{}, 0, 1u); step(J3{}, 0, 1u);
-                            if (u >= kPfUnits) ok = pf_wait(acc_empty_bar1, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
+                            if (lead) { step(J0{}, 0, 0u); step(J1{}, 0, 1u); step(J2{}, 0, 1u); step(J3{}, 0, 1u); }
+                            if (u >= kPfUnits) ok = pf_wait_all(acc_empty_bar1, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
                             if (!ok) break;
                             pf_tc_fence_after();
-                            step(J4{}, 1, 0u); step(J5{}, 1, 1u); step(J6{}, 1, 1u); step(J7{}, 1, 1u);
-                            pf_mma_commit(acc_full_bar);
+                            if (lead) {
+                                step(J4{}, 1, 0u); step(J5{}, 1, 1u); step(J6{}, 1, 1u); step(J7{}, 1, 1u);
+                                pf_mma_commit(acc_full_bar);
+                            }
                         }
                         next_stage();
                     }
@@ -262,7 +271,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                 for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, unit0 += units_per_tile) {
                     int group_idx = 0, pos = 0;     // group of this tile, stage inside the group
                     for (int it = 0; it < nstages && ok; ++it) {
-                        ok = pf_wait(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
+                        ok = pf_wait_all(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
                         if (!ok) break;
                         const int u = unit0 + (group_idx >> 1);
                         const bool mine = (u & 1) == w;
@@ -270,19 +279,21 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                             const int b = group_idx & 1;
                             if (pos == 0) {     // a new group: its buffer must have been read out since its last use
                                 const int uses = b ? uses1 : uses0;
-                                if (uses >= 1) ok = pf_wait(b ? acc_empty_bar1 : acc_empty_bar0, (uint32_t)(uses - 1) & 1u, abort_flag);
+                                if (uses >= 1) ok = pf_wait_all(b ? acc_empty_bar1 : acc_empty_bar0, (uint32_t)(uses - 1) & 1u, abort_flag);
                                 if (!ok) break;
                                 if (b) ++uses1; else ++uses0;
                             }
                             pf_tc_fence_after();
-                            step(J0{}, b, pos == 0 ? 0u : 1u);
-                            step(J1{}, b, 1u); step(J2{}, b, 1u); step(J3{}, b, 1u);
-                            step(J4{}, b, 1u); step(J5{}, b, 1u); step(J6{}, b, 1u); step(J7{}, b, 1u);
+                            if (lead) {
+                                step(J0{}, b, pos == 0 ? 0u : 1u);
+                                step(J1{}, b, 1u); step(J2{}, b, 1u); step(J3{}, b, 1u);
+                                step(J4{}, b, 1u); step(J5{}, b, 1u); step(J6{}, b, 1u); step(J7{}, b, 1u);
+                            }
                         }
                         if (++pos == spg) {
                             pos = 0;
                             const bool unit_done = (group_idx & 1) == 1 || group_idx == ngroups - 1;
-                            if (mine && unit_done) pf_mma_commit(acc_full_bar);
+                            if (mine && unit_done && lead) pf_mma_commit(acc_full_bar);
                             ++group_idx;
                         }
                         next_stage();
@@ -428,7 +439,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
             // Software pipeline over 32-column halves: while one half is converted and
             // accumulated, the next half (possibly of the next group) is on its way from TMEM.
             int v0[32], v1[32];                         // first / second half of the current group
-            ok = pf_wait_warp(pf_smem_u32(&bar_acc_full[unit0 & 1]), (unit0 >> 1) & 1, abort_flag);
+            ok = pf_wait_all(pf_smem_u32(&bar_acc_full[unit0 & 1]), (unit0 >> 1) & 1, abort_flag);
             if (ok) { pf_tc_fence_after(); pf_tmem_ld32(tlane + (2 * (unit0 & 1)) * kPfBN, v0); }
             for (int g0 = 0; g0 < ngroups && ok; g0 += 8) {
                 float sc_cur[8];

@@ -97,7 +97,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
     __shared__ int abort_flag_s;
     volatile int *abort_flag = &abort_flag_s;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: known to be uniform
     const int nstages = p.K / kHfBK;        // stages per tile
     const int dps = p.slices_per_group;     // 64-k slices between two drains
     const int ngroups = (p.K / 64) / dps;   // scale groups per tile
@@ -154,7 +154,9 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
         // set by the scalar instructions between two MMAs): specialised on the 64-k slices per
         // group (DPS = 1, 2, or 0 for groups of whole 256-k blocks), K-step offsets as immediates
         // on the low descriptor word.  A stage is two 64-k sub-tiles of four K = 16 steps each.
-        if (warp < 2 && lane == 0) {
+        // (The whole warp walks the loop and an elected lane issues, as in w2a8_prefill.cu.)
+        if (warp < 2) {
+            const bool lead = pf_elect();
             const int w = warp;
             const uint64_t a_desc0 = pf_smem_desc(smem_base);
             const uint64_t b_desc0 = pf_smem_desc(smem_base + 2 * kHfHalfBytes);
@@ -176,7 +178,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
                 pf_mma_f16(t0 + b * kHfBN, ad, bd, pf_instr_desc_bf16(kHfBM, kHfBN), accumulate);
             };
             auto next_stage = [&]() {
-                pf_mma_commit(pf_smem_u32(&bar_empty[s]));
+                if (lead) pf_mma_commit(pf_smem_u32(&bar_empty[s]));
                 so += kHfStageBytes >> 4;
                 if (++s == kHfStages) { s = 0; so = 0; full_parity ^= 1u; }
             };
@@ -189,19 +191,21 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
                 int u = 0;                  // unit (= stage) index across tiles
                 for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                     for (int it = 0; it < nstages && ok; ++it, ++u) {
-                        ok = pf_wait(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
+                        ok = pf_wait_all(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
                         if (!ok) break;
                         if ((u & 1) == w) {
                             // each buffer must have been read out by the drain warps since its last use
-                            if (u >= kHfUnits) ok = pf_wait(acc_empty_bar0, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
+                            if (u >= kHfUnits) ok = pf_wait_all(acc_empty_bar0, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
                             if (!ok) break;
                             pf_tc_fence_after();
-                            step(J0{}, 0, 0u); step(J1{}, 0, 1u); step(J2{}, 0, 1u); step(J3{}, 0, 1u);
-                            if (u >= kHfUnits) ok = pf_wait(acc_empty_bar1, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
+                            if (lead) { step(J0{}, 0, 0u); step(J1{}, 0, 1u); step(J2{}, 0, 1u); step(J3{}, 0, 1u); }
+                            if (u >= kHfUnits) ok = pf_wait_all(acc_empty_bar1, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
                             if (!ok) break;
                             pf_tc_fence_after();
-                            step(J4{}, 1, 0u); step(J5{}, 1, 1u); step(J6{}, 1, 1u); step(J7{}, 1, 1u);
-                            pf_mma_commit(acc_full_bar);
+                            if (lead) {
+                                step(J4{}, 1, 0u); step(J5{}, 1, 1u); step(J6{}, 1, 1u); step(J7{}, 1, 1u);
+                                pf_mma_commit(acc_full_bar);
+                            }
                         }
                         next_stage();
                     }
@@ -216,7 +220,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
                 for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, unit0 += units_per_tile) {
                     int group_idx = 0, pos = 0;     // group of this tile, stage inside the group
                     for (int it = 0; it < nstages && ok; ++it) {
-                        ok = pf_wait(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
+                        ok = pf_wait_all(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
                         if (!ok) break;
                         const int u = unit0 + (group_idx >> 1);
                         const bool mine = (u & 1) == w;
@@ -224,19 +228,21 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
                             const int b = group_idx & 1;
                             if (pos == 0) {     // a new group: its buffer must have been read out since its last use
                                 const int uses = b ? uses1 : uses0;
-                                if (uses >= 1) ok = pf_wait(b ? acc_empty_bar1 : acc_empty_bar0, (uint32_t)(uses - 1) & 1u, abort_flag);
+                                if (uses >= 1) ok = pf_wait_all(b ? acc_empty_bar1 : acc_empty_bar0, (uint32_t)(uses - 1) & 1u, abort_flag);
                                 if (!ok) break;
                                 if (b) ++uses1; else ++uses0;
                             }
                             pf_tc_fence_after();
-                            step(J0{}, b, (DPS == 2 || pos == 0) ? 0u : 1u);
-                            step(J1{}, b, 1u); step(J2{}, b, 1u); step(J3{}, b, 1u);
-                            step(J4{}, b, 1u); step(J5{}, b, 1u); step(J6{}, b, 1u); step(J7{}, b, 1u);
+                            if (lead) {
+                                step(J0{}, b, (DPS == 2 || pos == 0) ? 0u : 1u);
+                                step(J1{}, b, 1u); step(J2{}, b, 1u); step(J3{}, b, 1u);
+                                step(J4{}, b, 1u); step(J5{}, b, 1u); step(J6{}, b, 1u); step(J7{}, b, 1u);
+                            }
                         }
                         if (DPS == 2 || ++pos == spg) {
                             pos = 0;
                             const bool unit_done = (group_idx & 1) == 1 || group_idx == ngroups - 1;
-                            if (mine && unit_done) pf_mma_commit(acc_full_bar);
+                            if (mine && unit_done && lead) pf_mma_commit(acc_full_bar);
                             ++group_idx;
                         }
                         next_stage();
@@ -327,7 +333,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
             };
             refill(0);
             int v0[32], v1[32];                         // first / second half of the current group (fp32 bit patterns)
-            ok = pf_wait_warp(pf_smem_u32(&bar_acc_full[unit0 & 1]), (unit0 >> 1) & 1, abort_flag);
+            ok = pf_wait_all(pf_smem_u32(&bar_acc_full[unit0 & 1]), (unit0 >> 1) & 1, abort_flag);
             if (ok) { pf_tc_fence_after(); pf_tmem_ld32(tlane + (2 * (unit0 & 1)) * kHfBN, v0); }
             for (int g0 = 0; g0 < ngroups && ok; g0 += 8) {
                 float sc_cur[8];

@@ -61,7 +61,7 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
     __shared__ int abort_flag_s;
     volatile int *abort_flag = &abort_flag_s;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: known to be uniform
     const int nstages = p.K / kWdBK;        // stages per tile (even: K is a multiple of 256)
     const int tiles_m = (p.M + kWdBN - 1) / kWdBN;
     const int ntiles = (p.N / kWdBM) * tiles_m;
@@ -117,7 +117,9 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
         // depend on the order, except that the tile's first MMA (which overwrites the buffer) has to
         // come first: thread 0 issues all of stage 0 and commits `bar_first`; thread 1 waits for it
         // before its first MMA of the tile.  Straight-line issue: descriptors = 32-bit base + immediates.
-        if (warp < 2 && lane == 0) {
+        // (The whole warp walks the loop and an elected lane issues, as in w2a8_prefill.cu.)
+        if (warp < 2) {
+            const bool lead = pf_elect();
             const int w = warp;
             const uint64_t a_desc0 = pf_smem_desc(smem_base);
             const uint64_t b_desc0 = pf_smem_desc(smem_base + kWdABytes);
@@ -133,34 +135,38 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
                 const int buf = seq & 1;
                 const uint32_t d_tmem = tmem_base + buf * kWdBN;
                 for (int it = 0; it < nstages && ok; ++it) {
-                    ok = pf_wait(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
+                    ok = pf_wait_all(pf_smem_u32(&bar_full[s]), full_parity, abort_flag);
                     if (!ok) break;
                     const uint64_t ad = ((uint64_t)a_hi << 32) | (a_lo0 + so);
                     const uint64_t bd = ((uint64_t)b_hi << 32) | (b_lo0 + so);
                     if (it == 0) {
                         if (w == 0) {
                             if (seq >= 2) {     // the epilogue warps must have read out this buffer's last tile
-                                ok = pf_wait(pf_smem_u32(&bar_acc_empty[buf]), (uint32_t)((seq >> 1) - 1) & 1u, abort_flag);
+                                ok = pf_wait_all(pf_smem_u32(&bar_acc_empty[buf]), (uint32_t)((seq >> 1) - 1) & 1u, abort_flag);
                                 if (!ok) break;
                             }
                             pf_tc_fence_after();
-                            pf_mma_i8(d_tmem, ad, bd, idesc, 0u);
-                            pf_mma_i8(d_tmem, ad + 2, bd + 2, idesc, 1u);
-                            pf_mma_i8(d_tmem, ad + 4, bd + 4, idesc, 1u);
-                            pf_mma_i8(d_tmem, ad + 6, bd + 6, idesc, 1u);
-                            pf_mma_commit(pf_smem_u32(&bar_first));
+                            if (lead) {
+                                pf_mma_i8(d_tmem, ad, bd, idesc, 0u);
+                                pf_mma_i8(d_tmem, ad + 2, bd + 2, idesc, 1u);
+                                pf_mma_i8(d_tmem, ad + 4, bd + 4, idesc, 1u);
+                                pf_mma_i8(d_tmem, ad + 6, bd + 6, idesc, 1u);
+                                pf_mma_commit(pf_smem_u32(&bar_first));
+                            }
                         }
                     } else {
                         if (it == 1 && w == 1) {
-                            ok = pf_wait(pf_smem_u32(&bar_first), (uint32_t)seq & 1u, abort_flag);
+                            ok = pf_wait_all(pf_smem_u32(&bar_first), (uint32_t)seq & 1u, abort_flag);
                             if (!ok) break;
                         }
                         pf_tc_fence_after();
-                        pf_mma_i8(d_tmem, ad + 4 * w, bd + 4 * w, idesc, 1u);
-                        pf_mma_i8(d_tmem, ad + 4 * w + 2, bd + 4 * w + 2, idesc, 1u);
-                        if (it == nstages - 1) pf_mma_commit(pf_smem_u32(&bar_acc_full[buf]));
+                        if (lead) {
+                            pf_mma_i8(d_tmem, ad + 4 * w, bd + 4 * w, idesc, 1u);
+                            pf_mma_i8(d_tmem, ad + 4 * w + 2, bd + 4 * w + 2, idesc, 1u);
+                            if (it == nstages - 1) pf_mma_commit(pf_smem_u32(&bar_acc_full[buf]));
+                        }
                     }
-                    pf_mma_commit(pf_smem_u32(&bar_empty[s]));   // stage can be refilled once these MMAs are done
+                    if (lead) pf_mma_commit(pf_smem_u32(&bar_empty[s]));   // stage can be refilled once these MMAs are done
                     so += kWdStageBytes >> 4;
                     if (++s == kWdStages) { s = 0; so = 0; full_parity ^= 1u; }
                 }
