@@ -133,7 +133,7 @@ int w2a8_workspace_status(const void *workspace, void *stream);
  * read once per slab of up to 32 tokens): the one-shot kernel when the problem
  * is about one wave of its CTAs, the persistent one (at most 32 tokens,
  * K % 256 == 0) for small matrices with K <= 4096 and for problems of more
- * than one wave; and the one with stationary activations (5 .. 256 tokens,
+ * than one wave; and the one with stationary activations (up to 256 tokens,
  * K % 256 == 0), which unpacks every weight once per 64 tokens, where its estimate
  * is ahead: larger problems of few tokens, smaller ones of many.  w2a8_kernel_for reports tensor-core or streaming.
  * A problem given to the tensor-core kernel may leave its last (at most

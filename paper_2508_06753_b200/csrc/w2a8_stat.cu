@@ -1,4 +1,4 @@
-// Streaming kernel with stationary activations (a few to a few hundred tokens): the weights stream past
+// Streaming kernel with stationary activations (up to a few hundred tokens): the weights stream past
 // activations that stay in shared memory, and every weight is unpacked once per group of up to 64 tokens.
 //
 //  * Work.  A cluster of C CTAs owns a contiguous range of channel pairs (32 channels); rank r of it
@@ -55,6 +55,7 @@ struct StParams {
     int round_pairs;              // pairs per round = sum slots
     int tgroups;                  // token groups of 8 * MT tokens; neighbouring clusters take the same pairs of different groups
     int y16;
+    int s_wide;                   // scales are copied 16 bytes at a time (every row starts on a 16-byte boundary)
     int pairs;                    // (host)
 };
 
@@ -161,6 +162,13 @@ w2a8_stat_kernel(const __grid_constant__ StParams p) {
             else               cp_async4(sdst, q_s + 4 * gi);
         } else if constexpr (kScaleStep == 16) {          // whole blocks: a block's scales of a channel are one aligned unit
             cp_async16(sdst, q_s);
+        } else if (p.s_wide) {
+            // The 16 bytes around the block's scales, past L1: the rings leave it 28 KB, less than the lines that
+            // the 8 x 32 rows in flight would hold, so pieces of 8 or 4 bytes (which can only go through L1) missed
+            // it block after block (28672 x 8192, groups of 128: 24.8 / 17.5 us at 8 tokens, 38.9 / 37.8 at 32;
+            // 8192 x 28672 at 32 33.1 / 32.4).  Small launches are ahead with the pieces (4096 x 14336 at 32 tokens
+            // 10.97 / 11.12, 4096 x 4096 at 64 10.1 / 10.7): the host decides by the number of cells.
+            cp_async16(sdst, reinterpret_cast<const void *>(reinterpret_cast<uintptr_t>(q_s) & ~(uintptr_t)15));
         } else if constexpr (kScaleStep == 8) {
             cp_async8(sdst, q_s);
         } else {
@@ -286,9 +294,11 @@ w2a8_stat_kernel(const __grid_constant__ StParams p) {
                     for (int i = 0; i < 4; ++i)
                         odd_scale |= (((n0 + (i >> 1) * tile + (i & 1) * 8 + gq) * p.G + gi) & 1) << i;
                 }
+                // the block's scales inside their slot (whole 16 bytes: groups of 64, fp32)
+                const int s_off = SPP == 4 || kScaleStep == 16 || !p.s_wide ? 0 : ((kb_lo + kb) * kScaleStep) & 15;
                 // scale of slice s for rows gq, gq + 8 of both tiles (i = 0 .. 3)
                 auto scale = [&](int i, int s) -> float {
-                    const unsigned char *ss = sl + kStWSlot + (i * 8 + gq) * 16;
+                    const unsigned char *ss = sl + kStWSlot + (i * 8 + gq) * 16 + s_off;
                     if constexpr (!H16)          return reinterpret_cast<const float *>(ss)[s / SPP];
                     else if constexpr (SPP != 4) return __half2float(reinterpret_cast<const __half *>(ss)[s / SPP]);
                     else                         return __half2float(reinterpret_cast<const __half *>(ss)[(odd_scale >> i) & 1]);
@@ -422,6 +432,11 @@ static bool stat_supported(int M, int K, int group) {
 
 // Whether the kernel takes a launch over `count` matrices of `tiles` 16-channel tiles in all.  Measured on
 // B200 (us per GEMM call, group 64, back to back over rotating weight copies; before / this kernel):
+//   1 .. 4 tokens: only matrices of the size of the 70B layer's, where the shorter prologue of the other
+//     kernels no longer counts: 28672 x 8192 17.7 / 16.8 at 1 token, 22.2 / 17.4 at 4; 8192 x (28672 + 28672)
+//     31.5 / 30.2 at 3 (groups of 128 32.2 / 27.6, one scale 28.5 / 24.7), but 28.7 / 29.4 at 1; 8192 x 8192 7.1 / 7.2,
+//     q|k|v 8192 x 10240 8.8 / 9.0.  Binary16 scales: 8192 x 28672 21.5 / 16.2 at 1, 23.5 / 16.3 at 4; 8192 x 8192
+//     6.6 / 6.9, 4096 x 14336 5.2 / 6.1.
 //   5 .. 8 tokens: 8192 x 8192 8.3 / 7.7, 8192 x (28672 + 28672) 36.0 / 30.9, 28672 x 8192 23.0 / 18.3; but
 //     14336 x 4096 7.8 / 8.6, gate|up 4096 x (14336 + 14336) 9.0 / 11.0;
 //   9 .. 16 tokens: gate|up 13.9 / 13.0, 8192 x 8192 10.6 / 9.7, 8192 x (28672 + 28672) 65.2 / 35.3,
@@ -443,12 +458,13 @@ bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
     const int mode = env_int("W2A8_STAT", 1);
     if (mode == 0) return false;
     if (mode == 2) return true;
-    if (M < 5 || M > 256) return false;
+    if (M > 256) return false;
     for (const char *name : {"W2A8_CHUNKS", "W2A8_TG", "W2A8_RING", "W2A8_MT", "W2A8_CLUSTER", "W2A8_MIN_WARPS",
                              "W2A8_RELAX"})
         if (env_set(name)) return false;
     if (env_int("W2A8_GEMV", 1) == 2) return false;
     const long long blocks = K / kBlockK, cells = (long long)((tiles + 1) / 2) * blocks;
+    if (M <= 4) return cells >= 24576 && (h16 || blocks > (M == 1 ? 64 : 16));
     if (M <= 8) return gemv_preferred(M, K, group, tiles, count) && blocks > 16 && cells >= 8192;
     if (M <= 16 && !h16 && gemv_preferred(M, K, group, tiles, count)) return cells >= (blocks > 16 ? 8192 : 12288);
     if (M <= 32) return cells >= (count > 1 ? 1536 : 4096);
@@ -579,6 +595,9 @@ int launch_stat(const int8_t *a, const float *a_scale, int count, const uint32_t
     p.a = a; p.a_scale = a_scale; p.nmats = count; p.M = M; p.K = K; p.G = si.G; p.blocks = si.blocks;
     p.words_per_row = si.words_per_row; p.blocks_per_group = (group + kBlockK - 1) / kBlockK;
     p.pairs = pairs;
+    p.s_wide = (si.G * (h16 ? 2 : 4)) % 16 == 0 && (long long)pairs * si.blocks >= 12288;
+    for (int i = 0; i < count; ++i)
+        if (reinterpret_cast<uintptr_t>(w_scale[i]) % 16 != 0) p.s_wide = 0;
     p.y16 = y16 ? 1 : 0;
     const cudaError_t e = h16 ? launch_stat_mt<true>(p, si.spp, st) : launch_stat_mt<false>(p, si.spp, st);
     return e == cudaSuccess ? W2A8_OK : W2A8_ERR_CUDA;

@@ -43,6 +43,8 @@ CASES = [
     (64, 4096, [1024], 128, 0),               # eight: a full group
     (100, 2048, [272], 64, 2),                # two groups of seven slabs, the second not full
     (130, 512, [1024], 0, 0),                 # three groups
+    (3, 8192, [12304], 128, 0),               # large: the 16 bytes around the scales of a block
+    (2, 8192, [12288], 64, 0),
 ]
 
 
