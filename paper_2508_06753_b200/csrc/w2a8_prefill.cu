@@ -6,23 +6,32 @@
 // up-convert of Sec. II-C done into shared memory because the tensor core has
 // no 2-bit operand type.
 //
-// Persistent CTAs (12 warps, one CTA per SM) walk 128-channel x 128-token tiles of y.
-//   A operand (UMMA M = 128): weights.  Two "unpack" warps read the packed words
+// Persistent CTAs (16 warps, one CTA per SM) walk 128-channel x 128-token tiles of y.
+//   A operand (UMMA M = 128): weights.  Teams of two "unpack" warps read the packed words
 //     of 128 channels x one 256-k block, expand them to int8 lanes (value
 //     64 * (code - 2): one shift + one LOP3 per four weights) and store them
 //     K-major with the 128-byte swizzle the tensor core expects.
 //   B operand (UMMA N = 128): int8 activations, 128 tokens x 256 k, brought by TMA
-//     (issued by one lane of an unpack warp) with the same swizzle.
+//     with the same swizzle.
 //   D: int32 in tensor memory, lane = channel, column = token.  Because a lane is
 //     a channel, a drain thread needs one weight scale per group, not one per value.
 // Per 64-k group (or whatever the scale group is) an MMA thread issues K = 32 steps
 // into one of four accumulator buffers (all 512 TMEM columns).  MMA and drain hand
-// buffers over in units of two consecutive groups (a barrier round trip costs as much
-// as the MMAs of a 64-k group); two threads share the issuing, one unit slot each, in
+// buffers over in units of two consecutive groups (one by one was slower: 4096 x 14336
+// at 2048 tokens 286 against 243 us); two threads share the issuing, one unit slot each, in
 // straight-line code per stage (the kernel is specialised on the slices per group).
 // Eight "drain" warps (two per TMEM lane quarter, 64 token columns each) read finished
 // buffers with tcgen05.ld, software-pipelined in 32-column halves, convert to fp32 and
-// accumulate scale * value in registers with packed fp32 FMAs.  Stage slots and units
+// accumulate scale * value in registers with packed fp32 FMAs.  For groups of 64 and 128 one more
+// MMA, over a constant tile of 255s, starts every buffer from 32 * 255 * 255 instead of zero: the
+// sums are then positive integers below 2^24, whose bits read as a float are the (subnormal) number
+// sum * 2^-149, so the conversion is one packed FMA for two values that also takes the constant off
+// again, exactly.  The drain is two packed FMAs per two values and its loop two kilobytes of code; what bounds
+// the kernel at groups of 64 is the hand-off: buffers released, MMAs issued, finished and seen (800 cycles)
+// against 900 cycles of drain per unit, with unpack and drain sharing the issue slots.
+// Measured (4096 x 14336, us per call at 100 / 512 / 2048 tokens): conversion instructions, loop unrolled over
+// eight groups 26.6 / 76.3 / 283 (groups of 64) and 19.6 / 57.5 / 212 (128); loop over four groups, the scales of
+// four groups by one load, conversion by FMA 21.9 / 65.3 / 243 and 15.6 / 46.2 / 169.  Stage slots and units
 // are numbered across tiles, so the producers run ahead into the next tile while the
 // drain warps store y.  Every wait on an mbarrier is bounded; a wait that gives up
 // sets the status word of the workspace and the CTA winds down.
@@ -35,22 +44,29 @@
 #include "w2a8_tc.cuh"
 
 namespace w2a8 {
-// Of every eight drained values, how many are turned into floats by the integer-add route (the rest
-// by the conversion instruction): the two routes load different pipes -- the conversion instruction
-// issues at a quarter of the rate of an integer add, the add route takes one more issue slot per two
-// values -- and a mix beats either alone (4096 -> 14336, 2048 tokens, group 64: all conversions
-// 693 TOPS, all adds 702, half and half 760, two of eight by adds 772).
-constexpr int kPfMagicOfEight = 2;
-
-// Two warp layouts (template parameter UW = unpack warps):
-//   UW = 2: 12 warps -- 2 MMA issuers, 2 unpack warps (lane 0 of the first also issues the TMA
-//           loads), 8 drain warps; every thread has the same 168 registers.
-//   UW = 4: 16 warps in four warpgroups whose registers are re-balanced at entry (setmaxnreg):
-//           warps 0-3 two MMA issuers, the TMA producer, one spare (56 registers per thread);
-//           warps 4-7 unpack (104); warps 8-15 drain (176).
-__host__ __device__ constexpr int pf_threads(int uw) { return uw == 4 ? 512 : 384; }
-__host__ __device__ constexpr int pf_first_unpack(int uw) { return uw == 4 ? 4 : 2; }
-__host__ __device__ constexpr int pf_first_drain(int uw) { return uw == 4 ? 8 : 4; }
+// What the biased accumulators start from: one K step of unsigned 255 x 255.  It has to exceed every negative
+// sum of a group of 128 (at most 128 * 127 * 128 = kPfBias - 32), and bias + sum has to stay below 2^24.
+constexpr int kPfBias = 32 * 255 * 255;
+constexpr int kPfBiasBytes = 128 * 128;           // the tile of 255s, the A and the B operand of that step
+__host__ __device__ constexpr uint32_t pf_bias_desc(int m, int n) { return pf_instr_desc(m, n) & ~((7u << 7) | (7u << 10)); }
+// (acc0, acc1) += (d0 - kPfBias, d1 - kPfBias) * 2^-23 * sc.  d * 2^-149 (its bits as a float) times 2^126 minus
+// the bias is exact, and so is a scale that carries the factor 2^23: the sums are those of a conversion, bit for bit.
+__device__ __forceinline__ void pf_bias_fma2(float &acc0, float &acc1, int d0, int d1, float sc) {
+    asm("{\n\t.reg .b64 a, b, c, m, o;\n\t"
+        "mov.b64 a, {%2, %3};\n\t"
+        "mov.b64 m, {%5, %5};\n\t"
+        "mov.b64 o, {%6, %6};\n\t"
+        "fma.rn.f32x2 a, a, m, o;\n\t"
+        "mov.b64 b, {%4, %4};\n\t"
+        "mov.b64 c, {%0, %1};\n\t"
+        "fma.rn.f32x2 c, a, b, c;\n\t"
+        "mov.b64 {%0, %1}, c;\n\t}"
+        : "+f"(acc0), "+f"(acc1) : "r"(d0), "r"(d1), "f"(sc), "f"(0x1p126f), "f"(-(float)kPfBias * 0x1p-23f));
+}
+// 16 warps in four warpgroups whose registers are re-balanced at entry (setmaxnreg): warps 0-3 two MMA
+// issuers, the TMA producer, one spare (56 registers per thread); warps 4-7 unpack, two teams of two (104);
+// warps 8-15 drain (176).
+constexpr int kPfThreads = 512, kPfFirstUnpack = 4, kPfFirstDrain = 8;
 constexpr int kPfDrainCols = 64;         // token columns per drain warp (two warps share a lane quarter)
 constexpr int kPfBM = 128;               // channels per tile (UMMA M)
 constexpr int kPfBN = 128;               // tokens per tile (UMMA N)
@@ -86,8 +102,8 @@ __device__ __forceinline__ void pf_setmaxnreg_inc() { asm volatile("setmaxnreg.i
 
 // SPLIT: work items are (tile, K split) pairs; without it the split count is the constant 1 (the
 // general form costs 15 % on the unsplit problem: 596 against 702 TOPS at 2048 tokens, group 64).
-template <bool PARTIALS, bool H16, int DPS, int UW, bool SPLIT>
-__global__ void __launch_bounds__(pf_threads(UW), 1)
+template <bool PARTIALS, bool H16, int DPS, bool SPLIT>
+__global__ void __launch_bounds__(kPfThreads, 1)
 w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillParams p) {
     extern __shared__ unsigned char pf_smem_raw[];
     __shared__ __align__(8) unsigned long long bar_full[kPfStages], bar_empty[kPfStages];
@@ -130,6 +146,13 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
         pf_fence_proxy_async();
     }
     if (warp == 1) pf_tmem_alloc(pf_smem_u32(&tmem_base_slot), kPfTmemCols);
+    constexpr bool kBiased = DPS == 1 || DPS == 2;
+    const uint32_t bias_tile = smem_base + kPfStages * kPfStageBytes;
+    if constexpr (kBiased) {
+        for (int i = threadIdx.x; i < kPfBiasBytes / 16; i += kPfThreads)
+            pf_st_shared_v4(bias_tile + 16 * i, ~0u, ~0u, ~0u, ~0u);
+        pf_fence_proxy_async();
+    }
     pf_tc_fence_before();
     __syncthreads();
     pf_tc_fence_after();
@@ -140,31 +163,28 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
     // quantiser and one scale per channel, 2048 tokens, 119.5 / 110.7.
     pdl_launch_dependents();
 
-    constexpr int kFirstUnpack = pf_first_unpack(UW), kFirstDrain = pf_first_drain(UW);
-    if (warp < kFirstUnpack) {
-        if constexpr (UW == 4) {
-            pf_setmaxnreg_dec<56>();
-            if (warp == 2 && lane == 0) {
-                // ===== TMA producer: activations, 128 tokens x 256 k per stage ===============
-                pdl_wait();
-                int s = 0, round = 0;
-                for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-                    const int m0 = item_m0(tile), k0 = item_stage0(tile) * kPfBK;
-                    bool ok = true;
-                    for (int it = 0; it < nstages; ++it) {
-                        if (round > 0 && !pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) {
-                            ok = false;
-                            break;
-                        }
-                        const uint32_t bar = pf_smem_u32(&bar_full[s]);
-                        const uint32_t dst = smem_base + s * kPfStageBytes + 2 * kPfHalfBytes;
-                        pf_mbar_arrive_expect_tx(bar, 2 * kPfHalfBytes);
-                        pf_tma_load_2d(dst, &act_map, k0 + it * kPfBK, m0, bar);
-                        pf_tma_load_2d(dst + kPfHalfBytes, &act_map, k0 + it * kPfBK + 128, m0, bar);
-                        if (++s == kPfStages) { s = 0; ++round; }
+    if (warp < kPfFirstUnpack) {
+        pf_setmaxnreg_dec<56>();
+        if (warp == 2 && lane == 0) {
+            // ===== TMA producer: activations, 128 tokens x 256 k per stage ===============
+            pdl_wait();
+            int s = 0, round = 0;
+            for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+                const int m0 = item_m0(tile), k0 = item_stage0(tile) * kPfBK;
+                bool ok = true;
+                for (int it = 0; it < nstages; ++it) {
+                    if (round > 0 && !pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) {
+                        ok = false;
+                        break;
                     }
-                    if (!ok) break;
+                    const uint32_t bar = pf_smem_u32(&bar_full[s]);
+                    const uint32_t dst = smem_base + s * kPfStageBytes + 2 * kPfHalfBytes;
+                    pf_mbar_arrive_expect_tx(bar, 2 * kPfHalfBytes);
+                    pf_tma_load_2d(dst, &act_map, k0 + it * kPfBK, m0, bar);
+                    pf_tma_load_2d(dst + kPfHalfBytes, &act_map, k0 + it * kPfBK + 128, m0, bar);
+                    if (++s == kPfStages) { s = 0; ++round; }
                 }
+                if (!ok) break;
             }
         }
         // ===== MMA issuers (one thread in each of warps 0 and 1) =========================
@@ -203,6 +223,8 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                 const uint64_t bd = ((uint64_t)b_hi << 32) | (b_lo0 + so + koff);
                 pf_mma_i8(t0 + b * kPfBN, ad, bd, pf_instr_desc(kPfBM, kPfBN), accumulate);
             };
+            const uint64_t bias_desc = pf_smem_desc(bias_tile);
+            auto bias = [&](int b) { pf_mma_i8(t0 + b * kPfBN, bias_desc, bias_desc, pf_bias_desc(kPfBM, kPfBN), 0u); };
             auto next_stage = [&]() {
                 if (lead) pf_mma_commit(pf_smem_u32(&bar_empty[s]));   // stage can be refilled once these MMAs are done
                 so += kPfStageBytes >> 4;
@@ -225,15 +247,17 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                         if (!ok) break;
                         pf_tc_fence_after();
                         if (lead) {
-                            if (w == 0) { step(J0{}, 0, 0u); step(J1{}, 0, 1u); }
-                            else        { step(J4{}, 0, 0u); step(J5{}, 0, 1u); }
+                            bias(0);
+                            if (w == 0) { step(J0{}, 0, 1u); step(J1{}, 0, 1u); }
+                            else        { step(J4{}, 0, 1u); step(J5{}, 0, 1u); }
                         }
                         if (c >= 1) ok = pf_wait_all(acc_empty_bar1, (uint32_t)(c - 1) & 1u, abort_flag);
                         if (!ok) break;
                         pf_tc_fence_after();
                         if (lead) {
-                            if (w == 0) { step(J2{}, 1, 0u); step(J3{}, 1, 1u); }
-                            else        { step(J6{}, 1, 0u); step(J7{}, 1, 1u); }
+                            bias(1);
+                            if (w == 0) { step(J2{}, 1, 1u); step(J3{}, 1, 1u); }
+                            else        { step(J6{}, 1, 1u); step(J7{}, 1, 1u); }
                             pf_mma_commit(acc_full_bar);
                         }
                         next_stage();
@@ -250,12 +274,12 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                             if (u >= kPfUnits) ok = pf_wait_all(acc_empty_bar0, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
                             if (!ok) break;
                             pf_tc_fence_after();
-                            if (lead) { step(J0{}, 0, 0u); step(J1{}, 0, 1u); step(J2{}, 0, 1u); step(J3{}, 0, 1u); }
+                            if (lead) { bias(0); step(J0{}, 0, 1u); step(J1{}, 0, 1u); step(J2{}, 0, 1u); step(J3{}, 0, 1u); }
                             if (u >= kPfUnits) ok = pf_wait_all(acc_empty_bar1, (uint32_t)((u >> 1) - 1) & 1u, abort_flag);
                             if (!ok) break;
                             pf_tc_fence_after();
                             if (lead) {
-                                step(J4{}, 1, 0u); step(J5{}, 1, 1u); step(J6{}, 1, 1u); step(J7{}, 1, 1u);
+                                bias(1); step(J4{}, 1, 1u); step(J5{}, 1, 1u); step(J6{}, 1, 1u); step(J7{}, 1, 1u);
                                 pf_mma_commit(acc_full_bar);
                             }
                         }
@@ -301,16 +325,16 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                 }
             }
         }
-    } else if (warp < kFirstDrain) {
-        if constexpr (UW == 4) pf_setmaxnreg_dec<104>();
+    } else if (warp < kPfFirstDrain) {
+        pf_setmaxnreg_dec<104>();
         // ===== unpack warps: packed words -> int8 lanes, K-major, 128-byte swizzle =====
         // Teams of two warps; team j fills stages j, j + kTeams, ... (numbered across tiles).  With
         // two teams a stage's fixed costs -- the wait for the slot, the proxy fence, the arrive --
         // overlap the other team's unpack instead of adding to every stage.
-        constexpr int kTeams = UW / 2;
+        constexpr int kTeams = 2;
         constexpr int kUnits = 8;                   // 16-byte units per thread and stage
-        const int team = (warp - kFirstUnpack) >> 1;
-        const int ut = ((warp - kFirstUnpack) & 1) * 32 + lane;
+        const int team = (warp - kPfFirstUnpack) >> 1;
+        const int ut = ((warp - kPfFirstUnpack) & 1) * 32 + lane;
         // Unit u: 16 bytes of packed words (word t = u % 4 of the four slices) of one row.  The eight
         // lanes whose 16-byte stores share a shared-memory wavefront take rows that differ by four:
         // under the 128-byte swizzle (chunk ^= row % 8) their two groups of four chunks are then the
@@ -334,7 +358,6 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
         int s = team, round = 0;                    // slot and use count of the slot for this team's stage
         uint4 w_nxt[kUnits];
         if (tile < ntiles) request(w_nxt, tile, it);
-        if (UW == 2 && warp == kFirstUnpack) pdl_wait();      // its first lane brings the activations
         while (tile < ntiles) {
             uint4 w[kUnits];
 #pragma unroll
@@ -345,15 +368,6 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
             for (int j = 0; j < kTeams; ++j) advance(tile_nxt, it_nxt);
             if (tile_nxt < ntiles) request(w_nxt, tile_nxt, it_nxt);
             if (round > 0 && !pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
-            if (UW == 2 && warp == kFirstUnpack && lane == 0) {
-                // this lane is also the TMA producer: activations, 128 tokens x 256 k per stage
-                const int m0 = item_m0(tile), k = (item_stage0(tile) + it) * kPfBK;
-                const uint32_t bar = pf_smem_u32(&bar_full[s]);
-                const uint32_t dst = smem_base + s * kPfStageBytes + 2 * kPfHalfBytes;
-                pf_mbar_arrive_expect_tx(bar, 2 * kPfHalfBytes);
-                pf_tma_load_2d(dst, &act_map, k, m0, bar);
-                pf_tma_load_2d(dst + kPfHalfBytes, &act_map, k + 128, m0, bar);
-            }
             const uint32_t a_stage = smem_base + s * kPfStageBytes;      // shared-space address
 #pragma unroll
             for (int i = 0; i < kUnits; ++i) {
@@ -377,11 +391,21 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
     } else {
         // ===== drain warps: TMEM -> registers, fp32 accumulate with the group scale ======
         const int q4 = warp & 3;                    // TMEM lane quarter this warp may access
-        if constexpr (UW == 4) pf_setmaxnreg_inc<176>();
+        pf_setmaxnreg_inc<176>();
         pdl_wait();
-        const int col0 = ((warp - kFirstDrain) >> 2) * kPfDrainCols;   // first token column of this warp
+        const int col0 = ((warp - kPfFirstDrain) >> 2) * kPfDrainCols;   // first token column of this warp
         const int ch = q4 * 32 + lane;              // channel inside the tile = TMEM lane
         const uint32_t tlane = tmem_base + ((uint32_t)(q4 * 32) << 16) + col0;
+        auto add32 = [&](float *to, const int (&v)[32], float sc) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+                if constexpr (kBiased) pf_bias_fma2(to[j], to[j + 1], v[j], v[j + 1], sc);
+                else                   pf_fma2(to[j], to[j + 1], (float)v[j], (float)v[j + 1], sc);
+            }
+        };
+        // Groups per turn of the loop, and scales per load.  Unrolled over eight groups the loop was 17 KB of code,
+        // and drain and unpack warps waited for instructions; over two the scales arrive late (263 against 243 us).
+        constexpr int SR = 4;
         bool ok = true;
         int unit0 = 0;                              // units of the tiles before this one
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, unit0 += units_per_tile) {
@@ -392,35 +416,38 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
             float acc[kPfDrainCols];
 #pragma unroll
             for (int j = 0; j < kPfDrainCols; ++j) acc[j] = 0.f;
-            // Scales are fetched eight groups ahead (a drain takes a few hundred cycles, a
-            // global load several hundred): a ring of eight, refilled once per eight groups.
+            // Scales are fetched four groups ahead (a drain takes a few hundred cycles, a global load several
+            // hundred), as one load: the lanes' rows are G apart, so each load takes the load unit 32 sectors.
             const float *sc_row = PARTIALS ? nullptr : p.w_scale + (size_t)n * p.G + gbase;
             const unsigned short *sc_row_h = reinterpret_cast<const unsigned short *>(p.w_scale) + (size_t)n * p.G + gbase;
-            // The ring holds what the loads return, untouched: any instruction that reads a
-            // loaded register makes the warp wait for that load.  fp32: eight values.  binary16:
-            // eight values widened when they are taken out -- fetched as one 16-byte load when the
-            // row pitch allows (G % 8 == 0: registers 0..3 hold two scales each), else as eight
-            // 16-bit loads into 32-bit registers.
-            const bool vec8 = H16 && (p.G % 8 == 0) && (gbase % 8 == 0);
-            uint32_t sc_nxt[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+            // sc_nxt holds what the loads return, untouched: any instruction that reads a loaded register
+            // makes the warp wait for that load.  binary16: widened when they are taken out; as one load
+            // registers 0 and 1 hold two scales each.
+            uint32_t sc_nxt[SR] = {};
+            const bool vec = p.G % SR == 0 && gbase % SR == 0 && reinterpret_cast<uintptr_t>(p.w_scale) % ((H16 ? 2 : 4) * SR) == 0;
             auto refill = [&](int g0) {
                 if constexpr (PARTIALS) {
                     return;
                 } else if constexpr (H16) {
-                    if (vec8) {
+                    if (vec) {
                         if (g0 < ngroups) {
-                            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(sc_row_h + g0));
-                            sc_nxt[0] = v.x; sc_nxt[1] = v.y; sc_nxt[2] = v.z; sc_nxt[3] = v.w;
+                            const uint2 v = __ldg(reinterpret_cast<const uint2 *>(sc_row_h + g0));
+                            sc_nxt[0] = v.x; sc_nxt[1] = v.y;
                         }
                     } else {
 #pragma unroll
-                        for (int u = 0; u < 8; ++u)
+                        for (int u = 0; u < SR; ++u)
                             if (g0 + u < ngroups)
                                 asm volatile("ld.global.nc.u16 %0, [%1];" : "=r"(sc_nxt[u]) : "l"(sc_row_h + g0 + u));
                     }
+                } else if (vec) {
+                    if (g0 < ngroups) {
+                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(sc_row + g0));
+                        sc_nxt[0] = v.x; sc_nxt[1] = v.y; sc_nxt[2] = v.z; sc_nxt[3] = v.w;
+                    }
                 } else {
 #pragma unroll
-                    for (int u = 0; u < 8; ++u)
+                    for (int u = 0; u < SR; ++u)
                         if (g0 + u < ngroups) sc_nxt[u] = __float_as_uint(__ldg(sc_row + g0 + u));
                 }
             };
@@ -429,7 +456,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                     // one conversion that names the half of the register it reads
                     const __half2 pair = *reinterpret_cast<const __half2 *>(&sc_nxt[u >> 1]);
                     const __half2 lone = *reinterpret_cast<const __half2 *>(&sc_nxt[u]);
-                    if (vec8) return (u & 1) ? __high2float(pair) : __low2float(pair);
+                    if (vec) return (u & 1) ? __high2float(pair) : __low2float(pair);
                     return __low2float(lone);
                 } else {
                     return __uint_as_float(sc_nxt[u]);
@@ -441,15 +468,15 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
             int v0[32], v1[32];                         // first / second half of the current group
             ok = pf_wait_all(pf_smem_u32(&bar_acc_full[unit0 & 1]), (unit0 >> 1) & 1, abort_flag);
             if (ok) { pf_tc_fence_after(); pf_tmem_ld32(tlane + (2 * (unit0 & 1)) * kPfBN, v0); }
-            for (int g0 = 0; g0 < ngroups && ok; g0 += 8) {
-                float sc_cur[8];
+            for (int g0 = 0; g0 < ngroups && ok; g0 += SR) {
+                float sc_cur[SR];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    sc_cur[u] = take(u);
+                for (int u = 0; u < SR; ++u) {
+                    sc_cur[u] = take(u) * (kBiased ? 0x1p23f : 1.0f);
                 }
-                refill(g0 + 8);
+                refill(g0 + SR);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
+                for (int u = 0; u < SR; ++u) {
                     const int gi = g0 + u;
                     if (gi >= ngroups || !ok) break;
                     const int unit = unit0 + (gi >> 1);            // group gi lives in buffer 2 (unit % 2) + gi % 2
@@ -461,14 +488,10 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
                             const int m = m0 + col0 + j;
-                            if (m < p.M) p.partials[((size_t)m * p.N + n) * p.G + gi] = v0[j] >> 6;
+                            if (m < p.M) p.partials[((size_t)m * p.N + n) * p.G + gi] = (v0[j] - (kBiased ? kPfBias : 0)) >> 6;
                         }
                     } else {
-#pragma unroll
-                        for (int j = 0; j < 32; j += 2) {
-                            if ((j & 7) < kPfMagicOfEight) pf_cvt_fma2<DPS == 1 || DPS == 2>(acc[j], acc[j + 1], v0[j], v0[j + 1], sc);
-                            else                  pf_cvt_fma2<false>(acc[j], acc[j + 1], v0[j], v0[j + 1], sc);
-                        }
+add32(acc, v0, sc);
                     }
                     pf_tmem_ld_wait();                     // second half is in v1
                     {
@@ -490,13 +513,10 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
                             const int m = m0 + col0 + 32 + j;
-                            if (m < p.M) p.partials[((size_t)m * p.N + n) * p.G + gi] = v1[j] >> 6;
+                            if (m < p.M) p.partials[((size_t)m * p.N + n) * p.G + gi] = (v1[j] - (kBiased ? kPfBias : 0)) >> 6;
                         }
                     } else {
-#pragma unroll
-                        for (int j = 0; j < 32; j += 2)
-                            if ((j & 7) < kPfMagicOfEight) pf_cvt_fma2<DPS == 1 || DPS == 2>(acc[32 + j], acc[32 + j + 1], v1[j], v1[j + 1], sc);
-                            else                  pf_cvt_fma2<false>(acc[32 + j], acc[32 + j + 1], v1[j], v1[j + 1], sc);
+add32(acc + 32, v1, sc);
                     }
                 }
             }
@@ -552,16 +572,6 @@ __global__ void pf_splitk_reduce_kernel(const float *__restrict__ split_out, voi
 
 // ---- host side -----------------------------------------------------------------------
 
-// Unpack warps (warp layout) by scale group; W2A8_PF_UNPACK_WARPS = 2 or 4 overrides.
-int prefill_unpack_warps(int group) {
-    const int forced = env_int("W2A8_PF_UNPACK_WARPS", 0);
-    if (forced == 2 || forced == 4) return forced;
-    // Measured on B200 (4096 -> 14336, 2048 tokens, POPS with 2 / 4 unpack warps): group 64: 717 / 637;
-    // 128: 946 / 1006; 256: 1105 / 1328; K: 1130 / 1455.  With 64-k groups the drain warps are the
-    // bottleneck and two more warps competing for their issue slots cost more than a faster unpack
-    // gains; from 128 up the unpack is.
-    return group >= 128 ? 4 : 2;
-}
 bool prefill_supported(int M, int N, int K, int group) {
     if (M < 64) return false;
     if (N % kPfBM != 0 || K % kPfBK != 0) return false;
@@ -736,41 +746,29 @@ int launch_prefill(const int8_t *a, const float *a_scale, const uint32_t *packed
     const int nsplit = (partials || ldy != N) ? 1 : prefill_ksplit(M, N, K, group);
     p.ks_shift = nsplit == 8 ? 3 : nsplit == 4 ? 2 : nsplit == 2 ? 1 : 0;
     p.split_out = nsplit > 1 ? reinterpret_cast<float *>(reinterpret_cast<char *>(status) + kPfSplitOffset) : nullptr;
-    const size_t smem = (size_t)kPfStages * kPfStageBytes + 1024;
+    const size_t smem = (size_t)kPfStages * kPfStageBytes + kPfBiasBytes + 1024;
     const long long tiles = (long long)(N / kPfBM) * ((M + kPfBN - 1) / kPfBN) * nsplit;
     const int sms = sm_count();
     dim3 grid((unsigned)(tiles < sms ? tiles : sms));   // persistent CTAs, one per SM
-    static PerDeviceFlags configured[21];
-    auto launch = [&](auto kernel, int slot, int threads) -> bool {
+    static PerDeviceFlags configured[15];
+    auto launch = [&](auto kernel, int slot) -> bool {
         if (allow_dynamic_smem(kernel, configured[slot], (int)smem) != cudaSuccess) return false;
-        return launch_kernel(kernel, grid, dim3(threads), smem, st, pdl_enabled(), map, p) == cudaSuccess;
+        return launch_kernel(kernel, grid, dim3(kPfThreads), smem, st, pdl_enabled(), map, p) == cudaSuccess;
     };
     // The MMA-issuing code is specialised on the 64-k slices per scale group: 1, 2, or whole stages
-    // (0); the warp layout on the number of unpack warps (the parity export keeps the 12-warp one).
-    // A K split runs on the group's default layout only.
-    const int uw = nsplit > 1 ? (group >= 128 ? 4 : 2) : prefill_unpack_warps(group);
-    auto launch_dps = [&](auto partials_c, auto h16_c, auto uw_c, int slot0) -> bool {
-        constexpr bool P = decltype(partials_c)::value, H = decltype(h16_c)::value;
-        constexpr int U = decltype(uw_c)::value;
-        if (group == 64) return launch(w2a8_prefill_kernel<P, H, 1, U, false>, slot0, pf_threads(U));
-        if (group == 128) return launch(w2a8_prefill_kernel<P, H, 2, U, false>, slot0 + 1, pf_threads(U));
-        return launch(w2a8_prefill_kernel<P, H, 0, U, false>, slot0 + 2, pf_threads(U));
+    // (0).
+    auto launch_dps = [&](auto partials_c, auto h16_c, auto split_c, int slot0) -> bool {
+        constexpr bool P = decltype(partials_c)::value, H = decltype(h16_c)::value, S = decltype(split_c)::value;
+        if (group == 64) return launch(w2a8_prefill_kernel<P, H, 1, S>, slot0);
+        if (group == 128) return launch(w2a8_prefill_kernel<P, H, 2, S>, slot0 + 1);
+        return launch(w2a8_prefill_kernel<P, H, 0, S>, slot0 + 2);
     };
-    auto launch_split = [&](auto h16_c, int slot0) -> bool {
-        constexpr bool H = decltype(h16_c)::value;
-        if (group == 64) return launch(w2a8_prefill_kernel<false, H, 1, 2, true>, slot0, pf_threads(2));
-        if (group == 128) return launch(w2a8_prefill_kernel<false, H, 2, 4, true>, slot0 + 1, pf_threads(4));
-        return launch(w2a8_prefill_kernel<false, H, 0, 4, true>, slot0 + 2, pf_threads(4));
-    };
-    using U2 = std::integral_constant<int, 2>;
-    using U4 = std::integral_constant<int, 4>;
+    const std::true_type yes;
+    const std::false_type no;
     const bool launched =
-        partials     ? launch_dps(std::true_type{}, std::false_type{}, U2{}, 3)
-        : nsplit > 1 ? (h16 ? launch_split(std::true_type{}, 18) : launch_split(std::false_type{}, 15))
-        : h16        ? (uw == 4 ? launch_dps(std::false_type{}, std::true_type{}, U4{}, 12)
-                                : launch_dps(std::false_type{}, std::true_type{}, U2{}, 6))
-                     : (uw == 4 ? launch_dps(std::false_type{}, std::false_type{}, U4{}, 9)
-                                : launch_dps(std::false_type{}, std::false_type{}, U2{}, 0));
+        partials     ? launch_dps(yes, no, no, 0)
+        : nsplit > 1 ? (h16 ? launch_dps(no, yes, yes, 3) : launch_dps(no, no, yes, 6))
+                     : (h16 ? launch_dps(no, yes, no, 9) : launch_dps(no, no, no, 12));
     if (!launched) return W2A8_ERR_CUDA;
     if (nsplit > 1) {
         const size_t quads = (size_t)M * (N / 4);
