@@ -323,11 +323,20 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
 #pragma unroll
             for (int j = 0; j < kHfDrainCols; ++j) acc[j] = 0.f;
             const float *sc_row = PARTIALS ? nullptr : p.w_scale + (size_t)n * p.G;
-            uint32_t sc_nxt[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+            constexpr int SR = 4;        // groups per turn of the loop and scales per load, as in w2a8_prefill.cu
+            uint32_t sc_nxt[SR] = {};
+            const bool vec = !PARTIALS && p.G % SR == 0 && reinterpret_cast<uintptr_t>(p.w_scale) % (4 * SR) == 0;
             auto refill = [&](int g0) {
-                if constexpr (!PARTIALS) {
+                if constexpr (PARTIALS) {
+                    return;
+                } else if (vec) {
+                    if (g0 < ngroups) {
+                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(sc_row + g0));
+                        sc_nxt[0] = v.x; sc_nxt[1] = v.y; sc_nxt[2] = v.z; sc_nxt[3] = v.w;
+                    }
+                } else {
 #pragma unroll
-                    for (int u = 0; u < 8; ++u)
+                    for (int u = 0; u < SR; ++u)
                         if (g0 + u < ngroups) sc_nxt[u] = __float_as_uint(__ldg(sc_row + g0 + u));
                 }
             };
@@ -335,13 +344,13 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
             int v0[32], v1[32];                         // first / second half of the current group (fp32 bit patterns)
             ok = pf_wait_all(pf_smem_u32(&bar_acc_full[unit0 & 1]), (unit0 >> 1) & 1, abort_flag);
             if (ok) { pf_tc_fence_after(); pf_tmem_ld32(tlane + (2 * (unit0 & 1)) * kHfBN, v0); }
-            for (int g0 = 0; g0 < ngroups && ok; g0 += 8) {
-                float sc_cur[8];
+            for (int g0 = 0; g0 < ngroups && ok; g0 += SR) {
+                float sc_cur[SR];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) sc_cur[u] = __uint_as_float(sc_nxt[u]);
-                refill(g0 + 8);
+                for (int u = 0; u < SR; ++u) sc_cur[u] = __uint_as_float(sc_nxt[u]);
+                refill(g0 + SR);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
+                for (int u = 0; u < SR; ++u) {
                     const int gi = g0 + u;
                     if (gi >= ngroups || !ok) break;
                     const int unit = unit0 + (gi >> 1);
