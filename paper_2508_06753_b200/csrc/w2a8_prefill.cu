@@ -599,11 +599,11 @@ constexpr size_t kPfSplitOffset = 256;              // byte offset of the K-spli
 // Estimated time of the tensor-core path with the work of every tile split `nsplit` ways along K:
 // rounds of one work item per SM, each K / nsplit long, plus (split only) the launch of the summing
 // kernel and its traffic.
-static double prefill_seconds(int M, int N, int K, int group, int nsplit) {
+static double prefill_seconds(int M, int N, int K, int group, int nsplit, double round_seconds_per_k) {
     const long long items = (long long)(N / kPfBM) * ((M + kPfBN - 1) / kPfBN) * nsplit;
     const long long sms = sm_count();
     const long long rounds = (items + sms - 1) / sms;
-    double t = (double)rounds * (K / nsplit) * prefill_round_seconds_per_k(group);
+    double t = (double)rounds * (K / nsplit) * round_seconds_per_k;
     if (nsplit > 1) t += 2.0e-6 + (double)(nsplit + 1) * M * N * 4.0 / 3.0e12;
     return t;
 }
@@ -622,10 +622,10 @@ int prefill_ksplit(int M, int N, int K, int group) {
     const int forced = env_int("W2A8_PF_KSPLIT", 0);
     if (forced == 1 || forced == 2 || forced == 4 || forced == 8) return valid(forced) ? forced : 1;
     int best = 1;
-    double best_t = prefill_seconds(M, N, K, group, 1);
+    double best_t = prefill_seconds(M, N, K, group, 1, prefill_round_seconds_per_k(group));
     for (int sp = 2; sp <= 8; sp *= 2) {
         if (!valid(sp)) continue;
-        const double t = prefill_seconds(M, N, K, group, sp);
+        const double t = prefill_seconds(M, N, K, group, sp, prefill_round_seconds_per_k(group));
         if (t < best_t * 0.95) { best_t = t; best = sp; }      // a split has to pay by 5 % or more
     }
     return best;
@@ -644,7 +644,7 @@ size_t prefill_workspace_bytes(int M, int N, int K, int group) {
 // the streaming one) is kept with a split.  `can_split` = false: the caller's kernel has no K split.
 bool prefill_preferred(int M, int N, int K, int group, bool can_split) {
     const int sp = can_split ? prefill_ksplit(M, N, K, group) : 1;
-    double t_tc = prefill_seconds(M, N, K, group, sp);
+    double t_tc = prefill_seconds(M, N, K, group, sp, prefill_round_seconds_per_k(group));
     if (can_split && prefill_uses_wide(M, N, K, group)) {
         int c;
         const double t_wide = split_plan(M, N, K, 256, kWideRoundSecondsPerK, &c);
@@ -654,11 +654,16 @@ bool prefill_preferred(int M, int N, int K, int group, bool can_split) {
     return t_tc * (950000.0 / 875000.0) < t_stream;
 }
 
-// Expected time of a problem on the faster of the tensor-core path and the one-shot streaming kernel.
+// Expected time of a problem on the faster of the tensor-core path and the one-shot streaming kernel, for the
+// comparison with the kernel with stationary activations (65 to 256 tokens).  The 128-token tiles at what they
+// take now: 3 us and 4.9 / 3.4 / 3.0 / 2.4 ns per k and round for groups of 64 / 128 / 256 / more (us, estimate /
+// measured: 4096 x 14336 at 100 tokens 23.1 / 22.0, 4096 x 4096 12.7 / 13.1, 14336 x 4096 25.3 / 24.8, at 140 42.4 / 39.6).
+// The rules between the tensor-core and the streaming kernels keep the constants they were fitted with.
 double many_token_seconds(int M, int N, int K, int group) {
     double t = kStreamSecondsPerMac * (double)M * (double)N * (double)K;
     if (!prefill_supported(M, N, K, group)) return t;
-    const double t_tc = prefill_seconds(M, N, K, group, prefill_ksplit(M, N, K, group));
+    const double per_k = group <= 64 ? 4.9e-9 : group <= 128 ? 3.4e-9 : group <= 256 ? 3.0e-9 : 2.4e-9;
+    const double t_tc = 3.0e-6 + prefill_seconds(M, N, K, group, prefill_ksplit(M, N, K, group), per_k);
     if (t_tc < t) t = t_tc;
     if (prefill_uses_wide(M, N, K, group)) {
         int c;

@@ -450,7 +450,8 @@ static bool stat_supported(int M, int K, int group) {
 //     29.1 / 14.6, 34.4 / 22.1; 8192 x 8192 29.1 / 16.1, 37.2 / 23.5.
 //   65 .. 256 tokens: about 5 us + 0.27 ns per cell and slab (a little more for K > 8192, where clusters of six
 //     and eight leave SMs idle), against the model of the tensor-core kernels: 4096 x 4096 at 100 tokens
-//     15.1 / 12.6, at 200 20.9 / 19.8, but 4096 x 14336 at 100 29.6 / 31.3.
+//     13.1 / 12.5, 4096 x 14336 at 140 40.6 / 38.1, but at 100 22.0 / 31.1 and at 200 40.6 / 56.4, 14336 x 4096 at 140
+//     39.6 / 46.1.
 // W2A8_STAT = 0 never, 2 whenever it supports the shape; any switch that forces a plan of another kernel
 // keeps it out.
 bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
