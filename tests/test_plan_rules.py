@@ -1,0 +1,33 @@
+"""The automatic fuse rule at the edges of its range, on the host (no GPU needed)."""
+import pytest
+
+from paper_2508_06753_b200 import binding as b
+
+
+@pytest.fixture(autouse=True)
+def library(monkeypatch):
+    from paper_2508_06753_b200 import build
+    build.build()
+    for name in ("W2A8_FUSE_MAX_ELEMS", "W2A8_GEMV", "W2A8_STAT", "W2A8_GEMV_WARPS", "W2A8_GEMV_BCACHE"):
+        monkeypatch.delenv(name, raising=False)
+
+
+@pytest.mark.parametrize("Ns,M,K,fused", [
+    ([2048], 1, 2048, True),              # about one wave of CTAs
+    ([4736], 1, 4096, True),              # 296 tiles: the last of that range
+    ([4752], 1, 4096, False),
+    ([14192], 1, 4096, False),
+    ([14208], 1, 4096, True),             # 888 tiles: large enough again
+    ([14336, 14336], 1, 4096, True),
+    ([2048], 2, 2048, False),             # more than one token
+    ([4096], 1, 14336, False),            # activations do not stay in registers
+])
+def test_automatic_fuse_rule(Ns, M, K, fused):
+    assert b.w2a8_grouped_plan(Ns, M, K, 64)["fused"] is fused
+
+
+def test_limit_replaces_the_rule(monkeypatch):
+    monkeypatch.setenv("W2A8_FUSE_MAX_ELEMS", "0")
+    assert b.w2a8_grouped_plan([2048], 1, 2048, 64)["fused"] is False
+    monkeypatch.setenv("W2A8_FUSE_MAX_ELEMS", "4096")
+    assert b.w2a8_grouped_plan([2048], 2, 2048, 64)["fused"] is True
