@@ -16,8 +16,9 @@
 //    the compiler to keep many MMAs in flight.  Against two CTAs (128 registers) or 16 and 12 warps:
 //    14336 x 4096 at 32 tokens 12.9 / 13.7 us, at 64 tokens 22.1 / 26.9; 8192 x (28672 + 28672) at 16 tokens
 //    35.3 / 44.
-//  * Bound.  32 tokens: issue slots (about 540 warp instructions per cell, of which 64 MMAs, 128 packed
-//    promotions and 112 of unpack); 64 tokens: the MMA pipe at half its rate (425 of 1190 TOPS with 2 warps
+//  * Bound.  32 tokens: the chain unpack - MMA - promotion inside a warp (583 warp instructions per cell, of which
+//    64 MMAs, 128 packed promotions and 112 of unpack; with two warps per scheduler one issues every 3.2 clk: issue
+//    slots 32 %, tensor pipe 28 % busy, ncu at 14336 x 4096); 64 tokens: the MMA pipe at half its rate (425 of 1190 TOPS with 2 warps
 //    per scheduler); small problems: the 4 to 5 us that a launch costs beside the stream (a cold prologue, the
 //    activations after the dependency wait, two cluster barriers).
 #include "w2a8_cell.cuh"
