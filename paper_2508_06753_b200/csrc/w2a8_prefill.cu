@@ -159,6 +159,8 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
     const uint32_t tmem_base = tmem_base_slot;
     // Programmatic dependent launch: the set-up above and the first weights overlap the tail of the previous
     // kernel of the stream; the roles that touch anything else (activations, token scales, outputs) wait for it.
+    // So do the others before their first bounded wait (MMA issuers at once, unpack warps when a slot comes
+    // round again): the poll limit covers this kernel's own work, not whatever time its predecessor takes.
     // Measured (us per call, plain / dependent launch): 4096 x 14336 at 100 tokens 29.3 / 27.8, at 512 83.0 / 80.7;
     // quantiser and one scale per channel, 2048 tokens, 119.5 / 110.7.
     pdl_launch_dependents();
@@ -201,6 +203,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
         // The whole warp walks the loop and one elected lane issues: the waits cost a third of a lone lane's and
         // descriptors stay warp-uniform.
         if (warp < 2) {
+            pdl_wait();
             const bool lead = pf_elect();
             const int w = warp;             // this thread's unit slot: accumulator buffers 2 w and 2 w + 1
             const uint64_t a_desc0 = pf_smem_desc(smem_base);
@@ -367,7 +370,10 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
 #pragma unroll
             for (int j = 0; j < kTeams; ++j) advance(tile_nxt, it_nxt);
             if (tile_nxt < ntiles) request(w_nxt, tile_nxt, it_nxt);
-            if (round > 0 && !pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
+            if (round > 0) {
+                if (round == 1) pdl_wait();     // (a no-op once the previous kernel has completed)
+                if (!pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
+            }
             const uint32_t a_stage = smem_base + s * kPfStageBytes;      // shared-space address
 #pragma unroll
             for (int i = 0; i < kUnits; ++i) {

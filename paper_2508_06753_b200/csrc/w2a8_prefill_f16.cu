@@ -156,6 +156,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
         // on the low descriptor word.  A stage is two 64-k sub-tiles of four K = 16 steps each.
         // (The whole warp walks the loop and an elected lane issues, as in w2a8_prefill.cu.)
         if (warp < 2) {
+            pdl_wait();
             const bool lead = pf_elect();
             const int w = warp;
             const uint64_t a_desc0 = pf_smem_desc(smem_base);
@@ -283,7 +284,10 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
             int tile_nxt = tile, blk_nxt = blk + 1;
             if (blk_nxt == nblocks) { blk_nxt = 0; tile_nxt += gridDim.x; }
             if (tile_nxt < ntiles) request(w_nxt, tile_nxt, blk_nxt);
-            if (round > 0 && !pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
+            if (round > 0) {
+                if (round == 1) pdl_wait();     // (a no-op once the previous kernel has completed)
+                if (!pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
+            }
             unsigned char *a_stage = smem_gen + s * kHfStageBytes;
 #pragma unroll
             for (int i = 0; i < kUnits; ++i) {

@@ -119,6 +119,7 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
         // before its first MMA of the tile.  Straight-line issue: descriptors = 32-bit base + immediates.
         // (The whole warp walks the loop and an elected lane issues, as in w2a8_prefill.cu.)
         if (warp < 2) {
+            pdl_wait();
             const bool lead = pf_elect();
             const int w = warp;
             const uint64_t a_desc0 = pf_smem_desc(smem_base);
@@ -205,7 +206,10 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
             int tile_nxt = tile, blk_nxt = blk + 1;
             if (blk_nxt == nblocks) { blk_nxt = 0; tile_nxt += gridDim.x; }
             if (tile_nxt < ntiles) request(w_nxt, tile_nxt, blk_nxt);
-            if (round > 0 && !pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
+            if (round > 0) {
+                if (round == 1) pdl_wait();     // (a no-op once the previous kernel has completed)
+                if (!pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
+            }
             const uint32_t a_stage = smem_base + s * kWdStageBytes;
 #pragma unroll
             for (int i = 0; i < kUnits; ++i) {
