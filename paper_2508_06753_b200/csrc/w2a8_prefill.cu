@@ -79,6 +79,7 @@ constexpr int kPfTmemCols = kPfAccBufs * kPfBN;   // 512 columns: all of tensor 
 constexpr int kPfUnits = kPfAccBufs / 2;  // hand-off unit between MMA and drain: two groups (two buffers)
 
 struct PrefillParams {
+    const int8_t *a;
     const uint32_t *packed;
     const float *w_scale;
     const float *a_scale;
@@ -93,6 +94,29 @@ struct PrefillParams {
     int ks_shift;            // log2 of the K splits S: work item = tile * S + split; each split walks K / S
     float *split_out;        // S > 1: [S][M][N] fp32 partial outputs (summed in split order by a second kernel)
 };
+
+// The sum over groups [g0, g0 + n) of one output from memory, with the products and the order of the drain: for
+// channels with a scale that 2^23 takes out of range.
+__device__ __forceinline__ float pf_output_from_memory(const PrefillParams &p, int m, int n, int g0, int ngroups) {
+    const int8_t *a = p.a + (size_t)m * p.K;
+    const uint32_t *w = p.packed + (size_t)n * p.words_per_row;
+    float acc = 0.f;
+#pragma unroll 1
+    for (int gi = g0; gi < g0 + ngroups; ++gi) {
+        int sum = 0;
+#pragma unroll 1
+        for (int k = gi * p.group; k < (gi + 1) * p.group; k += 16) {
+            const uint32_t word = w[16 * (k >> 8) + 4 * ((k >> 4) & 3) + ((k >> 6) & 3)];
+            const int4 v = *reinterpret_cast<const int4 *>(a + k);
+            sum = __dp4a((int)lane_codes(word, 0), v.x, sum);
+            sum = __dp4a((int)lane_codes(word, 1), v.y, sum);
+            sum = __dp4a((int)lane_codes(word, 2), v.z, sum);
+            sum = __dp4a((int)lane_codes(word, 3), v.w, sum);
+        }
+        acc = fmaf((float)sum, p.w_scale[(size_t)n * p.G + gi], acc);
+    }
+    return acc;
+}
 
 // H16: w_scale points at IEEE binary16 values; the result is fp32 or, with p.y16, bf16.
 template <int N>
@@ -409,6 +433,8 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                 else                   pf_fma2(to[j], to[j + 1], (float)v[j], (float)v[j + 1], sc);
             }
         };
+        // fp32 scales may be too large for their factor of 2^23 (binary16 ones are not)
+        constexpr bool kLifted = kBiased && !H16 && !PARTIALS;
         // Groups per turn of the loop, and scales per load.  Unrolled over eight groups the loop was 17 KB of code,
         // and drain and unpack warps waited for instructions; over two the scales arrive late (263 against 243 us).
         constexpr int SR = 4;
@@ -497,7 +523,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                             if (m < p.M) p.partials[((size_t)m * p.N + n) * p.G + gi] = (v0[j] - (kBiased ? kPfBias : 0)) >> 6;
                         }
                     } else {
-add32(acc, v0, sc);
+                        add32(acc, v0, sc);
                     }
                     pf_tmem_ld_wait();                     // second half is in v1
                     {
@@ -522,21 +548,32 @@ add32(acc, v0, sc);
                             if (m < p.M) p.partials[((size_t)m * p.N + n) * p.G + gi] = (v1[j] - (kBiased ? kPfBias : 0)) >> 6;
                         }
                     } else {
-add32(acc + 32, v1, sc);
+                        add32(acc + 32, v1, sc);
                     }
                 }
             }
             pf_tmem_ld_wait();
             if (!PARTIALS && ok) {
+                auto store = [&](int m, float sum) {
+                    const float v = sum * (__ldg(p.a_scale + m) * (1.0f / kCodeGain));
+                    if (SPLIT)        p.split_out[((size_t)split * p.M + m) * p.N + n] = v;
+                    else if (H16 && p.y16) reinterpret_cast<__nv_bfloat16 *>(p.y)[(size_t)m * p.ldy + n] = __float2bfloat16_rn(v);
+                    else              p.y[(size_t)m * p.ldy + n] = v;
+                };
 #pragma unroll
                 for (int j = 0; j < kPfDrainCols; ++j) {
                     const int m = m0 + col0 + j;
-                    if (m < p.M) {
-                        const float v = acc[j] * (__ldg(p.a_scale + m) * (1.0f / kCodeGain));
-                        if (SPLIT)        p.split_out[((size_t)split * p.M + m) * p.N + n] = v;
-                        else if (H16 && p.y16) reinterpret_cast<__nv_bfloat16 *>(p.y)[(size_t)m * p.ldy + n] = __float2bfloat16_rn(v);
-                        else              p.y[(size_t)m * p.ldy + n] = v;
-                    }
+                    if (m < p.M) store(m, acc[j]);
+                }
+                if constexpr (kLifted) {
+                    // An fp32 scale of 2^105 or more became infinite with its factor of 2^23, and infinity times any
+                    // sum, zero too, leaves no running sum finite: one of them tells.  (Looking at the scales in the
+                    // loop costs 2 %.)  Ordinary weights never get here.
+                    if (!(fabsf(acc[0]) < __int_as_float(0x7F800000)))
+#pragma unroll 1
+                        for (int m = m0 + col0; m < min(m0 + col0 + kPfDrainCols, p.M); ++m)
+                            store(m, pf_output_from_memory(p, m, n, gbase, ngroups));
+                    __syncwarp();
                 }
             }
         }
@@ -745,7 +782,7 @@ int launch_prefill(const int8_t *a, const float *a_scale, const uint32_t *packed
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return W2A8_ERR_CUDA;
     PrefillParams p;
-    p.packed = packed; p.w_scale = reinterpret_cast<const float *>(w_scale); p.a_scale = a_scale;
+    p.a = a; p.packed = packed; p.w_scale = reinterpret_cast<const float *>(w_scale); p.a_scale = a_scale;
     p.y = reinterpret_cast<float *>(y); p.partials = partials; p.y16 = (h16 && y16) ? 1 : 0;
     p.ldy = ldy;
     p.status = status;
