@@ -396,7 +396,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
             if (tile_nxt < ntiles) request(w_nxt, tile_nxt, it_nxt);
             if (round > 0) {
                 if (round == 1) pdl_wait();     // (a no-op once the previous kernel has completed)
-                if (!pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
+                if (!pf_wait_all(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
             }
             const uint32_t a_stage = smem_base + s * kPfStageBytes;      // shared-space address
 #pragma unroll
@@ -499,8 +499,13 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
             // accumulated, the next half (possibly of the next group) is on its way from TMEM.
             int v0[32], v1[32];                         // first / second half of the current group
             ok = pf_wait_all(pf_smem_u32(&bar_acc_full[unit0 & 1]), (unit0 >> 1) & 1, abort_flag);
-            if (ok) { pf_tc_fence_after(); pf_tmem_ld32(tlane + (2 * (unit0 & 1)) * kPfBN, v0); }
-            for (int g0 = 0; g0 < ngroups && ok; g0 += SR) {
+            if (!ok) break;
+            pf_tc_fence_after();
+            pf_tmem_ld32(tlane + (2 * (unit0 & 1)) * kPfBN, v0);
+            // A lane whose wait gave up stays with its warp to the end of the tile (its later waits see the abort flag):
+            // the loads from tensor memory need all 32 lanes.
+            bool got = true;
+            for (int g0 = 0; g0 < ngroups; g0 += SR) {
                 float sc_cur[SR];
 #pragma unroll
                 for (int u = 0; u < SR; ++u) {
@@ -510,7 +515,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
 #pragma unroll
                 for (int u = 0; u < SR; ++u) {
                     const int gi = g0 + u;
-                    if (gi >= ngroups || !ok) break;
+                    if (gi >= ngroups) break;
                     const int unit = unit0 + (gi >> 1);            // group gi lives in buffer 2 (unit % 2) + gi % 2
                     const int buf = 2 * (unit & 1) + (gi & 1);
                     const float sc = sc_cur[u];
@@ -535,8 +540,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                     if (gi + 1 < ngroups) {                // request the first half of the next group
                         const int nunit = unit0 + ((gi + 1) >> 1);
                         if (((gi + 1) & 1) == 0) {         // it opens a new unit: wait for its MMAs
-                            ok = pf_wait(pf_smem_u32(&bar_acc_full[nunit & 1]), (nunit >> 1) & 1, abort_flag);   // all lanes poll: no broadcast step
-                            if (!ok) break;
+                            got &= pf_wait(pf_smem_u32(&bar_acc_full[nunit & 1]), (nunit >> 1) & 1, abort_flag);   // all lanes poll: no broadcast step
                             pf_tc_fence_after();
                         }
                         pf_tmem_ld32(tlane + (2 * (nunit & 1) + ((gi + 1) & 1)) * kPfBN, v0);
@@ -553,6 +557,7 @@ w2a8_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const PrefillPa
                 }
             }
             pf_tmem_ld_wait();
+            ok = __all_sync(0xFFFFFFFFu, got) != 0;
             if (!PARTIALS && ok) {
                 auto store = [&](int m, float sum) {
                     const float v = sum * (__ldg(p.a_scale + m) * (1.0f / kCodeGain));

@@ -286,7 +286,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
             if (tile_nxt < ntiles) request(w_nxt, tile_nxt, blk_nxt);
             if (round > 0) {
                 if (round == 1) pdl_wait();     // (a no-op once the previous kernel has completed)
-                if (!pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
+                if (!pf_wait_all(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
             }
             unsigned char *a_stage = smem_gen + s * kHfStageBytes;
 #pragma unroll
@@ -347,8 +347,13 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
             refill(0);
             int v0[32], v1[32];                         // first / second half of the current group (fp32 bit patterns)
             ok = pf_wait_all(pf_smem_u32(&bar_acc_full[unit0 & 1]), (unit0 >> 1) & 1, abort_flag);
-            if (ok) { pf_tc_fence_after(); pf_tmem_ld32(tlane + (2 * (unit0 & 1)) * kHfBN, v0); }
-            for (int g0 = 0; g0 < ngroups && ok; g0 += SR) {
+            if (!ok) break;
+            pf_tc_fence_after();
+            pf_tmem_ld32(tlane + (2 * (unit0 & 1)) * kHfBN, v0);
+            // A lane whose wait gave up stays with its warp to the end of the tile (its later waits see the abort flag):
+            // the loads from tensor memory need all 32 lanes.
+            bool got = true;
+            for (int g0 = 0; g0 < ngroups; g0 += SR) {
                 float sc_cur[SR];
 #pragma unroll
                 for (int u = 0; u < SR; ++u) sc_cur[u] = __uint_as_float(sc_nxt[u]);
@@ -356,7 +361,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
 #pragma unroll
                 for (int u = 0; u < SR; ++u) {
                     const int gi = g0 + u;
-                    if (gi >= ngroups || !ok) break;
+                    if (gi >= ngroups) break;
                     const int unit = unit0 + (gi >> 1);
                     const int buf = 2 * (unit & 1) + (gi & 1);
                     const float sc = sc_cur[u];
@@ -382,8 +387,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
                     if (gi + 1 < ngroups) {                // request the first half of the next group
                         const int nunit = unit0 + ((gi + 1) >> 1);
                         if (((gi + 1) & 1) == 0) {
-                            ok = pf_wait(pf_smem_u32(&bar_acc_full[nunit & 1]), (nunit >> 1) & 1, abort_flag);
-                            if (!ok) break;
+                            got &= pf_wait(pf_smem_u32(&bar_acc_full[nunit & 1]), (nunit >> 1) & 1, abort_flag);   // all lanes poll: no broadcast step
                             pf_tc_fence_after();
                         }
                         pf_tmem_ld32(tlane + (2 * (nunit & 1) + ((gi + 1) & 1)) * kHfBN, v0);
@@ -402,6 +406,7 @@ w2a16_prefill_kernel(const __grid_constant__ CUtensorMap act_map, const HfParams
                 }
             }
             pf_tmem_ld_wait();
+            ok = __all_sync(0xFFFFFFFFu, got) != 0;
             if (!PARTIALS && ok) {
 #pragma unroll
                 for (int j = 0; j < kHfDrainCols; ++j) {

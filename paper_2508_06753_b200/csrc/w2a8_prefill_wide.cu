@@ -208,7 +208,7 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
             if (tile_nxt < ntiles) request(w_nxt, tile_nxt, blk_nxt);
             if (round > 0) {
                 if (round == 1) pdl_wait();     // (a no-op once the previous kernel has completed)
-                if (!pf_wait(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
+                if (!pf_wait_all(pf_smem_u32(&bar_empty[s]), (round - 1) & 1, abort_flag)) break;
             }
             const uint32_t a_stage = smem_base + s * kWdStageBytes;
 #pragma unroll
@@ -246,7 +246,7 @@ w2a8_prefill_wide_kernel(const __grid_constant__ CUtensorMap act_map, const Wide
             float sc;
             if constexpr (H16) sc = __half2float(reinterpret_cast<const __half *>(p.w_scale)[n]);
             else               sc = __ldg(reinterpret_cast<const float *>(p.w_scale) + n);
-            ok = pf_wait(pf_smem_u32(&bar_acc_full[buf]), (uint32_t)(seq >> 1) & 1u, abort_flag);   // all lanes poll
+            ok = pf_wait_all(pf_smem_u32(&bar_acc_full[buf]), (uint32_t)(seq >> 1) & 1u, abort_flag);
             if (!ok) break;
             pf_tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q4 * 32) << 16) + buf * kWdBN + col0;
