@@ -281,11 +281,12 @@ int w2a8_gemm_partials(const int8_t *a, const uint32_t *packed, int32_t *partial
  *                                  the first three are DEVICE pointers as for w2a8_gemm
  *   workspace                      w2a8_grouped_workspace_bytes(count, N, M, K, group)
  * Each y[i] holds what w2a8_gemm computes for matrix i: bit for bit when both
- * calls take the same kernel, except that the kernel with stationary activations
- * (more than four tokens, larger problems) deals the work of a launch to its CTAs as a
- * whole, so there the order of the fp32 additions may differ.  With any kernel
- * it is within the tolerance of w2a8_gemm's contract and repeated calls give
- * equal bits.
+ * calls take the same kernel, unless that is the kernel with stationary
+ * activations (larger problems of up to 32 tokens; the largest from one token
+ * on).  It deals the channels of all matrices of a launch to its CTAs as one
+ * sequence, so with it the order of the fp32 additions depends on the group.
+ * With any kernel the result is within the tolerance of w2a8_gemm's contract
+ * and repeated calls on the same group give equal bits.
  */
 int w2a8_gemm_grouped(const int8_t *a, const float *a_scale, int count, const uint32_t *const *packed,
                       const float *const *w_scale, float *const *y, const int *N, int M, int K, int group,

@@ -81,3 +81,29 @@ def test_stat_against_reference(gpu, oracle, monkeypatch, M, K, Ns, group, share
         ref = oracle.gemm(a_ref, s_ref, codes, s_w.astype(np.float32), g)
         err = np.abs(y.cpu().numpy().astype(np.float64) - ref).max(axis=1)
         assert (err <= TOL * np.abs(ref).max(axis=1)).all(), float(err.max())
+
+
+@pytest.mark.parametrize("M,K,Ns,group", [
+    (2, 8192, [28672, 28672], 128),         # few tokens: each matrix alone is large enough for the kernel too
+    (32, 4096, [14336, 14336], 64),
+    (12, 8192, [8192, 1024, 1024], 0),      # and two that alone go to the persistent kernel
+])
+def test_grouped_against_single_calls(gpu, M, K, Ns, group):
+    """By default, i.e. by the dispatch rule: the fp32 additions may come in another order than alone (at most
+    K / 64 of them per output, so a few times 2^-24 of the largest output of a row), equal bits on repeats."""
+    torch, b = gpu
+    g = K if group == 0 else group
+    gen = torch.Generator(device="cuda").manual_seed(M + K)
+    rand = lambda *shape: torch.rand(shape, generator=gen, device="cuda")
+    packed = [b.w2_pack((4 * rand(N, K)).to(torch.uint8).clamp_(max=3)) for N in Ns]
+    scales = [0.01 + 0.02 * rand(N, K // g) for N in Ns]
+    a, s_a = b.a8_quantize((rand(M, K) - 0.5).to(torch.bfloat16))
+    ws = b.new_workspace(b.w2a8_grouped_workspace_bytes(Ns, M, K, g))
+    ys = [y.clone() for y in b.w2a8_gemm_grouped(a, s_a, b.Group(packed, scales), g, ws)]
+    again = b.w2a8_gemm_grouped(a, s_a, b.Group(packed, scales), g, ws)
+    for pk, sc, y, y2 in zip(packed, scales, ys, again):
+        assert torch.equal(y, y2)
+        alone = b.w2a8_gemm(a, s_a, pk, sc, g, ws)
+        assert torch.equal(alone, b.w2a8_gemm(a, s_a, pk, sc, g, ws))
+        err = (y.double() - alone.double()).abs().amax(dim=1)
+        assert bool((err <= 1e-5 * alone.double().abs().amax(dim=1)).all()), float(err.max())
