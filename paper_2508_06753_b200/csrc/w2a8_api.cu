@@ -46,10 +46,9 @@ int launch_a8_to_bf16(const int8_t *a, void *scratch, int M, int K, cudaStream_t
 
 // ---- W2A8_* switches of the environment ---------------------------------------------
 // A call asks for some forty of them; reading each with getenv was 2 us of a call that launches a 2 us
-// kernel.  Values are kept per thread, together with a fingerprint of the environment block: the
-// addresses of its strings (the C library makes a new string whenever a variable is set to a new value,
-// so any change moves the fingerprint).  Inside an EnvScope, i.e. once per call, the fingerprint is taken
-// once.
+// kernel.  Values are kept per thread, together with a fingerprint of the W2A8_* strings of the environment.
+// Of their contents: a string that was given to putenv may be edited in place.  Inside an EnvScope, i.e. once
+// per call, the fingerprint is taken once.
 extern "C" char **environ;
 namespace {
 struct EnvCache {
@@ -61,7 +60,11 @@ thread_local EnvCache t_env;
 
 uint64_t take_fingerprint() {
     uint64_t h = 1469598103934665603ull;
-    for (char **e = environ; e && *e; ++e) h = (h ^ (uint64_t)(uintptr_t)*e) * 1099511628211ull;
+    for (char **e = environ; e && *e; ++e) {
+        const char *c = *e;
+        if (c[0] != 'W' || c[1] != '2' || c[2] != 'A' || c[3] != '8') continue;
+        do h = (h ^ (unsigned char)*c) * 1099511628211ull; while (*c++);       // the terminator too
+    }
     return h;
 }
 void refresh_env(EnvCache &c) {
