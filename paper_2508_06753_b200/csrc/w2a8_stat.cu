@@ -471,10 +471,11 @@ bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
     if (M <= 16 && !h16 && gemv_preferred(M, K, group, tiles, count)) return cells >= (blocks > 16 ? 8192 : 12288);
     if (M <= 32) return cells >= (count > 1 ? 1536 : 4096);
     if (count > 1) return false;                  // (more than 32 tokens: a launch per matrix)
+    if (M >= 64)
+        for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE",
+                                 "W2A8_PF_UNPACK_WARPS"})
+            if (env_set(name)) return false;
     if (M <= 64) return cells >= 1024;
-    for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE",
-                             "W2A8_PF_UNPACK_WARPS"})
-        if (env_set(name)) return false;
     const double mine = 5.0e-6 + 0.27e-9 * (blocks > 32 ? 1.15 : 1.0) * (double)cells * st_tgroups(M) * st_slabs(M);
     return mine < 0.95 * many_token_seconds(M, tiles * 16, K, group);
 }

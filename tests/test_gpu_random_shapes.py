@@ -93,6 +93,8 @@ def test_gemm_random_prefill_shapes(gpu, oracle, monkeypatch, seed):
                           {"W2A8_PREFILL": "2", "W2A8_PF_UNPACK_WARPS": rng.choice(["2", "4"])}])
         for k, v in env.items():
             monkeypatch.setenv(k, v)
+        if env:
+            assert b.w2a8_kernel_for(M, N, K, g) == "tensor_core", (M, N, K, g, env)
         codes, s_w = synth.make_linear(rng.randrange(1 << 20), K, N, g)
         bits = synth.activations_bf16(rng.randrange(1 << 20), M, K)
         a, s_a = b.a8_quantize(_dev(torch, bits.view(np.int16)).view(torch.bfloat16))

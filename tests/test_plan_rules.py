@@ -1,4 +1,5 @@
-"""The automatic fuse rule at the edges of its range, on the host (no GPU needed)."""
+"""Dispatch rules on the host (no GPU needed): the automatic fuse rule at the edges of its range, and the switches
+that force the tensor-core kernel."""
 import pytest
 
 from paper_2508_06753_b200 import binding as b
@@ -8,7 +9,8 @@ from paper_2508_06753_b200 import binding as b
 def library(monkeypatch):
     from paper_2508_06753_b200 import build
     build.build()
-    for name in ("W2A8_FUSE_MAX_ELEMS", "W2A8_GEMV", "W2A8_STAT", "W2A8_GEMV_WARPS", "W2A8_GEMV_BCACHE"):
+    for name in ("W2A8_FUSE_MAX_ELEMS", "W2A8_GEMV", "W2A8_STAT", "W2A8_GEMV_WARPS", "W2A8_GEMV_BCACHE",
+                 "W2A8_PREFILL", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE", "W2A8_TC_KIND"):
         monkeypatch.delenv(name, raising=False)
 
 
@@ -31,3 +33,18 @@ def test_limit_replaces_the_rule(monkeypatch):
     assert b.w2a8_grouped_plan([2048], 1, 2048, 64)["fused"] is False
     monkeypatch.setenv("W2A8_FUSE_MAX_ELEMS", "4096")
     assert b.w2a8_grouped_plan([2048], 2, 2048, 64)["fused"] is True
+
+
+@pytest.mark.parametrize("M", [64, 65, 128, 256])
+@pytest.mark.parametrize("N,K", [(4096, 4096), (14336, 4096), (4096, 14336), (128, 256)])
+def test_tensor_core_kernel_when_forced(monkeypatch, M, N, K):
+    for more in ({}, {"W2A8_PF_KSPLIT": "2"}, {"W2A8_PF_WIDE": "2"}, {"W2A8_TC_KIND": "16"}):
+        monkeypatch.setenv("W2A8_PREFILL", "2")
+        for name, value in more.items():
+            monkeypatch.setenv(name, value)
+        assert b.w2a8_kernel_for(M, N, K, 64) == "tensor_core", more
+        assert b.w2a8_kernel_for(M, N, K, K) == "tensor_core", more
+        for name in more:
+            monkeypatch.delenv(name)
+    monkeypatch.setenv("W2A8_PREFILL", "0")
+    assert b.w2a8_kernel_for(M, N, K, 64) == "streaming"
