@@ -362,15 +362,19 @@ static int tensor_core_channels(int M, int N, int K, int group);
 
 static bool tensor_core_kind_is_16(int M, int N, int K, int group);
 
-// Workspace of the kernels themselves (status word, split-K counters and partial outputs).
+// Workspace of the kernels themselves (status word, split-K counters and partial outputs), whichever entry point
+// the call comes through: int8 activations may go to the tensor cores or not, and bf16 ones by a rule of their own.
 static size_t kernel_workspace_bytes(int M, int N, int K, int group) {
     ShapeInfo si;
     if (!shape_ok(M, N, K, group, &si)) return 0;
     size_t need = decode_workspace_bytes(M, N, K, si);
-    if (takes_tensor_core_kernel(M, N, K, group)) {
+    const bool int8_takes = takes_tensor_core_kernel(M, N, K, group);
+    if (int8_takes) {
         // partial outputs of a K split of the int8 tensor-core kernel
         const size_t split = prefill_workspace_bytes(M, N, K, group);
         if (split > need) need = split;
+    }
+    if (int8_takes || takes_tensor_core_kernel_ex(M, N, K, group, false)) {
         // the last channel tiles may be given to the streaming kernel, with a plan of its own
         const int n_tc = tensor_core_channels(M, N, K, group);
         ShapeInfo rest;

@@ -48,3 +48,26 @@ def test_tensor_core_kernel_when_forced(monkeypatch, M, N, K):
             monkeypatch.delenv(name)
     monkeypatch.setenv("W2A8_PREFILL", "0")
     assert b.w2a8_kernel_for(M, N, K, 64) == "streaming"
+
+
+def test_workspace_covers_the_channel_remainder_of_bf16_activations(monkeypatch):
+    """w2a16_gemm has a tensor-core rule of its own and may split channels where w2a8_gemm does not; one query
+    sizes the workspace of both."""
+    found = 0
+    for M in (65, 100, 136, 140, 180, 200, 256, 300, 512, 700):
+        for N in (4096, 8192, 14336, 19456, 28672):
+            for K in (1024, 2048, 4096, 8192):
+                for group in (64, 128, K):
+                    monkeypatch.setenv("W2A8_TC_KIND", "16")         # the rule for 16-bit operands
+                    takes = b.w2a8_kernel_for(M, N, K, group) == "tensor_core"
+                    channels = b.w2a8_tensor_core_channels(M, N, K, group)
+                    monkeypatch.delenv("W2A8_TC_KIND")
+                    if not takes or channels == N:
+                        continue
+                    found += 1
+                    size = b.w2a8_workspace_bytes(M, N, K, group)
+                    monkeypatch.setenv("W2A8_PREFILL", "0")          # the remainder runs on a streaming kernel
+                    rest = b.w2a8_workspace_bytes(M, N - channels, K, group)
+                    monkeypatch.delenv("W2A8_PREFILL")
+                    assert size >= rest, (M, N, K, group)
+    assert found > 10
