@@ -732,6 +732,10 @@ int launch_decode(const int8_t *a, const float *a_scale, const uint32_t *packed,
     p.status = reinterpret_cast<int *>(base);
     p.counters = reinterpret_cast<unsigned *>(base + kStatusBytes);
     p.ws = reinterpret_cast<float *>(base + kStatusBytes + counters);
+    if (pl.chunks > 1 && !p.cluster && !partials) {
+        // more chunks than a cluster holds: the arrival counters may lie where another shape's partial outputs lay
+        if (cudaMemsetAsync(p.counters, 0, counters, st) != cudaSuccess) return W2A8_ERR_CUDA;
+    }
     if (partials) {
         // several warps add their share of a large group: start from zero
         if (cudaMemsetAsync(partials, 0, (size_t)M * N * si.G * sizeof(int32_t), st) != cudaSuccess)
