@@ -521,8 +521,12 @@ size_t gemm_header_bytes(int M, int N, int K, int group) {
 int gemm_dispatch(const int8_t *a, const float *a_scale, const uint32_t *packed, const void *w_scale,
                   void *y, int32_t *partials, int M, int N, int K, int group, const ShapeInfo &si,
                   void *workspace, void *stream, bool h16, bool y16, bool a16) {
-    if (!a16 && !partials && stat_takes(M, K, group, N / 16, 1, h16))
-        return launch_stat(a, a_scale, 1, &packed, &w_scale, &y, &N, &N, M, K, group, (cudaStream_t)stream, h16, y16);
+    if (!a16 && !partials && stat_takes(M, K, group, N / 16, 1, h16)) {
+        const int st = launch_stat(a, a_scale, 1, &packed, &w_scale, &y, &N, &N, M, K, group, (cudaStream_t)stream, h16, y16);
+        if (st != kStatNoPlan) return st;
+        return launch_decode(a, a_scale, packed, w_scale, y, nullptr, M, N, K, group, si, workspace,
+                             (cudaStream_t)stream, h16, y16, false, N);
+    }
     const bool takes = a16 ? takes_tensor_core_kernel_ex(M, N, K, group, false) : takes_tensor_core_kernel(M, N, K, group);
     const bool tc16 = !h16 && takes && prefill_f16_supported(M, N, K, group) &&
                       (a16 || tensor_core_kind_is_16(M, N, K, group));
@@ -682,10 +686,14 @@ static int grouped_common(const void *x_bf16, const int8_t *a_in, const float *a
     }
     int tiles = 0;
     for (int i = 0; i < count; ++i) tiles += N[i] / 16;
-    if (plan == 1 && stat_takes(M, K, group, tiles, count, false))
-        return launch_stat(a_in, a_scale_in, count, packed, reinterpret_cast<const void *const *>(w_scale),
-                           reinterpret_cast<void *const *>(y), N, N, M, K, group, (cudaStream_t)stream, false, false);
-    if (plan == 1)          // one launch over all matrices
+    bool gemv = plan == 1;
+    if (plan == 1 && stat_takes(M, K, group, tiles, count, false)) {
+        const int st = launch_stat(a_in, a_scale_in, count, packed, reinterpret_cast<const void *const *>(w_scale),
+                                   reinterpret_cast<void *const *>(y), N, N, M, K, group, (cudaStream_t)stream, false, false);
+        if (st != kStatNoPlan) return st;
+        gemv = gemv_supported(M, K, group);
+    }
+    if (gemv)               // one launch over all matrices
         return launch_gemv(a_in, a_scale_in, nullptr, nullptr, nullptr, count, packed, w_scale, y, N, N, M, K, group,
                            (cudaStream_t)stream);
     for (int i = 0; i < count; ++i)     // one launch per matrix (same stream, so one workspace serves all)

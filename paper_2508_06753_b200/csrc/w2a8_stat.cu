@@ -553,7 +553,7 @@ static cudaError_t launch_stat_inst(StParams &p, cudaStream_t st) {
         cs.known.store(1, std::memory_order_release);
     }
     StPlan pl;
-    if (!stat_plan(p.M, p.K, p.pairs, cs.n, &pl)) return cudaErrorInvalidValue;
+    if (!stat_plan(p.M, p.K, p.pairs, cs.n, &pl)) return cudaErrorNotSupported;
     p.C = pl.C; p.round_pairs = pl.round_pairs;
     p.blk_per = p.blocks / pl.C; p.blk_extra = p.blocks % pl.C;
     for (int i = 0; i < 2; ++i) p.nb_inv[i] = (65536 + p.blk_per + i - 1) / (p.blk_per + i);
@@ -581,7 +581,9 @@ static cudaError_t launch_stat_mt(StParams &p, int spp, cudaStream_t st) {
     }
 }
 
-// Enqueue one launch over `count` matrices (1 .. 4) that share their activations.
+// Enqueue one launch over `count` matrices (1 .. 4) that share their activations.  kStatNoPlan: nothing was launched,
+// because no cluster size holds the activations and is resident for every token group (a small partition of a GPU,
+// or a forced W2A8_STAT_C); how many clusters are resident is only known here, with a context.
 int launch_stat(const int8_t *a, const float *a_scale, int count, const uint32_t *const *packed,
                 const void *const *w_scale, void *const *y, const int *N, const int *ldy, int M, int K, int group,
                 cudaStream_t st, bool h16, bool y16) {
@@ -603,7 +605,7 @@ int launch_stat(const int8_t *a, const float *a_scale, int count, const uint32_t
         if (reinterpret_cast<uintptr_t>(w_scale[i]) % 16 != 0) p.s_wide = 0;
     p.y16 = y16 ? 1 : 0;
     const cudaError_t e = h16 ? launch_stat_mt<true>(p, si.spp, st) : launch_stat_mt<false>(p, si.spp, st);
-    return e == cudaSuccess ? W2A8_OK : W2A8_ERR_CUDA;
+    return e == cudaSuccess ? W2A8_OK : e == cudaErrorNotSupported ? kStatNoPlan : W2A8_ERR_CUDA;
 }
 
 }  // namespace w2a8

@@ -107,3 +107,25 @@ def test_grouped_against_single_calls(gpu, M, K, Ns, group):
         assert torch.equal(alone, b.w2a8_gemm(a, s_a, pk, sc, g, ws))
         err = (y.double() - alone.double()).abs().amax(dim=1)
         assert bool((err <= 1e-5 * alone.double().abs().amax(dim=1)).all()), float(err.max())
+
+
+@pytest.mark.parametrize("M,K,Ns,shares", [
+    (64, 14336, [256], 1),               # eight slabs of 56 blocks do not fit one CTA
+    (32, 28672, [64, 32], 2),            # a group: to the persistent kernel
+    (40, 28672, [64, 32], 2),            # more tokens than that one takes
+])
+def test_shapes_without_a_plan_take_another_kernel(gpu, oracle, monkeypatch, M, K, Ns, shares):
+    torch, b = gpu
+    monkeypatch.setenv("W2A8_STAT", "2")
+    monkeypatch.setenv("W2A8_STAT_C", str(shares))
+    mats = [synth.make_linear(K + i, K, N, 64) for i, N in enumerate(Ns)]
+    bits = synth.activations_bf16(M, M, K)
+    a, s_a = b.a8_quantize(_dev(torch, bits.view(np.int16)).view(torch.bfloat16))
+    grp = b.Group([b.w2_pack(_dev(torch, c)) for c, _ in mats], [_dev(torch, s) for _, s in mats])
+    ws = b.new_workspace(b.w2a8_grouped_workspace_bytes(Ns, M, K, 64))
+    ys = b.w2a8_gemm_grouped(a, s_a, grp, 64, ws)
+    a_ref, s_ref = oracle.quantize(bits)
+    for (codes, s_w), y in zip(mats, ys):
+        ref = oracle.gemm(a_ref, s_ref, codes, s_w, 64)
+        err = np.abs(y.cpu().numpy().astype(np.float64) - ref).max(axis=1)
+        assert (err <= TOL * np.abs(ref).max(axis=1)).all(), float(err.max())
