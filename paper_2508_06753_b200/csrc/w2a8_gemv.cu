@@ -446,6 +446,8 @@ static int gemv_warps(int M, int K) {
     return fits ? 8 : 16;
 }
 
+bool gemv_half_sm(int M, int K) { return gemv_warps(M, K) == 8; }
+
 // Whether this kernel serves the shape at all: whole 256-k blocks only (a ragged last block is
 // left to the one-shot streaming kernel), at most kGvMaxTokens tokens.  W2A8_GEMV=0 switches the
 // kernel off, and so does any switch that forces a launch plan of the one-shot kernel.

@@ -26,6 +26,10 @@
 namespace w2a8 {
 
 bool gemv_preferred(int M, int K, int group, int tiles, int count);
+bool gemv_half_sm(int M, int K);
+bool decode_one_wave(int M, int N, int K, int group, bool h16);
+bool prefill_supported(int M, int N, int K, int group);
+bool prefill_preferred(int M, int N, int K, int group, bool can_split);
 double many_token_seconds(int M, int N, int K, int group);
 
 constexpr int kStMaxMats = 4;
@@ -438,8 +442,10 @@ static bool stat_supported(int M, int K, int group) {
 //     31.5 / 30.2 at 3 (groups of 128 32.2 / 27.6, one scale 28.5 / 24.7), but 28.7 / 29.4 at 1; 8192 x 8192 7.1 / 7.2,
 //     q|k|v 8192 x 10240 8.8 / 9.0.  Binary16 scales: 8192 x 28672 21.5 / 16.2 at 1, 23.5 / 16.3 at 4; 8192 x 8192
 //     6.6 / 6.9, 4096 x 14336 5.2 / 6.1.
-//   5 .. 8 tokens: 8192 x 8192 8.3 / 7.7, 8192 x (28672 + 28672) 36.0 / 30.9, 28672 x 8192 23.0 / 18.3; but
-//     14336 x 4096 7.8 / 8.6, gate|up 4096 x (14336 + 14336) 9.0 / 11.0;
+//   5 .. 8 tokens: 8192 x (28672 + 28672) 36.0 / 30.9, 28672 x 8192 23.0 / 18.3, 8192 x (10240 + 1024 + 1024) 10.3 / 9.8;
+//     but 14336 x 4096 7.8 / 8.6, gate|up 4096 x (14336 + 14336) 9.0 / 11.0, 8192 x (8192 + 1024 + 1024) 8.9 / 9.45 (groups of
+//     128 9.0 / 9.0, one scale 8.5 / 8.0).  Against the persistent kernel in its two-CTAs-per-SM form, 5120 x (8192 +
+//     8192) at 6 tokens: 8.3 / 9.3, of 128 8.0 / 9.1, one scale 7.8 / 7.7; 5120 x (14336 + 14336) 13.1 / 13.0;
 //   9 .. 16 tokens: gate|up 13.9 / 13.0, 8192 x 8192 10.6 / 9.7, 8192 x (28672 + 28672) 65.2 / 35.3,
 //     28672 x 8192 29.9 / 21.8; but 4096 x 14336 8.3 / 8.8, 14336 x 4096 9.5 / 9.7.  Where only the one-shot
 //     kernel is left (binary16 scales): 4096 x 14336 9.9 / 8.2, 14336 x 4096 11.1 / 9.6, 4096 x 4096 4.1 / 4.9.
@@ -448,8 +454,12 @@ static bool stat_supported(int M, int K, int group) {
 //     a launch costs 4 to 5 us beside the stream, so small problems stay where they were, unless the
 //     alternative is a launch per matrix (q|k|v 4096 x 6144 12.0 / 8.7).
 //   33 .. 64 tokens: 4096 x 4096 8.8 / 7.2, 11.8 / 9.9; 4096 x 14336 20.6 / 13.5, 27.9 / 20.3; 14336 x 4096
-//     29.1 / 14.6, 34.4 / 22.1; 8192 x 8192 29.1 / 16.1, 37.2 / 23.5.
-//   65 .. 256 tokens: about 5 us + 0.27 ns per cell and slab (a little more for K > 8192, where clusters of six
+//     29.1 / 14.6, 34.4 / 22.1; 8192 x 8192 29.1 / 16.1, 37.2 / 23.5.  But where the one-shot kernel has all its CTAs resident
+//     at once it stays: 4096 x 4096 at 48 tokens 6.1 / 7.7 (groups of 128) and 5.9 / 7.5 (one scale), 2560 x 4096 4.4 / 7.4,
+//     8192 x 2048 at 40 6.9 / 8.6; and on small ones of 5 to 10 blocks, 2048 x 5120 at 48 5.6 / 6.8.  At 64 tokens the tensor-core
+//     kernel takes what the estimate below gives it: 14336 x 4096 18.9 / 22.7 (128), 4096 x 14336 13.4 / 18.9 (one scale),
+//     8192 x 28672 40.1 / 63.8 (one scale), 52.3 / 66.2 (128).
+//   64 .. 256 tokens: about 5 us + 0.27 ns per cell and slab (a little more for K > 8192, where clusters of six
 //     and eight leave SMs idle), against the model of the tensor-core kernels: 4096 x 4096 at 100 tokens
 //     13.1 / 12.5, 4096 x 14336 at 140 40.6 / 38.1, but at 100 22.0 / 31.1 and at 200 40.6 / 56.4, 14336 x 4096 at 140
 //     39.6 / 46.1.
@@ -467,7 +477,10 @@ bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
     if (env_int("W2A8_GEMV", 1) == 2) return false;
     const long long blocks = K / kBlockK, cells = (long long)((tiles + 1) / 2) * blocks;
     if (M <= 4) return cells >= 24576 && (h16 || blocks > (M == 1 ? 64 : 16));
-    if (M <= 8) return gemv_preferred(M, K, group, tiles, count) && blocks > 16 && cells >= 8192;
+    if (M <= 8) {
+        const long long least = group <= 128 && gemv_half_sm(M, K) ? 16384 : group <= 64 ? 12288 : 8192;
+        return gemv_preferred(M, K, group, tiles, count) && blocks > 16 && cells >= least;
+    }
     if (M <= 16 && !h16 && gemv_preferred(M, K, group, tiles, count)) return cells >= (blocks > 16 ? 8192 : 12288);
     if (M <= 32) return cells >= (count > 1 ? 1536 : 4096);
     if (count > 1) return false;                  // (more than 32 tokens: a launch per matrix)
@@ -475,7 +488,8 @@ bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
         for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE",
                                  "W2A8_PF_UNPACK_WARPS"})
             if (env_set(name)) return false;
-    if (M <= 64) return cells >= 1024;
+    if (M < 64 || (M == 64 && !(prefill_supported(M, tiles * 16, K, group) && prefill_preferred(M, tiles * 16, K, group, true))))
+        return cells >= (blocks > 4 && blocks <= 10 ? 2048 : 1024) && !decode_one_wave(M, tiles * 16, K, group, h16);
     const double mine = 5.0e-6 + 0.27e-9 * (blocks > 32 ? 1.15 : 1.0) * (double)cells * st_tgroups(M) * st_slabs(M);
     return mine < 0.95 * many_token_seconds(M, tiles * 16, K, group);
 }

@@ -71,3 +71,17 @@ def test_workspace_covers_the_channel_remainder_of_bf16_activations(monkeypatch)
                     monkeypatch.delenv("W2A8_PREFILL")
                     assert size >= rest, (M, N, K, group)
     assert found > 10
+
+
+@pytest.mark.parametrize("N,K,group,kernel", [
+    (28672, 8192, 8192, "tensor_core"),
+    (28672, 8192, 128, "tensor_core"),
+    (14336, 4096, 4096, "tensor_core"),
+    (4096, 14336, 128, "tensor_core"),
+    (4096, 14336, 64, "streaming"),
+    (4096, 4096, 64, "streaming"),
+    (8192, 8192, 64, "streaming"),
+])
+def test_64_tokens(N, K, group, kernel):
+    """The fewest tokens of the tensor-core kernel, which is ahead there with large groups only."""
+    assert b.w2a8_kernel_for(64, N, K, group) == kernel
