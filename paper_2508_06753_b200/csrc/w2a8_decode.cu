@@ -332,8 +332,9 @@ w2a8_decode_kernel(const DecodeParams p) {
 
     // The cell loop is unrolled, except in the 64-register instance for groups of 64 and one slab of tokens:
     // unrolled, its scales and pointers spill (14336 x 4096 at 2 / 4 / 8 tokens 6.88 / 7.12 / 7.78 us, as a loop
-    // 6.67 / 6.75 / 6.94; 8192 x 8192 at 4 / 8 tokens 7.76 / 8.36 and 7.21 / 7.44).  The others lose 1 to 7 %.
-    constexpr bool kRolled = SPP == 1 && MT == 1 && !RELAX && !H16 && !A16 && !PARTIALS;
+    // 6.67 / 6.75 / 6.94; 8192 x 8192 at 4 / 8 tokens 7.76 / 8.36 and 7.21 / 7.44).  The others lose 1 to 7 %, its
+    // single-token form among them (14336 x 4096 6.34 / 6.58, 8192 x 8192 6.80 / 7.14).
+    constexpr bool kRolled = SPP == 1 && MT == 1 && !ONE && !RELAX && !H16 && !A16 && !PARTIALS;
 #pragma unroll(kRolled ? 1 : RING)
     for (int c = 0; c < RING; ++c) {
         if (c < full_cells) {                                 // warp-uniform
