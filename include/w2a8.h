@@ -306,9 +306,8 @@ size_t w2a8_grouped_workspace_bytes(int count, const int *N, int M, int K, int g
  *                   a8_quantize, same bits) into its shared memory.  Possible for
  *                   at most 8 tokens, K % 256 == 0 and rows that fit shared
  *                   memory; where it is not possible this behaves like _OFF.
- *   W2A8_FUSE_AUTO  fuses where that is measured to be faster: one token, rows of
- *                   1024, 2048 or 4096 values (activations in registers), and at
- *                   most one or at least three 16-channel tiles per CTA; else _OFF: the
+ *   W2A8_FUSE_AUTO  fuses where that is measured to be faster: one token and rows of
+ *                   1024, 2048 or 4096 values (activations in registers); else _OFF: the
  *                   separate quantiser launch hides behind the weight prefetch of
  *                   the launch that follows it (two tokens on: 0.5 us and more per
  *                   call).  W2A8_FUSE_MAX_ELEMS in the environment replaces the rule

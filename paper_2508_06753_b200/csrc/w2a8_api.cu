@@ -18,7 +18,7 @@ size_t decode_workspace_header_bytes(int M, int N, int K, const ShapeInfo &si);
 bool gemv_supported(int M, int K, int group);
 bool gemv_preferred(int M, int K, int group, int tiles, int count);
 bool gemv_can_fuse(int M, int K, int group);
-bool gemv_fuse_preferred(int M, int K, int group, int tiles);
+bool gemv_fuse_preferred(int M, int K, int group);
 int launch_gemv(const int8_t *a, const float *a_scale, const void *x_bf16, int8_t *a_out, float *a_scale_out,
                 int count, const uint32_t *const *packed, const float *const *w_scale, float *const *y,
                 const int *N, const int *ldy, int M, int K, int group, cudaStream_t st);
@@ -632,7 +632,7 @@ static int grouped_plan(int count, const int *N, int M, int K, int group, int fu
     }
     int plan = 0;
     if (have_x && fuse != W2A8_FUSE_OFF && gemv_can_fuse(M, K, group) &&
-        (fuse == W2A8_FUSE_ON || gemv_fuse_preferred(M, K, group, tiles)))
+        (fuse == W2A8_FUSE_ON || gemv_fuse_preferred(M, K, group)))
         plan = 3;
     else if (stat_takes(M, K, group, tiles, count, false) || gemv_preferred(M, K, group, tiles, count))
         plan = 1;

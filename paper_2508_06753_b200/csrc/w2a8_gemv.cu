@@ -508,21 +508,22 @@ bool gemv_can_fuse(int M, int K, int group) {
 // The paper exposes the abs-max scales "inside the GEMM or in a kernel of their own" as a knob
 // (Sec. II-D) and finds the fused form ahead for GEMV-sized problems only.  Here every CTA repeats the
 // abs-max, and under programmatic dependent launch a separate quantiser launch hides behind the weight
-// prefetch of the kernel that follows it.  Measured on B200 (us per call, fused / quantiser launch +
-// persistent kernel): one token with register-resident activations: 2.54 / 3.08 (2048 x 2048), 3.59 / 3.73
-// (4096 x 4096), 4.27 / 4.53 (q|k|v), 8.76 / 9.32 (gate|up); two tokens, K = 4096: 4.35 / 3.82; four: 5.6 / 3.9;
-// eight: 8.6 / 4.3; one token, K = 14336 (activations staged for the whole CTA): 9.3 / 7.7.  So one token
-// with register-resident activations is fused, which saves a launch on the host as well.  (From one to three
-// tiles per CTA, which is where q|k|v lies, the separate launch stays: the plan that the grouped entry point
-// reports there is part of its tests, and the gain is the smallest.)  W2A8_FUSE_MAX_ELEMS: fuse up to that many
+// prefetch of the kernel that follows it.  Measured on B200 (us per call, fused / quantiser launch + the kernel
+// that w2a8_gemm takes), groups of 64, one token with register-resident activations: 2.69 / 3.13 (2048 x 2048,
+// 128 tiles), 3.58 / 3.78 (4096 x 4096, 256), 3.79 / 4.20 (296), 4.25 / 4.47 (q|k|v, 384), 4.8 / 4.95 (512), 5.44 / 5.75
+// (688), 5.76 / 5.96 (768), 6.17 / 6.30 (896), 9.2 / 9.85 (gate|up, 1792), 16.1 / 16.7 (3584); one scale per channel and
+// rows of 1024 and 2048 the same way, up to 0.6 ahead.  In the pass of an 8B layer, where the calls follow one
+// another: all separate 25.6, all fused but down 25.4 (one scale per channel 24.1 / 23.5); with q|k|v left out there
+// was no gain (25.9 / 26.1, where all of them gave 25.5).  Two tokens, K = 4096: 4.35 / 3.82; four: 5.6 / 3.9; eight: 8.6 / 4.3;
+// one token, K = 14336 (activations staged for the whole CTA): 9.3 / 7.7.  So one token with register-resident
+// activations is fused, which saves a launch on the host as well.  W2A8_FUSE_MAX_ELEMS: fuse up to that many
 // values of M * K instead.
-bool gemv_fuse_preferred(int M, int K, int group, int tiles) {
+bool gemv_fuse_preferred(int M, int K, int group) {
     if (!gemv_can_fuse(M, K, group)) return false;
     const int limit = env_int("W2A8_FUSE_MAX_ELEMS", -1);
     if (limit >= 0) return (long long)M * K <= (long long)limit;
-    const int blocks = K / kBlockK, ctas = 2 * sm_count();
-    return M == 1 && (blocks == 4 || blocks == 8 || blocks == 16) && gemv_warps(M, K) == 8 &&
-           (tiles <= ctas || tiles >= 3 * ctas);
+    const int blocks = K / kBlockK;
+    return M == 1 && (blocks == 4 || blocks == 8 || blocks == 16) && gemv_warps(M, K) == 8;
 }
 
 static GemvPlan gemv_plan(int M, int K, int tiles, const ShapeInfo &si, bool fused) {

@@ -15,12 +15,15 @@ def library(monkeypatch):
 
 
 @pytest.mark.parametrize("Ns,M,K,fused", [
-    ([2048], 1, 2048, True),              # about one wave of CTAs
-    ([4736], 1, 4096, True),              # 296 tiles: the last of that range
-    ([4752], 1, 4096, False),
-    ([14192], 1, 4096, False),
-    ([14208], 1, 4096, True),             # 888 tiles: large enough again
+    ([2048], 1, 2048, True),
+    ([16], 1, 1024, True),                # one tile
+    ([4736], 1, 4096, True),              # one tile per CTA, the last such size
+    ([4752], 1, 4096, True),
+    ([4096, 1024, 1024], 1, 4096, True),
+    ([14192], 1, 4096, True),
     ([14336, 14336], 1, 4096, True),
+    ([2048], 1, 3072, False),             # no instance with these rows in registers
+    ([2048], 1, 8192, False),
     ([2048], 2, 2048, False),             # more than one token
     ([4096], 1, 14336, False),            # activations do not stay in registers
 ])
