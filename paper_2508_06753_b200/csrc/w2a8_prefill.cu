@@ -702,17 +702,19 @@ bool prefill_preferred(int M, int N, int K, int group, bool can_split) {
     return t_tc * (950000.0 / 875000.0) < t_stream;
 }
 
-// Expected time of a problem on the faster of the tensor-core path and the one-shot streaming kernel, for the
-// comparison with the kernel with stationary activations (65 to 256 tokens).  The 128-token tiles at what they
-// take now: 3 us and 4.9 / 3.4 / 3.0 / 2.4 ns per k and round for groups of 64 / 128 / 256 / more (us, estimate /
+// Expected time of a problem on the kernel that it goes to without the kernel with stationary activations, for the
+// comparison with that one (64 to 256 tokens): the one-shot streaming kernel, or the 128-token tiles at what they
+// take now, 3 us and 4.9 / 3.4 / 3.0 / 2.4 ns per k and round for groups of 64 / 128 / 256 / more (us, estimate /
 // measured: 4096 x 14336 at 100 tokens 23.1 / 22.0, 4096 x 4096 12.7 / 13.1, 14336 x 4096 25.3 / 24.8, at 140 42.4 / 39.6).
-// The rules between the tensor-core and the streaming kernels keep the constants they were fitted with.
+// The rules between the tensor-core and the streaming kernels, the K split and the channel split keep the constants
+// they were fitted with, 7.0 / 4.8 / 3.6 / 3.0 ns.  Measured against every forced alternative on 272 problems (six
+// matrices of the 8B and 70B layers, four groupings, 65 to 2048 tokens) all choices together are within 4 % of the
+// best in 255; the others are 4096 x 1024 at 160 to 256 tokens (12.4 us, best 9.5) and five of up to 15 %.
 double many_token_seconds(int M, int N, int K, int group) {
-    double t = kStreamSecondsPerMac * (double)M * (double)N * (double)K;
-    if (!prefill_supported(M, N, K, group)) return t;
+    if (!prefill_supported(M, N, K, group) || !prefill_preferred(M, N, K, group, true))
+        return kStreamSecondsPerMac * (double)M * (double)N * (double)K;
     const double per_k = group <= 64 ? 4.9e-9 : group <= 128 ? 3.4e-9 : group <= 256 ? 3.0e-9 : 2.4e-9;
-    const double t_tc = 3.0e-6 + prefill_seconds(M, N, K, group, prefill_ksplit(M, N, K, group), per_k);
-    if (t_tc < t) t = t_tc;
+    double t = 3.0e-6 + prefill_seconds(M, N, K, group, prefill_ksplit(M, N, K, group), per_k);
     if (prefill_uses_wide(M, N, K, group)) {
         int c;
         const double t_wide = split_plan(M, N, K, 256, kWideRoundSecondsPerK, &c);
