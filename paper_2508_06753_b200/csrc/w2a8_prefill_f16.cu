@@ -24,7 +24,6 @@
 
 namespace w2a8 {
 
-
 // Four warpgroups, with the register file re-balanced between them at kernel entry (setmaxnreg):
 //   warps 0-3   two MMA issuers, the TMA producer, one spare       (56 registers per thread)
 //   warps 4-7   unpack                                             (104)

@@ -485,8 +485,7 @@ bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
     if (M <= 32) return cells >= (count > 1 ? 1536 : 4096);
     if (count > 1) return false;                  // (more than 32 tokens: a launch per matrix)
     if (M >= 64)
-        for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE",
-                                 "W2A8_PF_UNPACK_WARPS"})
+        for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE"})
             if (env_set(name)) return false;
     if (M < 64 || (M == 64 && !(prefill_supported(M, tiles * 16, K, group) && prefill_preferred(M, tiles * 16, K, group, true))))
         return cells >= (blocks > 4 && blocks <= 10 ? 2048 : 1024) && !decode_one_wave(M, tiles * 16, K, group, h16);

@@ -1,7 +1,7 @@
 """Seeded random shapes through the public entry points against the CPU reference: the grouped
 operator (persistent kernel in both of its forms, fused and unfused quantiser, one-shot fallback)
 and w2a8_gemm at prefill sizes (default dispatch and forced variants: K split, 256-token tiles,
-both warp layouts).  Outputs within 1e-4 * max|row|; int8 activations bit-exact."""
+both operand types).  Outputs within 1e-4 * max|row|; int8 activations bit-exact."""
 import random
 
 import numpy as np
@@ -11,7 +11,7 @@ from paper_2508_06753_b200 import synth
 
 pytestmark = pytest.mark.gpu
 TOL = 1e-4
-SWITCHES = ("W2A8_PREFILL", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE", "W2A8_PF_UNPACK_WARPS", "W2A8_GEMV", "W2A8_GEMV_WARPS",
+SWITCHES = ("W2A8_PREFILL", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE", "W2A8_GEMV", "W2A8_GEMV_WARPS",
             "W2A8_FUSE_MAX_ELEMS", "W2A8_TC_KIND")
 
 
@@ -90,7 +90,7 @@ def test_gemm_random_prefill_shapes(gpu, oracle, monkeypatch, seed):
         env = rng.choice([{}, {}, {"W2A8_PREFILL": "2"},
                           {"W2A8_PREFILL": "2", "W2A8_PF_KSPLIT": rng.choice(["2", "4", "8"])},
                           {"W2A8_PREFILL": "2", "W2A8_PF_WIDE": "2"},
-                          {"W2A8_PREFILL": "2", "W2A8_PF_UNPACK_WARPS": rng.choice(["2", "4"])}])
+                          {"W2A8_PREFILL": "2", "W2A8_TC_KIND": rng.choice(["8", "16"])}])
         for k, v in env.items():
             monkeypatch.setenv(k, v)
         if env:
