@@ -34,13 +34,10 @@ from paper_2508_06753_b200 import synth
 CFG_INDEX = 1
 METRIC = "W2A8 GEMM HBM GB/s at M=1-16 (Llama-3-8B decoder-layer linears, M in {1,4,16}, group 64)"
 NOMINAL_HBM_GBS = 8000.0
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch of the decode kernel on the
-# 4096x14336, M=1, group-64 GEMM (ncu capture of one launch); the algorithmic bytes of that
-# launch are 18,411,524.
-NCU_TRAFFIC_BYTES_GATE_M1 = 18_378_752
-# the same for one grouped launch of the persistent kernel on gate|up, 4096x(14336+14336), M=1:
-# 36,818,948 algorithmic bytes, 36,734,720 read from DRAM (the activations come from L2), 256 written
-NCU_TRAFFIC_BYTES_GATEUP_M1 = 36_734_976
+# dram__bytes_read.sum + dram__bytes_write.sum of one launch over gate|up, 4096x(14336+14336), group 64, by tokens
+# (ncu, one launch each): the persistent kernel with the quantiser inside, the kernel with stationary activations
+# (algorithmic bytes 36,827,140 and 38,600,768; the activations and the results stay in L2)
+NCU_TRAFFIC_BYTES_GATEUP = {1: 36_747_264, 16: 36_787_456}
 
 
 # --------------------------------------------------------------------- accounting
@@ -389,9 +386,10 @@ def per_m_times(rep, mode, use_graph, blocks=10):
 
 
 def kernel_probe(device, peaks, l2_bytes, M, K, N, g, use_graph=True, seed=9000, count=1):
-    """One GEMM launch on its own -- w2a8_gemm, or w2a8_gemm_grouped over `count` matrices of the
-    same shape -- back to back in a graph over its own set of weight copies, at least twice L2 of
-    distinct weight bytes, CUDA events on the launching stream."""
+    """One GEMM launch on its own -- w2a8_gemm, or a grouped call over `count` matrices of the same
+    shape (w2a8_linear_grouped where that is one launch, else w2a8_gemm_grouped) -- back to back in a graph
+    over its own set of weight copies, at least twice L2 of distinct weight bytes, CUDA events on the
+    launching stream."""
     import torch
     from paper_2508_06753_b200 import binding as b
     codes, s_w = synth.make_linear(seed + K + N, K, N, g)
@@ -405,10 +403,13 @@ def kernel_probe(device, peaks, l2_bytes, M, K, N, g, use_graph=True, seed=9000,
     ys = [torch.empty((M, N), dtype=torch.float32, device=device) for _ in range(count)]
     ws = b.new_workspace(b.w2a8_workspace_bytes(M, N, K, g), device=device)
     groups = [b.Group([m[0] for m in grp], [m[1] for m in grp], ys) for grp in mats]
+    fused = count > 1 and b.w2a8_grouped_plan([N] * count, M, K, g)["fused"]
 
     def body():
         for grp, gargs in zip(mats, groups):
-            if count == 1:
+            if fused:
+                b.w2a8_linear_grouped(x, gargs, g, ws, a=a, a_scale=s_a)
+            elif count == 1:
                 b.w2a8_gemm(a, s_a, grp[0][0], grp[0][1], g, ws, ys[0])
             else:
                 b.w2a8_gemm_grouped(a, s_a, gargs, g, ws)
@@ -417,10 +418,13 @@ def kernel_probe(device, peaks, l2_bytes, M, K, N, g, use_graph=True, seed=9000,
     t = timed_blocks(torch, run, stream, blocks=12, reps=max(1, 48 // ncopy))
     torch.cuda.current_stream().wait_stream(stream)
     nbytes = count * gemm_bytes(M, N, K, g) - (count - 1) * (M * K + 4 * M)     # the activations are read once
+    if fused:
+        nbytes += 2 * M * K                                                     # bf16 read, int8 and scales written
     us = t["mean"] / ncopy * 1e3
     plan = b.w2a8_grouped_plan([N] * count, M, K, g, b.FUSE_OFF)
     return dict(shape=f"{K}x{N}" + (f" x{count}" if count > 1 else ""), M=M, group=g, us_per_launch=us,
-                kernel="persistent" if plan["one_launch"] else "one-shot", us_min=t["min"] / ncopy * 1e3,
+                kernel="persistent, quantiser inside" if fused else "one launch for the group" if plan["one_launch"] and count > 1
+                else "persistent" if plan["one_launch"] else "one-shot", us_min=t["min"] / ncopy * 1e3,
                 us_median=t["median"] / ncopy * 1e3, bytes_per_launch=nbytes, gbs=nbytes / us / 1e3,
                 frac_of_measured_hbm=nbytes / us / 1e3 / peaks["hbm_gbs"],
                 distinct_weight_bytes=per * ncopy, weight_copies=ncopy, launch=kind,
@@ -869,13 +873,11 @@ def run_ours(args):
         note("per-M rows done")
         name, K, N = max(cfg["shapes"], key=lambda s: s[1] * s[2])
         K, N = 4096, 14336
-        # the launches with the largest share of the step: gate|up as one grouped launch (M = 1, 4),
-        # gate alone (M = 16, and M = 1 for the one-shot kernel on its own), down
-        probes = [kernel_probe(device, peaks, l2, 1, K, N, 64, use_graph, count=2),
-                  kernel_probe(device, peaks, l2, 4, K, N, 64, use_graph, count=2),
-                  kernel_probe(device, peaks, l2, 16, K, N, 64, use_graph),
-                  kernel_probe(device, peaks, l2, 1, K, N, 64, use_graph),
-                  kernel_probe(device, peaks, l2, 1, 14336, 4096, 64, use_graph)]
+        # the launches with the largest share of the step, gate|up as one launch, and for the one-shot kernel
+        # gate alone and down
+        probes = [kernel_probe(device, peaks, l2, M, K, N, 64, use_graph, count=2) for M in cfg["Ms"]]
+        probes += [kernel_probe(device, peaks, l2, 1, K, N, 64, use_graph),
+                   kernel_probe(device, peaks, l2, 1, 14336, 4096, 64, use_graph)]
         extra["read_ceiling"] = read_ceiling_probe(device, l2)
         note("kernel probes done")
         extra["fused_vs_separate"] = fused_vs_separate(rep, use_graph)
@@ -915,14 +917,12 @@ def run_ours(args):
         cpu = cpu_baseline(cfg, budget_s=20.0)
         note("cpu baseline done")
 
-    dom = probes[0]
+    dom = max(probes[:len(cfg["Ms"])], key=lambda pr: pr["us_per_launch"])
     ceiling = extra["read_ceiling"]["gbs"]
     roofline = {"bound": "hbm", "achieved": dom["gbs"], "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": dom["gbs"] / peaks["hbm_gbs"], "traffic": NCU_TRAFFIC_BYTES_GATEUP_M1,
+                "frac": dom["gbs"] / peaks["hbm_gbs"], "traffic": NCU_TRAFFIC_BYTES_GATEUP.get(dom["M"]),
                 "peak_source": peaks["source"],
-                "kernel": "w2a8_gemv_kernel<MT=1,SPP=1,ONE,BCACHE,W=8> (persistent, two 8-warp CTAs per SM) on gate|up 4096x(14336+14336) as one "
-                          "grouped launch, M=1: the launch with the largest share of the step (the other large "
-                          "launches, and the one-shot kernel on gate alone, are in roofline_by_m)",
+                "kernel": f"gate|up {dom['shape']}, M={dom['M']}, {dom['kernel']}: the largest share of the step",
                 "bytes_per_launch": dom["bytes_per_launch"], "us_per_launch": dom["us_per_launch"],
                 "us_min": dom["us_min"], "us_median": dom["us_median"],
                 "distinct_weight_bytes": dom["distinct_weight_bytes"], "l2_bytes": l2,
@@ -951,7 +951,34 @@ def run_ours(args):
         "kernel_probes": probes, "other_configs": other, "prefill": prefill,
     }
     out.update(extra)
-    print(json.dumps(out))
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(out, f, indent=1)
+    print(json.dumps(compact(out)))
+
+
+def compact(full):
+    """The record as one short line: the headline with its clocks, end-to-end time, roofline and baseline, and of the
+    other rows the times alone.  `--details FILE` keeps all of it."""
+    line = {k: full[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+                                 "scaling", "vs_baseline", "dtype", "data", "config", "frac_of_measured_hbm", "clocks",
+                                 "e2e", "gpu_launches", "roofline", "cpu_baseline")}
+    line["us_per_launch"] = {f"{p['shape']} M={p['M']}": p["us_per_launch"] for p in full["kernel_probes"]}
+    line["us_per_layer"] = {name: {M: r["us_per_layer"] for M, r in rows.items()} for name, rows in
+                            [("grouped", full["per_m"]), ("separate_calls", full["per_m_separate_calls"])] +
+                            [(key, full[key]["per_m"]) for key in ("recipe_g128_binary16_scales_bf16_out",
+                                                                   "w2a16_no_quantiser") if full.get(key)] +
+                            [(row["name"], row["per_m"]) for row in full["other_configs"]]}
+    if full["prefill"]:
+        line["prefill_tops"] = {f"{r['shape']} M={r['M']}": r["tops"] for r in full["prefill"]["rows"]}
+
+    def short(v):
+        if isinstance(v, dict):
+            return {k: short(w) for k, w in v.items()}
+        if isinstance(v, list):
+            return [short(w) for w in v]
+        return float(f"{v:.6g}") if isinstance(v, float) else v
+    return short(line)
 
 
 def prefill_probe(device, peaks, Ms=(512, 2048, 8192), reps=5):
@@ -1183,14 +1210,17 @@ def run_kernel_profile(args):
 
         def gemm(pk, sw):
             b.w2a8_gemm_h16(a, s_a, pk, sw, g, ws, y)
-    elif args.profile_entry == "grouped2":
-        # two matrices of the shape as one grouped launch (gate|up): pairs of neighbouring copies
+    elif args.profile_entry in ("grouped2", "linear2"):
+        # two matrices of the shape as one grouped call (gate|up): pairs of neighbouring copies
         y2 = torch.empty((M, N), dtype=torch.float32, device=dev)
         pairs = {id(mats[i][0]): b.Group([mats[i][0], mats[(i + 1) % copies][0]],
                                          [mats[i][1], mats[(i + 1) % copies][1]], [y, y2]) for i in range(copies)}
 
         def gemm(pk, sw):
-            b.w2a8_gemm_grouped(a, s_a, pairs[id(pk)], g, ws)
+            if args.profile_entry == "linear2":
+                b.w2a8_linear_grouped(x, pairs[id(pk)], g, ws, a=a, a_scale=s_a)
+            else:
+                b.w2a8_gemm_grouped(a, s_a, pairs[id(pk)], g, ws)
     else:
         def gemm(pk, sw):
             b.w2a8_gemm(a, s_a, pk, sw, g, ws, y)
@@ -1244,12 +1274,15 @@ def main():
                          "short command for profilers")
     ap.add_argument("--sweep-config", type=int, default=1, choices=[1, 2, 3], help="configuration --sweep-plan runs")
     ap.add_argument("--sweep-ms", default="1,4,8,16", help="token counts --sweep-plan runs")
+    ap.add_argument("--details", default=None, metavar="FILE", help="write the whole record there (the printed line "
+                                                                    "holds the headline and the times)")
     ap.add_argument("--profile-shape", default=None, help="KxN: run only a few launches of this GEMM")
     ap.add_argument("--profile-m", type=int, default=1)
     ap.add_argument("--profile-group", type=int, default=64)
     ap.add_argument("--profile-reps", type=int, default=10)
-    ap.add_argument("--profile-entry", default="a8", choices=["a8", "h16", "a16", "grouped2"],
-                    help="entry point the profile run launches: w2a8_gemm, w2a8_gemm_h16 or w2a16_gemm")
+    ap.add_argument("--profile-entry", default="a8", choices=["a8", "h16", "a16", "grouped2", "linear2"],
+                    help="entry point the profile run launches: w2a8_gemm, w2a8_gemm_h16, w2a16_gemm, or w2a8_gemm_grouped / "
+                         "w2a8_linear_grouped over two matrices")
     args = ap.parse_args()
     if args.profile_shape:
         run_kernel_profile(args)

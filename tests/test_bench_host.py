@@ -83,3 +83,28 @@ def test_reference_arm_prints_contract_line():
     assert line["e2e"] == {"value": line["value"], "unit": "GB/s", "h2d_bytes_per_step": 0,
                            "d2h_bytes_per_step": 0}
     assert line["metric"] == bench.METRIC
+
+
+def test_printed_line_is_short():
+    """The whole record is some 24 KB; the printed line keeps the keys of the headline and stays below 6 KB."""
+    Ms = ["1", "4", "16"]
+    row = {M: {"us_per_layer": 25.123456789, "us_min": 25.0, "gbs": 2700.123456789, "bytes_per_layer": 1 << 26} for M in Ms}
+    probe = {"shape": "4096x14336 x2", "M": 1, "us_per_launch": 9.123456789, "gbs": 4000.0, "kernel": "persistent"}
+    full = {k: 1.0 / 3.0 for k in ("value", "ms_per_step", "frac_of_measured_hbm", "frac_of_nominal_8TBs")}
+    full.update(metric=bench.METRIC, unit="GB/s", n_gpus=1, steps=20, warmup=5, higher_is_better=True, scaling="weak",
+                vs_baseline=None, dtype="int8xint2->int32, fp32 scales", data="synthetic",
+                config={"workload": bench.WORKLOAD, "text": "x" * 600}, clocks={"sm_mhz": 1965, "reasons": []},
+                e2e={"value": 1000.0, "unit": "GB/s", "api": "x" * 300}, gpu_launches=420,
+                roofline={"frac": 0.61234567891, "kernel": "x" * 300}, cpu_baseline={"value": 1.0, "sample": "x" * 300},
+                kernel_probes=[dict(probe, M=m) for m in range(5)], roofline_by_m=[probe] * 5, per_m=row,
+                per_m_separate_calls=row, recipe_g128_binary16_scales_bf16_out={"what": "x", "per_m": row},
+                w2a16_no_quantiser={"what": "x", "per_m": row},
+                other_configs=[{"name": f"configuration {i}", "per_m": row} for i in range(3)],
+                prefill={"rows": [{"shape": "4096x14336", "M": m, "tops": 912.3456789} for m in range(6)]})
+    line = json.dumps(bench.compact(full))
+    assert len(line) < 6000 and "\n" not in line
+    back = json.loads(line)
+    assert back["value"] == 0.333333 and back["roofline"]["frac"] == 0.612346
+    assert back["us_per_layer"]["grouped"] == {"1": 25.1235, "4": 25.1235, "16": 25.1235}
+    for key in ("metric", "e2e", "clocks", "gpu_launches", "config", "vs_baseline", "n_gpus", "steps", "warmup"):
+        assert key in back
