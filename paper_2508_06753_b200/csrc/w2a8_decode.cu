@@ -586,14 +586,17 @@ static DecodePlan decode_plan(int M, int N, int K, const ShapeInfo &si, bool h16
     return cached;
 }
 
-// Whether all CTAs of the launch are resident at once (CTAs per SM by the registers of the instances: 8 for one
-// slab, 4 for two, 4 or, with groups of 64, 3 for three, 3 for four).
-bool decode_one_wave(int M, int N, int K, int group, bool h16) {
+// Whether the launch is one that the kernel with stationary activations does not catch up with at 33 to 64 tokens: all
+// its CTAs resident at once (CTAs per SM by the registers of the instances: 8 for one slab, 4 for two, 4 or, with groups
+// of 64, 3 for three, 3 for four), or a smaller matrix of 5 to 10 blocks with all of K in a CTA.
+bool one_shot_keeps(int M, int N, int K, int group, bool h16) {
     ShapeInfo si;
     if (!shape_ok(M, N, K, group, &si)) return false;
     const DecodePlan pl = decode_plan(M, N, K, si, h16);
     const int per_sm = pl.mt == 1 ? 8 : pl.mt == 2 || (pl.mt == 3 && group > 64) ? 4 : 3;
-    return (long long)pl.groups * pl.chunks * pl.slabs <= (long long)sm_count() * per_sm;
+    const long long resident = (long long)sm_count() * per_sm;
+    if (pl.chunks == 1 && si.blocks > 4 && si.blocks <= 10 && (long long)(N / 16) * si.blocks < 4096) return true;
+    return (long long)pl.groups * pl.chunks * pl.slabs <= resident;
 }
 
 constexpr size_t kStatusBytes = 256;   // workspace header: status word

@@ -27,7 +27,7 @@ namespace w2a8 {
 
 bool gemv_preferred(int M, int K, int group, int tiles, int count);
 bool gemv_half_sm(int M, int K);
-bool decode_one_wave(int M, int N, int K, int group, bool h16);
+bool one_shot_keeps(int M, int N, int K, int group, bool h16);
 bool prefill_supported(int M, int N, int K, int group);
 bool prefill_preferred(int M, int N, int K, int group, bool can_split);
 double many_token_seconds(int M, int N, int K, int group);
@@ -456,7 +456,8 @@ static bool stat_supported(int M, int K, int group) {
 //   33 .. 64 tokens: 4096 x 4096 8.8 / 7.2, 11.8 / 9.9; 4096 x 14336 20.6 / 13.5, 27.9 / 20.3; 14336 x 4096
 //     29.1 / 14.6, 34.4 / 22.1; 8192 x 8192 29.1 / 16.1, 37.2 / 23.5.  But where the one-shot kernel has all its CTAs resident
 //     at once it stays: 4096 x 4096 at 48 tokens 6.1 / 7.7 (groups of 128) and 5.9 / 7.5 (one scale), 2560 x 4096 4.4 / 7.4,
-//     8192 x 2048 at 40 6.9 / 8.6; and on small ones of 5 to 10 blocks, 2048 x 5120 at 48 5.6 / 6.8.  At 64 tokens the tensor-core
+//     8192 x 2048 at 40 6.9 / 8.6; and on short rows, 2048 x 5120 at 48 5.6 / 6.8 (not 2560 x 3840, whose K it splits over
+//     two waves of CTAs: 9.9 / 6.7).  At 64 tokens the tensor-core
 //     kernel takes what the estimate below gives it: 14336 x 4096 18.9 / 22.7 (128), 4096 x 14336 13.4 / 18.9 (one scale),
 //     8192 x 28672 40.1 / 63.8 (one scale), 52.3 / 66.2 (128).
 //   64 .. 256 tokens: about 5 us + 0.27 ns per cell and slab (a little more for K > 8192, where clusters of six
@@ -488,7 +489,7 @@ bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
         for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE"})
             if (env_set(name)) return false;
     if (M < 64 || (M == 64 && !(prefill_supported(M, tiles * 16, K, group) && prefill_preferred(M, tiles * 16, K, group, true))))
-        return cells >= (blocks > 4 && blocks <= 10 ? 2048 : 1024) && !decode_one_wave(M, tiles * 16, K, group, h16);
+        return cells >= 1024 && !one_shot_keeps(M, tiles * 16, K, group, h16);
     const double mine = 5.0e-6 + 0.27e-9 * (blocks > 32 ? 1.15 : 1.0) * (double)cells * st_tgroups(M) * st_slabs(M);
     return mine < 0.95 * many_token_seconds(M, tiles * 16, K, group);
 }
