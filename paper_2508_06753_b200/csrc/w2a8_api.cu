@@ -527,7 +527,12 @@ int gemm_dispatch(const int8_t *a, const float *a_scale, const uint32_t *packed,
         return launch_decode(a, a_scale, packed, w_scale, y, nullptr, M, N, K, group, si, workspace,
                              (cudaStream_t)stream, h16, y16, false, N);
     }
-    const bool takes = a16 ? takes_tensor_core_kernel_ex(M, N, K, group, false) : takes_tensor_core_kernel(M, N, K, group);
+    // The tensor-core export of partial sums stores four bytes per row and group: groups of up to 256 stream, where the
+    // stores are not what the time goes to (us, streaming / tensor cores: 4096 x 4096 at 100 tokens 251 / 837, 114 / 425 and
+    // 50 / 117 for groups of 64, 128 and 256, 24 / 12 for one; 4096 x 14336 at 64 tokens 207 / 488, 100 / 89 for 128, 256).
+    const bool exports = !partials || group > 256 || env_int("W2A8_PREFILL", 1) == 2;
+    const bool takes = a16 ? takes_tensor_core_kernel_ex(M, N, K, group, false)
+                           : exports && takes_tensor_core_kernel(M, N, K, group);
     const bool tc16 = !h16 && takes && prefill_f16_supported(M, N, K, group) &&
                       (a16 || tensor_core_kind_is_16(M, N, K, group));
     if (tc16 || (!a16 && takes)) {
