@@ -714,7 +714,7 @@ bool prefill_preferred(int M, int N, int K, int group, bool can_split) {
 // The rules between the tensor-core and the streaming kernels, the K split and the channel split keep the constants
 // they were fitted with, 7.0 / 4.8 / 3.6 / 3.0 ns.  Measured against every forced alternative on 272 problems (six
 // matrices of the 8B and 70B layers, four groupings, 65 to 2048 tokens) all choices together are within 4 % of the
-// best in 255; the others are 4096 x 1024 at 160 to 256 tokens (12.4 us, best 9.5) and five of up to 15 %.
+// best in 255; the others are eleven of 4096 x 1024 (at 200 tokens 12.4 us, best 8.5) and six of up to 15 %.
 double many_token_seconds(int M, int N, int K, int group) {
     if (!prefill_supported(M, N, K, group) || !prefill_preferred(M, N, K, group, true))
         return kStreamSecondsPerMac * (double)M * (double)N * (double)K;
