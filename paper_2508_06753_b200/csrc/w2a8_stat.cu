@@ -30,6 +30,7 @@ bool gemv_half_sm(int M, int K);
 bool one_shot_keeps(int M, int N, int K, int group, bool h16);
 bool prefill_supported(int M, int N, int K, int group);
 bool prefill_preferred(int M, int N, int K, int group, bool can_split);
+size_t prefill_workspace_bytes(int M, int N, int K, int group);
 double many_token_seconds(int M, int N, int K, int group);
 
 constexpr int kStMaxMats = 4;
@@ -459,7 +460,8 @@ static bool stat_supported(int M, int K, int group) {
 //     8192 x 2048 at 40 6.9 / 8.6; and on short rows, 2048 x 5120 at 48 5.6 / 6.8 (not 2560 x 3840, whose K it splits over
 //     two waves of CTAs: 9.9 / 6.7).  At 64 tokens the tensor-core
 //     kernel takes what the estimate below gives it: 14336 x 4096 18.9 / 22.7 (128), 4096 x 14336 13.4 / 18.9 (one scale),
-//     8192 x 28672 40.1 / 63.8 (one scale), 52.3 / 66.2 (128).
+//     8192 x 28672 40.1 / 63.8 (one scale), 52.3 / 66.2 (128); but not on a K split that needs more than the fixed scratch of
+//     w2a8_gemm_static, 14336 x 5120 (128) 32.0 / 31.5.
 //   64 .. 256 tokens: about 5 us + 0.27 ns per cell and slab (a little more for K > 8192, where clusters of six
 //     and eight leave SMs idle), against the model of the tensor-core kernels: 4096 x 4096 at 100 tokens
 //     13.1 / 12.5, 4096 x 14336 at 140 40.6 / 38.1, but at 100 22.0 / 31.1 and at 200 40.6 / 56.4, 14336 x 4096 at 140
@@ -488,7 +490,10 @@ bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
     if (M >= 64)
         for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE"})
             if (env_set(name)) return false;
-    if (M < 64 || (M == 64 && !(prefill_supported(M, tiles * 16, K, group) && prefill_preferred(M, tiles * 16, K, group, true))))
+    const bool tensor_cores = M >= 64 && prefill_supported(M, tiles * 16, K, group) &&
+                              prefill_preferred(M, tiles * 16, K, group, true) &&
+                              (M > 64 || prefill_workspace_bytes(M, tiles * 16, K, group) <= W2A8_STATIC_SCRATCH_BYTES);
+    if (M < 64 || (M == 64 && !tensor_cores))
         return cells >= 1024 && !one_shot_keeps(M, tiles * 16, K, group, h16);
     const double mine = 5.0e-6 + 0.27e-9 * (blocks > 32 ? 1.15 : 1.0) * (double)cells * st_tgroups(M) * st_slabs(M);
     return mine < 0.95 * many_token_seconds(M, tiles * 16, K, group);

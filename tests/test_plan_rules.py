@@ -84,7 +84,11 @@ def test_workspace_covers_the_channel_remainder_of_bf16_activations(monkeypatch)
     (4096, 14336, 64, "streaming"),
     (4096, 4096, 64, "streaming"),
     (8192, 8192, 64, "streaming"),
+    (5120, 14336, 128, "streaming"),
 ])
 def test_64_tokens(N, K, group, kernel):
-    """The fewest tokens of the tensor-core kernel, which is ahead there with large groups only."""
+    """The fewest tokens of the tensor-core kernel, which is ahead there with large groups only, and not by a K
+    split whose scratch w2a8_gemm_static does not have."""
     assert b.w2a8_kernel_for(64, N, K, group) == kernel
+    if (N, K) == (5120, 14336):
+        assert b.w2a8_workspace_bytes(64, N, K, group) <= 8 << 20
