@@ -136,6 +136,9 @@ int w2a8_workspace_status(const void *workspace, void *stream);
  * than one wave; and the one with stationary activations (up to 256 tokens,
  * K % 256 == 0), which unpacks every weight once per 64 tokens, where its estimate
  * is ahead: larger problems of few tokens, smaller ones of many.  w2a8_kernel_for reports tensor-core or streaming.
+ * From 9 to 64 tokens (K % 256 == 0) a larger problem goes to none of these but to a streaming kernel that feeds the
+ * weights to the tensor cores through tensor memory, where its estimate is ahead; the report functions say what the
+ * shape would get without it.
  * A problem given to the tensor-core kernel may leave its last (at most
  * eight) 128-channel tiles to the streaming kernel, as a second launch on the
  * same stream (w2a8_tensor_core_channels); the result does not depend on it
@@ -283,8 +286,9 @@ int w2a8_gemm_partials(const int8_t *a, const uint32_t *packed, int32_t *partial
  * Each y[i] holds what w2a8_gemm computes for matrix i: bit for bit when both
  * calls take the same kernel, unless that is the kernel with stationary
  * activations (larger problems of up to 32 tokens; the largest from one token
- * on).  It deals the channels of all matrices of a launch to its CTAs as one
- * sequence, so with it the order of the fp32 additions depends on the group.
+ * on) or the streaming one on the tensor cores (larger problems of 9 to 64
+ * tokens).  They deal the channels of all matrices of a launch to their CTAs as one
+ * sequence, so with them the order of the fp32 additions depends on the group.
  * With any kernel the result is within the tolerance of w2a8_gemm's contract
  * and repeated calls on the same group give equal bits.
  */
@@ -318,7 +322,8 @@ size_t w2a8_grouped_workspace_bytes(int count, const int *N, int M, int K, int g
  *              not be NULL otherwise (W2A8_ERR_NULL)
  *   the rest as for w2a8_gemm_grouped.
  * w2a8_grouped_plan reports what a call will do: bit 0 = one launch of the
- * persistent kernel for the whole group, bit 1 = that launch also quantises.
+ * persistent kernel for the whole group, bit 1 = that launch also quantises,
+ * bit 2 = one launch of the streaming kernel on the tensor cores in any case.
  * a and a_scale are bitwise those of a8_quantize; every y is bitwise that of
  * w2a8_gemm_grouped when that call takes the persistent kernel too, and differs
  * from it by fp32 summation order only otherwise.

@@ -28,6 +28,11 @@ int launch_stat(const int8_t *a, const float *a_scale, int count, const uint32_t
                 const void *const *w_scale, void *const *y, const int *N, const int *ldy, int M, int K, int group,
                 cudaStream_t st, bool h16, bool y16);
 
+bool tstream_takes(int M, int K, int group, int tiles16, int count);
+int launch_tstream(const int8_t *a, const float *a_scale, int count, const uint32_t *const *packed,
+                   const void *const *w_scale, void *const *y, const int *N, const int *ldy, int M, int K, int group,
+                   void *workspace, cudaStream_t st, bool h16, bool y16);
+
 bool prefill_supported(int M, int N, int K, int group);
 bool prefill_preferred(int M, int N, int K, int group, bool can_split);
 size_t prefill_workspace_bytes(int M, int N, int K, int group);
@@ -423,6 +428,7 @@ static bool takes_tensor_core_kernel_ex(int M, int N, int K, int group, bool can
     return prefill_preferred(M, N, K, group, can_split);
 }
 // int8 activations: the int8 kernel can split K for problems with few output tiles, the 16-bit one cannot
+// (9 to 64 tokens: among the kernels other than the streaming one on the tensor cores, which dispatch asks first)
 static bool takes_tensor_core_kernel(int M, int N, int K, int group) {
     return takes_tensor_core_kernel_ex(M, N, K, group, !tensor_core_kind_is_16(M, N, K, group)) &&
            !stat_takes(M, K, group, N / 16, 1, false);
@@ -521,6 +527,10 @@ size_t gemm_header_bytes(int M, int N, int K, int group) {
 int gemm_dispatch(const int8_t *a, const float *a_scale, const uint32_t *packed, const void *w_scale,
                   void *y, int32_t *partials, int M, int N, int K, int group, const ShapeInfo &si,
                   void *workspace, void *stream, bool h16, bool y16, bool a16) {
+    if (!a16 && !partials && tstream_takes(M, K, group, N / 16, 1)) {
+        const int st = launch_tstream(a, a_scale, 1, &packed, &w_scale, &y, &N, &N, M, K, group, workspace, (cudaStream_t)stream, h16, y16);
+        if (st != kStatNoPlan) return st;
+    }
     if (!a16 && !partials && stat_takes(M, K, group, N / 16, 1, h16)) {
         const int st = launch_stat(a, a_scale, 1, &packed, &w_scale, &y, &N, &N, M, K, group, (cudaStream_t)stream, h16, y16);
         if (st != kStatNoPlan) return st;
@@ -626,8 +636,8 @@ static inline size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 // ---- matrices that share their activations --------------------------------------------------
 constexpr int kMaxGroup = 4;
 
-// bit 0: the group runs as one launch of the persistent kernel; bit 1: that launch quantises the
-// activations itself.  fuse: W2A8_FUSE_AUTO / _OFF / _ON.  Negative: error.
+// bit 0: the group runs as one launch of the persistent kernel or of the one with stationary activations; bit 1: that
+// launch quantises the activations itself; bit 2: one launch of the streaming kernel on the tensor cores instead.  fuse: W2A8_FUSE_AUTO / _OFF / _ON.  Negative: error.
 static int grouped_plan(int count, const int *N, int M, int K, int group, int fuse, bool have_x) {
     if (count < 1 || count > kMaxGroup || !N) return W2A8_ERR_SHAPE;
     int tiles = 0;
@@ -641,6 +651,7 @@ static int grouped_plan(int count, const int *N, int M, int K, int group, int fu
         plan = 3;
     else if (stat_takes(M, K, group, tiles, count, false) || gemv_preferred(M, K, group, tiles, count))
         plan = 1;
+    if (plan != 3 && tstream_takes(M, K, group, tiles, count)) plan |= 4;
     return plan;
 }
 
@@ -691,8 +702,13 @@ static int grouped_common(const void *x_bf16, const int8_t *a_in, const float *a
     }
     int tiles = 0;
     for (int i = 0; i < count; ++i) tiles += N[i] / 16;
-    bool gemv = plan == 1;
-    if (plan == 1 && stat_takes(M, K, group, tiles, count, false)) {
+    bool gemv = plan & 1;
+    if (plan & 4) {
+        const int st = launch_tstream(a_in, a_scale_in, count, packed, reinterpret_cast<const void *const *>(w_scale),
+                                      reinterpret_cast<void *const *>(y), N, N, M, K, group, workspace, (cudaStream_t)stream, false, false);
+        if (st != kStatNoPlan) return st;
+    }
+    if ((plan & 1) && stat_takes(M, K, group, tiles, count, false)) {
         const int st = launch_stat(a_in, a_scale_in, count, packed, reinterpret_cast<const void *const *>(w_scale),
                                    reinterpret_cast<void *const *>(y), N, N, M, K, group, (cudaStream_t)stream, false, false);
         if (st != kStatNoPlan) return st;

@@ -203,7 +203,7 @@ bool env_set(const char *name);
 uint64_t env_fingerprint();      // changes whenever the environment does
 struct EnvScope { EnvScope(); ~EnvScope(); };      // one look at the environment for the calls inside
 
-constexpr int kStatNoPlan = 1;   // launch_stat: the caller takes another kernel (no status code is positive)
+constexpr int kStatNoPlan = 1;   // launch_stat, launch_tstream: the caller takes another kernel (no status code is positive)
 
 bool pdl_enabled();
 int check_device();  // W2A8_OK or W2A8_ERR_ARCH / W2A8_ERR_CUDA

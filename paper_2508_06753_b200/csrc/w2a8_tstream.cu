@@ -1,0 +1,764 @@
+// Streaming kernel on the 5th-generation tensor cores (up to 64 tokens): the packed weights stream through
+// shared memory once, are unpacked into tensor memory as the A operand of tcgen05.mma kind::i8 (UMMA M = 128
+// channels), and meet the tokens as a narrow B operand (UMMA N = 16, 32 or 64).
+//
+//  * Work.  A cluster of C CTAs (1, 2, 4 or 8) takes tiles of 128 channels, of up to four matrices that share their
+//    activations; rank r of it the r-th share of K (K-splitting of Sec. II-D), in blocks of 256 k = 8 KB of packed weights.
+//    The ranks exchange their sums of a tile through distributed shared memory, each adding up a part of the token
+//    columns in rank order: the order is fixed by the launch, so results repeat bit for bit.
+//  * Roles.  One thread brings weights (64-byte rows, 64-byte swizzle) and activations (128-byte swizzle) by TMA;
+//    four or eight warps unpack a channel per lane, 64 registers of int8 lanes for 256 k, into tensor memory
+//    (tcgen05.st), which the shared memory's 128 B/clk would not bear beside the copies; one warp issues the MMAs; four or
+//    eight warps drain the accumulators (lane = channel, column = token): a conversion and half a packed FMA per value.
+//  * Up to 32 tokens a CTA has 12 warps, 112 KB and 256 columns of tensor memory, so that two are resident per SM and one
+//    computes while the other waits or, under programmatic dependent launch, while the previous kernel ends; with 64
+//    tokens one CTA of 20 warps has them all.  Registers are dealt by setmaxnreg so that nothing spills: a few spilled
+//    words per block (local memory beside the copies) made 8192 x (28672 + 28672) at 32 tokens 94 us instead of 54.
+//  * Bound (8192 x (28672 + 28672), groups of 128, 32 tokens, 41 us, 3.2 TB/s): issue slots, 68 % busy: about 450 warp
+//    instructions of unpack per block, 800 of drain, the rest waits.  On the kernel with stationary activations
+//    (mma.sync) the same launch takes 58 us.  Not kept: conversion through the bits of 1.5 * 2^23, by integer adds (50 us);
+//    eight drain warps at 32 tokens (45); blocks dealt evenly over CTAs with cut tiles summed through global
+//    memory (3 us more per small launch).
+//  * A wait is one barrier per warp: lanes of a warp that polled different barriers saw phases that had not completed.
+//  * Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include "w2a8_tc.cuh"
+
+namespace w2a8 {
+
+constexpr int kTsMaxMats = 4;
+constexpr int kTsBM = 128;                  // channels of a tile (UMMA M, TMEM lanes)
+constexpr int kTsWBytes = kTsBM * 64;       // packed weights of a block
+constexpr int kTsMaxCluster = 8;
+
+struct TsMat {
+    const void *w_scale;
+    void *y;
+    int tile_end;         // tiles of this matrix and of all before it
+    int N;
+    int ldy;
+};
+
+struct TsParams {
+    TsMat mat[kTsMaxMats];
+    const float *a_scale;
+    int *status;
+    int nmats, M, G, KB;  // KB: blocks of a row
+    int C;                // CTAs per cluster = shares of K
+    int blk_per, blk_extra;       // rank r owns blk_per (+ 1 if r < blk_extra) blocks of every row
+    int tiles, nclusters; // cluster c takes tiles c, c + nclusters, ...
+    int bpg;              // blocks per scale group (groups of whole blocks)
+    int y16;
+};
+
+struct TsMaps {
+    CUtensorMap w[kTsMaxMats];
+    CUtensorMap act;
+};
+
+// NT: tokens of a tile (UMMA N, a multiple of 16); SPP: 64-k slices per scale group, 0 = groups of whole blocks.
+template <int NT, int SPP>
+struct TsCfg {
+    static constexpr int kCtasPerSm = NT <= 32 ? 2 : 1;
+    static constexpr int kDrainWarps = NT > 32 ? 8 : 4;
+    static constexpr int kUnpackSets = NT <= 32 ? 1 : 2;          // sets of four warps, on alternate blocks
+    static constexpr int DC = NT * 4 / kDrainWarps;               // token columns of a drain warp
+    static constexpr int kFirstUnpack = 4, kFirstDrain = 4 + 4 * kUnpackSets;
+    static constexpr int kThreads = 32 * (kFirstDrain + kDrainWarps);
+    static constexpr int kTmemCols = NT <= 32 ? 256 : 512;
+    static constexpr int AS = NT <= 32 ? 2 : 4;     // unpacked blocks in tensor memory
+    static constexpr int kAccCols = kTmemCols - 64 * AS;
+    static constexpr int GPB = SPP == 0 ? 1 : 4 / SPP;            // groups of a block
+    static constexpr int UG = SPP == 0 ? 1 : GPB * NT <= 64 ? GPB : 2;   // groups of a unit = hand-off between MMA and drain
+    static constexpr int UPB = GPB / UG;                          // units of a block
+    static constexpr int kUnitCols = UG * NT;
+    static constexpr int kUnits = kAccCols / kUnitCols;
+    // One barrier says that a block is unpacked and its accumulators are free, where both come round alike.
+    static constexpr bool kFold = SPP != 0 && UPB == 1 && kUnits >= AS;
+    static constexpr int NU = kFold ? AS : kUnits > 4 ? 4 : kUnits;      // units in flight
+    static constexpr int kStageBytes = kTsWBytes + NT * 256;
+    static constexpr int kSumBytes = kTsBM * NT * 4;              // a tile's sums
+    static constexpr int kRing = ((kCtasPerSm == 2 ? 112 : 224) * 1024 - 2048 - 2 * kSumBytes) / kStageBytes;
+    static constexpr size_t kSmem = (size_t)kRing * kStageBytes + 2 * kSumBytes + 1024;
+    static constexpr bool kUnitBarrier = SPP == 0 || UPB > 1;     // else a block's barrier says it all
+    static_assert(NU >= 2 && AS < kRing, "");
+};
+
+__device__ __forceinline__ void ts_mma_i8_tmem(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void ts_tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void ts_tmem_st32(uint32_t taddr, const uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+        ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+          "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
+          "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]),
+          "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+        : "memory");
+}
+__device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[32]) { pf_tmem_ld32(taddr, v); }
+template <int N>
+__device__ __forceinline__ void ts_maxreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void ts_maxreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+
+__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// N (1, 2, 4, 8, 16) floats into another CTA's shared memory, counted by its barrier
+template <int N>
+__device__ __forceinline__ void ts_send(uint32_t addr, uint32_t bar, int rank, const float *v) {
+    uint32_t ra, rb;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(bar), "r"(rank));
+    if constexpr (N == 1) {
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                     ::"r"(ra), "r"(__float_as_uint(v[0])), "r"(rb) : "memory");
+    } else if constexpr (N == 2) {
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+                     ::"r"(ra), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(rb) : "memory");
+    } else {
+#pragma unroll
+        for (int j = 0; j < N; j += 4)
+            asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                         ::"r"(ra + j * 4), "r"(__float_as_uint(v[j])), "r"(__float_as_uint(v[j + 1])), "r"(__float_as_uint(v[j + 2])),
+                           "r"(__float_as_uint(v[j + 3])), "r"(rb) : "memory");
+    }
+}
+template <int N>
+__device__ __forceinline__ void ts_ld_shared(float (&v)[N], uint32_t addr) {
+    if constexpr (N == 1) asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[0]) : "r"(addr) : "memory");
+    else if constexpr (N == 2) asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(addr) : "memory");
+    else {
+#pragma unroll
+        for (int j = 0; j < N; j += 4)
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[j]), "=f"(v[j + 1]), "=f"(v[j + 2]), "=f"(v[j + 3])
+                         : "r"(addr + j * 4) : "memory");
+    }
+}
+// pf_wait for data that other CTAs of the cluster wrote
+__device__ __forceinline__ bool ts_wait_cluster(uint32_t bar, unsigned parity, volatile int *abort_flag) {
+    for (unsigned i = 0; i < kPfWaitPolls; ++i) {
+        unsigned ok;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+        if ((i & 63u) == 63u && *abort_flag) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
+
+// Bounded wait of a converged warp (pf_wait_all) whose first look costs a poll, a vote and a branch: most waits find their
+// barrier complete, and what the warps spend on looking was a third of all instructions.
+__device__ __forceinline__ bool ts_wait(uint32_t bar, unsigned parity, volatile int *abort_flag) {
+    if (__all_sync(0xFFFFFFFFu, pf_mbar_try_wait(bar, parity))) return true;
+    return pf_wait_all(bar, parity, abort_flag);
+}
+
+template <int NT, int SPP, bool H16>
+__global__ void __launch_bounds__(TsCfg<NT, SPP>::kThreads, TsCfg<NT, SPP>::kCtasPerSm)
+w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__ TsParams p) {
+    using C = TsCfg<NT, SPP>;
+    constexpr int R = C::kRing, AS = C::AS, NU = C::NU, UG = C::UG, DC = C::DC;
+    extern __shared__ unsigned char ts_smem[];
+    __shared__ __align__(8) unsigned long long bar_w[R], bar_b[R], bar_done[R], bar_a[AS], bar_full[NU], bar_free[NU];
+    __shared__ __align__(8) unsigned long long bar_sum[2][C::kDrainWarps];
+    __shared__ float tok_scale[NT];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_s;
+    volatile int *abort_flag = &abort_s;
+
+    const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const uint32_t stage0 = (pf_smem_u32(ts_smem) + 1023u) & ~1023u;
+    // this CTA's share of K, and its tiles
+    const int nc = p.C, rank = nc > 1 ? (int)cluster_ctarank() : 0;
+    int cl;
+    asm("mov.u32 %0, %%clusterid.x;" : "=r"(cl));
+    const int kb_lo = rank * p.blk_per + min(rank, p.blk_extra), nb = p.blk_per + (rank < p.blk_extra ? 1 : 0);
+    const int ntiles = (p.tiles - cl + p.nclusters - 1) / p.nclusters, n = ntiles * nb;      // blocks of this CTA
+    // matrix of a tile, and the tile's first channel there
+    auto mat_of = [&](int tile, int &n0) -> int {
+        int i = 0, first = 0;
+#pragma unroll
+        for (int j = 1; j < kTsMaxMats; ++j)
+            if (j < p.nmats && tile >= p.mat[j - 1].tile_end) { i = j; first = p.mat[j - 1].tile_end; }
+        n0 = (tile - first) * kTsBM;
+        return i;
+    };
+
+    if (threadIdx.x == 0) {
+        abort_s = 0;
+        for (int i = 0; i < R; ++i) {
+            pf_mbar_init(pf_smem_u32(&bar_w[i]), 1);
+            pf_mbar_init(pf_smem_u32(&bar_b[i]), 1);
+            pf_mbar_init(pf_smem_u32(&bar_done[i]), 1);
+        }
+        for (int i = 0; i < AS; ++i) pf_mbar_init(pf_smem_u32(&bar_a[i]), 4 + (C::kFold ? C::kDrainWarps : 0));
+        for (int i = 0; i < NU; ++i) {
+            pf_mbar_init(pf_smem_u32(&bar_full[i]), 1);
+            pf_mbar_init(pf_smem_u32(&bar_free[i]), C::kDrainWarps);
+        }
+        for (int i = 0; i < 2 * C::kDrainWarps; ++i) pf_mbar_init(pf_smem_u32(&bar_sum[0][0] + i), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        pf_fence_proxy_async();
+    }
+    if (warp == 1) pf_tmem_alloc(pf_smem_u32(&tmem_slot), C::kTmemCols);
+    pf_tc_fence_before();
+    __syncthreads();
+    pf_tc_fence_after();
+    // every CTA of the cluster has its barriers: arrive here, wait before the first access to another CTA
+    if (nc > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    const uint32_t sums0 = stage0 + R * C::kStageBytes;
+    const uint32_t tmem_a = tmem_slot, tmem_acc = tmem_slot + 64 * AS;
+    // Programmatic dependent launch: weights and scales are frozen, everything up to the first unpacked blocks
+    // overlaps the tail of the previous kernel of the stream.  Roles that touch anything else, or that could wait for
+    // one that does, wait for that kernel first (a wait's limit covers this kernel's own work only).
+    pdl_launch_dependents();
+
+    if (warp < C::kFirstUnpack) {
+        if constexpr (NT <= 32) ts_maxreg_dec<40>(); else ts_maxreg_dec<32>();
+        if (warp == 0 && lane == 0) {
+            // ===== TMA producer =============================================================
+            int tile = cl, kb = 0, n0;
+            int mi = mat_of(tile, n0);
+            auto advance = [&]() {
+                if (++kb == nb) {
+                    kb = 0;
+                    tile += p.nclusters;
+                    if (tile < p.tiles) mi = mat_of(tile, n0);
+                }
+            };
+            auto load_w = [&](int s) {
+                pf_tma_load_2d(stage0 + s * C::kStageBytes, &maps.w[mi], (kb_lo + kb) * 16, n0, pf_smem_u32(&bar_w[s]));
+            };
+            auto load_b = [&](int s, int k, uint32_t bar) {
+                const uint32_t dst = stage0 + s * C::kStageBytes + kTsWBytes;
+                pf_tma_load_2d(dst, &maps.act, (kb_lo + k) * 256, 0, bar);
+                pf_tma_load_2d(dst + NT * 128, &maps.act, (kb_lo + k) * 256 + 128, 0, bar);
+            };
+            const int head = min(R, n);
+            for (int i = 0; i < head; ++i) {
+                pf_mbar_arrive_expect_tx(pf_smem_u32(&bar_w[i]), kTsWBytes);
+                load_w(i);
+                advance();
+            }
+            asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.act) : "memory");
+            pdl_wait();
+            for (int i = 0, k = 0; i < head; ++i) {
+                pf_mbar_arrive_expect_tx(pf_smem_u32(&bar_b[i]), NT * 256);
+                load_b(i, k, pf_smem_u32(&bar_b[i]));
+                if (++k == nb) k = 0;
+            }
+            int s = 0;
+            uint32_t ph = 0;
+            for (int i = R; i < n; ++i) {
+                if (!pf_wait(pf_smem_u32(&bar_done[s]), ph, abort_flag)) break;
+                // (the MMA warp learns of these activations from the unpack warps, which wait for both)
+                pf_mbar_arrive_expect_tx(pf_smem_u32(&bar_w[s]), C::kStageBytes);
+                load_w(s);
+                load_b(s, kb, pf_smem_u32(&bar_w[s]));
+                advance();
+                if (++s == R) { s = 0; ph ^= 1u; }
+            }
+        } else if (warp == 1) {
+            // ===== MMA issuer: the warp walks, one elected lane issues ========================
+            const bool lead = pf_elect();
+            if (lead) pdl_wait();
+            __syncwarp();
+            const uint64_t b_desc0 = pf_smem_desc(stage0 + kTsWBytes);
+            const uint32_t b_lo = (uint32_t)b_desc0, b_hi = (uint32_t)(b_desc0 >> 32);
+            constexpr uint32_t idesc = pf_instr_desc(kTsBM, NT);
+            int s = 0, as = 0, un = 0;
+            uint32_t aph = 0, uph = 0, so = 0, dph = 0;
+            bool ok = true;
+            [[maybe_unused]] int kb = 0;
+            [[maybe_unused]] bool fresh = true;         // (groups of whole blocks) the next block opens a unit
+            const int first_left = p.bpg - (SPP == 0 ? kb_lo % p.bpg : 0);
+            [[maybe_unused]] int left = first_left;
+            for (int i = 0; i < n; ++i) {
+                if (i < R) ok = ts_wait(pf_smem_u32(&bar_b[s]), 0, abort_flag);
+                if (SPP == 0 && fresh) ok = ok && ts_wait(pf_smem_u32(&bar_free[un]), uph, abort_flag);
+                ok = ok && ts_wait(pf_smem_u32(&bar_a[as]), aph, abort_flag);
+                if (!ok) break;
+                auto step = [&](int j, uint32_t d, uint32_t acc) {
+                    const uint32_t koff = ((j >> 2) * NT * 128 + (j & 3) * 32) >> 4;
+                    ts_mma_i8_tmem(d, tmem_a + as * 64 + 8 * j, ((uint64_t)b_hi << 32) | (b_lo + so + koff), idesc, acc);
+                };
+                if constexpr (SPP != 0) {
+#pragma unroll
+                    for (int u = 0; u < C::UPB; ++u) {
+                        if constexpr (!C::kFold) ok = ts_wait(pf_smem_u32(&bar_free[un]), uph, abort_flag);
+                        if (!ok) break;
+                        pf_tc_fence_after();
+                        if (lead) {
+                            const uint32_t d = tmem_acc + un * C::kUnitCols;
+#pragma unroll
+                            for (int j = 0; j < 8 / C::UPB; ++j) step(u * (8 / C::UPB) + j, d + (j / (2 * SPP)) * NT, j % (2 * SPP) != 0 ? 1u : 0u);
+                            if constexpr (C::kUnitBarrier) pf_mma_commit(pf_smem_u32(&bar_full[un]));
+                        }
+                        if (++un == NU) { un = 0; uph ^= 1u; }
+                    }
+                    if (!ok) break;
+                } else {
+                    pf_tc_fence_after();
+                    const bool last = --left == 0 || kb + 1 == nb;
+                    if (lead) {
+                        const uint32_t d = tmem_acc + un * C::kUnitCols;
+                        step(0, d, fresh ? 0u : 1u);
+#pragma unroll
+                        for (int j = 1; j < 8; ++j) step(j, d, 1u);
+                        if (last) pf_mma_commit(pf_smem_u32(&bar_full[un]));
+                    }
+                    fresh = last;
+                    if (last) {
+                        left = p.bpg;
+                        if (++un == NU) { un = 0; uph ^= 1u; }
+                    }
+                    if (++kb == nb) { kb = 0; left = first_left; }
+                }
+                if (lead) pf_mma_commit(pf_smem_u32(&bar_done[s]));
+                so += C::kStageBytes >> 4;
+                if (++s == R) { s = 0; so = 0; dph ^= 1u; }
+                if (++as == AS) { as = 0; aph ^= 1u; }
+            }
+            // (the drain warps need not have waited for a block's barrier: none may be signalled after this CTA has left)
+            if constexpr (C::kUnitBarrier)
+                if (ok) ts_wait(pf_smem_u32(&bar_done[s == 0 ? R - 1 : s - 1]), s == 0 ? dph ^ 1u : dph, abort_flag);
+        }
+    } else if (warp < C::kFirstDrain) {
+        // ===== unpack warps: a lane's channel of a block, 16 words -> 64 columns of int8 lanes ========
+        const int set = (warp - C::kFirstUnpack) >> 2, q = warp & 3;
+        const int row = q * 32 + lane;
+        const uint32_t tlane = tmem_a + ((uint32_t)(q * 32) << 16);
+        const uint32_t row_off = row * 64, sw = (row >> 1) & 3;
+        int s = set, as = set % AS;                     // ring slot, place in tensor memory
+        uint32_t ph = 0;
+        bool got = true;
+        uint32_t w[4][4];                               // [t][slice]
+        auto load = [&](int slot) {
+            const uint32_t base = stage0 + slot * C::kStageBytes + row_off;
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[t][0]), "=r"(w[t][1]), "=r"(w[t][2]), "=r"(w[t][3])
+                             : "r"(base + ((t ^ sw) << 4)));
+        };
+        if (set < n) {
+            got = ts_wait(pf_smem_u32(&bar_w[s]), 0, abort_flag);
+            load(s);
+        }
+        int ds = (set + 2 * R - AS) % R;                // slot of block i - AS
+        uint32_t dph = 1u;                              // its parity (flips whenever ds comes round to 0)
+        for (int i = set; i < n && got; i += C::kUnpackSets) {
+            if (i >= AS) {                              // the MMAs of block i - AS have read this place
+                if (i < AS + C::kUnpackSets) pdl_wait();
+                got = ts_wait(pf_smem_u32(&bar_done[ds]), dph, abort_flag);
+                pf_tc_fence_after();
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t v[32];
+#pragma unroll
+                for (int sl = 0; sl < 2; ++sl)
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) v[16 * sl + 4 * t + j] = lane_codes(w[t][2 * h + sl], j);
+                ts_tmem_st32(tlane + as * 64 + 32 * h, v);
+            }
+            // the next block's words on their way while the stores finish
+            s += C::kUnpackSets;
+            if (s >= R) { s -= R; ph ^= 1u; }
+            if (i + C::kUnpackSets < n) {
+                got = got && ts_wait(pf_smem_u32(&bar_w[s]), ph, abort_flag);
+                load(s);
+            }
+            ts_tmem_st_wait();
+            pf_tc_fence_before();
+            __syncwarp();
+            if (lane == 0) pf_mbar_arrive(pf_smem_u32(&bar_a[as]));
+            as = (as + C::kUnpackSets) % AS;
+            ds += C::kUnpackSets;
+            if (ds >= R) { ds -= R; dph ^= 1u; }
+        }
+    } else {
+        if constexpr (NT <= 32) ts_maxreg_inc<120>();
+        else ts_maxreg_inc<128>();
+        // ===== drain warps ==============================================================
+        const int q = warp & 3, d = warp - C::kFirstDrain, col0 = (d >> 2) * DC;
+        const uint32_t tlane = tmem_acc + ((uint32_t)(q * 32) << 16) + col0;
+#pragma unroll
+        for (int un = 0; un < NU; ++un) {
+            if (lane == 0) pf_mbar_arrive(pf_smem_u32(C::kFold ? &bar_a[un] : &bar_free[un]));
+        }
+        // scales of a block (groups of 64, 128) or group, two ahead of the block that is drained
+        struct Scales { uint32_t r[4]; };
+        int tile = cl, kb = 0;                          // block that is drained
+        int ptile = cl, pkb = 0, left = n;              // block whose scales are requested next
+        const char *srow = nullptr;
+        auto locate = [&](int t) {
+            int n0;
+            const int i = mat_of(t, n0);
+            const int ch = min(n0 + q * 32 + lane, p.mat[i].N - 1);
+            srow = reinterpret_cast<const char *>(p.mat[i].w_scale) + (size_t)ch * p.G * (H16 ? 2 : 4) +
+                   (SPP == 0 ? 0 : kb_lo * C::GPB * (H16 ? 2 : 4));
+        };
+        locate(ptile);
+        constexpr int kStep = SPP == 0 ? 0 : C::GPB * (H16 ? 2 : 4);      // scale bytes of a block
+        auto request = [&]() -> Scales {
+            Scales sc = {};
+            if (left == 0) return sc;
+            --left;
+            if constexpr (kStep == 16) {
+                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(srow)); sc.r[0] = v.x; sc.r[1] = v.y; sc.r[2] = v.z; sc.r[3] = v.w;
+            } else if constexpr (kStep == 8) {
+                const uint2 v = __ldg(reinterpret_cast<const uint2 *>(srow)); sc.r[0] = v.x; sc.r[1] = v.y;
+            } else if constexpr (kStep == 4) {
+                sc.r[0] = __ldg(reinterpret_cast<const uint32_t *>(srow));
+            } else {
+                const int gi = (kb_lo + pkb) / p.bpg;
+                if constexpr (H16) sc.r[0] = __ldg(reinterpret_cast<const unsigned short *>(srow) + gi);
+                else sc.r[0] = __ldg(reinterpret_cast<const uint32_t *>(srow) + gi);
+            }
+            srow += kStep;
+            if (++pkb == nb) { pkb = 0; ptile += p.nclusters; if (left > 0) locate(ptile); }
+            return sc;
+        };
+        auto scale = [&](const Scales &sc, int g) -> float {       // g is a constant after unrolling
+            if constexpr (!H16) return __uint_as_float(sc.r[g]);
+            else {
+                const __half2 h = *reinterpret_cast<const __half2 *>(&sc.r[g >> 1]);
+                return (g & 1) ? __high2float(h) : __low2float(h);
+            }
+        };
+        Scales sc_cur, sc_n1 = request(), sc_n2 = request();
+        pdl_wait();
+        if (warp == C::kFirstDrain)
+            for (int j = lane; j < NT; j += 32) tok_scale[j] = p.a_scale[min(j, p.M - 1)] * (1.0f / kCodeGain);
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * C::kDrainWarps) : "memory");
+        float acc[DC];
+#pragma unroll
+        for (int j = 0; j < DC; ++j) acc[j] = 0.f;
+        int s = 0, un = 0;
+        uint32_t ph = 0, uph = 0;
+        bool got = true;
+        const int first_left = SPP == 0 ? p.bpg - kb_lo % p.bpg : 0;
+        [[maybe_unused]] int gleft = first_left;
+        int nsum = 0;                                   // tiles summed so far
+        auto drain_unit = [&](int g0) {
+            // (at most CG groups of staged values: more spill, and local memory is slow beside the copies)
+            constexpr int CG = DC == 32 ? 1 : UG;
+            const uint32_t at = tlane + un * C::kUnitCols;
+#pragma unroll
+            for (int c = 0; c < UG; c += CG) {
+                int v[CG][DC];
+#pragma unroll
+                for (int g = 0; g < CG; ++g) ts_tmem_ld(at + (c + g) * NT, v[g]);
+                pf_tmem_ld_wait();
+                if (c + CG == UG) {
+                    pf_tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) pf_mbar_arrive(pf_smem_u32(C::kFold ? &bar_a[un] : &bar_free[un]));
+                    if (++un == NU) { un = 0; uph ^= 1u; }
+                }
+#pragma unroll
+                for (int g = 0; g < CG; ++g) {
+                    const float f = scale(sc_cur, g0 + c + g);
+#pragma unroll
+                    for (int j = 0; j < DC; j += 2) {
+                        pf_fma2(acc[j], acc[j + 1], (float)v[g][j], (float)v[g][j + 1], f);
+                    }
+                }
+            }
+        };
+        for (int i = 0; i < n; ++i) {
+            sc_cur = sc_n1; sc_n1 = sc_n2; sc_n2 = request();
+            const bool row_end = kb + 1 == nb;
+            if constexpr (SPP != 0) {
+#pragma unroll
+                for (int u = 0; u < C::UPB; ++u) {
+                    if constexpr (C::kUnitBarrier) got = got && ts_wait(pf_smem_u32(&bar_full[un]), uph, abort_flag);
+                    else                           got = ts_wait(pf_smem_u32(&bar_done[s]), ph, abort_flag);
+                    pf_tc_fence_after();
+                    drain_unit(u * UG);
+                }
+            } else if (--gleft == 0 || row_end) {
+                gleft = row_end ? first_left : p.bpg;
+                got = ts_wait(pf_smem_u32(&bar_full[un]), uph, abort_flag);
+                pf_tc_fence_after();
+                drain_unit(0);
+            }
+            if (++s == R) { s = 0; ph ^= 1u; }
+            if (!got) break;
+            if (row_end) {
+                // ---- this CTA's share of the tile's sums is complete ---------------------------
+                int n0;
+                const int mi = mat_of(tile, n0);
+                const int ch = n0 + q * 32 + lane;
+                const bool valid = ch < p.mat[mi].N;
+                const int ldy = p.mat[mi].ldy;
+                char *y = reinterpret_cast<char *>(p.mat[mi].y);
+                auto store = [&](int m, float sum) {
+                    const float v = sum * tok_scale[m];
+                    if (m < p.M && valid) {
+                        const size_t at = (size_t)m * ldy + ch;
+                        if (H16 && p.y16) reinterpret_cast<__nv_bfloat16 *>(y)[at] = __float2bfloat16_rn(v);
+                        else              reinterpret_cast<float *>(y)[at] = v;
+                    }
+                };
+                // Shares are exchanged through distributed shared memory: rank r adds up the r-th part of every
+                // thread's columns, in rank order.  The buffers alternate: a CTA that is two tiles ahead has received what
+                // its peers sent after reading theirs.
+                auto exchange = [&](auto cc) {
+                    constexpr int CC = decltype(cc)::value, PC = DC / CC;
+                    constexpr uint32_t kFrom = C::kDrainWarps * 32 * PC * 4;       // bytes from one rank
+                    const uint32_t buf = sums0 + (nsum & 1) * C::kSumBytes + (d * 32 + lane) * (PC * 4);
+                    const uint32_t bar = pf_smem_u32(&bar_sum[nsum & 1][d]);
+                    if (nsum == 0) cluster_wait_acquire();
+                    __syncwarp();
+                    if (lane == 0) pf_mbar_arrive_expect_tx(bar, (CC - 1) * 32 * PC * 4);
+#pragma unroll
+                    for (int r = 0; r < CC; ++r)
+                        if (r != rank) ts_send<PC>(buf + rank * kFrom, bar, r, acc + r * PC);
+                    float own[PC], sum[PC];
+#pragma unroll
+                    for (int r = 0; r < CC; ++r)
+                        if (r == rank) {
+#pragma unroll
+                            for (int j = 0; j < PC; ++j) own[j] = acc[r * PC + j];
+                        }
+                    got = __all_sync(0xFFFFFFFFu, ts_wait_cluster(bar, (nsum >> 1) & 1, abort_flag));
+#pragma unroll
+                    for (int r = 0; r < CC; ++r) {
+                        float v[PC];
+                        ts_ld_shared<PC>(v, buf + r * kFrom);
+#pragma unroll
+                        for (int j = 0; j < PC; ++j) {
+                            const float x = r == rank ? own[j] : v[j];
+                            sum[j] = r == 0 ? x : sum[j] + x;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < PC; ++j) store(col0 + rank * PC + j, sum[j]);
+                    ++nsum;
+                };
+                if (nc == 1) {
+#pragma unroll
+                    for (int j = 0; j < DC; ++j) store(col0 + j, acc[j]);
+                } else if (nc == 2) exchange(std::integral_constant<int, 2>{});
+                else if (nc == 4)   exchange(std::integral_constant<int, 4>{});
+                else                exchange(std::integral_constant<int, 8>{});
+#pragma unroll
+                for (int j = 0; j < DC; ++j) acc[j] = 0.f;
+            }
+            if (++kb == nb) { kb = 0; tile += p.nclusters; }
+        }
+    }
+
+    // ---- wind down ---------------------------------------------------------------------
+    __syncwarp();
+    if (nc > 1 && warp < C::kFirstDrain) cluster_wait_acquire();
+    pf_tc_fence_before();
+    __syncwarp();
+    __syncthreads();
+    if (threadIdx.x == 0 && abort_s) atomicExch(p.status, W2A8_ERR_TIMEOUT);
+    if (warp == 1) {
+        pf_tc_fence_after();
+        pf_tmem_dealloc(tmem_slot, C::kTmemCols);
+    }
+}
+
+// ---- host side -----------------------------------------------------------------------
+bool tstream_supported(int M, int K, int group) {
+    if (M < 1 || M > 64 || K % kBlockK != 0) return false;
+    if ((long long)64 * 254 * group >= (1ll << 31)) return false;           // int32 accumulator range
+    return group == 64 || group == 128 || group % 256 == 0;
+}
+static int ts_tokens(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : 64; }
+
+// Shares of K and clusters for a launch over `tiles` tiles of `KB` blocks: the least cost in blocks that one CTA works
+// off after the other.  A last round that not all clusters have counts 0.6 of a round (the CTAs left have the memory
+// for themselves), a second CTA on the SMs costs 20 %, an exchange of sums as much as a block.  Against the best of all C over
+// 456 launches (13 sets of matrices, 4 to 64 tokens) the choice loses 1.5 % on average and 17 % at most.
+static double ts_plan(int tiles, int KB, const int *resident, bool two_per_sm, int *C, int *nclusters) {
+    const int forced = env_int("W2A8_TSTREAM_C", 0);
+    double best = 1e30;
+    for (int c = 1; c <= kTsMaxCluster; c *= 2) {
+        if (c > KB || resident[c] < 1 || (forced > 0 && c != forced)) continue;
+        const int ncl = std::min(tiles, resident[c]), rounds = (tiles + ncl - 1) / ncl, sms = sm_count();
+        const double whole = (double)tiles / ncl, share = (KB + c - 1) / c;
+        double cost = (whole + 0.6 * (rounds - whole)) * share;
+        if (two_per_sm) cost *= 1.0 + 0.2 * std::min(1.0, std::max(0.0, (double)(ncl * c - sms) / sms));
+        if (c > 1) cost += rounds;
+        if (cost < best) { best = cost; *C = c; *nclusters = ncl; }
+    }
+    return best;
+}
+
+// Whether the kernel takes a launch over `count` matrices of `tiles16` 16-channel tiles in all (9 to 64 tokens).
+// Compared are its own time, a constant and a time per block of the plan's cost, and that of the kernel with stationary
+// activations, 4.6 us + 0.25 ns per 32 channels x 256 k and eight tokens.  Measured on B200 (us per call, before / this
+// kernel, groups of 64 | 128 | one scale per channel):
+//   16 tokens: 8192 x 8192 10.1 / 9.0 | 9.9 / 8.3 | 8.7 / 8.4; 4096 x (14336 + 14336) 13.2 / 12.7 | 12.5 / 11.6 | 11.7 / 11.0;
+//     28672 x 8192 21.9 / 21.9 | 21.4 / 19.5 | 19.9 / 17.8; but 8192 x 28672 20.3 / 23.1 | 19.7 / 20.5 | 18.8 / 18.5
+//   32 tokens: 8192 x 8192 14.1 / 12.1 | 13.3 / 10.1 | 12.5 / 9.4; 8192 x (28672 + 28672) 62.7 / 59.2 | 57.9 / 41.2 | 55.4 / 36.8;
+//     28672 x 8192 40.8 / 30.2 | 37.8 / 22.6 | 36.4 / 19.5; 4096 x 14336 12.1 / 11.7 | 11.5 / 9.5 | 10.9 / 9.1
+//   64 tokens: 4096 x 4096 10.0 / 8.8 | 10.7 / 7.3 | 9.7 / 7.3; 8192 x (28672 + 28672) 135 / 95 | 103 / 68 | 77 / 55;
+//     14336 x 4096 22.2 / 16.2 | 18.5 / 12.9 | 20.6 / 12.3
+// Small launches stay where they were (us, before / this kernel): at 32 tokens 4096 x 4096 5.7 / 6.6 | 5.7 / 5.4 | 5.0 / 5.4,
+// at 48 6.2 / 7.3 (128), 2048 x 2048 3.2 / 5.3; and so does everything of up to 8 tokens (4096 x (14336 + 14336) 9.4 / 11.2).
+// W2A8_TSTREAM = 0 never, 2 whenever it supports the shape; any switch that forces a plan of another kernel keeps it out.
+bool tstream_takes(int M, int K, int group, int tiles16, int count) {
+    if (!tstream_supported(M, K, group)) return false;
+    const int mode = env_int("W2A8_TSTREAM", 1);
+    if (mode == 0) return false;
+    if (mode == 2) return true;
+    if (M <= 8) return false;
+    const int KB = K / kBlockK, tiles = (tiles16 + 7) / 8, nt = ts_tokens(M), slabs = (M + 7) / 8;
+    const long long blocks = (long long)tiles * KB;
+    const long long least = M <= 32 ? (count > 1 && M > 24 ? 700 : 1536) : M <= 48 && count == 1 ? 1024 : 300;
+    if (blocks < least) return false;
+    if (env_int("W2A8_STAT", 1) == 2 || env_int("W2A8_GEMV", 1) == 2) return false;
+    for (const char *name : {"W2A8_STAT_C", "W2A8_CHUNKS", "W2A8_TG", "W2A8_RING", "W2A8_MT", "W2A8_CLUSTER",
+                             "W2A8_MIN_WARPS", "W2A8_RELAX"})
+        if (env_set(name)) return false;
+    if (M == 64)
+        for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE"})
+            if (env_set(name)) return false;
+    const int sms = sm_count(), spp = group == 64 ? 0 : group == 128 ? 1 : 2;
+    int resident[kTsMaxCluster + 1] = {}, C, ncl;       // (what the device reports for a whole B200: 148, 74, 33, 15)
+    for (int c = 1; c <= kTsMaxCluster; c *= 2) resident[c] = (int)(sms / c * (c == 4 ? 0.9 : c == 8 ? 0.84 : 1.0)) * (nt <= 32 ? 2 : 1);
+    if (nt <= 32) resident[8] = resident[8] * 3 / 4;
+    static const double base[3][3] = {{1.3, 1.35, 1.9}, {2.0, 2.15, 2.85}, {3.4, 3.75, 4.3}};
+    static const double per_block[3][3] = {{0.64, 0.555, 0.5}, {0.92, 0.66, 0.55}, {0.84, 0.58, 0.47}};
+    const int w = nt == 16 ? 0 : nt == 32 ? 1 : 2;
+    const double mine = base[w][spp] + per_block[w][spp] * ts_plan(tiles, KB, resident, nt <= 32, &C, &ncl);
+    static const double per_cell[3] = {0.27e-3, 0.25e-3, 0.235e-3};
+    // (more than 32 tokens: the other kernels take one matrix per launch)
+    const double other = 4.6 * (M > 32 ? count : 1) + per_cell[spp] * (KB > 32 ? 1.1 : 1.0) * 4.0 * (double)blocks * slabs;
+    return mine < (M <= 16 && spp == 2 ? 0.86 : 0.96) * other;
+}
+
+// Clusters of C CTAs that are resident at once, looked up once per device and instance.
+struct TsClusters { std::atomic<int> known; int n[kTsMaxCluster + 1]; };
+
+template <typename K>
+static int ts_resident(K kernel, int C, int threads, size_t smem) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
+template <int NT, int SPP, bool H16>
+static cudaError_t launch_ts_inst(const TsMaps &maps, TsParams &p, cudaStream_t st) {
+    using C = TsCfg<NT, SPP>;
+    auto kernel = w2a8_tstream_kernel<NT, SPP, H16>;
+    static PerDeviceFlags configured;   // per kernel instantiation
+    if (cudaError_t e = allow_dynamic_smem(kernel, configured, (int)C::kSmem)) return e;
+    if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) return e;
+    static TsClusters clusters[kMaxDevices];
+    TsClusters &cs = clusters[current_device()];
+    if (!cs.known.load(std::memory_order_acquire)) {      // racing threads write the same values
+        // The query answers for one CTA per SM; with 256 columns of tensor memory, 112 KB and half of the registers two
+        // are resident (clusters of eight: about three quarters of that).
+        for (int c = 1; c <= kTsMaxCluster; c *= 2) cs.n[c] = C::kCtasPerSm * ts_resident(kernel, c, C::kThreads, C::kSmem);
+        if (C::kCtasPerSm == 2 && cs.n[8] > 1) cs.n[8] = cs.n[8] * 3 / 4;
+        cs.known.store(1, std::memory_order_release);
+    }
+    if (ts_plan(p.tiles, p.KB, cs.n, C::kCtasPerSm == 2, &p.C, &p.nclusters) > 1e29) return cudaErrorNotSupported;
+    p.blk_per = p.KB / p.C; p.blk_extra = p.KB % p.C;
+    return launch_kernel_clusters(kernel, dim3((unsigned)(p.nclusters * p.C)), dim3(C::kThreads), C::kSmem, st, pdl_enabled(),
+                                  make_uint2((unsigned)p.C, 1u), maps, p);
+}
+template <int NT, bool H16>
+static cudaError_t launch_ts_spp(const TsMaps &maps, TsParams &p, int spp, cudaStream_t st) {
+    return spp == 1 ? launch_ts_inst<NT, 1, H16>(maps, p, st)
+         : spp == 2 ? launch_ts_inst<NT, 2, H16>(maps, p, st) : launch_ts_inst<NT, 0, H16>(maps, p, st);
+}
+template <bool H16>
+static cudaError_t launch_ts_nt(const TsMaps &maps, TsParams &p, int spp, cudaStream_t st) {
+    switch (ts_tokens(p.M)) {
+        case 16: return launch_ts_spp<16, H16>(maps, p, spp, st);
+        case 32: return launch_ts_spp<32, H16>(maps, p, spp, st);
+        default: return launch_ts_spp<64, H16>(maps, p, spp, st);
+    }
+}
+
+// Enqueue one launch over `count` matrices (1 .. 4) that share their activations.  kStatNoPlan: nothing was launched,
+// because no cluster is resident (a small partition of a GPU).
+int launch_tstream(const int8_t *a, const float *a_scale, int count, const uint32_t *const *packed,
+                   const void *const *w_scale, void *const *y, const int *N, const int *ldy, int M, int K, int group,
+                   void *workspace, cudaStream_t st, bool h16, bool y16) {
+    if (count < 1 || count > kTsMaxMats || !tstream_supported(M, K, group)) return W2A8_ERR_SHAPE;
+    EncodeTiledFn encode = encode_tiled_fn();
+    if (!encode) return W2A8_ERR_CUDA;
+    TsMaps maps = {};
+    TsParams p = {};
+    const cuuint32_t estr[2] = {1u, 1u};
+    int tiles = 0;
+    for (int i = 0; i < count; ++i) {
+        tiles += (N[i] + kTsBM - 1) / kTsBM;
+        p.mat[i].w_scale = w_scale[i]; p.mat[i].y = y[i]; p.mat[i].N = N[i]; p.mat[i].ldy = ldy[i]; p.mat[i].tile_end = tiles;
+        const cuuint64_t dims[2] = {(cuuint64_t)(K / 16), (cuuint64_t)N[i]};
+        const cuuint64_t strides[1] = {(cuuint64_t)(K / 4)};
+        const cuuint32_t box[2] = {16u, (cuuint32_t)kTsBM};                    // 64 bytes x 128 channels
+        if (encode(&maps.w[i], CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t *>(packed[i]), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return W2A8_ERR_CUDA;
+    }
+    {
+        const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
+        const cuuint64_t strides[1] = {(cuuint64_t)K};
+        const cuuint32_t box[2] = {128u, (cuuint32_t)ts_tokens(M)};
+        if (encode(&maps.act, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t *>(a), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return W2A8_ERR_CUDA;
+    }
+    p.a_scale = a_scale; p.nmats = count; p.M = M; p.G = K / group; p.KB = K / kBlockK;
+    p.bpg = group >= kBlockK ? group / kBlockK : 1;
+    p.y16 = h16 && y16 ? 1 : 0;
+    p.tiles = tiles;
+    p.status = reinterpret_cast<int *>(workspace);
+    const int spp = group == 64 ? 1 : group == 128 ? 2 : 0;
+    const cudaError_t e = h16 ? launch_ts_nt<true>(maps, p, spp, st) : launch_ts_nt<false>(maps, p, spp, st);
+    return e == cudaSuccess ? W2A8_OK : e == cudaErrorNotSupported ? kStatNoPlan : W2A8_ERR_CUDA;
+}
+
+}  // namespace w2a8

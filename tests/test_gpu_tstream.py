@@ -1,0 +1,163 @@
+"""GPU parity of the streaming kernel on the tensor cores (weights unpacked into tensor memory) against the CPU
+reference: edges of the token tiles, ragged last channel tiles, every scale group form, unequal shares of K, groups cut
+between shares, several tiles per cluster, grouped matrices, both scale types and result types."""
+import numpy as np
+import pytest
+
+from conftest import Guarded
+from paper_2508_06753_b200 import synth
+
+pytestmark = pytest.mark.gpu
+# y is a sum of K / group <= 448 fp32 terms from exact integer sums: about sqrt(448) * 2^-24 of its row's largest
+# value, 1e-6; the other kernels are held to the same 1e-4
+TOL = 1e-4
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2508_06753_b200 import binding, build
+    build.build()
+    binding.lib()
+    return torch, binding
+
+
+def _dev(torch, arr):
+    return torch.from_numpy(np.ascontiguousarray(arr)).cuda()
+
+
+CASES = [
+    # M, K, [N], group (0 = K), forced shares of K (0 = the plan's)
+    (1, 256, [16], 64, 0),                     # one block, an eighth of a tile
+    (8, 512, [128], 128, 2),
+    (9, 1280, [144], 64, 2),                   # shares of 3 and 2 blocks; a second tile of 16 channels
+    (16, 4096, [272, 16], 256, 4),
+    (16, 2048, [128 * 9], 0, 8),               # one scale per channel, a block per CTA
+    (17, 1792, [640, 32], 64, 4),              # shares of 2 and 1 blocks
+    (32, 1536, [384], 512, 4),                 # groups of two blocks cut between shares of 2, 2, 1, 1
+    (31, 768, [128 * 150], 64, 1),             # more tiles than SMs
+    (24, 1024, [128 * 170], 128, 2),           # two tiles for some clusters: both exchange buffers
+    (12, 512, [128 * 310], 64, 1),             # a second round
+    (33, 2048, [1024], 64, 8),
+    (48, 4096, [256, 128], 0, 0),
+    (64, 7168, [512], 64, 4),                  # the ring of stages comes round
+    (64, 512, [128 * 160], 128, 2),
+    (50, 3072, [144], 1024, 8),
+    (5, 14336, [256], 64, 8),
+]
+
+
+@pytest.mark.parametrize("h16", [False, True])
+@pytest.mark.parametrize("M,K,Ns,group,shares", CASES)
+def test_against_reference(gpu, oracle, monkeypatch, M, K, Ns, group, shares, h16):
+    torch, b = gpu
+    monkeypatch.setenv("W2A8_TSTREAM", "2")
+    if shares:
+        monkeypatch.setenv("W2A8_TSTREAM_C", str(shares))
+    g = K if group == 0 else group
+    mats = [synth.make_linear(7 * M + K + i, K, N, g) for i, N in enumerate(Ns)]
+    if h16:
+        mats = [(c, s.astype(np.float16)) for c, s in mats]
+    bits = synth.activations_bf16(M + K, M, K, 0.01)
+    a, s_a = b.a8_quantize(_dev(torch, bits.view(np.int16)).view(torch.bfloat16))
+    packed, scales = [b.w2_pack(_dev(torch, c)) for c, _ in mats], [_dev(torch, s) for _, s in mats]
+    ws = b.new_workspace(b.w2a8_grouped_workspace_bytes(Ns, M, K, g))
+    ys = []
+    for _ in range(2):
+        guards = [Guarded(torch, (M, N), torch.float32, float("nan")) for N in Ns]
+        if h16:
+            for pk, sc, gd in zip(packed, scales, guards):
+                b.w2a8_gemm_h16(a, s_a, pk, sc, g, ws, y=gd.view)
+        else:
+            b.w2a8_gemm_grouped(a, s_a, b.Group(packed, scales), g, ws, y=[gd.view for gd in guards])
+        torch.cuda.synchronize()
+        assert b.w2a8_workspace_status(ws) == 0
+        for gd in guards:
+            gd.check("y")
+        ys.append([gd.view.clone() for gd in guards])
+    a_ref, s_ref = oracle.quantize(bits)
+    for i, ((codes, s_w), y, again) in enumerate(zip(mats, *ys)):
+        assert torch.equal(y, again)
+        N = codes.shape[0]
+        sel = np.unique(np.concatenate([np.arange(min(N, 160)), np.arange(max(0, N - 160), N), np.arange(0, N, 37)]))
+        ref = oracle.gemm(a_ref, s_ref, codes[sel], s_w[sel].astype(np.float32), g)
+        err = np.abs(y.cpu().numpy()[:, sel].astype(np.float64) - ref).max(axis=1)
+        assert (err <= TOL * np.abs(ref).max(axis=1)).all(), float(err.max())
+        if h16:
+            y16 = b.w2a8_gemm_h16(a, s_a, packed[i], scales[i], g, ws,
+                                  y=torch.full((M, N), float("nan"), dtype=torch.bfloat16, device="cuda"))
+            assert torch.equal(y16, y.to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("group", [64, 2048])
+def test_largest_sums_and_scales(gpu, oracle, monkeypatch, group):
+    """Every product at its extreme (code 0 = -2 times +-127) and scales from 2^-100 to 2^95 (the running sums carry
+    64 times sums of up to 2^19, so that larger ones leave fp32)."""
+    torch, b = gpu
+    monkeypatch.setenv("W2A8_TSTREAM", "2")
+    M, N, K = 16, 128, 2048
+    codes = np.zeros((N, K), np.uint8)
+    codes[1::2] = 3
+    s_w = np.exp2(np.linspace(-100, 95, N * (K // group))).reshape(N, K // group).astype(np.float32)
+    a = np.where(np.arange(M)[:, None] % 2 == 0, 127, -127).astype(np.int8).repeat(K, axis=1)
+    s_a = np.full(M, 0.5, np.float32)
+    ws = b.new_workspace(b.w2a8_workspace_bytes(M, N, K, group))
+    y = b.w2a8_gemm(_dev(torch, a), _dev(torch, s_a), b.w2_pack(_dev(torch, codes)), _dev(torch, s_w), group, ws)
+    ref = oracle.gemm(a, s_a, codes, s_w, group)
+    err = np.abs(y.cpu().numpy().astype(np.float64) - ref)
+    assert (err <= 1e-5 * np.abs(ref)).all()          # all terms of an output have one sign: relative to each output
+
+
+@pytest.mark.parametrize("M,K,N", [(32, 8192, 8192), (64, 4096, 4096)])
+def test_default_dispatch_in_a_replayed_graph(gpu, monkeypatch, M, K, N):
+    """By the rule, captured and replayed on changed activations: the bits of a plain call."""
+    torch, b = gpu
+    gen = torch.Generator(device="cuda").manual_seed(M)
+    codes = torch.randint(0, 4, (N, K), generator=gen, device="cuda", dtype=torch.uint8)
+    packed, scale = b.w2_pack(codes), torch.rand((N, K // 128), generator=gen, device="cuda") + 0.01
+    x = torch.randn((M, K), generator=gen, device="cuda").to(torch.bfloat16)
+    a, s = b.a8_quantize(x)
+    ws = b.new_workspace(b.w2a8_workspace_bytes(M, N, K, 128))
+    y = torch.empty((M, N), device="cuda")
+    b.w2a8_gemm(a, s, packed, scale, 128, ws, y=y)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        b.a8_quantize(x, a, s)
+        b.w2a8_gemm(a, s, packed, scale, 128, ws, y=y)
+    x.copy_(torch.randn((M, K), generator=gen, device="cuda").to(torch.bfloat16))
+    graph.replay()
+    got = y.clone()
+    a2, s2 = b.a8_quantize(x)
+    plain = b.w2a8_gemm(a2, s2, packed, scale, 128, ws)
+    assert torch.equal(got, plain)
+    monkeypatch.setenv("W2A8_TSTREAM", "0")
+    other = b.w2a8_gemm(a2, s2, packed, scale, 128, b.new_workspace(b.w2a8_workspace_bytes(M, N, K, 128)))
+    assert not torch.equal(other, plain)              # another kernel, another order of the additions
+    assert (other - plain).abs().max() <= 1e-5 * plain.abs().max()
+
+
+def test_behind_a_long_kernel(gpu, monkeypatch):
+    """The bounded waits do not count the time of the kernel before (eight quantiser launches of 0.26 s)."""
+    torch, b = gpu
+    monkeypatch.setenv("W2A8_TSTREAM", "2")
+    M, N, K = 20, 512, 8192                            # four shares of eight blocks: the ring comes round
+    monkeypatch.setenv("W2A8_TSTREAM_C", "4")
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    packed = b.w2_pack(torch.randint(0, 4, (N, K), generator=gen, device="cuda", dtype=torch.uint8))
+    scale = torch.rand((N, K // 64), generator=gen, device="cuda")
+    a, s = b.a8_quantize(torch.randn((M, K), generator=gen, device="cuda").to(torch.bfloat16))
+    ws = b.new_workspace(b.w2a8_workspace_bytes(M, N, K, 64))
+    alone = b.w2a8_gemm(a, s, packed, scale, 64, ws)
+    x = torch.randn((1, 1 << 30), dtype=torch.bfloat16, device="cuda")
+    row, row_scale = torch.empty((1, 1 << 30), dtype=torch.int8, device="cuda"), torch.empty(1, device="cuda")
+    y = torch.full_like(alone, float("nan"))
+    torch.cuda.synchronize()
+    for _ in range(8):
+        b.a8_quantize(x, row, row_scale)
+    b.w2a8_gemm(a, s, packed, scale, 64, ws, y=y)
+    torch.cuda.synchronize()
+    assert b.w2a8_workspace_status(ws) == 0
+    assert torch.equal(y, alone)

@@ -92,3 +92,19 @@ def test_64_tokens(N, K, group, kernel):
     assert b.w2a8_kernel_for(64, N, K, group) == kernel
     if (N, K) == (5120, 14336):
         assert b.w2a8_workspace_bytes(64, N, K, group) <= 8 << 20
+
+
+@pytest.mark.parametrize("M,taken", [(8, False), (32, True), (33, True), (64, True), (65, False)])
+def test_streaming_tensor_core_kernel(monkeypatch, M, taken):
+    import ctypes
+    monkeypatch.delenv("W2A8_TSTREAM", raising=False)
+    plan = lambda: bool(b.lib().w2a8_grouped_plan(2, (ctypes.c_int * 2)(28672, 28672), M, 8192, 128, b.FUSE_OFF) & 4)
+    assert plan() is taken
+    for name in ("W2A8_GEMV", "W2A8_STAT"):           # another kernel forced, or kept out
+        monkeypatch.setenv(name, "2")
+        assert plan() is False
+        monkeypatch.setenv(name, "0")
+        assert plan() is taken
+        monkeypatch.delenv(name)
+    monkeypatch.setenv("W2A8_TSTREAM", "0")
+    assert plan() is False
