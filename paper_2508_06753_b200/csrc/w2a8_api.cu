@@ -28,7 +28,7 @@ int launch_stat(const int8_t *a, const float *a_scale, int count, const uint32_t
                 const void *const *w_scale, void *const *y, const int *N, const int *ldy, int M, int K, int group,
                 cudaStream_t st, bool h16, bool y16);
 
-bool tstream_takes(int M, int K, int group, int tiles16, int count);
+bool tstream_takes(int M, int K, int group, int tiles16, int count, bool h16);
 int launch_tstream(const int8_t *a, const float *a_scale, int count, const uint32_t *const *packed,
                    const void *const *w_scale, void *const *y, const int *N, const int *ldy, int M, int K, int group,
                    void *workspace, cudaStream_t st, bool h16, bool y16);
@@ -527,7 +527,7 @@ size_t gemm_header_bytes(int M, int N, int K, int group) {
 int gemm_dispatch(const int8_t *a, const float *a_scale, const uint32_t *packed, const void *w_scale,
                   void *y, int32_t *partials, int M, int N, int K, int group, const ShapeInfo &si,
                   void *workspace, void *stream, bool h16, bool y16, bool a16) {
-    if (!a16 && !partials && tstream_takes(M, K, group, N / 16, 1)) {
+    if (!a16 && !partials && tstream_takes(M, K, group, N / 16, 1, h16)) {
         const int st = launch_tstream(a, a_scale, 1, &packed, &w_scale, &y, &N, &N, M, K, group, workspace, (cudaStream_t)stream, h16, y16);
         if (st != kStatNoPlan) return st;
     }
@@ -651,7 +651,7 @@ static int grouped_plan(int count, const int *N, int M, int K, int group, int fu
         plan = 3;
     else if (stat_takes(M, K, group, tiles, count, false) || gemv_preferred(M, K, group, tiles, count))
         plan = 1;
-    if (plan != 3 && tstream_takes(M, K, group, tiles, count)) plan |= 4;
+    if (plan != 3 && tstream_takes(M, K, group, tiles, count, false)) plan |= 4;
     return plan;
 }
 

@@ -1,6 +1,6 @@
 // Streaming kernel on the 5th-generation tensor cores (up to 64 tokens): the packed weights stream through
 // shared memory once, are unpacked into tensor memory as the A operand of tcgen05.mma kind::i8 (UMMA M = 128
-// channels), and meet the tokens as a narrow B operand (UMMA N = 16, 32 or 64).
+// channels), and meet the tokens as a narrow B operand (UMMA N = 16, 32, 48 or 64).
 //
 //  * Work.  A cluster of C CTAs (1, 2, 4 or 8) takes tiles of 128 channels, of up to four matrices that share their
 //    activations; rank r of it the r-th share of K (K-splitting of Sec. II-D), in blocks of 256 k = 8 KB of packed weights.
@@ -62,9 +62,10 @@ struct TsMaps {
     CUtensorMap act;
 };
 
-// NT: tokens of a tile (UMMA N, a multiple of 16); SPP: 64-k slices per scale group, 0 = groups of whole blocks.
+// NT: tokens that are drained (16, 24, 32, 48, 64); SPP: 64-k slices per scale group, 0 = groups of whole blocks.
 template <int NT, int SPP>
 struct TsCfg {
+    static constexpr int BN = (NT + 15) / 16 * 16;                // UMMA N
     static constexpr int kCtasPerSm = NT <= 32 ? 2 : 1;
     static constexpr int kDrainWarps = NT > 32 ? 8 : 4;
     static constexpr int kUnpackSets = NT <= 32 ? 1 : 2;          // sets of four warps, on alternate blocks
@@ -75,15 +76,15 @@ struct TsCfg {
     static constexpr int AS = NT <= 32 ? 2 : 4;     // unpacked blocks in tensor memory
     static constexpr int kAccCols = kTmemCols - 64 * AS;
     static constexpr int GPB = SPP == 0 ? 1 : 4 / SPP;            // groups of a block
-    static constexpr int UG = SPP == 0 ? 1 : GPB * NT <= 64 ? GPB : 2;   // groups of a unit = hand-off between MMA and drain
+    static constexpr int UG = SPP == 0 ? 1 : GPB * BN <= 64 ? GPB : 2;   // groups of a unit = hand-off between MMA and drain
     static constexpr int UPB = GPB / UG;                          // units of a block
-    static constexpr int kUnitCols = UG * NT;
+    static constexpr int kUnitCols = UG * BN;
     static constexpr int kUnits = kAccCols / kUnitCols;
     // One barrier says that a block is unpacked and its accumulators are free, where both come round alike.
     static constexpr bool kFold = SPP != 0 && UPB == 1 && kUnits >= AS;
     static constexpr int NU = kFold ? AS : kUnits > 4 ? 4 : kUnits;      // units in flight
-    static constexpr int kStageBytes = kTsWBytes + NT * 256;
-    static constexpr int kSumBytes = kTsBM * NT * 4;              // a tile's sums
+    static constexpr int kStageBytes = kTsWBytes + BN * 256;
+    static constexpr int kSumBytes = kTsBM * (DC == 24 ? 32 : DC) * kDrainWarps;     // a tile's sums, in pieces of 16 bytes
     static constexpr int kRing = ((kCtasPerSm == 2 ? 112 : 224) * 1024 - 2048 - 2 * kSumBytes) / kStageBytes;
     static constexpr size_t kSmem = (size_t)kRing * kStageBytes + 2 * kSumBytes + 1024;
     static constexpr bool kUnitBarrier = SPP == 0 || UPB > 1;     // else a block's barrier says it all
@@ -120,6 +121,10 @@ __device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[16]) {
           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
         : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[24]) {
+    ts_tmem_ld(taddr, reinterpret_cast<int (&)[16]>(v[0]));
+    ts_tmem_ld(taddr + 16, reinterpret_cast<int (&)[8]>(v[16]));
+}
 __device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[32]) { pf_tmem_ld32(taddr, v); }
 template <int N>
 __device__ __forceinline__ void ts_maxreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
@@ -127,35 +132,39 @@ template <int N>
 __device__ __forceinline__ void ts_maxreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 
 __device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// N (1, 2, 4, 8, 16) floats into another CTA's shared memory, counted by its barrier
+// N floats into another CTA's shared memory, counted by its barrier, in the widest pieces that N divides into
 template <int N>
 __device__ __forceinline__ void ts_send(uint32_t addr, uint32_t bar, int rank, const float *v) {
     uint32_t ra, rb;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(bar), "r"(rank));
-    if constexpr (N == 1) {
-        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
-                     ::"r"(ra), "r"(__float_as_uint(v[0])), "r"(rb) : "memory");
-    } else if constexpr (N == 2) {
-        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
-                     ::"r"(ra), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(rb) : "memory");
-    } else {
+    constexpr int P = N % 4 == 0 ? 4 : N % 2 == 0 ? 2 : 1;
 #pragma unroll
-        for (int j = 0; j < N; j += 4)
+    for (int j = 0; j < N; j += P) {
+        if constexpr (P == 4)
             asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
                          ::"r"(ra + j * 4), "r"(__float_as_uint(v[j])), "r"(__float_as_uint(v[j + 1])), "r"(__float_as_uint(v[j + 2])),
                            "r"(__float_as_uint(v[j + 3])), "r"(rb) : "memory");
+        else if constexpr (P == 2)
+            asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+                         ::"r"(ra + j * 4), "r"(__float_as_uint(v[j])), "r"(__float_as_uint(v[j + 1])), "r"(rb) : "memory");
+        else
+            asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                         ::"r"(ra + j * 4), "r"(__float_as_uint(v[j])), "r"(rb) : "memory");
     }
 }
 template <int N>
 __device__ __forceinline__ void ts_ld_shared(float (&v)[N], uint32_t addr) {
-    if constexpr (N == 1) asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[0]) : "r"(addr) : "memory");
-    else if constexpr (N == 2) asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(addr) : "memory");
-    else {
+    constexpr int P = N % 4 == 0 ? 4 : N % 2 == 0 ? 2 : 1;
 #pragma unroll
-        for (int j = 0; j < N; j += 4)
+    for (int j = 0; j < N; j += P) {
+        if constexpr (P == 4)
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[j]), "=f"(v[j + 1]), "=f"(v[j + 2]), "=f"(v[j + 3])
                          : "r"(addr + j * 4) : "memory");
+        else if constexpr (P == 2)
+            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[j]), "=f"(v[j + 1]) : "r"(addr + j * 4) : "memory");
+        else
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[j]) : "r"(addr + j * 4) : "memory");
     }
 }
 // pf_wait for data that other CTAs of the cluster wrote
@@ -183,7 +192,7 @@ template <int NT, int SPP, bool H16>
 __global__ void __launch_bounds__(TsCfg<NT, SPP>::kThreads, TsCfg<NT, SPP>::kCtasPerSm)
 w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__ TsParams p) {
     using C = TsCfg<NT, SPP>;
-    constexpr int R = C::kRing, AS = C::AS, NU = C::NU, UG = C::UG, DC = C::DC;
+    constexpr int BN = C::BN, R = C::kRing, AS = C::AS, NU = C::NU, UG = C::UG, DC = C::DC;
     extern __shared__ unsigned char ts_smem[];
     __shared__ __align__(8) unsigned long long bar_w[R], bar_b[R], bar_done[R], bar_a[AS], bar_full[NU], bar_free[NU];
     __shared__ __align__(8) unsigned long long bar_sum[2][C::kDrainWarps];
@@ -258,7 +267,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             auto load_b = [&](int s, int k, uint32_t bar) {
                 const uint32_t dst = stage0 + s * C::kStageBytes + kTsWBytes;
                 pf_tma_load_2d(dst, &maps.act, (kb_lo + k) * 256, 0, bar);
-                pf_tma_load_2d(dst + NT * 128, &maps.act, (kb_lo + k) * 256 + 128, 0, bar);
+                pf_tma_load_2d(dst + BN * 128, &maps.act, (kb_lo + k) * 256 + 128, 0, bar);
             };
             const int head = min(R, n);
             for (int i = 0; i < head; ++i) {
@@ -269,7 +278,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.act) : "memory");
             pdl_wait();
             for (int i = 0, k = 0; i < head; ++i) {
-                pf_mbar_arrive_expect_tx(pf_smem_u32(&bar_b[i]), NT * 256);
+                pf_mbar_arrive_expect_tx(pf_smem_u32(&bar_b[i]), BN * 256);
                 load_b(i, k, pf_smem_u32(&bar_b[i]));
                 if (++k == nb) k = 0;
             }
@@ -291,7 +300,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             __syncwarp();
             const uint64_t b_desc0 = pf_smem_desc(stage0 + kTsWBytes);
             const uint32_t b_lo = (uint32_t)b_desc0, b_hi = (uint32_t)(b_desc0 >> 32);
-            constexpr uint32_t idesc = pf_instr_desc(kTsBM, NT);
+            constexpr uint32_t idesc = pf_instr_desc(kTsBM, BN);
             int s = 0, as = 0, un = 0;
             uint32_t aph = 0, uph = 0, so = 0, dph = 0;
             bool ok = true;
@@ -305,7 +314,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                 ok = ok && ts_wait(pf_smem_u32(&bar_a[as]), aph, abort_flag);
                 if (!ok) break;
                 auto step = [&](int j, uint32_t d, uint32_t acc) {
-                    const uint32_t koff = ((j >> 2) * NT * 128 + (j & 3) * 32) >> 4;
+                    const uint32_t koff = ((j >> 2) * BN * 128 + (j & 3) * 32) >> 4;
                     ts_mma_i8_tmem(d, tmem_a + as * 64 + 8 * j, ((uint64_t)b_hi << 32) | (b_lo + so + koff), idesc, acc);
                 };
                 if constexpr (SPP != 0) {
@@ -317,7 +326,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                         if (lead) {
                             const uint32_t d = tmem_acc + un * C::kUnitCols;
 #pragma unroll
-                            for (int j = 0; j < 8 / C::UPB; ++j) step(u * (8 / C::UPB) + j, d + (j / (2 * SPP)) * NT, j % (2 * SPP) != 0 ? 1u : 0u);
+                            for (int j = 0; j < 8 / C::UPB; ++j) step(u * (8 / C::UPB) + j, d + (j / (2 * SPP)) * BN, j % (2 * SPP) != 0 ? 1u : 0u);
                             if constexpr (C::kUnitBarrier) pf_mma_commit(pf_smem_u32(&bar_full[un]));
                         }
                         if (++un == NU) { un = 0; uph ^= 1u; }
@@ -470,13 +479,13 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
         int nsum = 0;                                   // tiles summed so far
         auto drain_unit = [&](int g0) {
             // (at most CG groups of staged values: more spill, and local memory is slow beside the copies)
-            constexpr int CG = DC == 32 ? 1 : UG;
+            constexpr int CG = DC > 16 ? 1 : UG;
             const uint32_t at = tlane + un * C::kUnitCols;
 #pragma unroll
             for (int c = 0; c < UG; c += CG) {
                 int v[CG][DC];
 #pragma unroll
-                for (int g = 0; g < CG; ++g) ts_tmem_ld(at + (c + g) * NT, v[g]);
+                for (int g = 0; g < CG; ++g) ts_tmem_ld(at + (c + g) * BN, v[g]);
                 pf_tmem_ld_wait();
                 if (c + CG == UG) {
                     pf_tc_fence_before();
@@ -530,27 +539,33 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                     }
                 };
                 // Shares are exchanged through distributed shared memory: rank r adds up the r-th part of every
-                // thread's columns, in rank order.  The buffers alternate: a CTA that is two tiles ahead has received what
+                // thread's columns, in rank order (of 24 columns eight ranks have parts of 4, not 3, and the last two none: with
+                // 4-byte stores 14336 x 4096 took 14 instead of 10 us at 24 tokens; a rank without columns gets a word, to keep step).  The buffers alternate: a CTA that is two tiles ahead has received what
                 // its peers sent after reading theirs.
                 auto exchange = [&](auto cc) {
-                    constexpr int CC = decltype(cc)::value, PC = DC / CC;
+                    constexpr int CC = decltype(cc)::value, PC = DC == 24 ? (24 / CC + 3) / 4 * 4 : DC / CC, kParts = DC / PC;
                     constexpr uint32_t kFrom = C::kDrainWarps * 32 * PC * 4;       // bytes from one rank
                     const uint32_t buf = sums0 + (nsum & 1) * C::kSumBytes + (d * 32 + lane) * (PC * 4);
                     const uint32_t bar = pf_smem_u32(&bar_sum[nsum & 1][d]);
                     if (nsum == 0) cluster_wait_acquire();
                     __syncwarp();
-                    if (lane == 0) pf_mbar_arrive_expect_tx(bar, (CC - 1) * 32 * PC * 4);
+                    if (lane == 0) pf_mbar_arrive_expect_tx(bar, (CC - 1) * (rank < kParts ? 32 * PC * 4 : 4));
 #pragma unroll
-                    for (int r = 0; r < CC; ++r)
-                        if (r != rank) ts_send<PC>(buf + rank * kFrom, bar, r, acc + r * PC);
+                    for (int r = 0; r < CC; ++r) {
+                        if (r == rank) continue;
+                        if (r < kParts)     ts_send<PC>(buf + rank * kFrom, bar, r, acc + (r < kParts ? r : 0) * PC);
+                        else if (lane == 0) ts_send<1>(buf + rank * kFrom, bar, r, acc);
+                    }
                     float own[PC], sum[PC];
 #pragma unroll
-                    for (int r = 0; r < CC; ++r)
+                    for (int r = 0; r < kParts; ++r)
                         if (r == rank) {
 #pragma unroll
                             for (int j = 0; j < PC; ++j) own[j] = acc[r * PC + j];
                         }
                     got = __all_sync(0xFFFFFFFFu, ts_wait_cluster(bar, (nsum >> 1) & 1, abort_flag));
+                    ++nsum;
+                    if (rank >= kParts) return;
 #pragma unroll
                     for (int r = 0; r < CC; ++r) {
                         float v[PC];
@@ -563,7 +578,6 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                     }
 #pragma unroll
                     for (int j = 0; j < PC; ++j) store(col0 + rank * PC + j, sum[j]);
-                    ++nsum;
                 };
                 if (nc == 1) {
 #pragma unroll
@@ -592,12 +606,14 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
 }
 
 // ---- host side -----------------------------------------------------------------------
+bool gemv_preferred(int M, int K, int group, int tiles, int count);
+
 bool tstream_supported(int M, int K, int group) {
     if (M < 1 || M > 64 || K % kBlockK != 0) return false;
     if ((long long)64 * 254 * group >= (1ll << 31)) return false;           // int32 accumulator range
     return group == 64 || group == 128 || group % 256 == 0;
 }
-static int ts_tokens(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : 64; }
+static int ts_tokens(int M) { return M <= 16 ? 16 : M <= 24 ? 24 : M <= 32 ? 32 : M <= 48 ? 48 : 64; }
 
 // Shares of K and clusters for a launch over `tiles` tiles of `KB` blocks: the least cost in blocks that one CTA works
 // off after the other.  A last round that not all clusters have counts 0.6 of a round (the CTAs left have the memory
@@ -624,14 +640,19 @@ static double ts_plan(int tiles, int KB, const int *resident, bool two_per_sm, i
 // kernel, groups of 64 | 128 | one scale per channel):
 //   16 tokens: 8192 x 8192 10.1 / 9.0 | 9.9 / 8.3 | 8.7 / 8.4; 4096 x (14336 + 14336) 13.2 / 12.7 | 12.5 / 11.6 | 11.7 / 11.0;
 //     28672 x 8192 21.9 / 21.9 | 21.4 / 19.5 | 19.9 / 17.8; but 8192 x 28672 20.3 / 23.1 | 19.7 / 20.5 | 18.8 / 18.5
+//   24 tokens: 8192 x 8192 11.8 / 10.9 | 11.1 / 9.8 | 10.8 / 9.0; 8192 x (28672 + 28672) 49.3 / 48.4 | 44.6 / 38.4 | 44.4 / 34.5
 //   32 tokens: 8192 x 8192 14.1 / 12.1 | 13.3 / 10.1 | 12.5 / 9.4; 8192 x (28672 + 28672) 62.7 / 59.2 | 57.9 / 41.2 | 55.4 / 36.8;
 //     28672 x 8192 40.8 / 30.2 | 37.8 / 22.6 | 36.4 / 19.5; 4096 x 14336 12.1 / 11.7 | 11.5 / 9.5 | 10.9 / 9.1
+//   48 tokens: 8192 x 8192 17.3 / 15.4 | 16.1 / 11.5 | 15.1 / 10.4; 28672 x 8192 80.4 / 42.2 | 71.8 / 29.8 | 68.3 / 24.9
 //   64 tokens: 4096 x 4096 10.0 / 8.8 | 10.7 / 7.3 | 9.7 / 7.3; 8192 x (28672 + 28672) 135 / 95 | 103 / 68 | 77 / 55;
 //     14336 x 4096 22.2 / 16.2 | 18.5 / 12.9 | 20.6 / 12.3
+// Rows of fewer than 4096 values that the persistent kernel does not hold in registers leave it at 9 to 16 tokens: 2560 x 3840 6.5 / 3.5 at
+// 12 and 7.6 / 3.5 at 16, 3072 x 12880 11.4 / 6.1 (128), 2560 x 1680 6.1 / 3.0.  Of 713 launches of random sets of
+// matrices (9 to 64 tokens) the rule moves 466 here, whose time falls by 1.47 on average; nine are slower by 2 to 10 %.
 // Small launches stay where they were (us, before / this kernel): at 32 tokens 4096 x 4096 5.7 / 6.6 | 5.7 / 5.4 | 5.0 / 5.4,
 // at 48 6.2 / 7.3 (128), 2048 x 2048 3.2 / 5.3; and so does everything of up to 8 tokens (4096 x (14336 + 14336) 9.4 / 11.2).
 // W2A8_TSTREAM = 0 never, 2 whenever it supports the shape; any switch that forces a plan of another kernel keeps it out.
-bool tstream_takes(int M, int K, int group, int tiles16, int count) {
+bool tstream_takes(int M, int K, int group, int tiles16, int count, bool h16) {
     if (!tstream_supported(M, K, group)) return false;
     const int mode = env_int("W2A8_TSTREAM", 1);
     if (mode == 0) return false;
@@ -640,7 +661,8 @@ bool tstream_takes(int M, int K, int group, int tiles16, int count) {
     const int KB = K / kBlockK, tiles = (tiles16 + 7) / 8, nt = ts_tokens(M), slabs = (M + 7) / 8;
     const long long blocks = (long long)tiles * KB;
     const long long least = M <= 32 ? (count > 1 && M > 24 ? 700 : 1536) : M <= 48 && count == 1 ? 1024 : 300;
-    if (blocks < least) return false;
+    const bool odd_row = M <= 16 && !h16 && KB < 16 && KB != 4 && KB != 8 && blocks >= 100;
+    if (blocks < least && !odd_row) return false;
     if (env_int("W2A8_STAT", 1) == 2 || env_int("W2A8_GEMV", 1) == 2) return false;
     for (const char *name : {"W2A8_STAT_C", "W2A8_CHUNKS", "W2A8_TG", "W2A8_RING", "W2A8_MT", "W2A8_CLUSTER",
                              "W2A8_MIN_WARPS", "W2A8_RELAX"})
@@ -648,18 +670,21 @@ bool tstream_takes(int M, int K, int group, int tiles16, int count) {
     if (M == 64)
         for (const char *name : {"W2A8_PREFILL", "W2A8_TC_KIND", "W2A8_PF_SPLIT", "W2A8_PF_KSPLIT", "W2A8_PF_WIDE"})
             if (env_set(name)) return false;
+    if (odd_row && gemv_preferred(M, K, group, tiles16, count)) return true;
+    if (blocks < least) return false;
     const int sms = sm_count(), spp = group == 64 ? 0 : group == 128 ? 1 : 2;
     int resident[kTsMaxCluster + 1] = {}, C, ncl;       // (what the device reports for a whole B200: 148, 74, 33, 15)
     for (int c = 1; c <= kTsMaxCluster; c *= 2) resident[c] = (int)(sms / c * (c == 4 ? 0.9 : c == 8 ? 0.84 : 1.0)) * (nt <= 32 ? 2 : 1);
     if (nt <= 32) resident[8] = resident[8] * 3 / 4;
-    static const double base[3][3] = {{1.3, 1.35, 1.9}, {2.0, 2.15, 2.85}, {3.4, 3.75, 4.3}};
-    static const double per_block[3][3] = {{0.64, 0.555, 0.5}, {0.92, 0.66, 0.55}, {0.84, 0.58, 0.47}};
-    const int w = nt == 16 ? 0 : nt == 32 ? 1 : 2;
+    static const double base[5][3] = {{1.5, 1.63, 2.36}, {2.63, 2.8, 3.34}, {2.8, 3.04, 3.88}, {3.77, 3.98, 4.56}, {4.24, 4.38, 5.24}};
+    static const double per_block[5][3] = {{0.636, 0.553, 0.479}, {0.764, 0.583, 0.494}, {0.848, 0.627, 0.507},
+                                           {0.714, 0.48, 0.409}, {0.798, 0.563, 0.432}};
+    const int w = nt == 16 ? 0 : nt == 24 ? 1 : nt == 32 ? 2 : nt == 48 ? 3 : 4;
     const double mine = base[w][spp] + per_block[w][spp] * ts_plan(tiles, KB, resident, nt <= 32, &C, &ncl);
     static const double per_cell[3] = {0.27e-3, 0.25e-3, 0.235e-3};
     // (more than 32 tokens: the other kernels take one matrix per launch)
     const double other = 4.6 * (M > 32 ? count : 1) + per_cell[spp] * (KB > 32 ? 1.1 : 1.0) * 4.0 * (double)blocks * slabs;
-    return mine < (M <= 16 && spp == 2 ? 0.86 : 0.96) * other;
+    return mine < (M <= 16 && spp == 2 ? 0.86 : 0.94) * other;
 }
 
 // Clusters of C CTAs that are resident at once, looked up once per device and instance.
@@ -714,7 +739,9 @@ template <bool H16>
 static cudaError_t launch_ts_nt(const TsMaps &maps, TsParams &p, int spp, cudaStream_t st) {
     switch (ts_tokens(p.M)) {
         case 16: return launch_ts_spp<16, H16>(maps, p, spp, st);
+        case 24: return launch_ts_spp<24, H16>(maps, p, spp, st);
         case 32: return launch_ts_spp<32, H16>(maps, p, spp, st);
+        case 48: return launch_ts_spp<48, H16>(maps, p, spp, st);
         default: return launch_ts_spp<64, H16>(maps, p, spp, st);
     }
 }
@@ -745,7 +772,7 @@ int launch_tstream(const int8_t *a, const float *a_scale, int count, const uint3
     {
         const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
         const cuuint64_t strides[1] = {(cuuint64_t)K};
-        const cuuint32_t box[2] = {128u, (cuuint32_t)ts_tokens(M)};
+        const cuuint32_t box[2] = {128u, (cuuint32_t)((ts_tokens(M) + 15) / 16 * 16)};
         if (encode(&maps.act, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t *>(a), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)

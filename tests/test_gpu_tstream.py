@@ -38,6 +38,7 @@ CASES = [
     (17, 1792, [640, 32], 64, 4),              # shares of 2 and 1 blocks
     (32, 1536, [384], 512, 4),                 # groups of two blocks cut between shares of 2, 2, 1, 1
     (31, 768, [128 * 150], 64, 1),             # more tiles than SMs
+    (20, 2048, [256], 128, 8),                 # three columns per rank and thread
     (24, 1024, [128 * 170], 128, 2),           # two tiles for some clusters: both exchange buffers
     (12, 512, [128 * 310], 64, 1),             # a second round
     (33, 2048, [1024], 64, 8),
