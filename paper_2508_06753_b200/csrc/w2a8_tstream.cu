@@ -479,7 +479,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
         int nsum = 0;                                   // tiles summed so far
         auto drain_unit = [&](int g0) {
             // (at most CG groups of staged values: more spill, and local memory is slow beside the copies)
-            constexpr int CG = DC > 16 ? 1 : UG;
+            constexpr int CG = DC == 32 ? 1 : UG;
             const uint32_t at = tlane + un * C::kUnitCols;
 #pragma unroll
             for (int c = 0; c < UG; c += CG) {
@@ -616,17 +616,17 @@ bool tstream_supported(int M, int K, int group) {
 static int ts_tokens(int M) { return M <= 16 ? 16 : M <= 24 ? 24 : M <= 32 ? 32 : M <= 48 ? 48 : 64; }
 
 // Shares of K and clusters for a launch over `tiles` tiles of `KB` blocks: the least cost in blocks that one CTA works
-// off after the other.  A last round that not all clusters have counts 0.6 of a round (the CTAs left have the memory
-// for themselves), a second CTA on the SMs costs 20 %, an exchange of sums as much as a block.  Against the best of all C over
-// 456 launches (13 sets of matrices, 4 to 64 tokens) the choice loses 1.5 % on average and 17 % at most.
+// off after the other.  A last round counts half of a round where a few clusters have it (they have the memory for
+// themselves) and a whole one from two thirds on, a second CTA on the SMs costs 20 %, an exchange of sums as much as a
+// block.  Against the best of all C over 440 launches (10 sets of matrices, 12 to 64 tokens) the choice loses 0.9 % on average and 13 % at most.
 static double ts_plan(int tiles, int KB, const int *resident, bool two_per_sm, int *C, int *nclusters) {
     const int forced = env_int("W2A8_TSTREAM_C", 0);
     double best = 1e30;
     for (int c = 1; c <= kTsMaxCluster; c *= 2) {
         if (c > KB || resident[c] < 1 || (forced > 0 && c != forced)) continue;
         const int ncl = std::min(tiles, resident[c]), rounds = (tiles + ncl - 1) / ncl, sms = sm_count();
-        const double whole = (double)tiles / ncl, share = (KB + c - 1) / c;
-        double cost = (whole + 0.6 * (rounds - whole)) * share;
+        const double left = (double)(tiles % ncl) / ncl, share = (KB + c - 1) / c;
+        double cost = (tiles / ncl + (left > 0 ? 0.5 + 0.5 * std::min(1.0, 1.5 * left) : 0.0)) * share;
         if (two_per_sm) cost *= 1.0 + 0.2 * std::min(1.0, std::max(0.0, (double)(ncl * c - sms) / sms));
         if (c > 1) cost += rounds;
         if (cost < best) { best = cost; *C = c; *nclusters = ncl; }
@@ -647,8 +647,8 @@ static double ts_plan(int tiles, int KB, const int *resident, bool two_per_sm, i
 //   64 tokens: 4096 x 4096 10.0 / 8.8 | 10.7 / 7.3 | 9.7 / 7.3; 8192 x (28672 + 28672) 135 / 95 | 103 / 68 | 77 / 55;
 //     14336 x 4096 22.2 / 16.2 | 18.5 / 12.9 | 20.6 / 12.3
 // Rows of fewer than 4096 values that the persistent kernel does not hold in registers leave it at 9 to 16 tokens: 2560 x 3840 6.5 / 3.5 at
-// 12 and 7.6 / 3.5 at 16, 3072 x 12880 11.4 / 6.1 (128), 2560 x 1680 6.1 / 3.0.  Of 713 launches of random sets of
-// matrices (9 to 64 tokens) the rule moves 466 here, whose time falls by 1.47 on average; nine are slower by 2 to 10 %.
+// 12 and 7.6 / 3.5 at 16, 3072 x 12880 11.4 / 6.1 (128), 2560 x 1680 6.1 / 3.0.  Of 757 launches of random sets of
+// matrices (9 to 64 tokens) the rule moves 521 here, whose time falls by 1.47 on average; eight are slower by 2 to 6 %.
 // Small launches stay where they were (us, before / this kernel): at 32 tokens 4096 x 4096 5.7 / 6.6 | 5.7 / 5.4 | 5.0 / 5.4,
 // at 48 6.2 / 7.3 (128), 2048 x 2048 3.2 / 5.3; and so does everything of up to 8 tokens (4096 x (14336 + 14336) 9.4 / 11.2).
 // W2A8_TSTREAM = 0 never, 2 whenever it supports the shape; any switch that forces a plan of another kernel keeps it out.
@@ -676,9 +676,16 @@ bool tstream_takes(int M, int K, int group, int tiles16, int count, bool h16) {
     int resident[kTsMaxCluster + 1] = {}, C, ncl;       // (what the device reports for a whole B200: 148, 74, 33, 15)
     for (int c = 1; c <= kTsMaxCluster; c *= 2) resident[c] = (int)(sms / c * (c == 4 ? 0.9 : c == 8 ? 0.84 : 1.0)) * (nt <= 32 ? 2 : 1);
     if (nt <= 32) resident[8] = resident[8] * 3 / 4;
-    static const double base[5][3] = {{1.5, 1.63, 2.36}, {2.63, 2.8, 3.34}, {2.8, 3.04, 3.88}, {3.77, 3.98, 4.56}, {4.24, 4.38, 5.24}};
-    static const double per_block[5][3] = {{0.636, 0.553, 0.479}, {0.764, 0.583, 0.494}, {0.848, 0.627, 0.507},
-                                           {0.714, 0.48, 0.409}, {0.798, 0.563, 0.432}};
+    static const double base[5][3] = {{1.82, 1.95, 2.59},
+                                      {3.06, 3.11, 3.56},
+                                      {3.21, 3.44, 4.14},
+                                      {3.82, 4.01, 4.58},
+                                      {4.3, 4.43, 5.26}};
+    static const double per_block[5][3] = {{0.592, 0.516, 0.453},
+                                           {0.707, 0.547, 0.474},
+                                           {0.795, 0.59, 0.486},
+                                           {0.705, 0.474, 0.404},
+                                           {0.789, 0.556, 0.427}};
     const int w = nt == 16 ? 0 : nt == 24 ? 1 : nt == 32 ? 2 : nt == 48 ? 3 : 4;
     const double mine = base[w][spp] + per_block[w][spp] * ts_plan(tiles, KB, resident, nt <= 32, &C, &ncl);
     static const double per_cell[3] = {0.27e-3, 0.25e-3, 0.235e-3};
