@@ -14,10 +14,11 @@
 //    computes while the other waits or, under programmatic dependent launch, while the previous kernel ends; with 64
 //    tokens one CTA of 20 warps has them all.  Registers are dealt by setmaxnreg so that nothing spills: a few spilled
 //    words per block (local memory beside the copies) made 8192 x (28672 + 28672) at 32 tokens 94 us instead of 54.
-//  * Bound (8192 x (28672 + 28672), groups of 128, 32 tokens, 41 us, 3.2 TB/s): issue slots, 68 % busy: about 450 warp
+//  * Bound (8192 x (28672 + 28672), groups of 128, 32 tokens, 42 us, 3.1 TB/s): issue slots, 68 % busy: about 450 warp
 //    instructions of unpack per block, 800 of drain, the rest waits.  On the kernel with stationary activations
 //    (mma.sync) the same launch takes 58 us.  Not kept: conversion through the bits of 1.5 * 2^23, by integer adds (50 us);
-//    eight drain warps at 32 tokens (45); blocks dealt evenly over CTAs with cut tiles summed through global
+//    eight drain warps at 32 tokens (45); a running sum that takes every group by itself (2 to 6 % faster, but up to 20 %
+//    further from sums in 64 bits than the other kernels, with the groups of a unit added up first it is level with them); blocks dealt evenly over CTAs with cut tiles summed through global
 //    memory (3 us more per small launch).
 //  * A wait is one barrier per warp: lanes of a warp that polled different barriers saw phases that had not completed.
 //  * Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
@@ -126,6 +127,15 @@ __device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[24]) {
     ts_tmem_ld(taddr + 16, reinterpret_cast<int (&)[8]>(v[16]));
 }
 __device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[32]) { pf_tmem_ld32(taddr, v); }
+// packed fp32: (t0, t1) = (x0, x1) * sc; (a0, a1) += (t0, t1)
+__device__ __forceinline__ void ts_mul2(float &t0, float &t1, float x0, float x1, float sc) {
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\tmul.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "=f"(t0), "=f"(t1) : "f"(x0), "f"(x1), "f"(sc));
+}
+__device__ __forceinline__ void ts_add2(float &a0, float &a1, float t0, float t1) {
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1) : "f"(t0), "f"(t1));
+}
 template <int N>
 __device__ __forceinline__ void ts_maxreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N>
@@ -478,27 +488,36 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
         [[maybe_unused]] int gleft = first_left;
         int nsum = 0;                                   // tiles summed so far
         auto drain_unit = [&](int g0) {
-            // (at most CG groups of staged values: more spill, and local memory is slow beside the copies)
-            constexpr int CG = DC == 32 ? 1 : UG;
+            // All groups of the unit for CH columns at a time (more staged values spill, and local memory is slow beside
+            // the copies).  The groups are added up before they join the running sum: one addition more for two or four
+            // groups, and the running sum, whose rounding is the larger, takes half or a quarter of the terms.
+            constexpr int CH = DC == 32 && UG > 1 ? 16 : DC;
             const uint32_t at = tlane + un * C::kUnitCols;
 #pragma unroll
-            for (int c = 0; c < UG; c += CG) {
-                int v[CG][DC];
+            for (int c = 0; c < DC; c += CH) {
+                int v[UG][CH];
 #pragma unroll
-                for (int g = 0; g < CG; ++g) ts_tmem_ld(at + (c + g) * BN, v[g]);
+                for (int g = 0; g < UG; ++g) ts_tmem_ld(at + g * BN + c, v[g]);
                 pf_tmem_ld_wait();
-                if (c + CG == UG) {
+                if (c + CH == DC) {
                     pf_tc_fence_before();
                     __syncwarp();
                     if (lane == 0) pf_mbar_arrive(pf_smem_u32(C::kFold ? &bar_a[un] : &bar_free[un]));
                     if (++un == NU) { un = 0; uph ^= 1u; }
                 }
+                float f[UG];
 #pragma unroll
-                for (int g = 0; g < CG; ++g) {
-                    const float f = scale(sc_cur, g0 + c + g);
+                for (int g = 0; g < UG; ++g) f[g] = scale(sc_cur, g0 + g);
 #pragma unroll
-                    for (int j = 0; j < DC; j += 2) {
-                        pf_fma2(acc[j], acc[j + 1], (float)v[g][j], (float)v[g][j + 1], f);
+                for (int j = 0; j < CH; j += 2) {
+                    if constexpr (UG == 1) {
+                        pf_fma2(acc[j], acc[j + 1], (float)v[0][j], (float)v[0][j + 1], f[0]);
+                    } else {
+                        float t0 = 0.f, t1 = 0.f;
+                        ts_mul2(t0, t1, (float)v[0][j], (float)v[0][j + 1], f[0]);
+#pragma unroll
+                        for (int g = 1; g < UG; ++g) pf_fma2(t0, t1, (float)v[g][j], (float)v[g][j + 1], f[g]);
+                        ts_add2(acc[c + j], acc[c + j + 1], t0, t1);
                     }
                 }
             }
@@ -648,7 +667,7 @@ static double ts_plan(int tiles, int KB, const int *resident, bool two_per_sm, i
 //     14336 x 4096 22.2 / 16.2 | 18.5 / 12.9 | 20.6 / 12.3
 // Rows of fewer than 4096 values that the persistent kernel does not hold in registers leave it at 9 to 16 tokens: 2560 x 3840 6.5 / 3.5 at
 // 12 and 7.6 / 3.5 at 16, 3072 x 12880 11.4 / 6.1 (128), 2560 x 1680 6.1 / 3.0.  Of 757 launches of random sets of
-// matrices (9 to 64 tokens) the rule moves 521 here, whose time falls by 1.47 on average; eight are slower by 2 to 6 %.
+// matrices (9 to 64 tokens) the rule moved 521 here, whose time fell by 1.47 on average; eight were slower by 2 to 6 %.
 // Small launches stay where they were (us, before / this kernel): at 32 tokens 4096 x 4096 5.7 / 6.6 | 5.7 / 5.4 | 5.0 / 5.4,
 // at 48 6.2 / 7.3 (128), 2048 x 2048 3.2 / 5.3; and so does everything of up to 8 tokens (4096 x (14336 + 14336) 9.4 / 11.2).
 // W2A8_TSTREAM = 0 never, 2 whenever it supports the shape; any switch that forces a plan of another kernel keeps it out.
@@ -681,17 +700,17 @@ bool tstream_takes(int M, int K, int group, int tiles16, int count, bool h16) {
                                       {3.21, 3.44, 4.14},
                                       {3.82, 4.01, 4.58},
                                       {4.3, 4.43, 5.26}};
-    static const double per_block[5][3] = {{0.592, 0.516, 0.453},
-                                           {0.707, 0.547, 0.474},
-                                           {0.795, 0.59, 0.486},
-                                           {0.705, 0.474, 0.404},
-                                           {0.789, 0.556, 0.427}};
+    static const double per_block[5][3] = {{0.616, 0.534, 0.453},
+                                           {0.735, 0.566, 0.474},
+                                           {0.827, 0.611, 0.486},
+                                           {0.733, 0.491, 0.404},
+                                           {0.821, 0.575, 0.427}};
     const int w = nt == 16 ? 0 : nt == 24 ? 1 : nt == 32 ? 2 : nt == 48 ? 3 : 4;
     const double mine = base[w][spp] + per_block[w][spp] * ts_plan(tiles, KB, resident, nt <= 32, &C, &ncl);
     static const double per_cell[3] = {0.27e-3, 0.25e-3, 0.235e-3};
     // (more than 32 tokens: the other kernels take one matrix per launch)
     const double other = 4.6 * (M > 32 ? count : 1) + per_cell[spp] * (KB > 32 ? 1.1 : 1.0) * 4.0 * (double)blocks * slabs;
-    return mine < (M <= 16 && spp == 2 ? 0.86 : 0.94) * other;
+    return mine < (M <= 16 && spp == 2 ? 0.86 : 0.92) * other;
 }
 
 // Clusters of C CTAs that are resident at once, looked up once per device and instance.
