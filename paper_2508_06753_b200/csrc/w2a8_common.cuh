@@ -7,6 +7,7 @@
 #include <atomic>
 
 #include "w2a8.h"
+#include "w2a8_table.h"
 
 namespace w2a8 {
 
@@ -212,7 +213,6 @@ int check_device();  // W2A8_OK or W2A8_ERR_ARCH / W2A8_ERR_CUDA
 // One process may drive several GPUs, and function attributes, the SM count and
 // the architecture check belong to a device, not to the process: everything that
 // is looked up once is kept per device ordinal.
-constexpr int kMaxDevices = 64;
 int current_device();   // ordinal of the current device, or -1
 int sm_count();         // multiprocessors of the current device (148 on B200), >= 1
 
@@ -230,6 +230,26 @@ inline cudaError_t allow_dynamic_smem(void (*kernel)(KArgs...), PerDeviceFlags &
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) flags.done[dev].store(true, std::memory_order_release);
     return e;
+}
+
+// Clusters of C CTAs of `kernel` that the current device holds at once (one CTA per SM), 0 if it cannot say.
+template <typename... KArgs>
+inline int resident_clusters(void (*kernel)(KArgs...), int C, int threads, size_t smem) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
 }
 
 }  // namespace w2a8

@@ -499,30 +499,6 @@ bool stat_takes(int M, int K, int group, int tiles, int count, bool h16) {
     return mine < 0.95 * many_token_seconds(M, tiles * 16, K, group);
 }
 
-// Clusters of C CTAs that are resident at once (clusters are placed inside one GPC, so the count is not
-// slots / C: 74, 45, 33, 26, 22, 15 for C = 2, 3, 4, 5, 6, 8).
-// A larger grid would run a second wave of a few clusters.  Looked up once per device and instance.
-struct StClusters { std::atomic<int> known; int n[kStMaxCluster + 1]; };
-
-template <typename K>
-static int stat_clusters(K kernel, int C, size_t smem, int fallback) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(kStWarps * 32);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
-        cudaGetLastError();
-        return fallback;
-    }
-    return n;
-}
-
 struct StPlan { int C, round_pairs, nclusters; size_t smem; };
 
 // The plan: C, pairs per round.  One cell of one warp is the unit of cost.  (C = 2 is ahead of 4 at equal
@@ -565,14 +541,17 @@ static cudaError_t launch_stat_inst(StParams &p, cudaStream_t st) {
     constexpr size_t budget = kStBudget;
     static PerDeviceFlags configured;   // per kernel instantiation
     if (cudaError_t e = allow_dynamic_smem(kernel, configured, (int)budget)) return e;
-    static StClusters clusters[kMaxDevices];
-    StClusters &cs = clusters[current_device()];
-    if (!cs.known.load(std::memory_order_acquire)) {      // racing threads write the same values
-        for (int C = 1; C <= kStMaxCluster; ++C) cs.n[C] = stat_clusters(kernel, C, budget, sm_count() / C);
-        cs.known.store(1, std::memory_order_release);
-    }
+    // Clusters of C CTAs that are resident at once (clusters are placed inside one GPC, so the count is not
+    // slots / C: 74, 45, 33, 26, 22, 15 for C = 2, 3, 4, 5, 6, 8).  A larger grid would run a second wave of a few clusters.
+    static PerDeviceTable<kStMaxCluster + 1> clusters;
+    const int *resident = clusters.get(current_device(), [&](int *n) {
+        for (int C = 1; C <= kStMaxCluster; ++C) {
+            const int found = resident_clusters(kernel, C, kStWarps * 32, budget);
+            n[C] = found > 0 ? found : sm_count() / C;
+        }
+    });
     StPlan pl;
-    if (!stat_plan(p.M, p.K, p.pairs, cs.n, &pl)) return cudaErrorNotSupported;
+    if (!stat_plan(p.M, p.K, p.pairs, resident, &pl)) return cudaErrorNotSupported;
     p.C = pl.C; p.round_pairs = pl.round_pairs;
     p.blk_per = p.blocks / pl.C; p.blk_extra = p.blocks % pl.C;
     for (int i = 0; i < 2; ++i) p.nb_inv[i] = (65536 + p.blk_per + i - 1) / (p.blk_per + i);

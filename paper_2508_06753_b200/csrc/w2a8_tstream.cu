@@ -713,28 +713,6 @@ bool tstream_takes(int M, int K, int group, int tiles16, int count, bool h16) {
     return mine < (M <= 16 && spp == 2 ? 0.86 : 0.92) * other;
 }
 
-// Clusters of C CTAs that are resident at once, looked up once per device and instance.
-struct TsClusters { std::atomic<int> known; int n[kTsMaxCluster + 1]; };
-
-template <typename K>
-static int ts_resident(K kernel, int C, int threads, size_t smem) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
-        cudaGetLastError();
-        return 0;
-    }
-    return n;
-}
-
 template <int NT, int SPP, bool H16>
 static cudaError_t launch_ts_inst(const TsMaps &maps, TsParams &p, cudaStream_t st) {
     using C = TsCfg<NT, SPP>;
@@ -742,16 +720,16 @@ static cudaError_t launch_ts_inst(const TsMaps &maps, TsParams &p, cudaStream_t 
     static PerDeviceFlags configured;   // per kernel instantiation
     if (cudaError_t e = allow_dynamic_smem(kernel, configured, (int)C::kSmem)) return e;
     if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) return e;
-    static TsClusters clusters[kMaxDevices];
-    TsClusters &cs = clusters[current_device()];
-    if (!cs.known.load(std::memory_order_acquire)) {      // racing threads write the same values
-        // The query answers for one CTA per SM; with 256 columns of tensor memory, 112 KB and half of the registers two
-        // are resident (clusters of eight: about three quarters of that).
-        for (int c = 1; c <= kTsMaxCluster; c *= 2) cs.n[c] = C::kCtasPerSm * ts_resident(kernel, c, C::kThreads, C::kSmem);
-        if (C::kCtasPerSm == 2 && cs.n[8] > 1) cs.n[8] = cs.n[8] * 3 / 4;
-        cs.known.store(1, std::memory_order_release);
-    }
-    if (ts_plan(p.tiles, p.KB, cs.n, C::kCtasPerSm == 2, &p.C, &p.nclusters) > 1e29) return cudaErrorNotSupported;
+    // Clusters of C CTAs that are resident at once.  The query answers for one CTA per SM; with 256 columns of tensor
+    // memory, 112 KB and half of the registers two are resident (clusters of eight: about three quarters of that).
+    static PerDeviceTable<kTsMaxCluster + 1> clusters;
+    const int *resident = clusters.get(current_device(), [&](int *n) {
+        for (int c = 1; c <= kTsMaxCluster; c *= 2) {
+            const int found = C::kCtasPerSm * resident_clusters(kernel, c, C::kThreads, C::kSmem);
+            n[c] = C::kCtasPerSm == 2 && c == 8 && found > 1 ? found * 3 / 4 : found;
+        }
+    });
+    if (ts_plan(p.tiles, p.KB, resident, C::kCtasPerSm == 2, &p.C, &p.nclusters) > 1e29) return cudaErrorNotSupported;
     p.blk_per = p.KB / p.C; p.blk_extra = p.KB % p.C;
     return launch_kernel_clusters(kernel, dim3((unsigned)(p.nclusters * p.C)), dim3(C::kThreads), C::kSmem, st, pdl_enabled(),
                                   make_uint2((unsigned)p.C, 1u), maps, p);
