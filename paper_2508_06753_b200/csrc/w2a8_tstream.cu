@@ -12,14 +12,19 @@
 //    eight warps drain the accumulators (lane = channel, column = token): a conversion and half a packed FMA per value.
 //  * Up to 32 tokens a CTA has 12 warps, 112 KB and 256 columns of tensor memory, so that two are resident per SM and one
 //    computes while the other waits or, under programmatic dependent launch, while the previous kernel ends; with 64
-//    tokens one CTA of 20 warps has them all.  Registers are dealt by setmaxnreg so that nothing spills: a few spilled
-//    words per block (local memory beside the copies) made 8192 x (28672 + 28672) at 32 tokens 94 us instead of 54.
-//  * Bound (8192 x (28672 + 28672), groups of 128, 32 tokens, 42 us, 3.1 TB/s): issue slots, 68 % busy: about 450 warp
-//    instructions of unpack per block, 800 of drain, the rest waits.  On the kernel with stationary activations
-//    (mma.sync) the same launch takes 58 us.  Not kept: conversion through the bits of 1.5 * 2^23, by integer adds (50 us);
-//    eight drain warps at 32 tokens (45); a running sum that takes every group by itself (2 to 6 % faster, but up to 20 %
-//    further from sums in 64 bits than the other kernels, with the groups of a unit added up first it is level with them); blocks dealt evenly over CTAs with cut tiles summed through global
-//    memory (3 us more per small launch).
+//    tokens one CTA of 20 warps has them all.  Registers are dealt by setmaxnreg so that hardly anything spills (28 bytes
+//    at most, in instances for 64 tokens; a few
+//    words per block, local memory beside the copies, made 8192 x (28672 + 28672) at 32 tokens 94 us instead of 54).
+//  * Sums.  Chains of eight groups by FMA; a chain joins the running sum with what that addition rounds away going into
+//    the next chain, and the ranks' shares are added in the same way: the error does not depend on the length of a row.
+//    Distance from sums in 64 bits, one running total / this: 4096 x (14336 + 14336) at 64 tokens, groups of 64, one share
+//    9.5e-8 / 4.6e-8; 28672 x 8192, groups of 64, four shares 7.5e-8 / 4.0e-8; 8192 x 8192, groups of 128, four shares
+//    5.5e-8 / 4.6e-8.  The other kernels are at 5.1e-8 and more at these sizes.
+//  * Bound (8192 x (28672 + 28672), groups of 128, 32 tokens): issue slots: per block of 8 KB unpack, drain (a conversion and
+//    half a packed FMA per value and group), and waits and bookkeeping.  On the kernel with stationary activations
+//    (mma.sync) the same launch takes 58 us.  Not kept: conversion through the bits of 1.5 * 2^23, by integer adds (50 us
+//    against 44); eight drain warps at 32 tokens (45); unpack warps with 64 registers (4 to 19 % more per launch); blocks dealt
+//    evenly over CTAs with cut tiles summed through global memory (3 us more per small launch).
 //  * A wait is one barrier per warp: lanes of a warp that polled different barriers saw phases that had not completed.
 //  * Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
 #include <cuda.h>
@@ -80,6 +85,11 @@ struct TsCfg {
     static constexpr int UG = SPP == 0 ? 1 : GPB * BN <= 64 ? GPB : 2;   // groups of a unit = hand-off between MMA and drain
     static constexpr int UPB = GPB / UG;                          // units of a block
     static constexpr int kUnitCols = UG * BN;
+    // A chain of additions is kChain blocks (groups of whole blocks: groups), eight groups, long.  The running sums of the
+    // second half of a thread's columns are in shared memory where the registers do not hold them.
+    static constexpr int kChain = SPP == 0 ? 8 : 8 / GPB;
+    static constexpr int kHiShared = DC > 16 ? DC / 2 : 0;
+    static constexpr int kHiBytes = kHiShared * 4 * 32 * kDrainWarps;
     static constexpr int kUnits = kAccCols / kUnitCols;
     // One barrier says that a block is unpacked and its accumulators are free, where both come round alike.
     static constexpr bool kFold = SPP != 0 && UPB == 1 && kUnits >= AS;
@@ -87,8 +97,13 @@ struct TsCfg {
     static constexpr int kStageBytes = kTsWBytes + BN * 256;
     static constexpr int kSumBytes = kTsBM * (DC == 24 ? 32 : DC) * kDrainWarps;     // a tile's sums, in pieces of 16 bytes
     static constexpr int kRing = ((kCtasPerSm == 2 ? 112 : 224) * 1024 - 2048 - 2 * kSumBytes) / kStageBytes;
-    static constexpr size_t kSmem = (size_t)kRing * kStageBytes + 2 * kSumBytes + 1024;
+    static constexpr size_t kSmem = (size_t)kRing * kStageBytes + 2 * kSumBytes + kHiBytes + 1024;
     static constexpr bool kUnitBarrier = SPP == 0 || UPB > 1;     // else a block's barrier says it all
+    // Registers per thread: the launch has 80 or 96 (what the launch bounds leave, rounded down to a multiple of eight, and
+    // what the compiler reports for every instance); setmaxnreg moves some of the first warps' to the drain warps.
+    static constexpr int kRegs = NT <= 32 ? 80 : 96, kRegsFirst = NT <= 32 ? 24 : 32, kRegsDrain = NT <= 32 ? 136 : 128;
+    static_assert(kFirstUnpack * (kRegs - kRegsFirst) >= kDrainWarps * (kRegsDrain - kRegs), "");
+    static_assert(kSmem + 1024 <= (kCtasPerSm == 2 ? 113 : 227) * 1024, "");
     static_assert(NU >= 2 && AS < kRing, "");
 };
 
@@ -127,14 +142,19 @@ __device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[24]) {
     ts_tmem_ld(taddr + 16, reinterpret_cast<int (&)[8]>(v[16]));
 }
 __device__ __forceinline__ void ts_tmem_ld(uint32_t taddr, int (&v)[32]) { pf_tmem_ld32(taddr, v); }
-// packed fp32: (t0, t1) = (x0, x1) * sc; (a0, a1) += (t0, t1)
-__device__ __forceinline__ void ts_mul2(float &t0, float &t1, float x0, float x1, float sc) {
-    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\tmul.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
-        : "=f"(t0), "=f"(t1) : "f"(x0), "f"(x1), "f"(sc));
+// Joins two chains (a0, a1) with the running sums (h0, h1), packed fp32.  What the addition rounds away stays behind in
+// the chains and goes into the next join.
+__device__ __forceinline__ void ts_join2(float &h0, float &h1, float &a0, float &a1) {
+    asm("{\n\t.reg .b64 h, a, s, z, m;\n\t"
+        "mov.b64 h, {%0, %1};\n\tmov.b64 a, {%2, %3};\n\tmov.b64 m, {%4, %4};\n\t"
+        "add.rn.f32x2 s, h, a;\n\t"
+        "fma.rn.f32x2 z, h, m, s;\n\t"        // s - h: the part of the chain that the sum took
+        "fma.rn.f32x2 a, z, m, a;\n\t"        // the rest
+        "mov.b64 {%0, %1}, s;\n\tmov.b64 {%2, %3}, a;\n\t}"
+        : "+f"(h0), "+f"(h1), "+f"(a0), "+f"(a1) : "f"(-1.f));
 }
-__device__ __forceinline__ void ts_add2(float &a0, float &a1, float t0, float t1) {
-    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
-        : "+f"(a0), "+f"(a1) : "f"(t0), "f"(t1));
+__device__ __forceinline__ void ts_st_shared2(uint32_t addr, float x, float y) {
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x), "f"(y) : "memory");
 }
 template <int N>
 __device__ __forceinline__ void ts_maxreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
@@ -259,7 +279,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
     pdl_launch_dependents();
 
     if (warp < C::kFirstUnpack) {
-        if constexpr (NT <= 32) ts_maxreg_dec<40>(); else ts_maxreg_dec<32>();
+        ts_maxreg_dec<C::kRegsFirst>();
         if (warp == 0 && lane == 0) {
             // ===== TMA producer =============================================================
             int tile = cl, kb = 0, n0;
@@ -424,8 +444,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             if (ds >= R) { ds -= R; dph ^= 1u; }
         }
     } else {
-        if constexpr (NT <= 32) ts_maxreg_inc<120>();
-        else ts_maxreg_inc<128>();
+        ts_maxreg_inc<C::kRegsDrain>();
         // ===== drain warps ==============================================================
         const int q = warp & 3, d = warp - C::kFirstDrain, col0 = (d >> 2) * DC;
         const uint32_t tlane = tmem_acc + ((uint32_t)(q * 32) << 16) + col0;
@@ -446,6 +465,9 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                    (SPP == 0 ? 0 : kb_lo * C::GPB * (H16 ? 2 : 4));
         };
         locate(ptile);
+        // (groups of whole blocks) group of the block that is requested next, blocks left of it
+        const int gi0 = SPP == 0 ? kb_lo / p.bpg : 0, first_left = (gi0 + 1) * p.bpg - kb_lo;
+        int pgi = gi0, pleft = first_left;
         constexpr int kStep = SPP == 0 ? 0 : C::GPB * (H16 ? 2 : 4);      // scale bytes of a block
         auto request = [&]() -> Scales {
             Scales sc = {};
@@ -458,12 +480,15 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             } else if constexpr (kStep == 4) {
                 sc.r[0] = __ldg(reinterpret_cast<const uint32_t *>(srow));
             } else {
-                const int gi = (kb_lo + pkb) / p.bpg;
-                if constexpr (H16) sc.r[0] = __ldg(reinterpret_cast<const unsigned short *>(srow) + gi);
-                else sc.r[0] = __ldg(reinterpret_cast<const uint32_t *>(srow) + gi);
+                if constexpr (H16) sc.r[0] = __ldg(reinterpret_cast<const unsigned short *>(srow) + pgi);
+                else sc.r[0] = __ldg(reinterpret_cast<const uint32_t *>(srow) + pgi);
+                if (--pleft == 0) { ++pgi; pleft = p.bpg; }
             }
             srow += kStep;
-            if (++pkb == nb) { pkb = 0; ptile += p.nclusters; if (left > 0) locate(ptile); }
+            if (++pkb == nb) {
+                pkb = 0; ptile += p.nclusters; pgi = gi0; pleft = first_left;
+                if (left > 0) locate(ptile);
+            }
             return sc;
         };
         auto scale = [&](const Scales &sc, int g) -> float {       // g is a constant after unrolling
@@ -478,20 +503,31 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
         if (warp == C::kFirstDrain)
             for (int j = lane; j < NT; j += 32) tok_scale[j] = p.a_scale[min(j, p.M - 1)] * (1.0f / kCodeGain);
         asm volatile("bar.sync 1, %0;" ::"n"(32 * C::kDrainWarps) : "memory");
-        float acc[DC];
+        constexpr int HS = C::kHiShared, HR = DC - HS;
+        float acc[DC], hi[HR];                          // chains, running sums (the last HS columns': hi_s, in pairs)
+        const uint32_t hi_s = sums0 + 2 * C::kSumBytes + (d * 32 + lane) * 8;
+        constexpr uint32_t kHiStep = C::kDrainWarps * 32 * 8;
+        int s = 0, un = 0, chain;
+        float largest;                                  // scale of this tile's row so far
+        auto clear = [&]() {
 #pragma unroll
-        for (int j = 0; j < DC; ++j) acc[j] = 0.f;
-        int s = 0, un = 0;
+            for (int j = 0; j < DC; ++j) acc[j] = 0.f;
+#pragma unroll
+            for (int j = 0; j < HR; ++j) hi[j] = 0.f;
+#pragma unroll
+            for (int j = 0; j < HS; j += 2) ts_st_shared2(hi_s + j / 2 * kHiStep, 0.f, 0.f);
+            chain = 0;
+            largest = 0.f;
+        };
+        clear();
         uint32_t ph = 0, uph = 0;
         bool got = true;
-        const int first_left = SPP == 0 ? p.bpg - kb_lo % p.bpg : 0;
         [[maybe_unused]] int gleft = first_left;
         int nsum = 0;                                   // tiles summed so far
         auto drain_unit = [&](int g0) {
             // All groups of the unit for CH columns at a time (more staged values spill, and local memory is slow beside
-            // the copies).  The groups are added up before they join the running sum: one addition more for two or four
-            // groups, and the running sum, whose rounding is the larger, takes half or a quarter of the terms.
-            constexpr int CH = DC == 32 && UG > 1 ? 16 : DC;
+            // the copies).
+            constexpr int CH = UG == 4 ? 8 : DC == 32 ? 16 : DC;
             const uint32_t at = tlane + un * C::kUnitCols;
 #pragma unroll
             for (int c = 0; c < DC; c += CH) {
@@ -507,19 +543,32 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                 }
                 float f[UG];
 #pragma unroll
-                for (int g = 0; g < UG; ++g) f[g] = scale(sc_cur, g0 + g);
-#pragma unroll
-                for (int j = 0; j < CH; j += 2) {
-                    if constexpr (UG == 1) {
-                        pf_fma2(acc[j], acc[j + 1], (float)v[0][j], (float)v[0][j + 1], f[0]);
-                    } else {
-                        float t0 = 0.f, t1 = 0.f;
-                        ts_mul2(t0, t1, (float)v[0][j], (float)v[0][j + 1], f[0]);
-#pragma unroll
-                        for (int g = 1; g < UG; ++g) pf_fma2(t0, t1, (float)v[g][j], (float)v[g][j + 1], f[g]);
-                        ts_add2(acc[c + j], acc[c + j + 1], t0, t1);
-                    }
+                for (int g = 0; g < UG; ++g) {
+                    f[g] = scale(sc_cur, g0 + g);
+                    if (c == 0) largest = fmaxf(largest, fabsf(f[g]));
                 }
+#pragma unroll
+                for (int g = 0; g < UG; ++g)
+#pragma unroll
+                    for (int j = 0; j < CH; j += 2) pf_fma2(acc[c + j], acc[c + j + 1], (float)v[g][j], (float)v[g][j + 1], f[g]);
+            }
+        };
+        auto join = [&]() {
+            chain = 0;
+#pragma unroll
+            for (int j = 0; j < HR; j += 2) ts_join2(hi[j], hi[j + 1], acc[j], acc[j + 1]);
+#pragma unroll
+            for (int j = 0; j < HS; j += 2) {
+                float h[2];
+                ts_ld_shared<2>(h, hi_s + j / 2 * kHiStep);
+                ts_join2(h[0], h[1], acc[HR + j], acc[HR + j + 1]);
+                ts_st_shared2(hi_s + j / 2 * kHiStep, h[0], h[1]);
+            }
+            // A row's integers add up to less than 2^31.  Sums that may be infinite are plain ones: an infinity minus itself is
+            // not what an addition left over.  (A vote in front of the branch cost 4 % of a launch at 16 tokens.)
+            if (largest >= 0x1p96f) {
+#pragma unroll
+                for (int j = 0; j < DC; ++j) acc[j] = 0.f;
             }
         };
         for (int i = 0; i < n; ++i) {
@@ -533,16 +582,27 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                     pf_tc_fence_after();
                     drain_unit(u * UG);
                 }
+                if (++chain == C::kChain) join();
             } else if (--gleft == 0 || row_end) {
                 gleft = row_end ? first_left : p.bpg;
                 got = ts_wait(pf_smem_u32(&bar_full[un]), uph, abort_flag);
                 pf_tc_fence_after();
                 drain_unit(0);
+                if (++chain == C::kChain) join();
             }
             if (++s == R) { s = 0; ph ^= 1u; }
             if (!got) break;
             if (row_end) {
                 // ---- this CTA's share of the tile's sums is complete ---------------------------
+#pragma unroll
+                for (int j = 0; j < HR; ++j) acc[j] += hi[j];
+#pragma unroll
+                for (int j = 0; j < HS; j += 2) {
+                    float h[2];
+                    ts_ld_shared<2>(h, hi_s + j / 2 * kHiStep);
+                    acc[HR + j] += h[0];
+                    acc[HR + j + 1] += h[1];
+                }
                 int n0;
                 const int mi = mat_of(tile, n0);
                 const int ch = n0 + q * 32 + lane;
@@ -575,28 +635,26 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                         if (r < kParts)     ts_send<PC>(buf + rank * kFrom, bar, r, acc + (r < kParts ? r : 0) * PC);
                         else if (lane == 0) ts_send<1>(buf + rank * kFrom, bar, r, acc);
                     }
-                    float own[PC], sum[PC];
-#pragma unroll
-                    for (int r = 0; r < kParts; ++r)
-                        if (r == rank) {
-#pragma unroll
-                            for (int j = 0; j < PC; ++j) own[j] = acc[r * PC + j];
-                        }
                     got = __all_sync(0xFFFFFFFFu, ts_wait_cluster(bar, (nsum >> 1) & 1, abort_flag));
                     ++nsum;
                     if (rank >= kParts) return;
+                    float sum[PC], rest[PC];
 #pragma unroll
                     for (int r = 0; r < CC; ++r) {
                         float v[PC];
                         ts_ld_shared<PC>(v, buf + r * kFrom);
 #pragma unroll
                         for (int j = 0; j < PC; ++j) {
-                            const float x = r == rank ? own[j] : v[j];
-                            sum[j] = r == 0 ? x : sum[j] + x;
+                            const float x = r < kParts && r == rank ? acc[(r < kParts ? r : 0) * PC + j] : v[j];
+                            if (r == 0) { sum[j] = x; rest[j] = 0.f; continue; }
+                            const float s2 = sum[j] + x, took = s2 - sum[j];      // exact sum = s2 + what is left of both terms
+                            rest[j] += (sum[j] - (s2 - took)) + (x - took);
+                            sum[j] = s2;
                         }
                     }
 #pragma unroll
-                    for (int j = 0; j < PC; ++j) store(col0 + rank * PC + j, sum[j]);
+                    for (int j = 0; j < PC; ++j)          // (an infinite sum has no rest)
+                        store(col0 + rank * PC + j, rest[j] == rest[j] ? sum[j] + rest[j] : sum[j]);
                 };
                 if (nc == 1) {
 #pragma unroll
@@ -604,8 +662,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                 } else if (nc == 2) exchange(std::integral_constant<int, 2>{});
                 else if (nc == 4)   exchange(std::integral_constant<int, 4>{});
                 else                exchange(std::integral_constant<int, 8>{});
-#pragma unroll
-                for (int j = 0; j < DC; ++j) acc[j] = 0.f;
+                clear();
             }
             if (++kb == nb) { kb = 0; tile += p.nclusters; }
         }

@@ -47,6 +47,10 @@ CASES = [
     (64, 512, [128 * 160], 128, 2),
     (50, 3072, [144], 1024, 8),
     (5, 14336, [256], 64, 8),
+    (48, 2048, [384, 16], 128, 2),
+    (24, 1024, [272], 0, 4),
+    (23, 3072, [256, 144], 1024, 2),
+    (32, 2048, [256], 128, 4),
 ]
 
 
@@ -162,3 +166,60 @@ def test_behind_a_long_kernel(gpu, monkeypatch):
     torch.cuda.synchronize()
     assert b.w2a8_workspace_status(ws) == 0
     assert torch.equal(y, alone)
+
+
+# One running total over the groups of these rows was up to 2.2 times as far from 64-bit sums as the kernels that had
+# such launches before.
+@pytest.mark.parametrize("M,K,N,group,shares", [
+    (16, 10240, 512, 64, 1), (24, 10240, 512, 128, 1), (32, 8192, 512, 64, 1), (32, 28672, 256, 128, 1),
+    (48, 10240, 512, 64, 1), (64, 10240, 512, 64, 1), (64, 28672, 256, 64, 2), (60, 16384, 256, 256, 1),
+])
+def test_error_does_not_grow_with_the_row(gpu, monkeypatch, M, K, N, group, shares):
+    """Distance from sums in 64 bits.  Chains of eight groups add 4.5 roundings of a relative size of 2.6e-8 (rms) at
+    most, a share's last addition, the sum of the shares and the token scale one each: sqrt(7.5) * 2.6e-8 = 7.1e-8 for
+    terms of equal size (7.3e-8 in numpy); a running total over the groups of these rows is at 1.0e-7 and more."""
+    torch, b = gpu
+    monkeypatch.setenv("W2A8_TSTREAM", "2")
+    monkeypatch.setenv("W2A8_TSTREAM_C", str(shares))
+    gen = torch.Generator(device="cuda").manual_seed(K + M)
+    codes = torch.randint(0, 4, (N, K), generator=gen, device="cuda", dtype=torch.uint8)
+    scale = 0.02 * torch.exp(0.5 * torch.randn((N, K // group), generator=gen, device="cuda"))
+    a = torch.randint(-127, 128, (M, K), generator=gen, device="cuda", dtype=torch.int8)
+    a_scale = torch.rand(M, generator=gen, device="cuda") + 0.5
+    ws = b.new_workspace(b.w2a8_workspace_bytes(M, N, K, group))
+    y = b.w2a8_gemm(a, a_scale, b.w2_pack(codes), scale, group, ws).double()
+    sums = torch.einsum("mgk,ngk->mng", a.double().view(M, -1, group), codes.double().view(N, -1, group) - 2)
+    exact = torch.einsum("mng,ng->mn", sums, scale.double()) * a_scale.double()[:, None]
+    assert b.w2a8_workspace_status(ws) == 0
+    assert ((y - exact).norm() / exact.norm()).item() <= 8e-8
+
+
+@pytest.mark.parametrize("group", [64, 128, 256])
+@pytest.mark.parametrize("M,shares", [(16, 1), (16, 8), (24, 4), (32, 1), (48, 2), (64, 4)])
+def test_infinities_and_nan(gpu, monkeypatch, M, shares, group):
+    """Infinite and NaN scales, and products that leave fp32: what a plain sum of the scaled group sums gives."""
+    torch, b = gpu
+    monkeypatch.setenv("W2A8_TSTREAM", "2")
+    monkeypatch.setenv("W2A8_TSTREAM_C", str(shares))
+    N, K = 160, 4096
+    G = K // group
+    gen = torch.Generator(device="cuda").manual_seed(M + group)
+    codes = torch.randint(0, 4, (N, K), generator=gen, device="cuda", dtype=torch.uint8)
+    a = torch.randint(-127, 128, (M, K), generator=gen, device="cuda", dtype=torch.int8)
+    scale = torch.rand((N, G), generator=gen, device="cuda") + 0.01
+    for ch in range(0, 64, 2):                        # one, then two infinite scales, somewhere in the row
+        scale[ch, (5 * ch) % G] = float("inf")
+        scale[ch, (11 * ch + 3) % G] = -float("inf") if ch % 4 else float("inf")
+    scale[64:80, G // 2] = float("nan")
+    scale[80:96, (G - 1) // 2] = 3.0e38               # finite, its products are not
+    ones = torch.ones(M, device="cuda")
+    ws = b.new_workspace(b.w2a8_workspace_bytes(M, N, K, group))
+    y = b.w2a8_gemm(a, ones, b.w2_pack(codes), scale, group, ws)
+    sums = 64 * torch.einsum("mgk,ngk->mng", a.double().view(M, G, group), codes.double().view(N, G, group) - 2)
+    ref = (sums * scale.double()).float().sum(dim=2) / 64        # (terms in fp32: infinite where theirs are)
+    assert b.w2a8_workspace_status(ws) == 0
+    assert torch.equal(y.isnan(), ref.isnan()) and torch.equal(y.isinf(), ref.isinf())
+    assert torch.equal(y.sign()[y.isinf()], ref.sign()[ref.isinf()])
+    fin = ref.isfinite()
+    assert int(fin.sum()) > M * 60
+    assert (y - ref)[fin].abs().max() <= 1e-5 * ref[fin].abs().max()
