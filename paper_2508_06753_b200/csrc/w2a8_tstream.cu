@@ -68,7 +68,9 @@ struct TsMaps {
     CUtensorMap act;
 };
 
-// NT: tokens that are drained (16, 24, 32, 48, 64); SPP: 64-k slices per scale group, 0 = groups of whole blocks.
+// NT: tokens that are drained (16, 24, 32, 48, 64); SPP: 64-k slices per scale group, 0 = groups of whole blocks, kTsRow = one
+// group per row.
+constexpr int kTsRow = -1;
 template <int NT, int SPP>
 struct TsCfg {
     static constexpr int BN = (NT + 15) / 16 * 16;                // UMMA N
@@ -81,24 +83,24 @@ struct TsCfg {
     static constexpr int kTmemCols = NT <= 32 ? 256 : 512;
     static constexpr int AS = NT <= 32 ? 2 : 4;     // unpacked blocks in tensor memory
     static constexpr int kAccCols = kTmemCols - 64 * AS;
-    static constexpr int GPB = SPP == 0 ? 1 : 4 / SPP;            // groups of a block
-    static constexpr int UG = SPP == 0 ? 1 : GPB * BN <= 64 ? GPB : 2;   // groups of a unit = hand-off between MMA and drain
+    static constexpr int GPB = SPP <= 0 ? 1 : 4 / SPP;            // groups of a block
+    static constexpr int UG = SPP <= 0 ? 1 : GPB * BN <= 64 ? GPB : 2;   // groups of a unit = hand-off between MMA and drain
     static constexpr int UPB = GPB / UG;                          // units of a block
     static constexpr int kUnitCols = UG * BN;
     // A chain of additions is kChain blocks (groups of whole blocks: groups), eight groups, long.  The running sums of the
     // second half of a thread's columns are in shared memory where the registers do not hold them.
-    static constexpr int kChain = SPP == 0 ? 8 : 8 / GPB;
-    static constexpr int kHiShared = DC > 16 ? DC / 2 : 0;
+    static constexpr int kChain = SPP <= 0 ? 8 : 8 / GPB;
+    static constexpr int kHiShared = SPP != kTsRow && DC > 16 ? DC / 2 : 0;
     static constexpr int kHiBytes = kHiShared * 4 * 32 * kDrainWarps;
     static constexpr int kUnits = kAccCols / kUnitCols;
     // One barrier says that a block is unpacked and its accumulators are free, where both come round alike.
-    static constexpr bool kFold = SPP != 0 && UPB == 1 && kUnits >= AS;
+    static constexpr bool kFold = SPP > 0 && UPB == 1 && kUnits >= AS;
     static constexpr int NU = kFold ? AS : kUnits > 4 ? 4 : kUnits;      // units in flight
     static constexpr int kStageBytes = kTsWBytes + BN * 256;
     static constexpr int kSumBytes = kTsBM * (DC == 24 ? 32 : DC) * kDrainWarps;     // a tile's sums, in pieces of 16 bytes
     static constexpr int kRing = ((kCtasPerSm == 2 ? 112 : 224) * 1024 - 2048 - 2 * kSumBytes) / kStageBytes;
     static constexpr size_t kSmem = (size_t)kRing * kStageBytes + 2 * kSumBytes + kHiBytes + 1024;
-    static constexpr bool kUnitBarrier = SPP == 0 || UPB > 1;     // else a block's barrier says it all
+    static constexpr bool kUnitBarrier = SPP <= 0 || UPB > 1;     // else a block's barrier says it all
     // Registers per thread: the launch has 80 or 96 (what the launch bounds leave, rounded down to a multiple of eight, and
     // what the compiler reports for every instance); setmaxnreg moves some of the first warps' to the drain warps.
     static constexpr int kRegs = NT <= 32 ? 80 : 96, kRegsFirst = NT <= 32 ? 24 : 32, kRegsDrain = NT <= 32 ? 136 : 128;
@@ -336,18 +338,18 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             bool ok = true;
             [[maybe_unused]] int kb = 0;
             [[maybe_unused]] bool fresh = true;         // (groups of whole blocks) the next block opens a unit
-            const int first_left = p.bpg - (SPP == 0 ? kb_lo % p.bpg : 0);
+            const int first_left = SPP == 0 ? p.bpg - kb_lo % p.bpg : nb;
             [[maybe_unused]] int left = first_left;
             for (int i = 0; i < n; ++i) {
                 if (i < R) ok = ts_wait(pf_smem_u32(&bar_b[s]), 0, abort_flag);
-                if (SPP == 0 && fresh) ok = ok && ts_wait(pf_smem_u32(&bar_free[un]), uph, abort_flag);
+                if (SPP <= 0 && fresh) ok = ok && ts_wait(pf_smem_u32(&bar_free[un]), uph, abort_flag);
                 ok = ok && ts_wait(pf_smem_u32(&bar_a[as]), aph, abort_flag);
                 if (!ok) break;
                 auto step = [&](int j, uint32_t d, uint32_t acc) {
                     const uint32_t koff = ((j >> 2) * BN * 128 + (j & 3) * 32) >> 4;
                     ts_mma_i8_tmem(d, tmem_a + as * 64 + 8 * j, ((uint64_t)b_hi << 32) | (b_lo + so + koff), idesc, acc);
                 };
-                if constexpr (SPP != 0) {
+                if constexpr (SPP > 0) {
 #pragma unroll
                     for (int u = 0; u < C::UPB; ++u) {
                         if constexpr (!C::kFold) ok = ts_wait(pf_smem_u32(&bar_free[un]), uph, abort_flag);
@@ -374,7 +376,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                     }
                     fresh = last;
                     if (last) {
-                        left = p.bpg;
+                        left = SPP == 0 ? p.bpg : nb;
                         if (++un == NU) { un = 0; uph ^= 1u; }
                     }
                     if (++kb == nb) { kb = 0; left = first_left; }
@@ -462,13 +464,13 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             const int i = mat_of(t, n0);
             const int ch = min(n0 + q * 32 + lane, p.mat[i].N - 1);
             srow = reinterpret_cast<const char *>(p.mat[i].w_scale) + (size_t)ch * p.G * (H16 ? 2 : 4) +
-                   (SPP == 0 ? 0 : kb_lo * C::GPB * (H16 ? 2 : 4));
+                   (SPP <= 0 ? 0 : kb_lo * C::GPB * (H16 ? 2 : 4));
         };
         locate(ptile);
         // (groups of whole blocks) group of the block that is requested next, blocks left of it
-        const int gi0 = SPP == 0 ? kb_lo / p.bpg : 0, first_left = (gi0 + 1) * p.bpg - kb_lo;
+        const int gi0 = SPP == 0 ? kb_lo / p.bpg : 0, first_left = SPP == 0 ? (gi0 + 1) * p.bpg - kb_lo : nb;
         int pgi = gi0, pleft = first_left;
-        constexpr int kStep = SPP == 0 ? 0 : C::GPB * (H16 ? 2 : 4);      // scale bytes of a block
+        constexpr int kStep = SPP <= 0 ? 0 : C::GPB * (H16 ? 2 : 4);      // scale bytes of a block
         auto request = [&]() -> Scales {
             Scales sc = {};
             if (left == 0) return sc;
@@ -482,7 +484,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             } else {
                 if constexpr (H16) sc.r[0] = __ldg(reinterpret_cast<const unsigned short *>(srow) + pgi);
                 else sc.r[0] = __ldg(reinterpret_cast<const uint32_t *>(srow) + pgi);
-                if (--pleft == 0) { ++pgi; pleft = p.bpg; }
+                if (SPP == 0 && --pleft == 0) { ++pgi; pleft = p.bpg; }
             }
             srow += kStep;
             if (++pkb == nb) {
@@ -522,6 +524,9 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
         clear();
         uint32_t ph = 0, uph = 0;
         bool got = true;
+        // One group per row: shares are summed as the integers they are and scaled once, so that the split of K adds no
+        // rounding (8192 x 8192 at 64 tokens 4.3e-8 from sums in 64 bits with scaled shares, 3.6e-8 with integers).
+        constexpr bool whole = SPP == kTsRow;
         [[maybe_unused]] int gleft = first_left;
         int nsum = 0;                                   // tiles summed so far
         auto drain_unit = [&](int g0) {
@@ -547,10 +552,15 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                     f[g] = scale(sc_cur, g0 + g);
                     if (c == 0) largest = fmaxf(largest, fabsf(f[g]));
                 }
+                if constexpr (whole) {
 #pragma unroll
-                for (int g = 0; g < UG; ++g)
+                    for (int j = 0; j < CH; ++j) acc[c + j] = __int_as_float(v[0][j]);
+                } else {
 #pragma unroll
-                    for (int j = 0; j < CH; j += 2) pf_fma2(acc[c + j], acc[c + j + 1], (float)v[g][j], (float)v[g][j + 1], f[g]);
+                    for (int g = 0; g < UG; ++g)
+#pragma unroll
+                        for (int j = 0; j < CH; j += 2) pf_fma2(acc[c + j], acc[c + j + 1], (float)v[g][j], (float)v[g][j + 1], f[g]);
+                }
             }
         };
         auto join = [&]() {
@@ -574,7 +584,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
         for (int i = 0; i < n; ++i) {
             sc_cur = sc_n1; sc_n1 = sc_n2; sc_n2 = request();
             const bool row_end = kb + 1 == nb;
-            if constexpr (SPP != 0) {
+            if constexpr (SPP > 0) {
 #pragma unroll
                 for (int u = 0; u < C::UPB; ++u) {
                     if constexpr (C::kUnitBarrier) got = got && ts_wait(pf_smem_u32(&bar_full[un]), uph, abort_flag);
@@ -584,25 +594,29 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                 }
                 if (++chain == C::kChain) join();
             } else if (--gleft == 0 || row_end) {
-                gleft = row_end ? first_left : p.bpg;
+                gleft = row_end ? first_left : SPP == 0 ? p.bpg : nb;
                 got = ts_wait(pf_smem_u32(&bar_full[un]), uph, abort_flag);
                 pf_tc_fence_after();
                 drain_unit(0);
-                if (++chain == C::kChain) join();
+                if (!whole && ++chain == C::kChain) join();
             }
             if (++s == R) { s = 0; ph ^= 1u; }
             if (!got) break;
             if (row_end) {
                 // ---- this CTA's share of the tile's sums is complete ---------------------------
+                if constexpr (!whole) {
 #pragma unroll
-                for (int j = 0; j < HR; ++j) acc[j] += hi[j];
+                    for (int j = 0; j < HR; ++j) acc[j] += hi[j];
 #pragma unroll
-                for (int j = 0; j < HS; j += 2) {
-                    float h[2];
-                    ts_ld_shared<2>(h, hi_s + j / 2 * kHiStep);
-                    acc[HR + j] += h[0];
-                    acc[HR + j + 1] += h[1];
+                    for (int j = 0; j < HS; j += 2) {
+                        float h[2];
+                        ts_ld_shared<2>(h, hi_s + j / 2 * kHiStep);
+                        acc[HR + j] += h[0];
+                        acc[HR + j + 1] += h[1];
+                    }
                 }
+                const float row_scale = whole ? scale(sc_cur, 0) : 0.f;
+                auto scaled = [&](float bits) -> float { return (float)__float_as_int(bits) * row_scale; };
                 int n0;
                 const int mi = mat_of(tile, n0);
                 const int ch = n0 + q * 32 + lane;
@@ -647,6 +661,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                         for (int j = 0; j < PC; ++j) {
                             const float x = r < kParts && r == rank ? acc[(r < kParts ? r : 0) * PC + j] : v[j];
                             if (r == 0) { sum[j] = x; rest[j] = 0.f; continue; }
+                            if (whole) { sum[j] = __int_as_float(__float_as_int(sum[j]) + __float_as_int(x)); continue; }
                             const float s2 = sum[j] + x, took = s2 - sum[j];      // exact sum = s2 + what is left of both terms
                             rest[j] += (sum[j] - (s2 - took)) + (x - took);
                             sum[j] = s2;
@@ -654,11 +669,11 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                     }
 #pragma unroll
                     for (int j = 0; j < PC; ++j)          // (an infinite sum has no rest)
-                        store(col0 + rank * PC + j, rest[j] == rest[j] ? sum[j] + rest[j] : sum[j]);
+                        store(col0 + rank * PC + j, whole ? scaled(sum[j]) : rest[j] == rest[j] ? sum[j] + rest[j] : sum[j]);
                 };
                 if (nc == 1) {
 #pragma unroll
-                    for (int j = 0; j < DC; ++j) store(col0 + j, acc[j]);
+                    for (int j = 0; j < DC; ++j) store(col0 + j, whole ? scaled(acc[j]) : acc[j]);
                 } else if (nc == 2) exchange(std::integral_constant<int, 2>{});
                 else if (nc == 4)   exchange(std::integral_constant<int, 4>{});
                 else                exchange(std::integral_constant<int, 8>{});
@@ -794,7 +809,8 @@ static cudaError_t launch_ts_inst(const TsMaps &maps, TsParams &p, cudaStream_t 
 template <int NT, bool H16>
 static cudaError_t launch_ts_spp(const TsMaps &maps, TsParams &p, int spp, cudaStream_t st) {
     return spp == 1 ? launch_ts_inst<NT, 1, H16>(maps, p, st)
-         : spp == 2 ? launch_ts_inst<NT, 2, H16>(maps, p, st) : launch_ts_inst<NT, 0, H16>(maps, p, st);
+         : spp == 2 ? launch_ts_inst<NT, 2, H16>(maps, p, st)
+         : p.G == 1 ? launch_ts_inst<NT, kTsRow, H16>(maps, p, st) : launch_ts_inst<NT, 0, H16>(maps, p, st);
 }
 template <bool H16>
 static cudaError_t launch_ts_nt(const TsMaps &maps, TsParams &p, int spp, cudaStream_t st) {

@@ -194,7 +194,7 @@ def test_error_does_not_grow_with_the_row(gpu, monkeypatch, M, K, N, group, shar
     assert ((y - exact).norm() / exact.norm()).item() <= 8e-8
 
 
-@pytest.mark.parametrize("group", [64, 128, 256])
+@pytest.mark.parametrize("group", [64, 128, 256, 4096])
 @pytest.mark.parametrize("M,shares", [(16, 1), (16, 8), (24, 4), (32, 1), (48, 2), (64, 4)])
 def test_infinities_and_nan(gpu, monkeypatch, M, shares, group):
     """Infinite and NaN scales, and products that leave fp32: what a plain sum of the scaled group sums gives."""
@@ -223,3 +223,25 @@ def test_infinities_and_nan(gpu, monkeypatch, M, shares, group):
     fin = ref.isfinite()
     assert int(fin.sum()) > M * 60
     assert (y - ref)[fin].abs().max() <= 1e-5 * ref[fin].abs().max()
+
+
+@pytest.mark.parametrize("N,K", [(1024, 8192), (1152, 2560)])
+@pytest.mark.parametrize("shares", [1, 2, 4, 8])
+def test_one_scale_per_channel_is_exact_up_to_the_scales(gpu, monkeypatch, N, K, shares):
+    """Integer sums, then the two scales: the bits of the int8 tensor-core kernel, whatever the shares of K."""
+    torch, b = gpu
+    M = 64
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    packed = b.w2_pack(torch.randint(0, 4, (N, K), generator=gen, device="cuda", dtype=torch.uint8))
+    scale = torch.rand((N, 1), generator=gen, device="cuda") + 0.01
+    a, s = b.a8_quantize(torch.randn((M, K), generator=gen, device="cuda").to(torch.bfloat16))
+    monkeypatch.setenv("W2A8_PREFILL", "2")
+    monkeypatch.setenv("W2A8_PF_KSPLIT", "1")
+    monkeypatch.setenv("W2A8_TSTREAM_C", str(shares))
+    ws = b.new_workspace(b.w2a8_workspace_bytes(M, N, K, K))
+    ys = {}
+    for mode in ("0", "2"):
+        monkeypatch.setenv("W2A8_TSTREAM", mode)
+        ys[mode] = b.w2a8_gemm(a, s, packed, scale, K, ws)
+        assert b.w2a8_workspace_status(ws) == 0
+    assert torch.equal(ys["0"], ys["2"])
