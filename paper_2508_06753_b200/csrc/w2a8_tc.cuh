@@ -39,8 +39,9 @@ __device__ __forceinline__ bool pf_mbar_try_wait(uint32_t bar, unsigned parity) 
     return ok != 0;
 }
 // Bounded wait; also gives up as soon as another role has raised the abort flag.
-__device__ __forceinline__ bool pf_wait(uint32_t bar, unsigned parity, volatile int *abort_flag) {
-    for (unsigned i = 0; i < kPfWaitPolls; ++i) {
+__device__ __forceinline__ bool pf_wait(uint32_t bar, unsigned parity, volatile int *abort_flag,
+                                        unsigned polls = kPfWaitPolls) {
+    for (unsigned i = 0; i < polls; ++i) {
         if (pf_mbar_try_wait(bar, parity)) return true;
         if ((i & 63u) == 63u && *abort_flag) return false;
     }
@@ -49,8 +50,13 @@ __device__ __forceinline__ bool pf_wait(uint32_t bar, unsigned parity, volatile 
 }
 // The same by a converged warp, all lanes polling: a ready barrier costs 75 clk this way, 250 when one lane
 // polls and the warp reconverges behind it (measured).
-__device__ __forceinline__ bool pf_wait_all(uint32_t bar, unsigned parity, volatile int *abort_flag) {
-    return __all_sync(0xFFFFFFFFu, pf_wait(bar, parity, abort_flag)) != 0;
+__device__ __forceinline__ bool pf_wait_all(uint32_t bar, unsigned parity, volatile int *abort_flag,
+                                            unsigned polls = kPfWaitPolls) {
+    return __all_sync(0xFFFFFFFFu, pf_wait(bar, parity, abort_flag, polls)) != 0;
+}
+// Bounded wait of a kernel that gives up for work of its own that is still on its way.
+__device__ __forceinline__ void pf_wait_own(uint32_t bar, unsigned parity) {
+    for (unsigned i = 0; i < kPfWaitPolls && !pf_mbar_try_wait(bar, parity); ++i) {}
 }
 __device__ __forceinline__ void pf_tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
     asm volatile(

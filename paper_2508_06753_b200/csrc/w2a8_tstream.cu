@@ -61,6 +61,7 @@ struct TsParams {
     int tiles, nclusters; // cluster c takes tiles c, c + nclusters, ...
     int bpg;              // blocks per scale group (groups of whole blocks)
     int y16;
+    unsigned polls;       // bound of every wait
 };
 
 struct TsMaps {
@@ -200,8 +201,8 @@ __device__ __forceinline__ void ts_ld_shared(float (&v)[N], uint32_t addr) {
     }
 }
 // pf_wait for data that other CTAs of the cluster wrote
-__device__ __forceinline__ bool ts_wait_cluster(uint32_t bar, unsigned parity, volatile int *abort_flag) {
-    for (unsigned i = 0; i < kPfWaitPolls; ++i) {
+__device__ __forceinline__ bool ts_wait_cluster(uint32_t bar, unsigned parity, volatile int *abort_flag, unsigned polls) {
+    for (unsigned i = 0; i < polls; ++i) {
         unsigned ok;
         asm volatile("{\n\t.reg .pred p;\n\t"
                      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
@@ -215,9 +216,9 @@ __device__ __forceinline__ bool ts_wait_cluster(uint32_t bar, unsigned parity, v
 
 // Bounded wait of a converged warp (pf_wait_all) whose first look costs a poll, a vote and a branch: most waits find their
 // barrier complete, and what the warps spend on looking was a third of all instructions.
-__device__ __forceinline__ bool ts_wait(uint32_t bar, unsigned parity, volatile int *abort_flag) {
+__device__ __forceinline__ bool ts_wait(uint32_t bar, unsigned parity, volatile int *abort_flag, unsigned polls) {
     if (__all_sync(0xFFFFFFFFu, pf_mbar_try_wait(bar, parity))) return true;
-    return pf_wait_all(bar, parity, abort_flag);
+    return pf_wait_all(bar, parity, abort_flag, polls);
 }
 
 template <int NT, int SPP, bool H16>
@@ -229,8 +230,9 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
     __shared__ __align__(8) unsigned long long bar_w[R], bar_b[R], bar_done[R], bar_a[AS], bar_full[NU], bar_free[NU];
     __shared__ __align__(8) unsigned long long bar_sum[2][C::kDrainWarps];
     __shared__ float tok_scale[NT];
+    __shared__ __align__(8) unsigned long long bar_mma;
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_s;
+    __shared__ int abort_s, copies_w_s, copies_b_s;
     volatile int *abort_flag = &abort_s;
 
     const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -252,7 +254,8 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
     };
 
     if (threadIdx.x == 0) {
-        abort_s = 0;
+        abort_s = copies_w_s = copies_b_s = 0;
+        pf_mbar_init(pf_smem_u32(&bar_mma), 1);
         for (int i = 0; i < R; ++i) {
             pf_mbar_init(pf_smem_u32(&bar_w[i]), 1);
             pf_mbar_init(pf_smem_u32(&bar_b[i]), 1);
@@ -272,6 +275,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
     __syncthreads();
     pf_tc_fence_after();
     // every CTA of the cluster has its barriers: arrive here, wait before the first access to another CTA
+    int nsum = 0;                                       // (drain warps) tiles summed so far
     if (nc > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     const uint32_t sums0 = stage0 + R * C::kStageBytes;
     const uint32_t tmem_a = tmem_slot, tmem_acc = tmem_slot + 64 * AS;
@@ -314,14 +318,17 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                 load_b(i, k, pf_smem_u32(&bar_b[i]));
                 if (++k == nb) k = 0;
             }
+            copies_b_s = head;
+            copies_w_s = head;
             int s = 0;
             uint32_t ph = 0;
             for (int i = R; i < n; ++i) {
-                if (!pf_wait(pf_smem_u32(&bar_done[s]), ph, abort_flag)) break;
+                if (!pf_wait(pf_smem_u32(&bar_done[s]), ph, abort_flag, p.polls)) break;
                 // (the MMA warp learns of these activations from the unpack warps, which wait for both)
                 pf_mbar_arrive_expect_tx(pf_smem_u32(&bar_w[s]), C::kStageBytes);
                 load_w(s);
                 load_b(s, kb, pf_smem_u32(&bar_w[s]));
+                copies_w_s = i + 1;
                 advance();
                 if (++s == R) { s = 0; ph ^= 1u; }
             }
@@ -334,16 +341,16 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             const uint32_t b_lo = (uint32_t)b_desc0, b_hi = (uint32_t)(b_desc0 >> 32);
             constexpr uint32_t idesc = pf_instr_desc(kTsBM, BN);
             int s = 0, as = 0, un = 0;
-            uint32_t aph = 0, uph = 0, so = 0, dph = 0;
+            uint32_t aph = 0, uph = 0, so = 0;
             bool ok = true;
             [[maybe_unused]] int kb = 0;
             [[maybe_unused]] bool fresh = true;         // (groups of whole blocks) the next block opens a unit
             const int first_left = SPP == 0 ? p.bpg - kb_lo % p.bpg : nb;
             [[maybe_unused]] int left = first_left;
             for (int i = 0; i < n; ++i) {
-                if (i < R) ok = ts_wait(pf_smem_u32(&bar_b[s]), 0, abort_flag);
-                if (SPP <= 0 && fresh) ok = ok && ts_wait(pf_smem_u32(&bar_free[un]), uph, abort_flag);
-                ok = ok && ts_wait(pf_smem_u32(&bar_a[as]), aph, abort_flag);
+                if (i < R) ok = ts_wait(pf_smem_u32(&bar_b[s]), 0, abort_flag, p.polls);
+                if (SPP <= 0 && fresh) ok = ok && ts_wait(pf_smem_u32(&bar_free[un]), uph, abort_flag, p.polls);
+                ok = ok && ts_wait(pf_smem_u32(&bar_a[as]), aph, abort_flag, p.polls);
                 if (!ok) break;
                 auto step = [&](int j, uint32_t d, uint32_t acc) {
                     const uint32_t koff = ((j >> 2) * BN * 128 + (j & 3) * 32) >> 4;
@@ -352,7 +359,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                 if constexpr (SPP > 0) {
 #pragma unroll
                     for (int u = 0; u < C::UPB; ++u) {
-                        if constexpr (!C::kFold) ok = ts_wait(pf_smem_u32(&bar_free[un]), uph, abort_flag);
+                        if constexpr (!C::kFold) ok = ts_wait(pf_smem_u32(&bar_free[un]), uph, abort_flag, p.polls);
                         if (!ok) break;
                         pf_tc_fence_after();
                         if (lead) {
@@ -383,12 +390,13 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                 }
                 if (lead) pf_mma_commit(pf_smem_u32(&bar_done[s]));
                 so += C::kStageBytes >> 4;
-                if (++s == R) { s = 0; so = 0; dph ^= 1u; }
+                if (++s == R) { s = 0; so = 0; }
                 if (++as == AS) { as = 0; aph ^= 1u; }
             }
-            // (the drain warps need not have waited for a block's barrier: none may be signalled after this CTA has left)
-            if constexpr (C::kUnitBarrier)
-                if (ok) ts_wait(pf_smem_u32(&bar_done[s == 0 ? R - 1 : s - 1]), s == 0 ? dph ^ 1u : dph, abort_flag);
+            // every MMA has ended, also where the drain warps need not have waited for it, and where a wait gave up
+            if (lead) pf_mma_commit(pf_smem_u32(&bar_mma));
+            pf_wait_own(pf_smem_u32(&bar_mma), 0);
+            __syncwarp();
         }
     } else if (warp < C::kFirstDrain) {
         // ===== unpack warps: a lane's channel of a block, 16 words -> 64 columns of int8 lanes ========
@@ -408,7 +416,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                              : "r"(base + ((t ^ sw) << 4)));
         };
         if (set < n) {
-            got = ts_wait(pf_smem_u32(&bar_w[s]), 0, abort_flag);
+            got = ts_wait(pf_smem_u32(&bar_w[s]), 0, abort_flag, p.polls);
             load(s);
         }
         int ds = (set + 2 * R - AS) % R;                // slot of block i - AS
@@ -416,7 +424,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
         for (int i = set; i < n && got; i += C::kUnpackSets) {
             if (i >= AS) {                              // the MMAs of block i - AS have read this place
                 if (i < AS + C::kUnpackSets) pdl_wait();
-                got = ts_wait(pf_smem_u32(&bar_done[ds]), dph, abort_flag);
+                got = ts_wait(pf_smem_u32(&bar_done[ds]), dph, abort_flag, p.polls);
                 pf_tc_fence_after();
             }
 #pragma unroll
@@ -434,7 +442,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             s += C::kUnpackSets;
             if (s >= R) { s -= R; ph ^= 1u; }
             if (i + C::kUnpackSets < n) {
-                got = got && ts_wait(pf_smem_u32(&bar_w[s]), ph, abort_flag);
+                got = got && ts_wait(pf_smem_u32(&bar_w[s]), ph, abort_flag, p.polls);
                 load(s);
             }
             ts_tmem_st_wait();
@@ -528,7 +536,6 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
         // rounding (8192 x 8192 at 64 tokens 4.3e-8 from sums in 64 bits with scaled shares, 3.6e-8 with integers).
         constexpr bool whole = SPP == kTsRow;
         [[maybe_unused]] int gleft = first_left;
-        int nsum = 0;                                   // tiles summed so far
         auto drain_unit = [&](int g0) {
             // All groups of the unit for CH columns at a time (more staged values spill, and local memory is slow beside
             // the copies).
@@ -587,15 +594,15 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
             if constexpr (SPP > 0) {
 #pragma unroll
                 for (int u = 0; u < C::UPB; ++u) {
-                    if constexpr (C::kUnitBarrier) got = got && ts_wait(pf_smem_u32(&bar_full[un]), uph, abort_flag);
-                    else                           got = ts_wait(pf_smem_u32(&bar_done[s]), ph, abort_flag);
+                    if constexpr (C::kUnitBarrier) got = got && ts_wait(pf_smem_u32(&bar_full[un]), uph, abort_flag, p.polls);
+                    else                           got = got && ts_wait(pf_smem_u32(&bar_done[s]), ph, abort_flag, p.polls);
                     pf_tc_fence_after();
                     drain_unit(u * UG);
                 }
                 if (++chain == C::kChain) join();
             } else if (--gleft == 0 || row_end) {
                 gleft = row_end ? first_left : SPP == 0 ? p.bpg : nb;
-                got = ts_wait(pf_smem_u32(&bar_full[un]), uph, abort_flag);
+                got = got && ts_wait(pf_smem_u32(&bar_full[un]), uph, abort_flag, p.polls);
                 pf_tc_fence_after();
                 drain_unit(0);
                 if (!whole && ++chain == C::kChain) join();
@@ -649,7 +656,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
                         if (r < kParts)     ts_send<PC>(buf + rank * kFrom, bar, r, acc + (r < kParts ? r : 0) * PC);
                         else if (lane == 0) ts_send<1>(buf + rank * kFrom, bar, r, acc);
                     }
-                    got = __all_sync(0xFFFFFFFFu, ts_wait_cluster(bar, (nsum >> 1) & 1, abort_flag));
+                    got = __all_sync(0xFFFFFFFFu, ts_wait_cluster(bar, (nsum >> 1) & 1, abort_flag, p.polls));
                     ++nsum;
                     if (rank >= kParts) return;
                     float sum[PC], rest[PC];
@@ -685,11 +692,26 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
 
     // ---- wind down ---------------------------------------------------------------------
     __syncwarp();
-    if (nc > 1 && warp < C::kFirstDrain) cluster_wait_acquire();
+    if (nc > 1 && nsum == 0) cluster_wait_acquire();
     pf_tc_fence_before();
     __syncwarp();
     __syncthreads();
-    if (threadIdx.x == 0 && abort_s) atomicExch(p.status, W2A8_ERR_TIMEOUT);
+    if (abort_s) {
+        // A wait gave up.  Nothing may be on its way into this CTA's shared memory when it leaves: neither its own copies
+        // nor sums of its peers, which have left or wait here as well once the cluster barrier opens (it counts the threads
+        // that have not exited).  The pause covers stores that were under way, many times over.
+        if (threadIdx.x == 0) {
+            atomicExch(p.status, W2A8_ERR_TIMEOUT);
+            for (int i = max(0, copies_w_s - R); i < copies_w_s; ++i) pf_wait_own(pf_smem_u32(&bar_w[i % R]), (uint32_t)(i / R) & 1u);
+            for (int i = 0; i < copies_b_s; ++i) pf_wait_own(pf_smem_u32(&bar_b[i]), 0);
+        }
+        __syncthreads();
+        if (nc > 1) {
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            cluster_wait_acquire();
+            __nanosleep(20000);
+        }
+    }
     if (warp == 1) {
         pf_tc_fence_after();
         pf_tmem_dealloc(tmem_slot, C::kTmemCols);
@@ -860,6 +882,7 @@ int launch_tstream(const int8_t *a, const float *a_scale, int count, const uint3
     p.y16 = h16 && y16 ? 1 : 0;
     p.tiles = tiles;
     p.status = reinterpret_cast<int *>(workspace);
+    p.polls = (unsigned)env_int("W2A8_TSTREAM_POLLS", (int)kPfWaitPolls);
     const int spp = group == 64 ? 1 : group == 128 ? 2 : 0;
     const cudaError_t e = h16 ? launch_ts_nt<true>(maps, p, spp, st) : launch_ts_nt<false>(maps, p, spp, st);
     return e == cudaSuccess ? W2A8_OK : e == cudaErrorNotSupported ? kStatNoPlan : W2A8_ERR_CUDA;

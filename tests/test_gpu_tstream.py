@@ -245,3 +245,28 @@ def test_one_scale_per_channel_is_exact_up_to_the_scales(gpu, monkeypatch, N, K,
         ys[mode] = b.w2a8_gemm(a, s, packed, scale, K, ws)
         assert b.w2a8_workspace_status(ws) == 0
     assert torch.equal(ys["0"], ys["2"])
+
+
+@pytest.mark.parametrize("M", [16, 32, 64])
+@pytest.mark.parametrize("shares", [1, 2, 8])
+@pytest.mark.parametrize("group", [64, 1024])
+def test_a_wait_that_gives_up(gpu, monkeypatch, M, shares, group):
+    """With no polls allowed the waits give up: the call ends, the status word says so, and the next call is whole."""
+    torch, b = gpu
+    monkeypatch.setenv("W2A8_TSTREAM", "2")
+    monkeypatch.setenv("W2A8_TSTREAM_C", str(shares))
+    N, K = 1024, 32768
+    gen = torch.Generator(device="cuda").manual_seed(M)
+    packed = b.w2_pack(torch.randint(0, 4, (N, K), generator=gen, device="cuda", dtype=torch.uint8))
+    scale = torch.rand((N, K // group), generator=gen, device="cuda") + 0.01
+    a, s = b.a8_quantize(torch.randn((M, K), generator=gen, device="cuda").to(torch.bfloat16))
+    ws = b.new_workspace(b.w2a8_workspace_bytes(M, N, K, group))
+    whole = b.w2a8_gemm(a, s, packed, scale, group, ws)
+    assert b.w2a8_workspace_status(ws) == 0
+    monkeypatch.setenv("W2A8_TSTREAM_POLLS", "0")
+    b.w2a8_gemm(a, s, packed, scale, group, ws)
+    assert b.w2a8_workspace_status(ws) == -7                  # W2A8_ERR_TIMEOUT
+    monkeypatch.delenv("W2A8_TSTREAM_POLLS")
+    ws.zero_()
+    assert torch.equal(b.w2a8_gemm(a, s, packed, scale, group, ws), whole)
+    assert b.w2a8_workspace_status(ws) == 0
