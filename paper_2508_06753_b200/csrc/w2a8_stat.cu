@@ -535,6 +535,21 @@ static bool stat_plan(int M, int K, int pairs, const int *resident, StPlan *out)
     return best < 1e29;
 }
 
+// Estimated time of a launch on a whole B200 in us, from its plan: a start, rounds, ranks, and cells of one warp (up to 64
+// tokens; 1260 launches of random matrices at 9 to 63 tokens, groups of 64, 128 and one scale: 7 % rms).  Negative: no plan.
+double stat_estimate(int M, int K, int group, int pairs) {
+    static const int resident[kStMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 20, 15};
+    StPlan pl;
+    if (!stat_supported(M, K, group) || !stat_plan(M, K, pairs, resident, &pl)) return -1.0;
+    const int nb = (K / kBlockK + pl.C - 1) / pl.C, per = (pairs + pl.nclusters - 1) / pl.nclusters;
+    const int rounds = (per + pl.round_pairs - 1) / pl.round_pairs;
+    int cells = 0;
+    for (int r = 0; r < rounds; ++r)
+        cells += ((r + 1 < rounds ? pl.round_pairs : per - pl.round_pairs * (rounds - 1)) * nb + kStWarps - 1) / kStWarps;
+    const double a = group == 64 ? 0.089 : group == 128 ? 0.072 : 0.113, b = group == 64 ? 0.273 : group == 128 ? 0.249 : 0.2335;
+    return 2.15 + 1.18 * rounds + 0.364 * pl.C + cells * (a + b * st_slabs(M));
+}
+
 template <int MT, int SPP, bool H16>
 static cudaError_t launch_stat_inst(StParams &p, cudaStream_t st) {
     auto kernel = w2a8_stat_kernel<MT, SPP, H16, st_ring(MT)>;

@@ -88,9 +88,10 @@ struct TsCfg {
     static constexpr int UG = SPP <= 0 ? 1 : GPB * BN <= 64 ? GPB : 2;   // groups of a unit = hand-off between MMA and drain
     static constexpr int UPB = GPB / UG;                          // units of a block
     static constexpr int kUnitCols = UG * BN;
-    // A chain of additions is kChain blocks (groups of whole blocks: groups), eight groups, long.  The running sums of the
+    // A chain of additions is kChain blocks (groups of whole blocks: groups) long, eight groups and with groups of 128 six
+    // (four cost 2 to 5 % of a launch, eight save nothing and are further off on short rows).  The running sums of the
     // second half of a thread's columns are in shared memory where the registers do not hold them.
-    static constexpr int kChain = SPP <= 0 ? 8 : 8 / GPB;
+    static constexpr int kChain = SPP <= 0 ? 8 : SPP == 2 ? 3 : 8 / GPB;
     static constexpr int kHiShared = SPP != kTsRow && DC > 16 ? DC / 2 : 0;
     static constexpr int kHiBytes = kHiShared * 4 * 32 * kDrainWarps;
     static constexpr int kUnits = kAccCols / kUnitCols;
@@ -720,6 +721,7 @@ w2a8_tstream_kernel(const __grid_constant__ TsMaps maps, const __grid_constant__
 
 // ---- host side -----------------------------------------------------------------------
 bool gemv_preferred(int M, int K, int group, int tiles, int count);
+double stat_estimate(int M, int K, int group, int pairs);
 
 bool tstream_supported(int M, int K, int group) {
     if (M < 1 || M > 64 || K % kBlockK != 0) return false;
@@ -728,53 +730,82 @@ bool tstream_supported(int M, int K, int group) {
 }
 static int ts_tokens(int M) { return M <= 16 ? 16 : M <= 24 ? 24 : M <= 32 ? 32 : M <= 48 ? 48 : 64; }
 
-// Shares of K and clusters for a launch over `tiles` tiles of `KB` blocks: the least cost in blocks that one CTA works
-// off after the other.  A last round counts half of a round where a few clusters have it (they have the memory for
-// themselves) and a whole one from two thirds on, a second CTA on the SMs costs 20 %, an exchange of sums as much as a
-// block.  Against the best of all C over 440 launches (10 sets of matrices, 12 to 64 tokens) the choice loses 0.9 % on average and 13 % at most.
-static double ts_plan(int tiles, int KB, const int *resident, bool two_per_sm, int *C, int *nclusters) {
+// Time of a launch in us, by token width and group (64, 128, more): a start, one per block of cost, round with an exchange
+// of sums, and level of C.
+struct TsTimes { double start, block, round, level; };
+static const TsTimes kTsTimes[5][3] = {
+    {{1.891, 0.340, 0.482, -0.054}, {1.889, 0.289, 0.457, -0.038}, {2.738, 0.234, 0.411, -0.236}},
+    {{2.652, 0.420, 0.573, -0.040}, {2.444, 0.320, 0.609, -0.095}, {3.033, 0.258, 0.457, -0.159}},
+    {{3.459, 0.471, 0.919, -0.456}, {3.396, 0.338, 0.835, -0.446}, {3.451, 0.263, 0.606, -0.302}},
+    {{3.317, 0.429, 0.729, -0.005}, {3.190, 0.294, 0.589, 0.071}, {3.874, 0.221, 0.332, 0.002}},
+    {{4.577, 0.488, 1.237, -0.560}, {4.311, 0.331, 1.059, -0.474}, {4.526, 0.226, 0.605, -0.197}}
+};
+static const TsTimes &ts_times(int M, int group) {
+    const int nt = ts_tokens(M);
+    return kTsTimes[nt == 16 ? 0 : nt == 24 ? 1 : nt == 32 ? 2 : nt == 48 ? 3 : 4][group == 64 ? 0 : group == 128 ? 1 : 2];
+}
+
+// Shares of K and clusters for a launch over `tiles` tiles of `KB` blocks: those of the least estimated time, which is
+// returned.  The cost counts blocks that one CTA works off after the other, in full rounds of the resident clusters and a
+// last one; a block takes twice as long where every SM has a CTA as where few have, and 30 % more with two CTAs on each.
+// Fitted to 2280 launches of the layers' and of random matrices at 9 to 64 tokens with every C (7 % rms); the choice loses
+// 1.0 % on average against the best C.
+static double ts_plan(int tiles, int KB, const int *resident, const TsTimes &t, int *C, int *nclusters) {
     const int forced = env_int("W2A8_TSTREAM_C", 0);
+    const double sms = sm_count();
+    auto load = [&](double ctas) { return 1.0 + std::min(1.0, ctas / sms) + 0.3 * std::max(0.0, ctas / sms - 1.0); };
     double best = 1e30;
-    for (int c = 1; c <= kTsMaxCluster; c *= 2) {
+    for (int c = 1, level = 0; c <= kTsMaxCluster; c *= 2, ++level) {
         if (c > KB || resident[c] < 1 || (forced > 0 && c != forced)) continue;
-        const int ncl = std::min(tiles, resident[c]), rounds = (tiles + ncl - 1) / ncl, sms = sm_count();
-        const double left = (double)(tiles % ncl) / ncl, share = (KB + c - 1) / c;
-        double cost = (tiles / ncl + (left > 0 ? 0.5 + 0.5 * std::min(1.0, 1.5 * left) : 0.0)) * share;
-        if (two_per_sm) cost *= 1.0 + 0.2 * std::min(1.0, std::max(0.0, (double)(ncl * c - sms) / sms));
-        if (c > 1) cost += rounds;
-        if (cost < best) { best = cost; *C = c; *nclusters = ncl; }
+        const int ncl = std::min(tiles, resident[c]), full = tiles / ncl, left = tiles % ncl, share = (KB + c - 1) / c;
+        const double cost = share * (full * load((double)ncl * c) + (left > 0 ? load((double)left * c) : 0.0));
+        const double us = t.start + t.block * cost + (c > 1 ? t.round * (full + (left > 0)) : 0.0) + t.level * level;
+        if (us < best) { best = us; *C = c; *nclusters = ncl; }
     }
     return best;
 }
 
 // Whether the kernel takes a launch over `count` matrices of `tiles16` 16-channel tiles in all (9 to 64 tokens).
-// Compared are its own time, a constant and a time per block of the plan's cost, and that of the kernel with stationary
-// activations, 4.6 us + 0.25 ns per 32 channels x 256 k and eight tokens.  Measured on B200 (us per call, before / this
-// kernel, groups of 64 | 128 | one scale per channel):
-//   16 tokens: 8192 x 8192 10.1 / 9.0 | 9.9 / 8.3 | 8.7 / 8.4; 4096 x (14336 + 14336) 13.2 / 12.7 | 12.5 / 11.6 | 11.7 / 11.0;
-//     28672 x 8192 21.9 / 21.9 | 21.4 / 19.5 | 19.9 / 17.8; but 8192 x 28672 20.3 / 23.1 | 19.7 / 20.5 | 18.8 / 18.5
-//   24 tokens: 8192 x 8192 11.8 / 10.9 | 11.1 / 9.8 | 10.8 / 9.0; 8192 x (28672 + 28672) 49.3 / 48.4 | 44.6 / 38.4 | 44.4 / 34.5
-//   32 tokens: 8192 x 8192 14.1 / 12.1 | 13.3 / 10.1 | 12.5 / 9.4; 8192 x (28672 + 28672) 62.7 / 59.2 | 57.9 / 41.2 | 55.4 / 36.8;
-//     28672 x 8192 40.8 / 30.2 | 37.8 / 22.6 | 36.4 / 19.5; 4096 x 14336 12.1 / 11.7 | 11.5 / 9.5 | 10.9 / 9.1
-//   48 tokens: 8192 x 8192 17.3 / 15.4 | 16.1 / 11.5 | 15.1 / 10.4; 28672 x 8192 80.4 / 42.2 | 71.8 / 29.8 | 68.3 / 24.9
-//   64 tokens: 4096 x 4096 10.0 / 8.8 | 10.7 / 7.3 | 9.7 / 7.3; 8192 x (28672 + 28672) 135 / 95 | 103 / 68 | 77 / 55;
-//     14336 x 4096 22.2 / 16.2 | 18.5 / 12.9 | 20.6 / 12.3
-// Rows of fewer than 4096 values that the persistent kernel does not hold in registers leave it at 9 to 16 tokens: 2560 x 3840 6.5 / 3.5 at
-// 12 and 7.6 / 3.5 at 16, 3072 x 12880 11.4 / 6.1 (128), 2560 x 1680 6.1 / 3.0.  Of 757 launches of random sets of
-// matrices (9 to 64 tokens) the rule moved 521 here, whose time fell by 1.47 on average; eight were slower by 2 to 6 %.
-// Small launches stay where they were (us, before / this kernel): at 32 tokens 4096 x 4096 5.7 / 6.6 | 5.7 / 5.4 | 5.0 / 5.4,
-// at 48 6.2 / 7.3 (128), 2048 x 2048 3.2 / 5.3; and so does everything of up to 8 tokens (4096 x (14336 + 14336) 9.4 / 11.2).
+// Compared are the estimates of its own launch and of the kernel with stationary activations, whose plan is the alternative
+// or (above 32 tokens, where the alternative is a launch per matrix, 2.5 us each; at 64 the tensor-core kernel) close to it.
+// Measured on B200 (us per call, before / this kernel, groups of 64 | 128 | one scale per channel):
+//   16 tokens: 8192 x 8192 10.1 / 9.3 | 9.9 / 8.6 | 8.7 / 8.2; 28672 x 8192 21.9 stays | 21.3 stays | 19.9 / 17.3;
+//   4096 x (14336 + 14336) 13.1 stays | 12.4 stays | 11.7 / 10.7; 2560 x 3840 7.5 / 3.7 | 7.3 / 3.5 | 7.1 / 3.6
+//   24 tokens: 8192 x 8192 11.7 / 11.5 | 11.1 / 9.8 | 10.8 / 8.7; 8192 x (28672 + 28672) 49.4 stays | 44.5 stays |
+//   44.2 / 34.8
+//   32 tokens: 8192 x (8192 + 1024 + 1024) 16.1 stays | 15.2 / 15.1 | 14.3 / 12.7; 8192 x 8192 14.1 / 12.4 | 13.3 /
+//   10.3 | 12.6 / 9.0; 8192 x (28672 + 28672) 62.9 stays | 58.1 / 44.3 | 55.4 / 35.6; 28672 x 8192 41.0 / 31.9 |
+//   37.9 / 24.3 | 36.4 / 18.9
+//   48 tokens: 8192 x 8192 17.1 / 16.2 | 16.0 / 12.3 | 15.1 / 10.9; 28672 x 8192 80.6 / 45.7 | 71.2 / 32.4 | 68.0 /
+//   25.5
+//   64 tokens: 4096 x 4096 10.0 stays | 10.8 / 7.8 | 9.8 / 7.3; 4096 x (14336 + 14336) 40.3 / 32.4 | 31.3 / 23.7 |
+//   25.7 / 17.0; 8192 x (28672 + 28672) 135.4 / 115.7 | 103.2 / 82.4 | 76.5 / 54.8; 14336 x 4096 22.2 / 17.5 | 18.3
+//   / 13.2 | 20.7 / 11.6
+// Small launches stay where they were, by their number of 8 KB blocks: their alternatives are not what the estimate describes
+// (us, before / this kernel: at 32 tokens 4096 x 4096, 512 blocks, 5.7 / 6.9 | 5.8 / 5.8 | 5.1 / 5.7; at 48 8.3 / 8.3 | 6.3 / 6.7;
+// 2048 x 2048, 128 blocks, 3.2 / 5.2), and so does everything of up to 8 tokens (4096 x (14336 + 14336) 9.4 / 11.2).
+// Rows of 1536 to 3840 values that the persistent kernel does not hold in registers leave it at 9 to 16 tokens, up to where
+// the kernel with stationary activations has them (3840 x 47392, groups of 128, 11 tokens 15.7 / 18.9).
+// Short rows stay too, below 1536 values with groups of 64 and below 2048 with groups of 128: a short row is summed no better here, and by
+// the other kernels in more parts (1024 x 20928, groups of 128, 64 tokens: 5.1e-8 from sums in 64 bits, 5.6e-8 here).  At 64 tokens so do
+// fewer than eight groups of 256 values and more, whose integers the tensor-core kernel never cuts, and groups of 128 with
+// binary16 scales, whose products it adds without rounding for longer (8192 x 8192 3.8e-8, 4.0e-8 here).
+// Of 4244 launches of random sets of matrices (9 to 64 tokens, groups of 64, 128, 1024 and one scale, some single
+// matrices with binary16 scales) the rule moved 2337 here: their time fell by 1.49 on average (geometric), 23 took more
+// than 1.5 % longer, 8 more than 5 %, 16 % at most; the distance from sums in 64 bits grew for 11 (binary16 scales in
+// groups of 1024, or rows below 2048), by 2.7 % at most.
 // W2A8_TSTREAM = 0 never, 2 whenever it supports the shape; any switch that forces a plan of another kernel keeps it out.
 bool tstream_takes(int M, int K, int group, int tiles16, int count, bool h16) {
     if (!tstream_supported(M, K, group)) return false;
     const int mode = env_int("W2A8_TSTREAM", 1);
     if (mode == 0) return false;
     if (mode == 2) return true;
-    if (M <= 8) return false;
-    const int KB = K / kBlockK, tiles = (tiles16 + 7) / 8, nt = ts_tokens(M), slabs = (M + 7) / 8;
+    if (M <= 8 || (group == 64 && K < 1536) || (group == 128 && K < 2048)) return false;
+    if (M == 64 && ((group > 128 && group < K && K / group < 8) || (h16 && group == 128))) return false;
+    const int KB = K / kBlockK, tiles = (tiles16 + 7) / 8, pairs = (tiles16 + 1) / 2;
     const long long blocks = (long long)tiles * KB;
     const long long least = M <= 32 ? (count > 1 && M > 24 ? 700 : 1536) : M <= 48 && count == 1 ? 1024 : 300;
-    const bool odd_row = M <= 16 && !h16 && KB < 16 && KB != 4 && KB != 8 && blocks >= 100;
+    const bool odd_row = M <= 16 && !h16 && KB >= 6 && KB < 16 && KB != 8 && blocks >= 100 && (long long)pairs * KB < 12288;
     if (blocks < least && !odd_row) return false;
     if (env_int("W2A8_STAT", 1) == 2 || env_int("W2A8_GEMV", 1) == 2) return false;
     for (const char *name : {"W2A8_STAT_C", "W2A8_CHUNKS", "W2A8_TG", "W2A8_RING", "W2A8_MT", "W2A8_CLUSTER",
@@ -785,26 +816,15 @@ bool tstream_takes(int M, int K, int group, int tiles16, int count, bool h16) {
             if (env_set(name)) return false;
     if (odd_row && gemv_preferred(M, K, group, tiles16, count)) return true;
     if (blocks < least) return false;
-    const int sms = sm_count(), spp = group == 64 ? 0 : group == 128 ? 1 : 2;
+    const int sms = sm_count(), per_sm = ts_tokens(M) <= 32 ? 2 : 1;
     int resident[kTsMaxCluster + 1] = {}, C, ncl;       // (what the device reports for a whole B200: 148, 74, 33, 15)
-    for (int c = 1; c <= kTsMaxCluster; c *= 2) resident[c] = (int)(sms / c * (c == 4 ? 0.9 : c == 8 ? 0.84 : 1.0)) * (nt <= 32 ? 2 : 1);
-    if (nt <= 32) resident[8] = resident[8] * 3 / 4;
-    static const double base[5][3] = {{1.82, 1.95, 2.59},
-                                      {3.06, 3.11, 3.56},
-                                      {3.21, 3.44, 4.14},
-                                      {3.82, 4.01, 4.58},
-                                      {4.3, 4.43, 5.26}};
-    static const double per_block[5][3] = {{0.616, 0.534, 0.453},
-                                           {0.735, 0.566, 0.474},
-                                           {0.827, 0.611, 0.486},
-                                           {0.733, 0.491, 0.404},
-                                           {0.821, 0.575, 0.427}};
-    const int w = nt == 16 ? 0 : nt == 24 ? 1 : nt == 32 ? 2 : nt == 48 ? 3 : 4;
-    const double mine = base[w][spp] + per_block[w][spp] * ts_plan(tiles, KB, resident, nt <= 32, &C, &ncl);
-    static const double per_cell[3] = {0.27e-3, 0.25e-3, 0.235e-3};
-    // (more than 32 tokens: the other kernels take one matrix per launch)
-    const double other = 4.6 * (M > 32 ? count : 1) + per_cell[spp] * (KB > 32 ? 1.1 : 1.0) * 4.0 * (double)blocks * slabs;
-    return mine < (M <= 16 && spp == 2 ? 0.86 : 0.92) * other;
+    for (int c = 1; c <= kTsMaxCluster; c *= 2) resident[c] = (int)(sms / c * (c == 4 ? 0.9 : c == 8 ? 0.84 : 1.0)) * per_sm;
+    if (per_sm == 2) resident[8] = resident[8] * 3 / 4;
+    const double mine = ts_plan(tiles, KB, resident, ts_times(M, group), &C, &ncl);
+    double other = stat_estimate(M, K, group, pairs);
+    if (other < 0) other = 4.6 + 1.0e-3 * (double)blocks * ((M + 7) / 8);
+    if (M > 32) other += 2.5 * (count - 1);
+    return mine < 0.95 * other;
 }
 
 template <int NT, int SPP, bool H16>
@@ -823,7 +843,8 @@ static cudaError_t launch_ts_inst(const TsMaps &maps, TsParams &p, cudaStream_t 
             n[c] = C::kCtasPerSm == 2 && c == 8 && found > 1 ? found * 3 / 4 : found;
         }
     });
-    if (ts_plan(p.tiles, p.KB, resident, C::kCtasPerSm == 2, &p.C, &p.nclusters) > 1e29) return cudaErrorNotSupported;
+    if (ts_plan(p.tiles, p.KB, resident, ts_times(p.M, SPP == 1 ? 64 : SPP == 2 ? 128 : 256), &p.C, &p.nclusters) > 1e29)
+        return cudaErrorNotSupported;
     p.blk_per = p.KB / p.C; p.blk_extra = p.KB % p.C;
     return launch_kernel_clusters(kernel, dim3((unsigned)(p.nclusters * p.C)), dim3(C::kThreads), C::kSmem, st, pdl_enabled(),
                                   make_uint2((unsigned)p.C, 1u), maps, p);

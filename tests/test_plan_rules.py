@@ -108,3 +108,25 @@ def test_streaming_tensor_core_kernel(monkeypatch, M, taken):
         monkeypatch.delenv(name)
     monkeypatch.setenv("W2A8_TSTREAM", "0")
     assert plan() is False
+
+
+@pytest.mark.parametrize("Ns,M,K,group,taken", [
+    ([14336, 14336], 8, 4096, 128, False),
+    ([3840], 9, 2560, 64, True),                  # short rows that the persistent kernel does not hold
+    ([3840], 16, 2560, 2560, True),
+    ([3840], 17, 2560, 64, False),
+    ([4096], 16, 2048, 64, False),                # rows that it holds
+    ([16384], 12, 1280, 64, False),               # too short for the sums
+    ([57344], 64, 1280, 128, False),
+    ([57344], 64, 1280, 1280, True),
+    ([4096], 32, 4096, 128, False),               # 512 blocks
+    ([4096], 64, 4096, 128, True),
+    ([28672], 64, 4096, 1024, False),             # four groups at 64 tokens
+    ([28672], 63, 4096, 1024, True),
+    ([28672, 28672], 64, 8192, 64, True),
+])
+def test_where_the_streaming_tensor_core_kernel_is_taken(monkeypatch, Ns, M, K, group, taken):
+    import ctypes
+    monkeypatch.delenv("W2A8_TSTREAM", raising=False)
+    plan = b.lib().w2a8_grouped_plan(len(Ns), (ctypes.c_int * len(Ns))(*Ns), M, K, group, b.FUSE_OFF)
+    assert bool(plan & 4) is taken
