@@ -423,8 +423,7 @@ def kernel_probe(device, peaks, l2_bytes, M, K, N, g, use_graph=True, seed=9000,
     us = t["mean"] / ncopy * 1e3
     plan = b.w2a8_grouped_plan([N] * count, M, K, g, b.FUSE_OFF)
     return dict(shape=f"{K}x{N}" + (f" x{count}" if count > 1 else ""), M=M, group=g, us_per_launch=us,
-                kernel="persistent, quantiser inside" if fused else "one launch for the group" if plan["one_launch"] and count > 1
-                else "persistent" if plan["one_launch"] else "one-shot", us_min=t["min"] / ncopy * 1e3,
+                kernel="persistent, quantiser inside" if fused else "one launch" if plan["one_launch"] else "one-shot", us_min=t["min"] / ncopy * 1e3,
                 us_median=t["median"] / ncopy * 1e3, bytes_per_launch=nbytes, gbs=nbytes / us / 1e3,
                 frac_of_measured_hbm=nbytes / us / 1e3 / peaks["hbm_gbs"],
                 distinct_weight_bytes=per * ncopy, weight_copies=ncopy, launch=kind,

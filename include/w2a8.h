@@ -137,8 +137,7 @@ int w2a8_workspace_status(const void *workspace, void *stream);
  * K % 256 == 0), which unpacks every weight once per 64 tokens, where its estimate
  * is ahead: larger problems of few tokens, smaller ones of many.  w2a8_kernel_for reports tensor-core or streaming.
  * From 9 to 64 tokens (K % 256 == 0) a larger problem goes to none of these but to a streaming kernel that feeds the
- * weights to the tensor cores through tensor memory, where its estimate is ahead; the report functions say what the
- * shape would get without it.
+ * weights to the tensor cores through tensor memory, where its estimate is ahead (w2a8_kernel_for: streaming).
  * A problem given to the tensor-core kernel may leave its last (at most
  * eight) 128-channel tiles to the streaming kernel, as a second launch on the
  * same stream (w2a8_tensor_core_channels); the result does not depend on it
@@ -321,9 +320,9 @@ size_t w2a8_grouped_workspace_bytes(int count, const int *N, int M, int K, int g
  *              be NULL when the call fuses (then nothing is written), and must
  *              not be NULL otherwise (W2A8_ERR_NULL)
  *   the rest as for w2a8_gemm_grouped.
- * w2a8_grouped_plan reports what a call will do: bit 0 = one launch of the
- * persistent kernel for the whole group, bit 1 = that launch also quantises,
- * bit 2 = one launch of the streaming kernel on the tensor cores in any case.
+ * w2a8_grouped_plan reports what a call will do: bit 0 = one launch for the whole
+ * group, bit 1 = that launch also quantises, bit 2 = it is the streaming kernel
+ * on the tensor cores.
  * a and a_scale are bitwise those of a8_quantize; every y is bitwise that of
  * w2a8_gemm_grouped when that call takes the persistent kernel too, and differs
  * from it by fp32 summation order only otherwise.

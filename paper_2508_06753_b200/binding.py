@@ -321,7 +321,7 @@ def w2a8_grouped_workspace_bytes(N, M: int, K: int, group: int) -> int:
 
 
 def w2a8_grouped_plan(N, M: int, K: int, group: int, fuse: int = FUSE_AUTO) -> dict:
-    """What a grouped call will do: {'one_launch': bool, 'fused': bool}."""
+    """What a grouped call will do: {'one_launch': bool (whichever kernel), 'fused': bool (quantiser inside it)}."""
     arr = (ctypes.c_int * len(N))(*[int(n) for n in N])
     r = int(lib().w2a8_grouped_plan(len(N), arr, M, K, group, fuse))
     _check(r if r < 0 else 0, "w2a8_grouped_plan")

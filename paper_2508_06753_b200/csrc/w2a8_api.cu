@@ -427,11 +427,17 @@ static bool takes_tensor_core_kernel_ex(int M, int N, int K, int group, bool can
     if (mode == 2) return true;
     return prefill_preferred(M, N, K, group, can_split);
 }
-// int8 activations: the int8 kernel can split K for problems with few output tiles, the 16-bit one cannot
-// (9 to 64 tokens: among the kernels other than the streaming one on the tensor cores, which dispatch asks first)
+// int8 activations: the int8 kernel can split K for problems with few output tiles, the 16-bit one cannot.
+// (9 to 64 tokens: among the kernels other than the streaming one on the tensor cores, which dispatch asks first; a
+// workspace serves these too, in case that one has no plan.)
 static bool takes_tensor_core_kernel(int M, int N, int K, int group) {
     return takes_tensor_core_kernel_ex(M, N, K, group, !tensor_core_kind_is_16(M, N, K, group)) &&
            !stat_takes(M, K, group, N / 16, 1, false);
+}
+
+// The kernel that a call gets, for the queries.
+static bool reports_tensor_core_kernel(int M, int N, int K, int group) {
+    return takes_tensor_core_kernel(M, N, K, group) && !tstream_takes(M, K, group, N / 16, 1, false);
 }
 
 // Channels the tensor-core kernel takes (the rest, if any, goes to the streaming kernel in a
@@ -465,9 +471,10 @@ static bool tensor_core_kind_is_16(int M, int N, int K, int group) {
 }
 
 int w2a8_tensor_core_kind(int M, int N, int K, int group) {
+    EnvScope scope;
     ShapeInfo si;
     if (!shape_ok(M, N, K, group, &si)) return W2A8_ERR_SHAPE;
-    if (!takes_tensor_core_kernel(M, N, K, group)) return 0;
+    if (!reports_tensor_core_kernel(M, N, K, group)) return 0;
     return tensor_core_kind_is_16(M, N, K, group) ? 16 : 8;
 }
 
@@ -475,27 +482,30 @@ int w2a8_kernel_for(int M, int N, int K, int group) {
     EnvScope scope;
     ShapeInfo si;
     if (!shape_ok(M, N, K, group, &si)) return W2A8_ERR_SHAPE;
-    return takes_tensor_core_kernel(M, N, K, group) ? 1 : 0;
+    return reports_tensor_core_kernel(M, N, K, group) ? 1 : 0;
 }
 
 int w2a8_tensor_core_channels(int M, int N, int K, int group) {
+    EnvScope scope;
     ShapeInfo si;
     if (!shape_ok(M, N, K, group, &si)) return W2A8_ERR_SHAPE;
-    return takes_tensor_core_kernel(M, N, K, group) ? tensor_core_channels(M, N, K, group) : 0;
+    return reports_tensor_core_kernel(M, N, K, group) ? tensor_core_channels(M, N, K, group) : 0;
 }
 
 int w2a8_tensor_core_ksplit(int M, int N, int K, int group) {
+    EnvScope scope;
     ShapeInfo si;
     if (!shape_ok(M, N, K, group, &si)) return W2A8_ERR_SHAPE;
-    if (!takes_tensor_core_kernel(M, N, K, group)) return 0;
+    if (!reports_tensor_core_kernel(M, N, K, group)) return 0;
     if (tensor_core_kind_is_16(M, N, K, group)) return 1;
     return prefill_ksplit(M, N, K, group);
 }
 
 int w2a8_tensor_core_tile_tokens(int M, int N, int K, int group) {
+    EnvScope scope;
     ShapeInfo si;
     if (!shape_ok(M, N, K, group, &si)) return W2A8_ERR_SHAPE;
-    if (!takes_tensor_core_kernel(M, N, K, group)) return 0;
+    if (!reports_tensor_core_kernel(M, N, K, group)) return 0;
     if (tensor_core_kind_is_16(M, N, K, group)) return 128;
     return prefill_uses_wide(M, N, K, group) ? 256 : 128;
 }
@@ -636,23 +646,21 @@ static inline size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 // ---- matrices that share their activations --------------------------------------------------
 constexpr int kMaxGroup = 4;
 
-// bit 0: the group runs as one launch of the persistent kernel or of the one with stationary activations; bit 1: that
-// launch quantises the activations itself; bit 2: one launch of the streaming kernel on the tensor cores instead.  fuse: W2A8_FUSE_AUTO / _OFF / _ON.  Negative: error.
-static int grouped_plan(int count, const int *N, int M, int K, int group, int fuse, bool have_x) {
+// bit 0: the group runs as one launch; bit 1: that launch quantises the activations itself (persistent kernel); bit 2: it
+// is the streaming kernel on the tensor cores (tstream: whether that one is asked).  fuse: W2A8_FUSE_AUTO / _OFF / _ON.
+// Negative: error.
+static int grouped_plan(int count, const int *N, int M, int K, int group, int fuse, bool have_x, bool tstream = true) {
     if (count < 1 || count > kMaxGroup || !N) return W2A8_ERR_SHAPE;
     int tiles = 0;
     for (int i = 0; i < count; ++i) {
         if (!shape_ok(M, N[i], K, group, nullptr)) return W2A8_ERR_SHAPE;
         tiles += N[i] / 16;
     }
-    int plan = 0;
     if (have_x && fuse != W2A8_FUSE_OFF && gemv_can_fuse(M, K, group) &&
         (fuse == W2A8_FUSE_ON || gemv_fuse_preferred(M, K, group)))
-        plan = 3;
-    else if (stat_takes(M, K, group, tiles, count, false) || gemv_preferred(M, K, group, tiles, count))
-        plan = 1;
-    if (plan != 3 && tstream_takes(M, K, group, tiles, count, false)) plan |= 4;
-    return plan;
+        return 3;
+    if (tstream && tstream_takes(M, K, group, tiles, count, false)) return 5;
+    return stat_takes(M, K, group, tiles, count, false) || gemv_preferred(M, K, group, tiles, count) ? 1 : 0;
 }
 
 size_t w2a8_grouped_workspace_bytes(int count, const int *N, int M, int K, int group) {
@@ -677,7 +685,7 @@ static int grouped_common(const void *x_bf16, const int8_t *a_in, const float *a
                           void *stream) {
     EnvScope scope;
     if (!packed || !w_scale || !y || !N) return W2A8_ERR_NULL;
-    const int plan = grouped_plan(count, N, M, K, group, fuse, x_bf16 != nullptr);
+    int plan = grouped_plan(count, N, M, K, group, fuse, x_bf16 != nullptr);
     if (plan < 0) return plan;
     for (int i = 0; i < count; ++i) {
         if (!packed[i] || !w_scale[i] || !y[i]) return W2A8_ERR_NULL;
@@ -702,13 +710,14 @@ static int grouped_common(const void *x_bf16, const int8_t *a_in, const float *a
     }
     int tiles = 0;
     for (int i = 0; i < count; ++i) tiles += N[i] / 16;
-    bool gemv = plan & 1;
-    if (plan & 4) {
+    if (plan == 5) {
         const int st = launch_tstream(a_in, a_scale_in, count, packed, reinterpret_cast<const void *const *>(w_scale),
                                       reinterpret_cast<void *const *>(y), N, N, M, K, group, workspace, (cudaStream_t)stream, false, false);
         if (st != kStatNoPlan) return st;
+        plan = grouped_plan(count, N, M, K, group, W2A8_FUSE_OFF, false, false);
     }
-    if ((plan & 1) && stat_takes(M, K, group, tiles, count, false)) {
+    bool gemv = plan == 1;
+    if (plan == 1 && stat_takes(M, K, group, tiles, count, false)) {
         const int st = launch_stat(a_in, a_scale_in, count, packed, reinterpret_cast<const void *const *>(w_scale),
                                    reinterpret_cast<void *const *>(y), N, N, M, K, group, (cudaStream_t)stream, false, false);
         if (st != kStatNoPlan) return st;

@@ -156,6 +156,8 @@ def test_grouped_plan_needs_no_gpu(lib, monkeypatch):
     assert b.w2a8_grouped_plan(qkv, 4, 4096, 64, b.FUSE_ON) == {"one_launch": True, "fused": True}
     assert b.w2a8_grouped_plan(qkv, 16, 4096, 64, b.FUSE_ON)["fused"] is False                     # too many tokens
     assert b.w2a8_grouped_plan([48, 32], 3, 1600, 64) == {"one_launch": False, "fused": False}     # ragged K
+    assert b.w2a8_grouped_plan(qkv, 64, 4096, 64) == {"one_launch": True, "fused": False}          # tensor memory
+    monkeypatch.setenv("W2A8_TSTREAM", "0")
     assert b.w2a8_grouped_plan(qkv, 64, 4096, 64) == {"one_launch": False, "fused": False}
     monkeypatch.setenv("W2A8_GEMV", "0")
     assert b.w2a8_grouped_plan(qkv, 1, 4096, 64) == {"one_launch": False, "fused": False}

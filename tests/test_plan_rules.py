@@ -86,9 +86,10 @@ def test_workspace_covers_the_channel_remainder_of_bf16_activations(monkeypatch)
     (8192, 8192, 64, "streaming"),
     (5120, 14336, 128, "streaming"),
 ])
-def test_64_tokens(N, K, group, kernel):
-    """The fewest tokens of the tensor-core kernel, which is ahead there with large groups only, and not by a K
-    split whose scratch w2a8_gemm_static does not have."""
+def test_64_tokens(monkeypatch, N, K, group, kernel):
+    """The fewest tokens of the tensor-core kernel, which is ahead there with large groups only (of the kernels other
+    than the streaming one on the tensor cores), and not by a K split whose scratch w2a8_gemm_static does not have."""
+    monkeypatch.setenv("W2A8_TSTREAM", "0")
     assert b.w2a8_kernel_for(64, N, K, group) == kernel
     if (N, K) == (5120, 14336):
         assert b.w2a8_workspace_bytes(64, N, K, group) <= 8 << 20
@@ -130,3 +131,20 @@ def test_where_the_streaming_tensor_core_kernel_is_taken(monkeypatch, Ns, M, K, 
     monkeypatch.delenv("W2A8_TSTREAM", raising=False)
     plan = b.lib().w2a8_grouped_plan(len(Ns), (ctypes.c_int * len(Ns))(*Ns), M, K, group, b.FUSE_OFF)
     assert bool(plan & 4) is taken
+
+
+@pytest.mark.parametrize("M", [32, 48, 64])
+def test_reports_say_what_runs(monkeypatch, M):
+    """Two matrices that the streaming kernel on the tensor cores takes: one launch, and no tensor-core kernel with its
+    splits and tiles; without it a launch per matrix above 32 tokens, on the tensor-core kernel at 64."""
+    plan = lambda: b.w2a8_grouped_plan([28672, 28672], M, 8192, 8192, b.FUSE_OFF)
+    reports = lambda: (b.w2a8_kernel_for(M, 28672, 8192, 8192), b.w2a8_tensor_core_kind(M, 28672, 8192, 8192),
+                       b.w2a8_tensor_core_channels(M, 28672, 8192, 8192) > 0, b.w2a8_tensor_core_ksplit(M, 28672, 8192, 8192) > 0,
+                       b.w2a8_tensor_core_tile_tokens(M, 28672, 8192, 8192) > 0)
+    monkeypatch.delenv("W2A8_TSTREAM", raising=False)
+    assert plan() == {"one_launch": True, "fused": False}
+    assert reports() == ("streaming", 0, False, False, False)
+    monkeypatch.setenv("W2A8_TSTREAM", "0")
+    assert plan()["one_launch"] is (M == 32)
+    assert reports() == (("tensor_core", 8, True, True, True) if M == 64 else ("streaming", 0, False, False, False))
+
