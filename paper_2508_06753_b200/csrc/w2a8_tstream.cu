@@ -12,19 +12,21 @@
 //    eight warps drain the accumulators (lane = channel, column = token): a conversion and half a packed FMA per value.
 //  * Up to 32 tokens a CTA has 12 warps, 112 KB and 256 columns of tensor memory, so that two are resident per SM and one
 //    computes while the other waits or, under programmatic dependent launch, while the previous kernel ends; with 64
-//    tokens one CTA of 20 warps has them all.  Registers are dealt by setmaxnreg so that hardly anything spills (28 bytes
-//    at most, in instances for 64 tokens; a few
-//    words per block, local memory beside the copies, made 8192 x (28672 + 28672) at 32 tokens 94 us instead of 54).
-//  * Sums.  Chains of eight groups by FMA; a chain joins the running sum with what that addition rounds away going into
+//    tokens one CTA of 20 warps has them all.  Registers are dealt by setmaxnreg so that hardly anything spills (16 bytes
+//    at most, in two instances for 64 tokens; a few words per block, local memory beside the copies, made
+//    8192 x (28672 + 28672) at 32 tokens 94 us instead of 54).
+//  * Sums.  Chains of eight or six groups by FMA; a chain joins the running sum with what that addition rounds away going into
 //    the next chain, and the ranks' shares are added in the same way: the error does not depend on the length of a row.
 //    Distance from sums in 64 bits, one running total / this: 4096 x (14336 + 14336) at 64 tokens, groups of 64, one share
 //    9.5e-8 / 4.6e-8; 28672 x 8192, groups of 64, four shares 7.5e-8 / 4.0e-8; 8192 x 8192, groups of 128, four shares
 //    5.5e-8 / 4.6e-8.  The other kernels are at 5.1e-8 and more at these sizes.
-//  * Bound (8192 x (28672 + 28672), groups of 128, 32 tokens): issue slots: per block of 8 KB unpack, drain (a conversion and
-//    half a packed FMA per value and group), and waits and bookkeeping.  On the kernel with stationary activations
-//    (mma.sync) the same launch takes 58 us.  Not kept: conversion through the bits of 1.5 * 2^23, by integer adds (50 us
-//    against 44); eight drain warps at 32 tokens (45); unpack warps with 64 registers (4 to 19 % more per launch); blocks dealt
-//    evenly over CTAs with cut tiles summed through global memory (3 us more per small launch).
+//  * Bound (8192 x (28672 + 28672), groups of 128, 32 tokens, 44 us, 3.0 TB/s): issue slots, 59 % busy: 2000 warp instructions
+//    per block of 8 KB, of which unpack and drain (a conversion and half a packed FMA per value and group) are a good half
+//    and waits and bookkeeping the rest.  On the kernel with stationary activations (mma.sync) the same launch takes 58 us.
+//    Not kept: conversion through the bits of 1.5 * 2^23, by integer adds (50 us); eight drain warps at 32 tokens (45);
+//    unpack warps with 64 registers (4 to 19 % more per launch); blocks dealt evenly over CTAs with cut tiles summed through
+//    global memory (3 us more per small launch); one running total, or pairs of groups added first, which are 4 to 6 % faster
+//    at 64 tokens and groups of 64 or 128, and too far off (above).
 //  * A wait is one barrier per warp: lanes of a warp that polled different barriers saw phases that had not completed.
 //  * Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
 #include <cuda.h>
@@ -189,16 +191,15 @@ __device__ __forceinline__ void ts_send(uint32_t addr, uint32_t bar, int rank, c
 }
 template <int N>
 __device__ __forceinline__ void ts_ld_shared(float (&v)[N], uint32_t addr) {
-    constexpr int P = N % 4 == 0 ? 4 : N % 2 == 0 ? 2 : 1;
+    constexpr int P = N % 4 == 0 ? 4 : 2;
+    static_assert(N % P == 0, "");
 #pragma unroll
     for (int j = 0; j < N; j += P) {
         if constexpr (P == 4)
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[j]), "=f"(v[j + 1]), "=f"(v[j + 2]), "=f"(v[j + 3])
                          : "r"(addr + j * 4) : "memory");
-        else if constexpr (P == 2)
-            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[j]), "=f"(v[j + 1]) : "r"(addr + j * 4) : "memory");
         else
-            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[j]) : "r"(addr + j * 4) : "memory");
+            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[j]), "=f"(v[j + 1]) : "r"(addr + j * 4) : "memory");
     }
 }
 // pf_wait for data that other CTAs of the cluster wrote
@@ -831,9 +832,12 @@ template <int NT, int SPP, bool H16>
 static cudaError_t launch_ts_inst(const TsMaps &maps, TsParams &p, cudaStream_t st) {
     using C = TsCfg<NT, SPP>;
     auto kernel = w2a8_tstream_kernel<NT, SPP, H16>;
-    static PerDeviceFlags configured;   // per kernel instantiation
+    static PerDeviceFlags configured, carved;   // per kernel instantiation
     if (cudaError_t e = allow_dynamic_smem(kernel, configured, (int)C::kSmem)) return e;
-    if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) return e;
+    if (!carved.done[current_device()].load(std::memory_order_acquire)) {
+        if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) return e;
+        carved.done[current_device()].store(true, std::memory_order_release);
+    }
     // Clusters of C CTAs that are resident at once.  The query answers for one CTA per SM; with 256 columns of tensor
     // memory, 112 KB and half of the registers two are resident (clusters of eight: about three quarters of that).
     static PerDeviceTable<kTsMaxCluster + 1> clusters;

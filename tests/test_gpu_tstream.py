@@ -8,8 +8,8 @@ from conftest import Guarded
 from paper_2508_06753_b200 import synth
 
 pytestmark = pytest.mark.gpu
-# y is a sum of K / group <= 448 fp32 terms from exact integer sums: about sqrt(448) * 2^-24 of its row's largest
-# value, 1e-6; the other kernels are held to the same 1e-4
+# y is a sum of K / group <= 512 fp32 terms from exact integer sums, 1e-6 of its row's largest value; the other kernels are
+# held to the same 1e-4, and test_error_does_not_grow_with_the_row holds the sums to their bound
 TOL = 1e-4
 
 
@@ -38,7 +38,7 @@ CASES = [
     (17, 1792, [640, 32], 64, 4),              # shares of 2 and 1 blocks
     (32, 1536, [384], 512, 4),                 # groups of two blocks cut between shares of 2, 2, 1, 1
     (31, 768, [128 * 150], 64, 1),             # more tiles than SMs
-    (20, 2048, [256], 128, 8),                 # three columns per rank and thread
+    (20, 2048, [256], 128, 8),                 # parts of four of 24 columns: two ranks have none
     (24, 1024, [128 * 170], 128, 2),           # two tiles for some clusters: both exchange buffers
     (12, 512, [128 * 310], 64, 1),             # a second round
     (33, 2048, [1024], 64, 8),
@@ -138,9 +138,10 @@ def test_default_dispatch_in_a_replayed_graph(gpu, monkeypatch, M, K, N):
     a2, s2 = b.a8_quantize(x)
     plain = b.w2a8_gemm(a2, s2, packed, scale, 128, ws)
     assert torch.equal(got, plain)
+    import ctypes
+    assert b.lib().w2a8_grouped_plan(1, (ctypes.c_int * 1)(N), M, K, 128, b.FUSE_OFF) & 4
     monkeypatch.setenv("W2A8_TSTREAM", "0")
     other = b.w2a8_gemm(a2, s2, packed, scale, 128, b.new_workspace(b.w2a8_workspace_bytes(M, N, K, 128)))
-    assert not torch.equal(other, plain)              # another kernel, another order of the additions
     assert (other - plain).abs().max() <= 1e-5 * plain.abs().max()
 
 
@@ -270,3 +271,37 @@ def test_a_wait_that_gives_up(gpu, monkeypatch, M, shares, group):
     ws.zero_()
     assert torch.equal(b.w2a8_gemm(a, s, packed, scale, group, ws), whole)
     assert b.w2a8_workspace_status(ws) == 0
+
+
+@pytest.mark.parametrize("M,K,Ns,group,h16", [
+    (12, 2560, [3840], 64, False),                 # short rows, 9 to 16 tokens
+    (16, 3072, [1984], 3072, False),
+    (32, 8192, [8192], 128, True),                 # binary16 scales
+    (24, 8192, [8192], 8192, True),
+    (48, 4096, [4096, 1024, 1024], 64, False),     # matrices that share their activations
+    (32, 8192, [8192, 1024, 1024], 8192, False),
+    (63, 14336, [4096], 1024, False),
+])
+def test_by_the_rule(gpu, monkeypatch, M, K, Ns, group, h16):
+    """Launches that come here by the rule: the bits of the forced kernel, which plans alike."""
+    torch, b = gpu
+    gen = torch.Generator(device="cuda").manual_seed(K + M)
+    packed = [b.w2_pack(torch.randint(0, 4, (N, K), generator=gen, device="cuda", dtype=torch.uint8)) for N in Ns]
+    scales = [torch.rand((N, K // group), generator=gen, device="cuda") + 0.01 for N in Ns]
+    if h16:
+        scales = [s.half() for s in scales]
+    a, s_a = b.a8_quantize(torch.randn((M, K), generator=gen, device="cuda").to(torch.bfloat16))
+    ws = b.new_workspace(b.w2a8_grouped_workspace_bytes(Ns, M, K, group))
+    run = lambda: ([b.w2a8_gemm_h16(a, s_a, packed[0], scales[0], group, ws)] if h16 else
+                   [y.clone() for y in b.w2a8_gemm_grouped(a, s_a, b.Group(packed, scales), group, ws)])
+    ys = {}
+    for mode in (None, "2", "0"):
+        if mode is None:
+            monkeypatch.delenv("W2A8_TSTREAM", raising=False)
+        else:
+            monkeypatch.setenv("W2A8_TSTREAM", mode)
+        ys[mode] = run()
+        assert b.w2a8_workspace_status(ws) == 0
+    for rule, forced, other in zip(ys[None], ys["2"], ys["0"]):
+        assert torch.equal(rule, forced)
+        assert (rule - other).abs().max() <= 1e-5 * other.abs().max()
